@@ -74,6 +74,11 @@ enum { APFC_LATTICE_CUSTOM = 0, APFC_LATTICE_HEX2D = 1, APFC_LATTICE_BCC3D = 2 }
 
 enum { APFC_FP64 = 0,         /* fields, Krylov iterates and reductions in FP64 */
        APFC_FP32_REFINED = 1  /* FP32 Krylov inside FP64 iterative refinement   */ };
+/* The only value.  Systems with constant coefficients on 2D grids (no Jacobian, fused 1,
+ * cheb_degree 1..4) are solved to the same tolerance by a Chebyshev iteration on the Schur
+ * complement of the block system, a_j + kap_j Bx G_h^2 (preconditioned by Eq. preconditioner's
+ * second factor squared where that pays, on fine grids); the others by BiCGStab, as is a system
+ * whose Chebyshev iteration could need more operator applications than max_iter allows. */
 enum { APFC_BICGSTAB = 0 };
 enum { APFC_TAU_FOLD = 0,     /* preconditioner uses 1/tau = 1/dt + kap dB      */
        APFC_TAU_PLAIN = 1     /* preconditioner uses tau = dt                    */ };
@@ -97,28 +102,29 @@ typedef struct {
 typedef struct {
   int precision;             /* APFC_FP64 or APFC_FP32_REFINED                     */
   int krylov;                /* APFC_BICGSTAB                                       */
-  int max_iter;              /* cap on Krylov iterations per solve (per refinement) */
+  int max_iter;              /* cap on iterations per solve (per refinement); an iteration
+                                applies the operator twice                          */
   int cheb_degree;           /* applications of D per diffusion solve in P^{-1}, 0..16 */
   int tau_mode;              /* APFC_TAU_FOLD or APFC_TAU_PLAIN                     */
   int max_refine;            /* cap on FP64 refinement sweeps (FP32_REFINED)        */
-  int check_every;           /* Krylov iterations between convergence checks        */
+  int check_every;           /* BiCGStab iterations between convergence checks      */
   int fused;                 /* 1: fused row-streaming A P^{-1} kernels on 2D grids (default);
                                 0: one kernel per stencil pass                         */
   double tol;                /* stop at ||b - A x||_2 <= tol ||b||_2 (block norm, per amplitude) */
   double tol_inner;          /* relative tolerance of each FP32 inner solve         */
   int tile;                  /* fused 2D kernel variant 0..5 (columns per block and
                                 rows of look-ahead), default 3                     */
-  int tile_rows;             /* rows per block of the fused 2D kernels of the Krylov
-                                iteration; 0 (default): the tallest of 128, 64, 32
-                                rows that gives the first fused kernel's launch
-                                >= 1.5 blocks per SM (x += P^{-1} u always takes
-                                that automatic height)                             */
+  int tile_rows;             /* rows per block of the fused 2D kernels of the
+                                iteration; 0 (default): automatic, by the grid size
+                                (BiCGStab: the tallest of 128, 64, 32 rows that
+                                gives the first fused kernel's launch >= 1.5 blocks
+                                per SM; x += P^{-1} u always takes that height)    */
   int picard_iters;          /* K of Alg. 1: Picard iterations per step, 1..100;
                                 1 (default) with jacobian 0 is the explicit step   */
   int jacobian;              /* 1: linearise N_j with D_j = dN_j/d eta_j (the
                                 paper's J^j, h^j) in every Picard iteration        */
   int tile_t;                /* variant 0..5 of the fused kernel t = A P^{-1} s of
-                                the merged iteration (-1: same as tile), default 1 */
+                                BiCGStab (-1: same as tile), default 1             */
   int guess;                 /* initial guess of each explicit step's solve:
                                 APFC_GUESS_PREV (the previous state, Alg. 1) or
                                 APFC_GUESS_EXTRAP (2 x^n - x^(n-1), after a
@@ -128,8 +134,9 @@ enum { APFC_GUESS_PREV = 0, APFC_GUESS_EXTRAP = 1 };
 
 typedef struct {
   long long steps;           /* steps taken since apfc_set_amplitudes             */
-  long long iters_total;     /* Krylov iterations summed over steps (of each solve,
-                                the iterations of its slowest amplitude)           */
+  long long iters_total;     /* iterations (two operator applications each) summed
+                                over steps (of each solve, those of its slowest
+                                amplitude)                                         */
   int iters_last;            /* max over amplitudes of iterations in the last step */
   int refine_last;           /* refinement sweeps in the last step (FP32_REFINED)  */
   double resid_last;         /* max over amplitudes of ||b-Ax||/||b|| after the last step */
@@ -173,7 +180,7 @@ apfc_status apfc_get_zeta(apfc_ctx* ctx, void* zeta, int where);
 
 /* Advance n steps of size dt (Alg. 1).  Default (picard_iters 1, jacobian 0):
  * one nonlinear iterate, explicit nonlinear right-hand side from eta^n for all
- * amplitudes, then one preconditioned Krylov solve per amplitude from the
+ * amplitudes, then one iterative solve per amplitude (see APFC_BICGSTAB) from the
  * initial guess (zeta^n, eta^n).  With picard_iters K > 1 or jacobian 1: K
  * iterations k, each solving per amplitude (all amplitudes reading eta^(k-1))
  *   [ I, -G_h ; kap Bx G_h, (1/dt + kap dB) I + kap D_j ] (zeta, eta)
@@ -187,9 +194,11 @@ apfc_status apfc_step(apfc_ctx* ctx, double dt, int n);
 /* Choose the rows per segment of the fused 2D kernels (opts.tile_rows) and the
  * variant of the merged iteration's t-kernel (opts.tile_t) by timing: from the
  * current state, one step of size dt per candidate, each from the same state,
- * after one untimed step; first the automatic height, 32, 48 and 64 rows and every
- * height ceil(ny / s) between 96 and 256 rows (t-kernel variant as set), then every
- * t-kernel variant at the best height.  Keeps the fastest in the context's options.  The state and the
+ * after one untimed step; first the automatic height, BiCGStab's automatic height, 32, 48 and
+ * 64 rows and every height ceil(ny / s) between 96 and 256 rows (t-kernel variant as set),
+ * then, where the solve is BiCGStab, every t-kernel variant at the best height.  Keeps the
+ * fastest in the context's options (opts.tile_rows stays 0 where the automatic height is;
+ * *tile_rows is then BiCGStab's automatic height).  The state and the
  * statistics are restored (the next step takes a stencil initial residual).  Only
  * the FP32-refined fused path on 2D grids has a choice to make: other
  * configurations return APFC_OK with their options unchanged and ms_per_step 0.
@@ -375,22 +384,21 @@ apfc_status apfc_rotation_field(apfc_ctx* ctx, void* omega, void* amp, void* hma
 /* ---- batched independent runs ----------------------------------------------
  * Many independent 2D simulations of one lattice, one parameter set and one
  * spacing (hx, hy) on periodic grids of different sizes nx[r] x ny[r], advanced
- * together by the step of apfc_step (Alg. 1 with one nonlinear iterate; the
- * Sec. II.B preconditioner inside BiCGStab) in precision APFC_FP32_REFINED with
- * the fused pipeline.  Every stage of the step is one launch over the work of
- * all runs; each (run, amplitude) keeps its own Krylov scalars and stops on its
- * own, and a run whose refinement has converged waits unchanged for the
+ * together by the step of apfc_step (Alg. 1 with one nonlinear iterate; Chebyshev
+ * solves of the Schur complement) in precision APFC_FP32_REFINED with the fused
+ * pipeline.  Every stage of the step is one launch over the work of
+ * all runs; each (run, amplitude) takes its own number of iterations, and a run whose refinement has converged waits unchanged for the
  * others.  Run r follows the same arithmetic as run r alone on an apfc_ctx
- * with the same options (the same per-run reductions in the same order).
+ * with the same options (its solves do not depend on the split into tiles, and its
+ * norms are reduced in the same order).
  *
  * Storage: the batch owns the concatenated block vectors of all runs (FP64
- * state, right-hand sides and residuals; FP32 Krylov vectors), about
- * 2 J sum_r(nx ny) x (4 x 16 + 10 x 8) bytes.  Amplitude buffers of run r are
+ * state, right-hand sides and residuals; FP32 solver fields), about
+ * J sum_r(nx ny) x (7 x 16 + 5 x 8) bytes.  Amplitude buffers of run r are
  * [J][ny[r]][nx[r]] complex128, owned by the caller, copied in or out.
  *
- * flags: APFC_BATCH_GRAPH replays the Krylov iteration blocks (check_every
- * merged iterations) from captured CUDA graphs; the first block of each solve
- * runs uncaptured.  With that flag a NULL stream makes the batch create and own
+ * flags: APFC_BATCH_GRAPH replays the passes of a solve from captured CUDA
+ * graphs (one per number of passes); the first solve runs uncaptured.  With that flag a NULL stream makes the batch create and own
  * a non-blocking stream (graphs cannot be captured on the legacy stream).
  * Errors are sticky as on a context; ENAN / ENOCONV name the failing run in
  * apfc_batch_last_error(). */
@@ -422,13 +430,11 @@ apfc_status apfc_batch_energy(apfc_batch* b, int run, double* F);
 apfc_status apfc_batch_stats(const apfc_batch* b, int run, apfc_stats_t* out);
 
 /* Tile autotuner: from the first refinement residual of a step of the current
- * state (the state itself is not changed), time a fixed number of merged
- * BiCGStab iterations over all runs, first for every tile variant (0..5) and
- * segment height (32, 48, 64, 96, 128, 192, 256 rows) shared by both fused
- * kernels, then for every variant of the t-kernel alone with the rest fixed;
- * keep the fastest in the
- * batch's options (tile, tile_rows, tile_t; see apfc_batch_get_opts) and return
- * tile, rows and ms per iteration (null pointers skipped). */
+ * state (the amplitudes are not changed), time a fixed number of Chebyshev
+ * passes over all runs for the narrow and the wide strips (tile 3 and 5) and every
+ * segment height (32, 48, 64, 96, 128, 192, 256 rows); keep the fastest in the
+ * batch's options (tile, tile_rows; see apfc_batch_get_opts) and return tile, rows
+ * and ms per pass (null pointers skipped). */
 apfc_status apfc_batch_autotune(apfc_batch* b, double dt, int* tile, int* tile_rows, double* ms_per_iter);
 
 /* Number of captured-graph replays since creation (-1 for a null batch). */

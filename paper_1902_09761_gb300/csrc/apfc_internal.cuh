@@ -10,6 +10,7 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
 
 #include "apfc.h"
@@ -133,30 +134,19 @@ __device__ __forceinline__ void prof_add(const OpCoef& c, int kid, unsigned long
 }
 
 // Batched runs: every run's block vectors sit one after another in shared
-// arrays; elem_off is the run's first element (of [J][2][pts]), part_off its
-// first 16-byte partial-sum slot.
+// arrays; elem_off is the run's first element (of [J][2][pts]).
 struct RunGeom {
   int nx, ny;
   long long pts, elem_off;
-  long long part_off, part_off_t;  // first partial-sum slot: v-kernel layout, t-kernel layout
-  int npart, npart_t;              // partial-sum slots per amplitude in each layout
+  long long field_off;             // the run's first element in a [run][J][pts] field (even)
+  long long part_off_r;            // residual kernel: first partial sum, partials, rows per segment
+  int npart_r, rows_r;
 };
 struct BatchLaunch {
   const RunGeom* dev;   // device copy of the run table (per-point kernels, reductions)
   const RunGeom* host;  // host copy (the fused kernels carry it in their parameters)
   int R;
-  int tlay;  // 1: partial sums in the t-kernel layout (its own tile variant)
 };
-
-// Point a kernel's grid sizes at run `run`; returns the run's first element.
-__device__ __forceinline__ long long select_run(const RunGeom* rg, int run, OpCoef& c) {
-  const RunGeom& q = rg[run];
-  c.nx = q.nx;
-  c.ny = q.ny;
-  c.nz = 1;
-  c.pts = q.pts;
-  return q.elem_off;
-}
 
 // Chebyshev recurrence weights for one application (per amplitude):
 // d_{k+1} = c1 d_k + c2 r_{k+1}.
@@ -203,6 +193,45 @@ struct KScal {
 
 enum KStatus { KS_RUNNING = 0, KS_CONVERGED = 1, KS_NOCONV = 2, KS_BREAKDOWN = 3, KS_NAN = 4 };
 enum KOp { OP_INIT = 0, OP_ALPHA = 1, OP_SNORM = 2, OP_OMEGA = 3, OP_RHO = 4, OP_NORMS = 5, OP_OMEGA3 = 6, OP_RNORM = 7, OP_BNORM = 8, OP_OMEGA5 = 9, OP_INIT3 = 10 };
+
+// Weights of one pass of the Chebyshev iteration on the Schur complement (cheb2d.cuh): per
+// amplitude, iteration i of the pass takes d = c1 d + c2 p^2 r; the first pass of a solve
+// starts with d_0 = p^2 r / theta.
+struct ChebPass {
+  double c1[2][kMaxJ], c2[2][kMaxJ];
+  double inv_theta[kMaxJ];
+};
+// The same for the iteration on S itself (gauge2d.cuh): term i of the pass is
+// v_(n+1) = v_n + c1 (v_n - v_(n-1)) + c2 (b - S v_n), v_1 = b / theta.
+constexpr int kGaugeMaxNI = 6;
+struct GaugeWeights {
+  double c1[kGaugeMaxNI][kMaxJ], c2[kGaugeMaxNI][kMaxJ];
+  double inv_theta[kMaxJ];
+};
+// e^{i phi_d i} per amplitude, [J][tx + ty (+ tz)]: dimension d's entries 0 .. n_d
+template <typename T>
+struct GaugeTab {
+  const cplx<T>* tab;
+  int tx, ty, tz;
+};
+// weight of the shifts in dimension d: sqrt(1 + (k_d h_d)^2) / h_d^2 (kh = k_d / h_d, ih2 = 1 / h_d^2)
+inline double gauge_w(const OpCoef& c, int j, int d) {
+  return std::sqrt(c.ih2[d] * c.ih2[d] + c.kh[j][d] * c.kh[j][d]);
+}
+inline double gauge_phi(const OpCoef& c, int j, int d) { return std::atan2(c.kh[j][d], c.ih2[d]); }
+
+// Fields [J][pts] of such a solve: r0 the initial residual, r and d ping-pong pairs (r0 may be
+// r[0]), u the sum of the d; x64 the state block that receives u; ks[j].iters the passes of
+// amplitude j (0: none).
+template <typename T>
+struct ChebBufs {
+  const cplx<T>* r0;
+  cplx<T>* r[2];
+  cplx<T>* d[2];
+  cplx<T>* u;
+  double2* x64;
+  const KScal* ks;
+};
 
 // Up to three (u, v) pairs of block vectors for conj(u).v per amplitude.
 template <typename T>
@@ -291,11 +320,6 @@ void launch_extrapolate(double2* x, double2* xp, const OpCoef& c, cudaStream_t s
 // complex64 [J][pts] <-> part (0 zeta, 1 eta) of the FP64 state block, rounding to nearest
 void launch_c64_to_part(const float2* src, double2* x, long long pts, int J, int part, cudaStream_t s);
 void launch_part_to_c64(const double2* x, float2* dst, long long pts, int J, int part, cudaStream_t s);
-void launch_residual_refine(const double2* b, const double2* x, float2* r32, double* partials, const OpCoef& c,
-                            cudaStream_t s);
-// 2D only: FP64 residual with FP32 (and optional FP64) output
-void launch_residual_refine2d(const double2* b, const double2* x, float2* r32, double2* r64, double* partials,
-                              const OpCoef& c, cudaStream_t s, const BatchLaunch* bl = nullptr);
 // One 2D or 3D grid: the residual with its tiles staged by TMA and the partial ||r||^2
 // per amplitude (resid2d.cu); false, with *err set, if the tensor maps cannot be built
 // (nothing is launched then)
@@ -308,11 +332,12 @@ unsigned long long stream3d_timeouts();
 // Start of an FP32 solve from x0 = 0: r = b, rhat = b rounded to bf16 with its packed copy
 // rh16 [J][pts] (bf16pair.cuh), partials of (r, r), (b, b), (rhat, r) in slots 0-2 (k_dots' layout)
 void launch_init32(const float2* b, float2* r, float2* rhat, uint2* rh16, void* partials, const OpCoef& c,
-                   cudaStream_t s, const BatchLaunch* bl = nullptr);
+                   cudaStream_t s);
 // new RHS and initial residual r0 = b - b_prev + r_prev (pointwise); b_prev = r_prev = null:
-// the RHS and the ||b||^2 partials only (the ||r0||^2 slot holds 0, r32 is not written)
+// the RHS and the ||b||^2 partials only (the ||r0||^2 slot holds 0, r32 is not written).
+// schur: r_prev and r32 are [J][pts] fields (the Schur complement's residual), else block vectors
 void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const double2* r_prev, float2* r32,
-                      double* partials, const OpCoef& c, const NonlinTable& nt, cudaStream_t s,
+                      double* partials, const OpCoef& c, const NonlinTable& nt, bool schur, cudaStream_t s,
                       const BatchLaunch* bl = nullptr);
 void launch_energy(const double2* x, double* partials, double* out, const OpCoef& c, const EnergyTable& et,
                    double Bx, cudaStream_t s);
@@ -350,19 +375,10 @@ void launch_energy_grad(const double2* x, double2* grad, double scale, double dB
 int fused2d_max_degree(int elem_bytes);
 int fused2d_npart(const OpCoef& c, int m, int Ly, int elem_bytes, int tile);  // elem_bytes = sizeof(complex)
 int fused2d_tiles();  // number of tile variants
-// p_new = r + beta (p_old - omega v_old); v_new = A P^{-1} p_new; partial (rhat, v_new)
-template <typename T>
-bool launch_fused_v(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* p_old,
-                    const cplx<T>* v_old, cplx<T>* p_new, cplx<T>* v_new, const cplx<T>* rhat, const uint2* rh16,
-                    const KScal* act, void* partials, cudaStream_t s);
-// t = A P^{-1} (r - alpha v); partials (t, s), (t, t), (s, s)
-template <typename T>
-bool launch_fused_t(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
-                    cplx<T>* t_out, const KScal* act, void* partials, cudaStream_t s);
 // x64 += P^{-1} u
 template <typename T>
 bool launch_fused_pinv_add(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* u, double2* x64,
-                           cudaStream_t s, const BatchLaunch* bl = nullptr);
+                           cudaStream_t s);
 // blocks of one fused launch over an nx x ny grid (J amplitudes); *npart = blocks per amplitude
 int fused2d_blocks(int nx, int ny, int J, int m, int Ly, int elem_bytes, int tile, bool with_a, int* npart);
 // x = P^{-1} b
@@ -376,38 +392,90 @@ template <typename T>
 bool launch_fused_merged_v(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
                            const cplx<T>* t, const cplx<T>* p, cplx<T>* u, cplx<T>* r_new, cplx<T>* p_new,
                            cplx<T>* v_new, const cplx<T>* rhat, const uint2* rh16, const KScal* act, void* partials,
-                           cudaStream_t s, const BatchLaunch* bl = nullptr);
+                           cudaStream_t s);
 // t = A P^{-1} s, s = r - alpha v; partials (t, s), (t, t), (s, s), (rhat, s), (rhat, t)
 template <typename T>
 bool launch_fused_merged_t(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
-                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s,
-                           const BatchLaunch* bl = nullptr);
+                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s);
 // the pending u += alpha p + omega (r - alpha v) of amplitudes that stopped in this iteration
 template <typename T>
 void launch_final_update(const cplx<T>* r, const cplx<T>* v, const cplx<T>* p, cplx<T>* u, const KScal* ks,
-                         const OpCoef& c, cudaStream_t s, const BatchLaunch* bl = nullptr);
-// s = r - alpha v; u += alpha p + omega s; r = s - omega t; partials (rhat, r), (r, r) in [J][kDotSlots][kDotBlocks]
+                         const OpCoef& c, cudaStream_t s);
+// ---------------------------------------------------------------------------
+// cheb2d_f32.cu, cheb2d_f64.cu: passes of the Chebyshev iteration on the Schur complement (2D
+// grids, degree m in 1..4 of p).  schur.cu: its spectrum, weights, outer residual and plan.
+// ---------------------------------------------------------------------------
+struct SchurCoef {
+  bool plain;                       // the iteration on S itself (gauge2d.cuh), else on S p(D)^2 (cheb2d.cuh)
+  double lmin[kMaxJ], lmax[kMaxJ];  // bounds of its spectrum
+  double lnrate[kMaxJ];             // acosh(sigma): each term shrinks the residual by about exp(-lnrate)
+};
+// L passes make schur_t0 + L schur_ni terms of the solve's polynomial
+constexpr int kGaugeNI32 = 3, kGaugeNI64 = 1;
 template <typename T>
-void launch_bicg_update(cplx<T>* r, const cplx<T>* v, const cplx<T>* p, cplx<T>* u, const cplx<T>* t,
-                        const cplx<T>* rhat, const KScal* ks, void* partials, const OpCoef& c, cudaStream_t s);
+int schur_ni(const SchurCoef& s, int m) {
+  if (s.plain) return sizeof(T) == 4 ? kGaugeNI32 : kGaugeNI64;
+  return sizeof(T) == 4 && m == 1 ? 2 : 1;
+}
+template <typename T>
+int schur_t0(const SchurCoef& s, int m) {
+  return s.plain ? 1 : 2 - schur_ni<T>(s, m);
+}
+bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s);
+ChebPass schur_pass(const SchurCoef& s, int J, int pass, int ni);
+GaugeWeights gauge_weights(const SchurCoef& s, int J, int pass, int ni);
+int schur_terms(double tin, double lnrate);  // terms that reduce the residual by tin
+// rows per segment of the passes over grids nx[i] x ny[i] stepped together (automatic height)
+int schur_auto_rows(const SchurCoef& sc, const int* nx, const int* ny, int n, int J, int m, int elem_bytes, int tile,
+                    int sms);
+template <typename T>
+bool launch_cheb2d(int m, const OpCoef& c, const ChebStep* w, const ChebPass& cp, int Ly, const ChebBufs<T>& b,
+                   int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
+template <typename T>
+bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Ly,
+                    const ChebBufs<T>& b, int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
+// tab[j][d][i] = e^{i phi_d i}, 0 <= i <= n_d (sizes of GaugeTab)
+template <typename T>
+void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s);
+// pass `pass` of a solve, by either iteration
+template <typename T>
+bool launch_schur_pass(const SchurCoef& sc, int m, int tile, const OpCoef& c, const ChebStep* w,
+                       const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int pass, cudaStream_t s,
+                       const BatchLaunch* bl = nullptr) {
+  const int ni = schur_ni<T>(sc, m);
+  return sc.plain ? launch_gauge2d<T>(tile, c, gt, gauge_weights(sc, c.J, pass, ni), Ly, b, pass, s, bl)
+                  : launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, pass, ni), Ly, b, pass, s, bl);
+}
+// r = b - (a + kt G^2) eta from the eta-parts of x, b; zeta = G eta written into x; r [J][pts] in
+// T, r64 (nullable) the same in FP64; part [J][2][schur_resid_parts] sums of ||r||^2, ||b||^2
+template <typename T>
+void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
+                          bool want_b, cudaStream_t s, const BatchLaunch* bl = nullptr);
+int schur_resid_rows(int nx, int ny, int J);
+int schur_resid_parts(int nx, int ny, int J);
+// ks[j].rnorm2 / bnorm2 from partial sums and ks[j].iters, the passes of the next solve
+struct SchurPlan {
+  const double* part;
+  int npart, elem;                   // partials per slot, doubles between two of them
+  long long slot_stride, amp_stride; // in doubles
+  int by_run;                        // batched: the residual kernel's layout of each run
+  int have;                          // 1: slot 0 holds ||r||^2, 2: slot 1 holds ||b||^2
+  double tol, tol_inner;
+  double lnrate[kMaxJ];
+  int t0, ni, max_pass, fp64, J;      // L passes make t0 + ni L terms
+};
+void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl = nullptr);
 
 // ---------------------------------------------------------------------------
 // reduce.cu
 // ---------------------------------------------------------------------------
-// bl != nullptr: one launch over every run of a batch (partials of run r from slot r J kDotSlots kDotBlocks)
 template <typename T>
 void launch_dots(int npair, const DotPairs<T>& pr, void* partials, const OpCoef& c, const KScal* act,
-                 cudaStream_t s, const BatchLaunch* bl = nullptr);
+                 cudaStream_t s);
 // npart: partial-sum slots per (amplitude, pair); layout [J][kDotSlots][npart].
 template <typename T>
 void launch_finalize(int npair, const void* partials, KScal* k, int op, int J, cudaStream_t s,
                      int npart = kDotBlocks);
 // partials in FP64 double2 layout regardless of T (for the fused FP64 residual)
 void launch_finalize64(int npair, const void* partials, KScal* k, int op, int J, cudaStream_t s);
-// batched runs: Krylov scalars k[run J + j]; npart_fixed > 0 for the k_dots layout
-// (kDotBlocks), 0 for the fused-pipeline layout (RunGeom part_off, npart)
-template <typename T>
-void launch_finalize_batch(int npair, const void* partials, int npart_fixed, const BatchLaunch& bl, int J, KScal* k,
-                           int op, cudaStream_t s);
-
 }  // namespace apfc

@@ -32,6 +32,15 @@ struct Work {
   bool ready = false;
 };
 
+// Fields [J][pts] of the Chebyshev iteration on the Schur complement (cheb2d.cuh).
+template <typename T>
+struct SchurWork {
+  cplx<T>* r[2] = {};
+  cplx<T>* d[2] = {};
+  cplx<T>* u = nullptr;
+  cplx<T>* tab = nullptr;  // phases of the gauge (gauge2d.cuh), of the lattice and the grid alone
+};
+
 }  // namespace
 
 // Process-wide measurement state (see apfc_profile_start in apfc.h).
@@ -188,6 +197,13 @@ struct apfc_ctx {
   KScal* ks64 = nullptr;       // refinement norms (device)
   KScal* ks64_host = nullptr;  // pinned
   void* part64 = nullptr;      // refinement partials
+  SchurWork<double> s64;
+  SchurWork<float> s32;
+  double* rpart = nullptr;     // partial sums of the Schur-complement residual
+  SchurCoef schur{};           // of the current coefficients
+  bool schur_ok = false;       // they allow the Chebyshev iteration (2D, degree 1..4)
+  bool prev_schur = false;     // r64_prev holds that path's residual field
+  double resid = 0.0;          // max over amplitudes of ||r|| / ||b|| after the last solve
   bool has_state = false;
   bool failed = false;
   std::string err;
@@ -385,6 +401,9 @@ bool build_coef(apfc_ctx* c, double dt, std::string& err) {
   if (c->coef_dt == dt) return true;
   if (!make_coef(c->lat, c->par, c->grid, c->opts.tau_mode, dt, c->coef, err)) return false;
   c->coef_dt = dt;
+  const int m = c->opts.cheb_degree;
+  c->schur_ok = c->dim == 2 && m >= 1 && m <= fused2d_max_degree((int)sizeof(float2)) &&
+                schur_build(c->coef, c->grid, m, c->schur);
   return true;
 }
 
@@ -746,6 +765,152 @@ apfc_status status_of(apfc_ctx* ctx, int worst) {
   return APFC_OK;
 }
 
+// Whether the solve runs as the Chebyshev iteration on the Schur complement: constant
+// coefficients (no Jacobian) on a 2D grid with the fused pipeline, and no more operator
+// applications than max_iter BiCGStab iterations (two each) may take.
+bool use_schur(const apfc_ctx* ctx) {
+  if (!ctx->schur_ok || ctx->opts.fused == 0 || ctx->coef.jd != nullptr) return false;
+  const double tin = ctx->opts.precision == APFC_FP64 ? 0.9 * ctx->opts.tol : ctx->opts.tol_inner;
+  for (int j = 0; j < ctx->J; ++j)
+    if (schur_terms(tin, ctx->schur.lnrate[j]) > 2LL * ctx->opts.max_iter) return false;
+  return true;
+}
+
+template <typename T>
+apfc_status alloc_schur(apfc_ctx* ctx, SchurWork<T>& w) {
+  if (w.u) return APFC_OK;
+  for (auto& p : w.r)
+    if (!p) CK(cudaMalloc(&p, field_bytes<T>(ctx)));
+  for (auto& p : w.d)
+    if (!p) CK(cudaMalloc(&p, field_bytes<T>(ctx)));
+  if (!ctx->rpart)
+    CK(cudaMalloc(&ctx->rpart,
+                  2 * sizeof(double) * ctx->J * (size_t)schur_resid_parts(ctx->grid.n[0], ctx->grid.n[1], ctx->J)));
+  const int tx = ctx->grid.n[0] + 1, ty = ctx->grid.n[1] + 1;
+  if (!w.tab) CK(cudaMalloc(&w.tab, sizeof(cplx<T>) * ctx->J * (size_t)(tx + ty)));
+  launch_gauge_table<T>(w.tab, ctx->coef, tx, ty, 0, ctx->stream);
+  CK(cudaGetLastError());
+  CK(cudaMalloc(&w.u, field_bytes<T>(ctx)));
+  return APFC_OK;
+}
+template <typename T>
+void free_schur(SchurWork<T>& w) {
+  for (auto& p : w.r) cudaFree(p), p = nullptr;
+  for (auto& p : w.d) cudaFree(p), p = nullptr;
+  cudaFree(w.u);
+  cudaFree(w.tab);
+  w.u = w.tab = nullptr;
+}
+
+// A x = b by Chebyshev solves of the Schur complement between outer residuals, from x's eta
+// part; zeta = G_h eta comes with every residual.  FP32 passes inside FP64-accurate refinement
+// (at most max_refine solves), or FP64 passes (at most four, restarted from the residual).
+// resid_ready: the FP32 residual field and the partial sums of ||r0||^2 and ||b||^2 come from
+// the right-hand-side kernel; bnorm_ready: its ||b||^2 does.
+template <typename T>
+apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double2* x, double2* r64_keep,
+                        bool resid_ready, bool bnorm_ready, int* total_it, int* sweeps, int* worst_out,
+                        bool* stencil_last) {
+  apfc_status st = alloc_schur<T>(ctx, w);
+  if (st != APFC_OK) return st;
+  constexpr bool fp64 = sizeof(T) == 8;
+  cudaStream_t s = ctx->stream;
+  const apfc_opts& o = ctx->opts;
+  const int m = o.cheb_degree, ni = schur_ni<T>(ctx->schur, m), nt0 = schur_t0<T>(ctx->schur, m), J = ctx->J;
+  const int most = fp64 ? 4 : o.max_refine;
+  const auto cw = cheb_weights(ctx);
+  const int rows = o.tile_rows > 0 ? o.tile_rows
+                                   : schur_auto_rows(ctx->schur, &ctx->grid.n[0], &ctx->grid.n[1], 1, J, m,
+                                                     (int)sizeof(cplx<T>), o.tile, ctx->sms);
+  SchurPlan plan{};
+  plan.tol = o.tol;
+  plan.tol_inner = o.tol_inner;
+  for (int j = 0; j < J; ++j) plan.lnrate[j] = ctx->schur.lnrate[j];
+  plan.t0 = nt0;
+  plan.ni = ni;
+  plan.max_pass = (int)std::min<long long>(1 << 30, std::max(1LL, (2LL * o.max_iter - nt0 + ni - 1) / ni));
+  plan.fp64 = fp64;
+  plan.J = J;
+  // the right-hand-side kernel's partial sums: (value, 0) pairs [J][kDotSlots][kDotBlocks]
+  SchurPlan prhs = plan;
+  prhs.part = reinterpret_cast<const double*>(ctx->part64);
+  prhs.npart = kDotBlocks;
+  prhs.elem = 2;
+  prhs.slot_stride = 2 * kDotBlocks;
+  prhs.amp_stride = 2 * kDotSlots * kDotBlocks;
+  // the residual kernel's: [J][2][npart]
+  plan.part = ctx->rpart;
+  plan.npart = schur_resid_parts(ctx->grid.n[0], ctx->grid.n[1], J);
+  plan.elem = 1;
+  plan.slot_stride = plan.npart;
+  plan.amp_stride = 2LL * plan.npart;
+  const GaugeTab<T> gt{w.tab, ctx->grid.n[0] + 1, ctx->grid.n[1] + 1, 0};
+  const ChebBufs<T> bufs{w.r[0], {w.r[0], w.r[1]}, {w.d[0], w.d[1]}, w.u, x, ctx->ks64};
+  int total = 0, worst = KS_CONVERGED, sweep = 0;
+  const double tol2 = o.tol * o.tol;
+  for (;; ++sweep) {
+    if (resid_ready) {
+      prhs.have = 3;
+      launch_schur_plan(prhs, ctx->ks64, s);
+    } else {
+      const bool want_b = sweep == 0 && !bnorm_ready;
+      if (sweep == 0 && bnorm_ready) {
+        prhs.have = 2;
+        launch_schur_plan(prhs, ctx->ks64, s);
+      }
+      launch_resid_schur2d<T>(b, x, w.r[0], r64_keep, ctx->rpart, ctx->coef, want_b, s);
+      plan.have = want_b ? 3 : 1;
+      launch_schur_plan(plan, ctx->ks64, s);
+    }
+    *stencil_last = !resid_ready;
+    resid_ready = false;
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(ctx->ks64_host, ctx->ks64, sizeof(KScal) * J, cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
+    bool done = true, bad = false;
+    int np = 0;
+    for (int j = 0; j < J; ++j) {
+      const KScal& k = ctx->ks64_host[j];
+      if (!std::isfinite(k.rnorm2) || !std::isfinite(k.bnorm2)) bad = true;
+      if (k.rnorm2 > tol2 * k.bnorm2) done = false;
+      np = std::max(np, k.iters);
+    }
+    if (bad) {
+      worst = KS_NAN;
+      break;
+    }
+    if (done) break;
+    if (sweep >= most) {
+      worst = KS_NOCONV;
+      break;
+    }
+    for (int p = 0; p < np; ++p)
+      if (!launch_schur_pass<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, p, s))
+        return fail(ctx, APFC_ECUDA, "the Chebyshev pass cannot be launched");
+    if (np > 0) total += (nt0 + ni * np + 1) / 2;  // two applications, as in a BiCGStab iteration
+  }
+  CK(cudaGetLastError());
+  *total_it = total;
+  *sweeps = sweep;
+  *worst_out = worst;
+  ctx->resid = max_rel_resid(ctx->ks64_host, J);
+  return APFC_OK;
+}
+
+// A x = b in FP64 from x.
+apfc_status solve_fp64(apfc_ctx* ctx, const double2* b, double2* x, int* iters, int* worst) {
+  if (use_schur(ctx)) {
+    int sweeps = 0;
+    bool stencil = false;
+    return schur_solve<double>(ctx, ctx->s64, b, x, nullptr, false, false, iters, &sweeps, worst, &stencil);
+  }
+  apfc_status st = alloc_work<double>(ctx, ctx->w64);
+  if (st != APFC_OK) return st;
+  st = krylov<double>(ctx, ctx->w64, b, x, ctx->opts.tol, ctx->opts.max_iter, iters, worst);
+  if (st == APFC_OK) ctx->resid = max_rel_resid(ctx->w64.ks_host, ctx->J);
+  return st;
+}
+
 // One step in FP64.
 // APFC_GUESS_EXTRAP, after the right-hand side has been formed from the state: replace the
 // state by the extrapolated guess 2 x^n - x^(n-1) (keeping x^n) when the history is that of
@@ -778,19 +943,17 @@ void guess_done(apfc_ctx* ctx, int worst) {
 
 apfc_status step_fp64(apfc_ctx* ctx) {
   ctx->have_prev = false;
-  apfc_status st = alloc_work<double>(ctx, ctx->w64);
-  if (st != APFC_OK) return st;
+  apfc_status st;
   launch_rhs(ctx->x64, ctx->b64, ctx->coef, ctx->nt, ctx->stream);
   bool ex = false;
   if ((st = guess_prepare(ctx, &ex)) != APFC_OK) return st;
   int iters = 0, worst = 0;
-  st = krylov<double>(ctx, ctx->w64, ctx->b64, ctx->x64, ctx->opts.tol, ctx->opts.max_iter, &iters, &worst);
-  if (st != APFC_OK) return st;
+  if ((st = solve_fp64(ctx, ctx->b64, ctx->x64, &iters, &worst)) != APFC_OK) return st;
   guess_done(ctx, worst);
   ctx->stats.iters_last = iters;
   ctx->stats.iters_total += iters;
   ctx->stats.refine_last = 0;
-  ctx->stats.resid_last = max_rel_resid(ctx->w64.ks_host, ctx->J);
+  ctx->stats.resid_last = ctx->resid;
   return status_of(ctx, worst);
 }
 
@@ -802,6 +965,9 @@ apfc_status step_fp64(apfc_ctx* ctx) {
 // bnorm_ready: the partial sums hold ||b||^2 (slot 1) from the right-hand-side kernel
 apfc_status refine_solve(apfc_ctx* ctx, const double2* b, double2* x, double2* r64_keep, bool resid_ready,
                          int* total_it, int* sweeps, int* worst_out, bool* stencil_last, bool bnorm_ready = false) {
+  if (use_schur(ctx))
+    return schur_solve<float>(ctx, ctx->s32, b, x, r64_keep, resid_ready, bnorm_ready, total_it, sweeps, worst_out,
+                              stencil_last);
   apfc_status st = alloc_work<float>(ctx, ctx->w32);
   if (st != APFC_OK) return st;
   cudaStream_t s = ctx->stream;
@@ -871,6 +1037,7 @@ apfc_status refine_solve(apfc_ctx* ctx, const double2* b, double2* x, double2* r
   *sweeps = sweep;
   *worst_out = worst;
   *stencil_last = stencil;
+  ctx->resid = max_rel_resid(ctx->ks64_host, ctx->J);
   return APFC_OK;
 }
 
@@ -884,20 +1051,21 @@ apfc_status step_refined(apfc_ctx* ctx) {
     CK(cudaMemsetAsync(ctx->b64_prev, 0, blk, s));
     ctx->have_prev = false;
   }
-  apfc_status st = alloc_work<float>(ctx, ctx->w32);
+  const bool schur = use_schur(ctx);
+  apfc_status st = schur ? alloc_schur<float>(ctx, ctx->s32) : alloc_work<float>(ctx, ctx->w32);
   if (st != APFC_OK) return st;
-  float2* r32 = ctx->w32.blk[7];
+  float2* r32 = schur ? ctx->s32.r[0] : ctx->w32.blk[7];
   double* part = reinterpret_cast<double*>(ctx->part64);
   bool resid_ready = false, bnorm_ready = false;
-  if (ctx->have_prev && ctx->prev_dt == ctx->coef_dt) {
+  if (ctx->have_prev && ctx->prev_dt == ctx->coef_dt && ctx->prev_schur == schur) {
     // r0 = b - b_prev + r_prev with the previous step's final residual r_prev = b_prev - A x;
     // b_prev is the RHS that residual was taken against; the new RHS goes to the other buffer
-    launch_rhs_resid(ctx->x64, ctx->b64_prev, ctx->b64, ctx->r64_prev, r32, part, ctx->coef, ctx->nt, s);
+    launch_rhs_resid(ctx->x64, ctx->b64_prev, ctx->b64, ctx->r64_prev, r32, part, ctx->coef, ctx->nt, schur, s);
     std::swap(ctx->b64, ctx->b64_prev);
     resid_ready = true;
   } else {
     // no previous residual: the new RHS and its norm, the initial residual by stencil below
-    launch_rhs_resid(ctx->x64, ctx->b64, nullptr, nullptr, r32, part, ctx->coef, ctx->nt, s);
+    launch_rhs_resid(ctx->x64, ctx->b64, nullptr, nullptr, r32, part, ctx->coef, ctx->nt, schur, s);
     bnorm_ready = true;
   }
   ctx->have_prev = false;
@@ -916,17 +1084,19 @@ apfc_status step_refined(apfc_ctx* ctx) {
   if (st != APFC_OK) return st;
   guess_done(ctx, worst);
   // a TMA wait that gave up leaves its kernel's results incomplete: fail the step
-  if (tma_timeouts() != 0) return fail(ctx, APFC_ECUDA, "a TMA tile load did not complete within its wait limit");
+  if (!schur && tma_timeouts() != 0)
+    return fail(ctx, APFC_ECUDA, "a TMA tile load did not complete within its wait limit");
   if (worst == KS_CONVERGED) {
     // after at least one sweep the last check was a stencil residual of the final
     // state, kept in r64_prev: it seeds the next step's initial residual
     ctx->have_prev = sweeps > 0 && stencil_last;
     ctx->prev_dt = ctx->coef_dt;
+    ctx->prev_schur = schur;
   }
   ctx->stats.iters_last = total_it;
   ctx->stats.iters_total += total_it;
   ctx->stats.refine_last = sweeps;
-  ctx->stats.resid_last = max_rel_resid(ctx->ks64_host, ctx->J);
+  ctx->stats.resid_last = ctx->resid;
   return status_of(ctx, worst);
 }
 
@@ -1037,8 +1207,7 @@ apfc_status solve_block(apfc_ctx* ctx, const double2* b, double2* x, int* iters)
   int worst = KS_CONVERGED;
   apfc_status st;
   if (ctx->opts.precision == APFC_FP64) {
-    if ((st = alloc_work<double>(ctx, ctx->w64)) != APFC_OK) return st;
-    st = krylov<double>(ctx, ctx->w64, b, x, ctx->opts.tol, ctx->opts.max_iter, iters, &worst);
+    st = solve_fp64(ctx, b, x, iters, &worst);
   } else {
     int sweeps = 0;
     bool stencil = false;
@@ -1125,7 +1294,7 @@ apfc_status step_picard(apfc_ctx* ctx) {
   ctx->stats.iters_last = total;
   ctx->stats.iters_total += total;
   ctx->stats.refine_last = ctx->opts.picard_iters;
-  ctx->stats.resid_last = max_rel_resid(ctx->opts.precision == APFC_FP64 ? ctx->w64.ks_host : ctx->ks64_host, ctx->J);
+  ctx->stats.resid_last = ctx->resid;
   return APFC_OK;
 }
 
@@ -1382,6 +1551,8 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
   const int saved_rows = ctx->opts.tile_rows, saved_tt = ctx->opts.tile_t;
   std::vector<int> cand;
   ctx->opts.tile_rows = 0;
+  const bool schur = use_schur(ctx);  // its automatic height is a candidate of its own, kept as 0
+  if (schur) cand.push_back(0);
   cand.push_back(fused_rows(ctx));
   for (int rows : {32, 48, 64})
     if (rows < ny && std::find(cand.begin(), cand.end(), rows) == cand.end()) cand.push_back(rows);
@@ -1413,7 +1584,8 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
     st = fail(ctx, APFC_ECUDA, "autotune: copy or event creation failed");
   // pass 1: the heights with the t-kernel variant as set; pass 2: every t-kernel variant at
   // the best height
-  const int nrows = (int)cand.size(), ntt = fused2d_tiles();
+  // (the Chebyshev passes have no t-kernel)
+  const int nrows = (int)cand.size(), ntt = schur ? 0 : fused2d_tiles();
   for (int i = -1; i < nrows + ntt && st == APFC_OK; ++i) {  // i = -1: untimed warm-up
     if (i >= nrows && i - nrows == (saved_tt < 0 ? ctx->opts.tile : saved_tt)) continue;  // timed in pass 1
     ctx->opts.tile_rows = i < nrows ? cand[i < 0 ? 0 : i] : best_rows;
@@ -1441,7 +1613,7 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
   ctx->opts.tile_rows = st == APFC_OK ? best_rows : saved_rows;
   ctx->opts.tile_t = st == APFC_OK ? best_tt : saved_tt;
   if (st != APFC_OK) return st;
-  if (tile_rows) *tile_rows = best_rows;
+  if (tile_rows) *tile_rows = fused_rows(ctx);
   if (tile_t) *tile_t = best_tt;
   if (ms_per_step) *ms_per_step = best;
   return APFC_OK;
@@ -1487,6 +1659,9 @@ void apfc_destroy(apfc_ctx* ctx) {
   cudaFree(ctx->part64);
   free_work(ctx->w64);
   free_work(ctx->w32);
+  free_schur(ctx->s64);
+  free_schur(ctx->s32);
+  cudaFree(ctx->rpart);
   cudaFree(ctx->xadj);
   cudaFree(ctx->badj);
   cudaFree(ctx->eblk);

@@ -508,119 +508,6 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   }
 }
 
-// FP64 outer residual of the refinement: r = b - A x (x, b FP64), written as FP32;
-// partials: ||r||^2 and ||b||^2 per amplitude (double2 layout [J][2][kDotBlocks]).
-__global__ void k_residual_refine(const double2* __restrict__ b, const double2* __restrict__ x, float2* __restrict__ r32,
-                                  double2* __restrict__ partials, OpCoef c) {
-  const int j = blockIdx.y;
-  prof_add(c, KID_RESID_REFINE, (unsigned long long)c.pts * (4 * sizeof(double2) + 2 * sizeof(float2)));
-  const long long o = 2LL * j * c.pts;
-  const double2* z = x + o;
-  const double2* e = z + c.pts;
-  const double kt = c.kt[j], a = c.a[j];
-  double acc[2] = {0.0, 0.0};
-  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < c.pts;
-       p += (long long)gridDim.x * blockDim.x) {
-    const Nb n = neighbours(p, c);
-    const double2 gz = opG<double>(z, n, c, j), ge = opG<double>(e, n, c, j);
-    const double2 zc = z[p], ec = e[p];
-    const double2 b1 = b[o + p], b2 = b[o + c.pts + p];
-    const double r1x = b1.x - (zc.x - ge.x), r1y = b1.y - (zc.y - ge.y);
-    const double ap = c.jd == nullptr ? a : a_at(c, j, p);
-    const double r2x = b2.x - (kt * gz.x + ap * ec.x), r2y = b2.y - (kt * gz.y + ap * ec.y);
-    r32[o + p] = make_float2((float)r1x, (float)r1y);
-    r32[o + c.pts + p] = make_float2((float)r2x, (float)r2y);
-    acc[0] += r1x * r1x + r1y * r1y + r2x * r2x + r2y * r2y;
-    acc[1] += b1.x * b1.x + b1.y * b1.y + b2.x * b2.x + b2.y * b2.y;
-  }
-  block_sum<2>(acc);
-  if (threadIdx.x == 0) {
-    partials[(j * kDotSlots + 0) * kDotBlocks + blockIdx.x] = make_double2(acc[0], 0.0);
-    partials[(j * kDotSlots + 1) * kDotBlocks + blockIdx.x] = make_double2(acc[1], 0.0);
-  }
-}
-
-// FP64-accurate outer residual on 2D grids, r = b - A x with x, b FP64 in memory,
-// evaluated without the FP64 pipe: every input double is split into an FP32 pair
-// (h, l) by integer operations and each component of r1 = b1 - zeta + G_h eta and
-// r2 = b2 - kt G_h zeta - a eta is one compensated sum of products (dfloat.cuh);
-// residuals to about 1e-14 of the terms' size, beneath the 1e-10 and 1e-13
-// tolerances of the refinement.  Writes r as FP32 (the inner solve's right-hand
-// side) and, if r64 != nullptr, as FP64 (kept as the previous residual of the
-// next step).  32 x 8 point tiles whose (zeta, eta) values and one-point halo are
-// split once into shared memory.  The partial ||r||^2 per amplitude is
-// accumulated from the FP32-rounded residual (it only decides convergence,
-// where a relative error of 1e-5 in the norm is immaterial); ||b||^2 is not
-// recomputed: b is fixed within a step.
-constexpr int kRTX = 32, kRTY = 8;
-__global__ void __launch_bounds__(256, 3) k_residual_refine2d(const double2* __restrict__ b,
-                                                           const double2* __restrict__ x, float2* __restrict__ r32,
-                                                           double2* __restrict__ r64, double2* __restrict__ partials,
-                                                           const __grid_constant__ OpCoef c, const RunGeom* rg) {
-  const int j = blockIdx.y;
-  int nx = c.nx, ny = c.ny;
-  long long pts = c.pts;
-  if (rg != nullptr) {  // batched runs: blockIdx.z selects the run (the Jacobian is never on here)
-    const RunGeom& q = rg[blockIdx.z];
-    nx = q.nx;
-    ny = q.ny;
-    pts = q.pts;
-    b += q.elem_off;
-    x += q.elem_off;
-    r32 += q.elem_off;
-    if (r64 != nullptr) r64 += q.elem_off;
-    partials += (long long)blockIdx.z * c.J * kDotSlots * kDotBlocks;
-  }
-  if (c.prof != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
-    atomicAdd(c.prof + KID_RESID_REFINE, (unsigned long long)pts * (4 * sizeof(double2) + 2 * sizeof(float2) +
-                                                                   (r64 ? 2 * sizeof(double2) : 0)));
-  __shared__ float4 sz[kRTY + 2][kRTX + 2], se[kRTY + 2][kRTX + 2];
-  const long long o = 2LL * j * pts;
-  const double2* z = x + o;
-  const double2* e = z + pts;
-  const ResidCoef<2> q = resid_coef<2>(c, j);
-  LaneC ma = lane_c(c.a[j], -1.f, -1.f);
-  const int tx_count = (nx + kRTX - 1) / kRTX, ntiles = tx_count * ((ny + kRTY - 1) / kRTY);
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  float rr = 0.f;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int tyi = tile / tx_count;
-    const int x0 = (tile - tyi * tx_count) * kRTX, y0 = tyi * kRTY;
-    __syncthreads();  // the previous tile's shared values are no longer read
-    for (int i = threadIdx.x; i < (kRTX + 2) * (kRTY + 2); i += 256) {
-      const int ry = i / (kRTX + 2), rx = i - ry * (kRTX + 2);
-      int gxx = x0 - 1 + rx, gyy = y0 - 1 + ry;
-      gxx = gxx < 0 ? gxx + nx : (gxx >= nx ? gxx % nx : gxx);
-      gyy = gyy < 0 ? gyy + ny : (gyy >= ny ? gyy % ny : gyy);
-      const long long q = (long long)gyy * nx + gxx;
-      sz[ry][rx] = pdf_pack(pdf_split(z[q]));
-      se[ry][rx] = pdf_pack(pdf_split(e[q]));
-    }
-    __syncthreads();
-    const int xx = x0 + tx, yy = y0 + ty;
-    if (xx >= nx || yy >= ny) continue;
-    const long long pc = (long long)yy * nx + xx;
-    const PDF zn[2][2] = {{pdf_unpack(sz[ty + 1][tx]), pdf_unpack(sz[ty + 1][tx + 2])},
-                          {pdf_unpack(sz[ty][tx + 1]), pdf_unpack(sz[ty + 2][tx + 1])}};
-    const PDF en[2][2] = {{pdf_unpack(se[ty + 1][tx]), pdf_unpack(se[ty + 1][tx + 2])},
-                          {pdf_unpack(se[ty][tx + 1]), pdf_unpack(se[ty + 2][tx + 1])}};
-    if (c.jd != nullptr) ma = lane_c(a_at(c, j, pc), -1.f, -1.f);
-    float2 f1, l1, f2, l2;
-    resid_point<2>(q, ma, pdf_split(b[o + pc]), pdf_split(b[o + pts + pc]), pdf_unpack(sz[ty + 1][tx + 1]),
-                   pdf_unpack(se[ty + 1][tx + 1]), zn, en, f1, l1, f2, l2);
-    r32[o + pc] = f1;
-    r32[o + pts + pc] = f2;
-    if (r64 != nullptr) {
-      r64[o + pc] = make_double2(df_to_d(DF{f1.x, l1.x}), df_to_d(DF{f1.y, l1.y}));
-      r64[o + pts + pc] = make_double2(df_to_d(DF{f2.x, l2.x}), df_to_d(DF{f2.y, l2.y}));
-    }
-    rr = fmaf(f1.x, f1.x, fmaf(f1.y, f1.y, fmaf(f2.x, f2.x, fmaf(f2.y, f2.y, rr))));
-  }
-  double acc[1] = {(double)rr};
-  block_sum<1>(acc);
-  if (threadIdx.x == 0) partials[(j * kDotSlots + 0) * kDotBlocks + blockIdx.x] = make_double2(acc[0], 0.0);
-}
-
 // New right-hand side plus the initial outer residual of the step without a
 // stencil: with the previous step's final residual r_prev = b_prev - A x0,
 // r0 = b - A x0 = b - b_prev + r_prev (exact algebra, pointwise).  Writes b
@@ -637,22 +524,25 @@ __global__ void __launch_bounds__(kRhsThreads, 2) k_rhs_resid_hex(const double2*
                                                        const double2* __restrict__ b_prev,
                                                        const double2* __restrict__ r_prev, float2* __restrict__ r32,
                                                        double2* __restrict__ partials, const __grid_constant__ OpCoef c,
-                                                       const __grid_constant__ NonlinTable nt, const RunGeom* rg) {
+                                                       const __grid_constant__ NonlinTable nt, int schur,
+                                                       const RunGeom* rg) {
   long long pts = c.pts;
   if (rg != nullptr) {  // batched runs: blockIdx.y selects the run
     const RunGeom& q = rg[blockIdx.y];
+    const long long ro = schur ? q.field_off : q.elem_off;
     pts = q.pts;
     x += q.elem_off;
     b += q.elem_off;
     if (b_prev != nullptr) {  // null: no previous step (kept null, not offset)
       b_prev += q.elem_off;
-      r_prev += q.elem_off;
+      r_prev += ro;
     }
-    r32 += q.elem_off;
+    r32 += ro;
     partials += (long long)blockIdx.y * 3 * kDotSlots * kDotBlocks;
   }
   if (c.prof != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
-    atomicAdd(c.prof + KID_RHS, 3ull * pts * (b_prev ? 5 * sizeof(double2) + 2 * sizeof(float2) : 2 * sizeof(double2)));
+    atomicAdd(c.prof + KID_RHS, 3ull * pts * (b_prev ? (schur ? 4 : 5) * sizeof(double2) + (schur ? 1 : 2) * sizeof(float2)
+                                                      : 2 * sizeof(double2)));
   const DF v3 = split_d(3.0 * nt.v), t2 = split_d(2.0 * nt.t), idt = split_d(c.inv_dt);
   DF kap[3];
 #pragma unroll
@@ -680,6 +570,15 @@ __global__ void __launch_bounds__(kRhsThreads, 2) k_rhs_resid_hex(const double2*
       const long long q1 = 2LL * j * pts + p, q2 = q1 + pts;
       b[q2] = cdf_to_d(bn);
       if (b_prev != nullptr) {  // without a previous step: b and ||b||^2 only (r0 by stencil)
+        if (schur) {  // the Schur complement's residual: one field
+          const long long qf = (long long)j * pts + p;
+          const CDF rs = cdf_add(cdf_sub(bn, cdf_split(b_prev[q2])), cdf_split(r_prev[qf]));
+          const float2 fs = make_float2(rs.x.h, rs.y.h);
+          r32[qf] = fs;
+          accf[2 * j] = fmaf(fs.x, fs.x, fmaf(fs.y, fs.y, accf[2 * j]));
+          accf[2 * j + 1] = fmaf(bn.x.h, bn.x.h, fmaf(bn.y.h, bn.y.h, accf[2 * j + 1]));
+          continue;
+        }
         const CDF r2 = cdf_add(cdf_sub(bn, cdf_split(b_prev[q2])), cdf_split(r_prev[q2]));
         const DF p1x = split_d(r_prev[q1].x), p1y = split_d(r_prev[q1].y);
         const float2 f1 = make_float2(__fadd_rn(p1x.h, p1x.l), __fadd_rn(p1y.h, p1y.l));
@@ -720,24 +619,27 @@ __global__ void __launch_bounds__(256) k_rhs_resid_tab(const double2* __restrict
                                                        const double2* __restrict__ b_prev,
                                                        const double2* __restrict__ r_prev, float2* __restrict__ r32,
                                                        double2* __restrict__ partials, const __grid_constant__ OpCoef c,
-                                                       const __grid_constant__ NonlinTable nt, const RunGeom* rg) {
+                                                       const __grid_constant__ NonlinTable nt, int schur,
+                                                       const RunGeom* rg) {
   long long pts = c.pts;
   if (rg != nullptr) {  // batched runs: blockIdx.y selects the run
     const RunGeom& q = rg[blockIdx.y];
+    const long long ro = schur ? q.field_off : q.elem_off;
     pts = q.pts;
     x += q.elem_off;
     b += q.elem_off;
     if (b_prev != nullptr) {  // null: no previous step (kept null, not offset)
       b_prev += q.elem_off;
-      r_prev += q.elem_off;
+      r_prev += ro;
     }
-    r32 += q.elem_off;
+    r32 += ro;
     partials += (long long)blockIdx.y * c.J * kDotSlots * kDotBlocks;
   }
   const int J = c.J, t = threadIdx.x;
   if (c.prof != nullptr && blockIdx.x == 0 && t == 0)
     atomicAdd(c.prof + KID_RHS, (unsigned long long)J * pts *
-                                    (b_prev ? 5 * sizeof(double2) + 2 * sizeof(float2) : 2 * sizeof(double2)));
+                                    (b_prev ? (schur ? 4 : 5) * sizeof(double2) + (schur ? 1 : 2) * sizeof(float2)
+                                            : 2 * sizeof(double2)));
   __shared__ float4 se4[kMaxJ][kThreads];  // split amplitudes of each thread's point (re h, re l, im h, im l)
   __shared__ float2 sn2[kMaxJ][kThreads];  // |eta_m|^2 as (h, l)
   __shared__ float2 swd[kMaxJ][kMaxJ];
@@ -793,6 +695,15 @@ __global__ void __launch_bounds__(256) k_rhs_resid_tab(const double2* __restrict
       const long long q1 = 2LL * j * pts + p, q2 = q1 + pts;
       b[q2] = cdf_to_d(bn);
       if (b_prev != nullptr) {  // without a previous step: b and ||b||^2 only (r0 by stencil)
+        if (schur) {  // the Schur complement's residual: one field
+          const long long qf = (long long)j * pts + p;
+          const CDF rs = cdf_add(cdf_sub(bn, cdf_split(b_prev[q2])), cdf_split(r_prev[qf]));
+          const float2 fs = make_float2(rs.x.h, rs.y.h);
+          r32[qf] = fs;
+          accf[2 * j] = fmaf(fs.x, fs.x, fmaf(fs.y, fs.y, accf[2 * j]));
+          accf[2 * j + 1] = fmaf(bn.x.h, bn.x.h, fmaf(bn.y.h, bn.y.h, accf[2 * j + 1]));
+          continue;
+        }
         const CDF r2 = cdf_add(cdf_sub(bn, cdf_split(b_prev[q2])), cdf_split(r_prev[q2]));
         const DF p1x = split_d(r_prev[q1].x), p1y = split_d(r_prev[q1].y);
         const float2 f1 = make_float2(__fadd_rn(p1x.h, p1x.l), __fadd_rn(p1y.h, p1y.l));
@@ -1307,28 +1218,17 @@ void launch_zeta(double2* x, const OpCoef& c, cudaStream_t s) {
   ProfScope ps_(KID_ZETA, s);
   k_zeta<2><<<grid_pts3(c), kThreads, 0, s>>>(x, c);
 }
-void launch_residual_refine(const double2* b, const double2* x, float2* r32, double* partials, const OpCoef& c,
-                            cudaStream_t s) {
-  ProfScope ps_(KID_RESID_REFINE, s);
-  k_residual_refine<<<dim3(kDotBlocks, c.J), kThreads, 0, s>>>(b, x, r32, reinterpret_cast<double2*>(partials), c);
-}
-void launch_residual_refine2d(const double2* b, const double2* x, float2* r32, double2* r64, double* partials,
-                              const OpCoef& c, cudaStream_t s, const BatchLaunch* bl) {
-  ProfScope ps_(KID_RESID_REFINE, s);
-  k_residual_refine2d<<<dim3(kDotBlocks, c.J, bl ? bl->R : 1), 256, 0, s>>>(
-      b, x, r32, r64, reinterpret_cast<double2*>(partials), c, bl ? bl->dev : nullptr);
-}
 void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const double2* r_prev, float2* r32,
-                      double* partials, const OpCoef& c, const NonlinTable& nt, cudaStream_t s,
+                      double* partials, const OpCoef& c, const NonlinTable& nt, bool schur, cudaStream_t s,
                       const BatchLaunch* bl) {
   ProfScope ps_(KID_RHS, s);
   if (nt.hex) {
     k_rhs_resid_hex<<<dim3(kDotBlocks, bl ? bl->R : 1), kRhsThreads, 0, s>>>(
-        x, b, b_prev, r_prev, r32, reinterpret_cast<double2*>(partials), c, nt, bl ? bl->dev : nullptr);
+        x, b, b_prev, r_prev, r32, reinterpret_cast<double2*>(partials), c, nt, schur ? 1 : 0, bl ? bl->dev : nullptr);
     return;
   }
   k_rhs_resid_tab<<<dim3(kDotBlocks, bl ? bl->R : 1), kThreads, 0, s>>>(
-      x, b, b_prev, r_prev, r32, reinterpret_cast<double2*>(partials), c, nt, bl ? bl->dev : nullptr);
+      x, b, b_prev, r_prev, r32, reinterpret_cast<double2*>(partials), c, nt, schur ? 1 : 0, bl ? bl->dev : nullptr);
 }
 void launch_energy(const double2* x, double* partials, double* out, const OpCoef& c, const EnergyTable& et, double Bx,
                    cudaStream_t s) {

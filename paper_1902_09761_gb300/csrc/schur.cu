@@ -1,0 +1,561 @@
+// The Schur-complement solve of constant-coefficient systems: spectrum of S p(D)^2, the weights
+// of the Chebyshev iteration, the outer residual r = b - (a + kt G_h^2) eta on 2D grids, and the
+// device-side choice of each amplitude's number of passes (cheb2d.cuh runs them).
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <vector>
+
+#include "apfc_internal.cuh"
+#include "dfloat.cuh"
+#include "host_common.h"
+#include "resid_point.cuh"
+
+namespace apfc {
+
+// ---------------------------------------------------------------------------
+// Host: spectrum and weights
+// ---------------------------------------------------------------------------
+namespace {
+
+// Symbol of S p(D)^2 at wave numbers q (radians per grid point) for amplitude j.
+struct Symbol {
+  const OpCoef& c;
+  const double* h;
+  int m;
+  double theta[kMaxJ], delta[kMaxJ], tsig[kMaxJ];
+  static double cheb(int n, double x) {
+    double t0 = 1.0, t1 = x;
+    if (n == 0) return t0;
+    for (int k = 1; k < n; ++k) {
+      const double t2 = 2.0 * x * t1 - t0;
+      t0 = t1;
+      t1 = t2;
+    }
+    return t1;
+  }
+  Symbol(const OpCoef& c_, const double* h_, int m_) : c(c_), h(h_), m(m_) {
+    double lapmax = 0.0;
+    for (int d = 0; d < c.dim; ++d) lapmax += 4.0 / (h[d] * h[d]);
+    for (int j = 0; j < c.J; ++j) {
+      const double lo = c.sD[j], hi = c.sD[j] + c.mu[j] * lapmax;
+      theta[j] = 0.5 * (hi + lo);
+      delta[j] = 0.5 * (hi - lo);
+      tsig[j] = cheb(m + 1, theta[j] / delta[j]);
+    }
+  }
+  // from K = -L_h's symbol and g = G_h's
+  double of(int j, double K, double g) const {
+    const double d = c.sD[j] + c.mu[j] * K;
+    const double p = (1.0 - cheb(m + 1, (theta[j] - d) / delta[j]) / tsig[j]) / d;
+    return (c.a[j] + c.kt[j] * g * g) * p * p;
+  }
+  double at(int j, const double* q) const {
+    double K = 0.0, A = 0.0;
+    for (int d = 0; d < c.dim; ++d) {
+      const double s = std::sin(0.5 * q[d]);
+      K += 4.0 * s * s / (h[d] * h[d]);
+      A += 2.0 * c.kh[j][d] * std::sin(q[d]);
+    }
+    return of(j, K, -K - A);
+  }
+};
+
+}  // namespace
+
+// Bounds of the spectrum of S_j p(D)^2 over all wave numbers: sampled on a mesh, then the best
+// few samples improved by a pattern search, with 1% to spare on both sides.
+void schur_spectrum(const OpCoef& c, const apfc_grid& grid, int m, double* lmin, double* lmax) {
+  const Symbol sym(c, grid.h, m);
+  const int n = c.dim == 2 ? 32 : 20;
+  constexpr double kTwoPi = 6.283185307179586476925286766559;
+  std::vector<double> K1(3 * n, 0.0), S1(3 * n, 0.0);
+  for (int d = 0; d < c.dim; ++d)
+    for (int i = 0; i < n; ++i) {
+      const double q = kTwoPi * i / n, s = std::sin(0.5 * q);
+      K1[d * n + i] = 4.0 * s * s / (grid.h[d] * grid.h[d]);
+      S1[d * n + i] = 2.0 * std::sin(q);
+    }
+  constexpr int kBest = 4;
+  struct Cand {
+    double v;
+    int i[3];
+  };
+  for (int j = 0; j < c.J; ++j) {
+    Cand best[2][kBest];
+    for (auto& b : best)
+      for (auto& e : b) e = Cand{1e300, {0, 0, 0}};
+    const int nz = c.dim == 3 ? n : 1;
+    for (int iz = 0; iz < nz; ++iz)
+      for (int iy = 0; iy < n; ++iy)
+        for (int ix = 0; ix < n; ++ix) {
+          double K = K1[ix] + K1[n + iy], A = c.kh[j][0] * S1[ix] + c.kh[j][1] * S1[n + iy];
+          if (c.dim == 3) K += K1[2 * n + iz], A += c.kh[j][2] * S1[2 * n + iz];
+          const double v = sym.of(j, K, -K - A);
+          for (int w = 0; w < 2; ++w) {
+            const double key = w == 0 ? v : -v;
+            if (key >= best[w][kBest - 1].v) continue;
+            int p = kBest - 1;
+            while (p > 0 && best[w][p - 1].v > key) best[w][p] = best[w][p - 1], --p;
+            best[w][p] = Cand{key, {ix, iy, iz}};
+          }
+        }
+    double ext[2] = {1e300, 1e300};
+    for (int w = 0; w < 2; ++w)
+      for (const Cand& e : best[w]) {
+        if (e.v >= 1e300) continue;
+        double q[3], v = e.v;
+        for (int d = 0; d < 3; ++d) q[d] = kTwoPi * e.i[d] / n;
+        for (double step = kTwoPi / (2 * n); step > 1e-3;) {
+          bool moved = false;
+          for (int d = 0; d < c.dim; ++d)
+            for (double sg : {-1.0, 1.0}) {
+              const double old = q[d];
+              q[d] += sg * step;
+              const double f = w == 0 ? sym.at(j, q) : -sym.at(j, q);
+              if (f < v)
+                v = f, moved = true;
+              else
+                q[d] = old;
+            }
+          if (!moved) step *= 0.5;
+        }
+        ext[w] = std::min(ext[w], v);
+      }
+    lmin[j] = 0.99 * ext[0];
+    lmax[j] = -1.01 * ext[1];
+  }
+}
+
+// S's own bounds are those of its symbol a + kt g^2, g = c0 + 2 sum_d w_d cos(q_d + phi_d) (which
+// takes the value 0).  A term of the plain iteration costs about half of one with p(D)^2 (measured
+// at 4096^2: 123 against 245 us in FP32), so the latter is taken where it halves their number;
+// below a condition number of 40 it cannot.
+bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s) {
+  SchurCoef q{};
+  auto finish = [&](SchurCoef& r) {
+    for (int j = 0; j < c.J; ++j) {
+      if (!(r.lmin[j] > 0.0) || !(r.lmax[j] > r.lmin[j]) || !std::isfinite(r.lmax[j])) return false;
+      r.lnrate[j] = std::acosh((r.lmax[j] + r.lmin[j]) / (r.lmax[j] - r.lmin[j]));
+    }
+    return true;
+  };
+  double slow = 1e300, kappa = 0.0;
+  s = SchurCoef{};
+  s.plain = true;
+  for (int j = 0; j < c.J; ++j) {
+    double g = -c.c0;
+    for (int d = 0; d < c.dim; ++d) g += 2.0 * gauge_w(c, j, d);
+    s.lmin[j] = c.a[j];
+    s.lmax[j] = c.a[j] + c.kt[j] * g * g;
+    kappa = std::max(kappa, s.lmax[j] / s.lmin[j]);
+  }
+  if (!finish(s)) return false;
+  if (!(kappa > 40.0) || c.dim != 2) return true;
+  schur_spectrum(c, grid, m, q.lmin, q.lmax);
+  if (!finish(q)) return true;
+  double slow_q = 1e300;
+  for (int j = 0; j < c.J; ++j) {
+    slow = std::min(slow, s.lnrate[j]);
+    slow_q = std::min(slow_q, q.lnrate[j]);
+  }
+  if (slow_q > 2.0 * slow) s = q;
+  return true;
+}
+
+// Saad, Alg. 12.1: rho_0 = 1/sigma, d_0 = z/theta; rho_k = 1/(2 sigma - rho_(k-1)),
+// d_k = rho_k rho_(k-1) d_(k-1) + (2 rho_k / delta) z_k: weights of d_first .. d_(first+count-1).
+namespace {
+template <typename F>
+void chebyshev_weights(const SchurCoef& s, int j, int first, int count, F&& put) {
+  const double theta = 0.5 * (s.lmax[j] + s.lmin[j]), delta = 0.5 * (s.lmax[j] - s.lmin[j]), sigma = theta / delta;
+  double rho = 1.0 / sigma;
+  for (int k = 1; k < first + count; ++k) {
+    const double rn = 1.0 / (2.0 * sigma - rho);
+    if (k >= first) put(k - first, rn * rho, 2.0 * rn / delta);
+    rho = rn;
+  }
+}
+}  // namespace
+// Pass 0 makes d_0 and d_1, pass k >= 1 the next ni terms.
+ChebPass schur_pass(const SchurCoef& s, int J, int pass, int ni) {
+  ChebPass cp;
+  std::memset(&cp, 0, sizeof(cp));
+  for (int j = 0; j < J; ++j) {
+    cp.inv_theta[j] = 2.0 / (s.lmax[j] + s.lmin[j]);
+    chebyshev_weights(s, j, pass == 0 ? 1 : 2 + (pass - 1) * ni, pass == 0 ? 1 : ni, [&](int i, double c1, double c2) {
+      cp.c1[i][j] = c1;
+      cp.c2[i][j] = c2;
+    });
+  }
+  return cp;
+}
+// Pass 0 makes d_0 = r / theta and ni terms, later ones ni.
+GaugeWeights gauge_weights(const SchurCoef& s, int J, int pass, int ni) {
+  GaugeWeights w;
+  std::memset(&w, 0, sizeof(w));
+  for (int j = 0; j < J; ++j) {
+    w.inv_theta[j] = 2.0 / (s.lmax[j] + s.lmin[j]);
+    chebyshev_weights(s, j, 1 + pass * ni, ni, [&](int i, double c1, double c2) {
+      w.c1[i][j] = c1;
+      w.c2[i][j] = c2;
+    });
+  }
+  return w;
+}
+
+int schur_terms(double tin, double lnrate) {
+  const double x = 1.0 / tin;
+  const double need = x > 1.0 ? std::log(x + std::sqrt(x * x - 1.0)) / lnrate : 0.0;
+  return need < 1e9 ? std::max(2, (int)std::ceil(need)) : 1000000000;
+}
+
+// ---------------------------------------------------------------------------
+// Device: norms and passes
+// ---------------------------------------------------------------------------
+namespace {
+
+constexpr double kSchurLast64 = 0.4, kSchurLast32 = 1.0 / 16.0;
+
+// Sums the partials of ||r||^2 and ||b||^2 (have bits 1, 2) of amplitude blockIdx.x of the run
+// and sets the number of passes of its next solve.
+__global__ void __launch_bounds__(256) k_schur_plan(const __grid_constant__ SchurPlan p, KScal* ks, const RunGeom* rg) {
+  const int run = rg != nullptr ? blockIdx.x / p.J : 0, j = blockIdx.x - run * p.J;
+  const double* part = p.part;
+  int npart = p.npart;
+  long long ss = p.slot_stride, sj = p.amp_stride;
+  if (rg != nullptr) {
+    if (p.by_run) {  // the residual kernel's layout [run][J][2][npart of the run]
+      npart = rg[run].npart_r;
+      part += rg[run].part_off_r;
+      ss = npart;
+      sj = 2ll * npart;
+    } else {
+      part += (long long)run * p.J * sj;
+    }
+  }
+  __shared__ double sh[2][8];
+  for (int q = 0; q < 2; ++q) {
+    double v = 0.0;
+    if (p.have & (1 << q))
+      for (int i = threadIdx.x; i < npart; i += 256) v += part[j * sj + q * ss + (long long)i * p.elem];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[q][threadIdx.x >> 5] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  KScal& k = ks[blockIdx.x];
+  double s[2] = {0.0, 0.0};
+  for (int q = 0; q < 2; ++q)
+    for (int w = 0; w < 8; ++w) s[q] += sh[q][w];
+  if (p.have & 1) k.rnorm2 = s[0];
+  if (p.have & 2) k.bnorm2 = s[1];
+  const double r2 = k.rnorm2, b2 = k.bnorm2;
+  k.iters = 0;
+  if (!isfinite(r2) || !isfinite(b2) || r2 <= p.tol * p.tol * b2) return;
+  // The residual that a Chebyshev solve leaves sits in the low end of the spectrum, where it
+  // weighs most in the error: the solve that is to meet the outer tolerance goes further below
+  // it than a Krylov solve has to for the same error.
+  const double want = b2 > 0.0 ? p.tol * sqrt(b2 / r2) : p.tol_inner;
+  double tin;
+  if (p.fp64) {
+    tin = kSchurLast64 * (b2 > 0.0 ? want : p.tol);
+  } else {
+    tin = fmin(0.5, fmax(p.tol_inner, 0.25 * want));
+    if (tin <= want) tin = fmin(tin, fmax(0.05 * p.tol_inner, kSchurLast32 * want));
+  }
+  const double x = 1.0 / tin;
+  const double need = x > 1.0 ? log(x + sqrt(x * x - 1.0)) / p.lnrate[j] : 0.0;
+  const double n = fmin(fmax(2.0, ceil(need)), 1e9);
+  k.iters = min(max(1, (int)ceil((n - p.t0) / p.ni)), p.max_pass);
+}
+
+// e^{i phi_d i}: blockIdx.y = amplitude
+template <typename T>
+__global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, int tx, int ty, int tz) {
+  const int j = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x, n = tx + ty + tz;
+  if (i >= n) return;
+  const int d = i < tx ? 0 : (i < tx + ty ? 1 : 2), k = i - (d > 0 ? tx : 0) - (d > 1 ? ty : 0);
+  double sn, cs;
+  sincos(atan2(c.kh[j][d], c.ih2[d]) * k, &sn, &cs);
+  tab[(long long)j * n + i] = mkc<T>((T)cs, (T)sn);
+}
+
+// ---------------------------------------------------------------------------
+// Outer residual r = b - a eta - kt G_h (G_h eta) on 2D grids, streamed down the rows: a block
+// owns 256 columns (252 of them valid) and a segment of rows; at step t a thread forms zeta =
+// G_h eta at row t - 1 and r at row t - 2 of its column, the y-neighbours in registers (the row
+// below is the one just formed), the x-neighbours from two-row shared-memory rings.  Every
+// double is split once.  Writes zeta into the state (the solve never reads it, so it always
+// belongs to the latest eta), r as FP32 (RED: or FP64), optionally r in FP64, and per block the
+// sums ||r||^2 and, on request, ||b||^2.
+// ---------------------------------------------------------------------------
+constexpr int kRsNT = 256, kRsPF = 2, kRsV = kRsNT - 4;
+
+template <bool F64>
+struct RsVal;
+template <>
+struct RsVal<false> {
+  using V = PDF;
+  using S = float4;
+  static __device__ __forceinline__ V in(double2 v) { return pdf_split(v); }
+  static __device__ __forceinline__ S pack(V v) { return pdf_pack(v); }
+  static __device__ __forceinline__ V unpack(S v) { return pdf_unpack(v); }
+  static __device__ __forceinline__ V zero() { return PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+};
+template <>
+struct RsVal<true> {
+  using V = double2;
+  using S = double2;
+  static __device__ __forceinline__ V in(double2 v) { return v; }
+  static __device__ __forceinline__ S pack(V v) { return v; }
+  static __device__ __forceinline__ V unpack(S v) { return v; }
+  static __device__ __forceinline__ V zero() { return make_double2(0.0, 0.0); }
+};
+
+__device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src));
+}
+
+template <bool F64>
+__global__ void __launch_bounds__(kRsNT, 2)
+    k_resid_schur2d(const double2* __restrict__ b, double2* x, void* r_out, double2* __restrict__ r64,
+                    double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
+                    int want_b, const RunGeom* rg) {
+  using RV = RsVal<F64>;
+  using V = typename RV::V;
+  using SV = typename RV::S;
+  __shared__ SV ring[2][2][kRsNT + 2];             // eta, zeta
+  __shared__ double2 stg[kRsPF + 1][2][kRsNT];     // eta, b rows in flight
+  __shared__ double shn[2][kRsNT / 32];
+  const int j = blockIdx.y, t = threadIdx.x;
+  int nx = c.nx, ny = c.ny;
+  long long pts = c.pts, fo = 0;
+  if (rg != nullptr) {
+    const RunGeom& q = rg[blockIdx.z];
+    nx = q.nx;
+    ny = q.ny;
+    pts = q.pts;
+    b += q.elem_off;
+    x += q.elem_off;
+    fo = q.field_off;
+    part += q.part_off_r;
+    Ly = q.rows_r;
+    nstrips = (nx + kRsV - 1) / kRsV;
+    nsegs = (ny + Ly - 1) / Ly;
+  }
+  const int npart = nstrips * nsegs;
+  if ((int)blockIdx.x >= npart) return;
+  const int sy = blockIdx.x / nstrips, sx = blockIdx.x - sy * nstrips;
+  if (c.prof != nullptr && blockIdx.x == 0 && t == 0)
+    atomicAdd(c.prof + KID_RESID_REFINE,
+              (unsigned long long)pts * (3 * sizeof(double2) + (F64 ? sizeof(double2) : sizeof(float2)) +
+                                         (r64 != nullptr ? sizeof(double2) : 0)));
+  double2* zt = x + 2LL * j * pts;
+  const double2* et = zt + pts;
+  const double2* bt = b + (2LL * j + 1) * pts;
+  fo += (long long)j * pts;
+  [[maybe_unused]] float2* r32 = reinterpret_cast<float2*>(r_out) + fo;
+  [[maybe_unused]] double2* rd = reinterpret_cast<double2*>(r_out) + fo;
+  if (r64 != nullptr) r64 += fo;
+
+  [[maybe_unused]] ResidCoef<2> q;
+  [[maybe_unused]] LaneC ma;
+  [[maybe_unused]] double g0, gx, gy, ax, ay, kt, aa;
+  if constexpr (F64) {
+    g0 = c.c0, gx = c.ih2[0], gy = c.ih2[1], ax = c.kh[j][0], ay = c.kh[j][1], kt = c.kt[j], aa = c.a[j];
+  } else {
+    q = resid_coef<2>(c, j);
+    ma = lane_c(c.a[j], -1.f, -1.f);
+  }
+
+  const int x_first = sx * kRsV - 2;
+  int gxx = (x_first + t) % nx;
+  if (gxx < 0) gxx += nx;
+  const int xo = x_first + t;
+  const bool col_own = t >= 2 && t < kRsNT - 2 && xo < nx;
+  const int y0 = sy * Ly, rows = min(ny, y0 + Ly) - y0, steps = rows + 4;
+  int fy = (y0 - 2) % ny;
+  if (fy < 0) fy += ny;
+  auto issue = [&](int tf, int slot) {
+    if (tf < steps) {
+      rs_copy16(&stg[slot][0][t], et + (long long)fy * nx + gxx);
+      fy = fy + 1 == ny ? 0 : fy + 1;
+      const int lr = tf - 2;  // row of r: local rows 2 .. rows + 1
+      if (col_own && lr >= 2) rs_copy16(&stg[slot][1][t], bt + (long long)(y0 + lr - 2) * nx + xo);
+    }
+    asm volatile("cp.async.commit_group;\n" ::);
+  };
+  if (t == 0) {
+    for (int k = 0; k < 2; ++k)
+      for (int p = 0; p < 2; ++p) ring[k][p][0] = ring[k][p][kRsNT + 1] = RV::pack(RV::zero());
+  }
+  for (int k = 0; k < 2; ++k)
+    for (int p = 0; p < 2; ++p) ring[k][p][t + 1] = RV::pack(RV::zero());
+  for (int tf = 0; tf < kRsPF; ++tf) issue(tf, tf);
+  __syncthreads();
+  V e1 = RV::zero(), e2 = RV::zero(), z1 = RV::zero(), z2 = RV::zero();  // rows formed 1 and 2 steps ago
+  float rr = 0.f, bb = 0.f;
+  double rrd = 0.0, bbd = 0.0;
+  int slot = 0, islot = kRsPF, par = 0;
+  for (int tt = 0; tt < steps; ++tt) {
+    issue(tt + kRsPF, islot);
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kRsPF));
+    const V e0 = RV::in(stg[slot][0][t]);
+    ring[0][par][t + 1] = RV::pack(e0);
+    // zeta at row tt - 1
+    const V el = RV::unpack(ring[0][par ^ 1][t]), er = RV::unpack(ring[0][par ^ 1][t + 2]);
+    V z0;
+    double2 zd;
+    if constexpr (F64) {
+      const double lx = fma(gy, e2.x + e0.x, fma(gx, el.x + er.x, g0 * e1.x));
+      const double ly = fma(gy, e2.y + e0.y, fma(gx, el.y + er.y, g0 * e1.y));
+      z0 = make_double2(lx - (ax * (er.y - el.y) + ay * (e0.y - e2.y)), ly + (ax * (er.x - el.x) + ay * (e0.x - e2.x)));
+      zd = z0;
+    } else {
+      PAcc a;
+      a.init(RV::zero());
+      a.fma(q.g0.h, q.g0.l, e1);
+      a.fma(q.gl[0].h, q.gl[0].l, pdf_add(er, el));
+      a.fma(q.gl[1].h, q.gl[1].l, pdf_add(e0, e2));
+      a.fma(q.ga[0].h, q.ga[0].l, pdf_swap(pdf_sub(er, el)));
+      a.fma(q.ga[1].h, q.ga[1].l, pdf_swap(pdf_sub(e0, e2)));
+      a.result(z0.h, z0.l);
+      zd = make_double2(df_to_d(DF{z0.h.x, z0.l.x}), df_to_d(DF{z0.h.y, z0.l.y}));
+    }
+    ring[1][par][t + 1] = RV::pack(z0);
+    const int lz = tt - 1;
+    if (col_own && lz >= 2 && lz < rows + 2) zt[(long long)(y0 + lz - 2) * nx + xo] = zd;
+    // r at row tt - 2
+    const int lr = tt - 2;
+    if (lr >= 2) {
+      const V zl = RV::unpack(ring[1][par ^ 1][t]), zr = RV::unpack(ring[1][par ^ 1][t + 2]);
+      if (col_own) {
+        const double2 bv = stg[slot][1][t];
+        const long long p = (long long)(y0 + lr - 2) * nx + xo;
+        if constexpr (F64) {
+          const double lx = fma(gy, z2.x + z0.x, fma(gx, zl.x + zr.x, g0 * z1.x));
+          const double ly = fma(gy, z2.y + z0.y, fma(gx, zl.y + zr.y, g0 * z1.y));
+          const double Gx = lx - (ax * (zr.y - zl.y) + ay * (z0.y - z2.y));
+          const double Gy = ly + (ax * (zr.x - zl.x) + ay * (z0.x - z2.x));
+          const double2 rv = make_double2(bv.x - (kt * Gx + aa * e2.x), bv.y - (kt * Gy + aa * e2.y));
+          rd[p] = rv;
+          rrd += rv.x * rv.x + rv.y * rv.y;
+          if (want_b) bbd += bv.x * bv.x + bv.y * bv.y;
+        } else {
+          const PDF bp = pdf_split(bv);
+          PAcc a;
+          a.init(bp);
+          a.fma(q.k0.h, q.k0.l, z1);
+          a.fma(q.kl[0].h, q.kl[0].l, pdf_add(zr, zl));
+          a.fma(q.kl[1].h, q.kl[1].l, pdf_add(z0, z2));
+          a.fma(q.ka[0].h, q.ka[0].l, pdf_swap(pdf_sub(zr, zl)));
+          a.fma(q.ka[1].h, q.ka[1].l, pdf_swap(pdf_sub(z0, z2)));
+          a.fma(ma.h, ma.l, e2);
+          float2 f, l;
+          a.result(f, l);
+          r32[p] = f;
+          if (r64 != nullptr) r64[p] = make_double2(df_to_d(DF{f.x, l.x}), df_to_d(DF{f.y, l.y}));
+          rr = fmaf(f.x, f.x, fmaf(f.y, f.y, rr));
+          if (want_b) bb = fmaf(bp.h.x, bp.h.x, fmaf(bp.h.y, bp.h.y, bb));
+        }
+      }
+    }
+    e2 = e1;
+    e1 = e0;
+    z2 = z1;
+    z1 = z0;
+    slot = slot == kRsPF ? 0 : slot + 1;
+    islot = islot == kRsPF ? 0 : islot + 1;
+    par ^= 1;
+    __syncthreads();
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::);
+  if constexpr (!F64) rrd = (double)rr, bbd = (double)bb;
+  for (int o = 16; o > 0; o >>= 1) {
+    rrd += __shfl_xor_sync(0xffffffffu, rrd, o);
+    bbd += __shfl_xor_sync(0xffffffffu, bbd, o);
+  }
+  if ((t & 31) == 0) shn[0][t >> 5] = rrd, shn[1][t >> 5] = bbd;
+  __syncthreads();
+  if (t < 2) {
+    double v = 0.0;
+    for (int w = 0; w < kRsNT / 32; ++w) v += shn[t][w];
+    part[(2LL * j + t) * npart + blockIdx.x] = v;
+  }
+}
+
+}  // namespace
+
+// Rows per segment of the passes: each step of a block costs about the same, so the heights
+// are compared by (what the busiest multiprocessor has to run) x (rows + 2S).
+int schur_auto_rows(const SchurCoef& sc, const int* nx, const int* ny, int n, int J, int m, int elem_bytes, int tile,
+                    int sms) {
+  const bool f32 = elem_bytes == 8, wide = f32 && sc.plain && (tile == 2 || tile == 4 || tile == 5);
+  const int S = sc.plain ? 2 * (f32 ? kGaugeNI32 : kGaugeNI64) : (f32 && m == 1 ? 8 : 2 + 2 * m);
+  const int NC = wide ? 256 : 128;
+  const int res = wide ? 3 : 6;       // resident blocks per SM
+  const double thr = wide ? 0.5 : 0.26;  // a step of one among several, a lone block's being 1
+  int most = 1;
+  for (int i = 0; i < n; ++i) most = std::max(most, ny[i]);
+  double best = 1e300;
+  int best_rows = std::min(most, 128);
+  for (int rows = 4; rows <= 512; rows += rows < 64 ? 4 : 8) {
+    long long blocks = 0;
+    for (int i = 0; i < n; ++i)
+      blocks += (long long)((nx[i] + NC - 2 * S - 1) / (NC - 2 * S)) * ((ny[i] + rows - 1) / rows) * J;
+    const long long per = (blocks + sms - 1) / sms;  // blocks of the busiest SM
+    const long long full = per / res, rest = per - full * res;
+    double t = full * std::max(1.0, res * thr);
+    if (rest > 0) t += std::max(1.0, rest * thr);
+    t *= std::min(rows, most) + 2 * S + 4;
+    if (t < best) best = t, best_rows = rows;
+    if (rows >= most) break;
+  }
+  return best_rows;
+}
+
+int schur_resid_rows(int nx, int ny, int J) {
+  const long long strips = (nx + kRsV - 1) / kRsV;
+  const long long rows = (long long)ny * strips * J / 912;  // about six blocks per SM
+  return (int)std::min<long long>(128, std::max<long long>(8, rows));
+}
+int schur_resid_parts(int nx, int ny, int J) {
+  const int Ly = schur_resid_rows(nx, ny, J);
+  return ((nx + kRsV - 1) / kRsV) * ((ny + Ly - 1) / Ly);
+}
+
+template <typename T>
+void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
+                          bool want_b, cudaStream_t s, const BatchLaunch* bl) {
+  ProfScope ps_(KID_RESID_REFINE, s);
+  constexpr bool F64 = sizeof(T) == 8;
+  if (bl != nullptr) {
+    int most = 0;
+    for (int i = 0; i < bl->R; ++i) most = std::max(most, bl->host[i].npart_r);
+    k_resid_schur2d<F64><<<dim3(most, c.J, bl->R), kRsNT, 0, s>>>(b, x, r, r64, part, c, 0, 0, 0, want_b, bl->dev);
+    return;
+  }
+  const int Ly = schur_resid_rows(c.nx, c.ny, c.J);
+  const int ns = (c.nx + kRsV - 1) / kRsV, ng = (c.ny + Ly - 1) / Ly;
+  k_resid_schur2d<F64><<<dim3(ns * ng, c.J), kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, nullptr);
+}
+template void launch_resid_schur2d<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool,
+                                          cudaStream_t, const BatchLaunch*);
+template void launch_resid_schur2d<double>(const double2*, double2*, double2*, double2*, double*, const OpCoef&, bool,
+                                           cudaStream_t, const BatchLaunch*);
+
+template <typename T>
+void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s) {
+  k_gauge_table<T><<<dim3((tx + ty + tz + 127) / 128, c.J), 128, 0, s>>>(tab, c, tx, ty, tz);
+}
+template void launch_gauge_table<float>(float2*, const OpCoef&, int, int, int, cudaStream_t);
+template void launch_gauge_table<double>(double2*, const OpCoef&, int, int, int, cudaStream_t);
+
+void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl) {
+  ProfScope ps_(kid_of<double>(KID_FINALIZE), s);
+  k_schur_plan<<<(bl ? bl->R : 1) * p.J, 256, 0, s>>>(p, ks, bl ? bl->dev : nullptr);
+}
+
+}  // namespace apfc

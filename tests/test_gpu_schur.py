@@ -1,0 +1,100 @@
+"""The Chebyshev solves of the Schur complement against the oracle, at the sizes and spacings
+where the kernels' edges lie.
+
+A step stops at relative residual tol; the error of eta is at most cond(S_j) tol with
+cond(S_j) <= 1 + Bx g^2 / (1/dt + dB) and g <= 2 sum_d (2/h_d^2) sqrt(1 + h_d^2) for |k_j| = 1.
+At h = pi/2 that is below 25: with tol = 1e-13 the bound 1e-10 holds as in the other parity
+tests.  At h = 0.5 (where the preconditioned iteration is taken) it is below 1400, and the
+FP64 rounding of the residual is about 1e-13: tol = 1e-12 and the bound 2e-9.
+"""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1902_09761_gb300 import apfc as A
+from paper_1902_09761_gb300 import inputs
+
+from gpu_common import H2, P, context, ensure_built, rel_l2_per_amp
+
+pytestmark = pytest.mark.gpu
+
+PRECISIONS = [A.APFC_FP64, A.APFC_FP32_REFINED]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    return ensure_built()
+
+
+def _steps(shape, h, n, bound, dt=1.0, seed=81, **opts):
+    ctx, L = context("hex", shape, h, **opts)
+    eta = inputs.random_amplitudes(3, shape, seed=seed, scale=0.15)
+    ctx.set_amplitudes(eta)
+    for _ in range(n):
+        ctx.step(dt)
+        eta, zeta = O.step(eta, dt, P, L, h)
+        assert max(rel_l2_per_amp(ctx.get_amplitudes(), eta)) <= bound
+        assert max(rel_l2_per_amp(ctx.get_zeta(), zeta)) <= bound
+    st = ctx.stats()
+    assert st["resid_last"] <= opts["tol"] and st["iters_last"] > 0
+    ctx.close()
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("shape", [(3, 3), (3, 4), (4, 3), (5, 130), (131, 6), (16, 116), (40, 117), (33, 244), (29, 245)])
+def test_grids_around_strip_and_halo_widths(prec, shape):
+    # grids smaller than the halo wrap several times; 116 and 244 columns are one strip of 128
+    # or 256 exactly, one more starts a second strip; odd rows take single-value copies
+    _steps(shape, H2, 2, 1e-10, tol=1e-13, precision=prec)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("rows", [1, 5, 70])
+@pytest.mark.parametrize("tile", [3, 5])
+def test_segment_heights(prec, rows, tile):
+    _steps((70, 130), (1.4, 1.7), 2, 1e-10, tol=1e-13, precision=prec, tile_rows=rows, tile=tile)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("m", [1, 2, 3, 4])
+@pytest.mark.parametrize("shape", [(24, 30), (37, 131), (130, 115)])
+def test_fine_grids_take_the_preconditioned_iteration(prec, m, shape):
+    _steps(shape, (0.5, 0.5), 2, 2e-9, tol=1e-12, precision=prec, cheb_degree=m)
+
+
+@pytest.mark.parametrize("dt", [0.01, 30.0])
+@pytest.mark.parametrize("prec", PRECISIONS)
+def test_small_and_large_time_steps(prec, dt):
+    # cond(S) from 1.2 (dt 0.01) to 370 (dt 30): bound cond(S) tol
+    _steps((48, 52), H2, 2, 1e-9, dt=dt, tol=1e-12, precision=prec)
+
+
+def test_more_applications_than_max_iter_allows_fall_back_to_bicgstab():
+    # the Chebyshev iteration needs about 45 applications of S for 1e-10, 10 iterations allow 20
+    shape = (40, 44)
+    eta = inputs.random_amplitudes(3, shape, seed=82, scale=0.15)
+    ctx, L = context("hex", shape, H2, tol=1e-10, max_iter=10)
+    ctx.set_amplitudes(eta)
+    ctx.step(1.0)
+    ref, _ = O.step(eta, 1.0, P, L, H2)
+    assert max(rel_l2_per_amp(ctx.get_amplitudes(), ref)) <= 25e-10
+    ctx.close()
+
+
+def test_batch_on_a_fine_grid_equals_the_runs_alone():
+    L = O.hex_lattice()
+    shapes = [(40, 48), (33, 131), (64, 64)]
+    o = A.apfc_default_opts(precision=A.APFC_FP32_REFINED, tol=1e-12)
+    states = [inputs.random_amplitudes(3, s, seed=90 + r, scale=0.15) for r, s in enumerate(shapes)]
+    h = (0.5, 0.5)
+    with A.Batch(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), shapes, h, o) as b:
+        for r, e in enumerate(states):
+            b.set_amplitudes(r, e)
+        b.step(1.0, 2)
+        got = [b.get_amplitudes(r) for r in range(len(shapes))]
+    for r, s in enumerate(shapes):
+        ctx, _ = context("hex", s, h, precision=A.APFC_FP32_REFINED, tol=1e-12)
+        ctx.set_amplitudes(states[r])
+        ctx.step(1.0, 2)
+        assert np.array_equal(ctx.get_amplitudes(), got[r]), s
+        ctx.close()
