@@ -285,7 +285,7 @@ struct PcFin {
   FieldRef<T> chi1;  // chi1 (stride 2 pts)
 };
 // 3D grids (stream3d.cu): the passes behind launch_apply_A, launch_residual, launch_pc_rhs,
-// launch_cheb_first / _sweep (fin: step 4 of P^{-1} in this last pass) and launch_zeta.
+// launch_cheb_first / _sweep (fin: step 4 of P^{-1} in this last pass).
 template <typename T>
 void launch3d_apply_A(const cplx<T>* x, cplx<T>* y, const OpCoef& c, const KScal* act, cudaStream_t s);
 template <typename T>
@@ -299,7 +299,6 @@ void launch3d_cheb_first(CFieldRef<T> f, FieldRef<T> X, FieldRef<T> R, FieldRef<
 template <typename T>
 void launch3d_cheb_sweep(CFieldRef<T> Dd, FieldRef<T> X, FieldRef<T> R, FieldRef<T> Dn, const ChebStep& w, int last,
                          const OpCoef& c, const KScal* act, cudaStream_t s, const PcFin<T>* fin);
-void launch3d_zeta(double2* x, const OpCoef& c, cudaStream_t s);
 // fin != nullptr (3D grids, last pass only): also step 4 of P^{-1}, see PcFin
 template <typename T>
 void launch_cheb_first(CFieldRef<T> f, FieldRef<T> X, FieldRef<T> R, FieldRef<T> Dn, const ChebStep& w, int last,
@@ -409,17 +408,24 @@ struct SchurCoef {
   bool plain;                       // the iteration on S itself (gauge2d.cuh), else on S p(D)^2 (cheb2d.cuh)
   double lmin[kMaxJ], lmax[kMaxJ];  // bounds of its spectrum
   double lnrate[kMaxJ];             // acosh(sigma): each term shrinks the residual by about exp(-lnrate)
+  // condition number of S.  A rounding of eta enters b - S eta amplified by up to kappa relative
+  // to b, so the residual's own noise is a few kappa units of the last place kept: about 8 kappa
+  // 2^-48 when eta is split into FP32 pairs, 8 kappa 2^-53 in FP64.
+  double kappa;
 };
+inline bool schur_resid_f64(const SchurCoef& s, double tol) { return tol < 2.9e-14 * s.kappa; }
+inline bool schur_resid_ok(const SchurCoef& s, double tol) { return tol >= 9e-16 * s.kappa; }
 // L passes make schur_t0 + L schur_ni terms of the solve's polynomial
 constexpr int kGaugeNI32 = 3, kGaugeNI64 = 1;
 template <typename T>
-int schur_ni(const SchurCoef& s, int m) {
+int schur_ni(const SchurCoef& s, int dim, int m) {
+  if (dim == 3) return 1;
   if (s.plain) return sizeof(T) == 4 ? kGaugeNI32 : kGaugeNI64;
   return sizeof(T) == 4 && m == 1 ? 2 : 1;
 }
 template <typename T>
-int schur_t0(const SchurCoef& s, int m) {
-  return s.plain ? 1 : 2 - schur_ni<T>(s, m);
+int schur_t0(const SchurCoef& s, int dim, int m) {
+  return s.plain ? 1 : 2 - schur_ni<T>(s, dim, m);
 }
 bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s);
 ChebPass schur_pass(const SchurCoef& s, int J, int pass, int ni);
@@ -434,6 +440,9 @@ bool launch_cheb2d(int m, const OpCoef& c, const ChebStep* w, const ChebPass& cp
 template <typename T>
 bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Ly,
                     const ChebBufs<T>& b, int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
+template <typename T>
+bool launch_gauge3d(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, const ChebBufs<T>& b, int pass,
+                    int sms, cudaStream_t s);
 // tab[j][d][i] = e^{i phi_d i}, 0 <= i <= n_d (sizes of GaugeTab)
 template <typename T>
 void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s);
@@ -441,16 +450,23 @@ void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, c
 template <typename T>
 bool launch_schur_pass(const SchurCoef& sc, int m, int tile, const OpCoef& c, const ChebStep* w,
                        const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int pass, cudaStream_t s,
-                       const BatchLaunch* bl = nullptr) {
-  const int ni = schur_ni<T>(sc, m);
+                       int sms, const BatchLaunch* bl = nullptr) {
+  const int ni = schur_ni<T>(sc, c.dim, m);
+  if (c.dim == 3) return launch_gauge3d<T>(c, gt, gauge_weights(sc, c.J, pass, ni), b, pass, sms, s);
   return sc.plain ? launch_gauge2d<T>(tile, c, gt, gauge_weights(sc, c.J, pass, ni), Ly, b, pass, s, bl)
                   : launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, pass, ni), Ly, b, pass, s, bl);
 }
 // r = b - (a + kt G^2) eta from the eta-parts of x, b; zeta = G eta written into x; r [J][pts] in
-// T, r64 (nullable) the same in FP64; part [J][2][schur_resid_parts] sums of ||r||^2, ||b||^2
+// T, r64 (nullable) the same in FP64; part [J][2][schur_resid_parts] sums of ||r||^2, ||b||^2;
+// f64 (always so for T = double): in FP64 arithmetic, else in FP32 pairs
 template <typename T>
 void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
-                          bool want_b, cudaStream_t s, const BatchLaunch* bl = nullptr);
+                          bool want_b, bool f64, cudaStream_t s, const BatchLaunch* bl = nullptr);
+// the same on 3D grids (part [J][2][schur_resid3_parts])
+template <typename T>
+bool launch_resid_schur3d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
+                          bool want_b, bool f64, cudaStream_t s);
+int schur_resid3_parts(int nx, int ny, int nz, int J);
 int schur_resid_rows(int nx, int ny, int J);
 int schur_resid_parts(int nx, int ny, int J);
 // ks[j].rnorm2 / bnorm2 from partial sums and ks[j].iters, the passes of the next solve

@@ -201,7 +201,7 @@ struct apfc_ctx {
   SchurWork<float> s32;
   double* rpart = nullptr;     // partial sums of the Schur-complement residual
   SchurCoef schur{};           // of the current coefficients
-  bool schur_ok = false;       // they allow the Chebyshev iteration (2D, degree 1..4)
+  bool schur_ok = false;       // they allow the Chebyshev iteration (degree 1..4)
   bool prev_schur = false;     // r64_prev holds that path's residual field
   double resid = 0.0;          // max over amplitudes of ||r|| / ||b|| after the last solve
   bool has_state = false;
@@ -402,8 +402,7 @@ bool build_coef(apfc_ctx* c, double dt, std::string& err) {
   if (!make_coef(c->lat, c->par, c->grid, c->opts.tau_mode, dt, c->coef, err)) return false;
   c->coef_dt = dt;
   const int m = c->opts.cheb_degree;
-  c->schur_ok = c->dim == 2 && m >= 1 && m <= fused2d_max_degree((int)sizeof(float2)) &&
-                schur_build(c->coef, c->grid, m, c->schur);
+  c->schur_ok = m >= 1 && m <= fused2d_max_degree((int)sizeof(float2)) && schur_build(c->coef, c->grid, m, c->schur);
   return true;
 }
 
@@ -766,14 +765,23 @@ apfc_status status_of(apfc_ctx* ctx, int worst) {
 }
 
 // Whether the solve runs as the Chebyshev iteration on the Schur complement: constant
-// coefficients (no Jacobian) on a 2D grid with the fused pipeline, and no more operator
-// applications than max_iter BiCGStab iterations (two each) may take.
+// coefficients (no Jacobian), the fused pipeline, a tolerance above the residual's noise, and no
+// more operator applications than max_iter BiCGStab iterations (two each) may take.
 bool use_schur(const apfc_ctx* ctx) {
   if (!ctx->schur_ok || ctx->opts.fused == 0 || ctx->coef.jd != nullptr) return false;
+  if (!schur_resid_ok(ctx->schur, ctx->opts.tol)) return false;
   const double tin = ctx->opts.precision == APFC_FP64 ? 0.9 * ctx->opts.tol : ctx->opts.tol_inner;
   for (int j = 0; j < ctx->J; ++j)
     if (schur_terms(tin, ctx->schur.lnrate[j]) > 2LL * ctx->opts.max_iter) return false;
   return true;
+}
+
+int resid_parts(const apfc_ctx* ctx) {
+  const int* n = ctx->grid.n;
+  return ctx->dim == 3 ? schur_resid3_parts(n[0], n[1], n[2], ctx->J) : schur_resid_parts(n[0], n[1], ctx->J);
+}
+GaugeTab<float> gauge_sizes(const apfc_ctx* ctx) {
+  return {nullptr, ctx->grid.n[0] + 1, ctx->grid.n[1] + 1, ctx->dim == 3 ? ctx->grid.n[2] + 1 : 0};
 }
 
 template <typename T>
@@ -783,12 +791,10 @@ apfc_status alloc_schur(apfc_ctx* ctx, SchurWork<T>& w) {
     if (!p) CK(cudaMalloc(&p, field_bytes<T>(ctx)));
   for (auto& p : w.d)
     if (!p) CK(cudaMalloc(&p, field_bytes<T>(ctx)));
-  if (!ctx->rpart)
-    CK(cudaMalloc(&ctx->rpart,
-                  2 * sizeof(double) * ctx->J * (size_t)schur_resid_parts(ctx->grid.n[0], ctx->grid.n[1], ctx->J)));
-  const int tx = ctx->grid.n[0] + 1, ty = ctx->grid.n[1] + 1;
-  if (!w.tab) CK(cudaMalloc(&w.tab, sizeof(cplx<T>) * ctx->J * (size_t)(tx + ty)));
-  launch_gauge_table<T>(w.tab, ctx->coef, tx, ty, 0, ctx->stream);
+  if (!ctx->rpart) CK(cudaMalloc(&ctx->rpart, 2 * sizeof(double) * ctx->J * (size_t)resid_parts(ctx)));
+  const auto [none, tx, ty, tz] = gauge_sizes(ctx);
+  if (!w.tab) CK(cudaMalloc(&w.tab, sizeof(cplx<T>) * ctx->J * ((size_t)tx + ty + tz)));
+  launch_gauge_table<T>(w.tab, ctx->coef, tx, ty, tz, ctx->stream);
   CK(cudaGetLastError());
   CK(cudaMalloc(&w.u, field_bytes<T>(ctx)));
   return APFC_OK;
@@ -816,7 +822,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   constexpr bool fp64 = sizeof(T) == 8;
   cudaStream_t s = ctx->stream;
   const apfc_opts& o = ctx->opts;
-  const int m = o.cheb_degree, ni = schur_ni<T>(ctx->schur, m), nt0 = schur_t0<T>(ctx->schur, m), J = ctx->J;
+  const int m = o.cheb_degree, ni = schur_ni<T>(ctx->schur, ctx->dim, m), nt0 = schur_t0<T>(ctx->schur, ctx->dim, m), J = ctx->J;
   const int most = fp64 ? 4 : o.max_refine;
   const auto cw = cheb_weights(ctx);
   const int rows = o.tile_rows > 0 ? o.tile_rows
@@ -840,11 +846,13 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   prhs.amp_stride = 2 * kDotSlots * kDotBlocks;
   // the residual kernel's: [J][2][npart]
   plan.part = ctx->rpart;
-  plan.npart = schur_resid_parts(ctx->grid.n[0], ctx->grid.n[1], J);
+  plan.npart = resid_parts(ctx);
   plan.elem = 1;
   plan.slot_stride = plan.npart;
   plan.amp_stride = 2LL * plan.npart;
-  const GaugeTab<T> gt{w.tab, ctx->grid.n[0] + 1, ctx->grid.n[1] + 1, 0};
+  const auto [none, tx, ty, tz] = gauge_sizes(ctx);
+  const GaugeTab<T> gt{w.tab, tx, ty, tz};
+  const bool f64 = fp64 || schur_resid_f64(ctx->schur, o.tol);
   const ChebBufs<T> bufs{w.r[0], {w.r[0], w.r[1]}, {w.d[0], w.d[1]}, w.u, x, ctx->ks64};
   int total = 0, worst = KS_CONVERGED, sweep = 0;
   const double tol2 = o.tol * o.tol;
@@ -858,7 +866,10 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
         prhs.have = 2;
         launch_schur_plan(prhs, ctx->ks64, s);
       }
-      launch_resid_schur2d<T>(b, x, w.r[0], r64_keep, ctx->rpart, ctx->coef, want_b, s);
+      if (ctx->dim == 2)
+        launch_resid_schur2d<T>(b, x, w.r[0], r64_keep, ctx->rpart, ctx->coef, want_b, f64, s);
+      else if (!launch_resid_schur3d<T>(b, x, w.r[0], r64_keep, ctx->rpart, ctx->coef, want_b, f64, s))
+        return fail(ctx, APFC_ECUDA, "the residual kernel cannot be launched");
       plan.have = want_b ? 3 : 1;
       launch_schur_plan(plan, ctx->ks64, s);
     }
@@ -885,7 +896,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       break;
     }
     for (int p = 0; p < np; ++p)
-      if (!launch_schur_pass<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, p, s))
+      if (!launch_schur_pass<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, p, s, ctx->sms))
         return fail(ctx, APFC_ECUDA, "the Chebyshev pass cannot be launched");
     if (np > 0) total += (nt0 + ni * np + 1) / 2;  // two applications, as in a BiCGStab iteration
   }

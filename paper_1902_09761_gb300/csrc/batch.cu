@@ -60,6 +60,12 @@ struct apfc_batch {
   double* rpart = nullptr;   // residual kernel partials, [run][J][2][npart_r]
   void* part_fix = nullptr;  // right-hand-side kernel partials: R J kDotSlots kDotBlocks slots
   SchurCoef schur{};
+  bool schur_ok = false;
+  // runs stepped alone where the Chebyshev iteration does not serve (very fine grids, tolerances
+  // beneath its residual's noise), each by a context of its own; fresh[r]: it holds run r's state
+  std::vector<apfc_ctx*> alone;
+  std::vector<char> fresh;
+  double2* field = nullptr;  // [J][pts] of the largest run
   KScal* ks64 = nullptr;
   KScal* ks64_host = nullptr;
   double* epart = nullptr;
@@ -139,10 +145,9 @@ bool set_coef(apfc_batch* b, double dt, std::string& e) {
   if (b->coef_dt == dt) return true;
   if (!make_coef(b->lat, b->par, b->gmax, b->opts.tau_mode, dt, b->coef, e)) return false;
   b->cw = cheb_weights_for(b->coef, b->gmax, b->opts.cheb_degree);
-  if (!schur_build(b->coef, b->gmax, b->opts.cheb_degree, b->schur)) {
-    e = "the Schur complement's spectrum is not positive and finite";
-    return false;
-  }
+  b->schur_ok = schur_build(b->coef, b->gmax, b->opts.cheb_degree, b->schur) && schur_resid_ok(b->schur, b->opts.tol);
+  for (int j = 0; j < b->J && b->schur_ok; ++j)
+    b->schur_ok = schur_terms(b->opts.tol_inner, b->schur.lnrate[j]) <= 2LL * b->opts.max_iter;
   b->coef_dt = dt;
   set_rows(b);
   drop_graphs(b);  // the captured launches hold the coefficients by value
@@ -164,7 +169,7 @@ bool issue_passes(apfc_batch* b, int np, int tile, int rows) {
   const GaugeTab<float> gt{b->tab, b->gmax.n[0] + 1, b->gmax.n[1] + 1, 0};
   const ChebBufs<float> bufs{b->r[0], {b->r[0], b->r[1]}, {b->d[0], b->d[1]}, b->u, b->x64, b->ks64};
   for (int p = 0; p < np; ++p)
-    if (!launch_schur_pass<float>(b->schur, m, tile, b->coef, b->cw.data(), gt, rows, bufs, p, b->stream, &b->bl))
+    if (!launch_schur_pass<float>(b->schur, m, tile, b->coef, b->cw.data(), gt, rows, bufs, p, b->stream, b->sms, &b->bl))
       return false;
   return true;
 }
@@ -178,11 +183,11 @@ apfc_status sync_ks(apfc_batch* b) {
 
 SchurPlan plan_of(const apfc_batch* b) {
   SchurPlan p{};
-  const int m = b->opts.cheb_degree, ni = schur_ni<float>(b->schur, m);
+  const int m = b->opts.cheb_degree, ni = schur_ni<float>(b->schur, 2, m);
   p.tol = b->opts.tol;
   p.tol_inner = b->opts.tol_inner;
   for (int j = 0; j < b->J; ++j) p.lnrate[j] = b->schur.lnrate[j];
-  p.t0 = schur_t0<float>(b->schur, m);
+  p.t0 = schur_t0<float>(b->schur, 2, m);
   p.ni = ni;
   p.max_pass = (int)std::min<long long>(1 << 30, std::max(1LL, (2LL * b->opts.max_iter - p.t0 + ni - 1) / ni));
   p.J = b->J;
@@ -220,8 +225,66 @@ apfc_status solve(apfc_batch* b, int np) {
   return APFC_OK;
 }
 
+// One part (0 zeta, 1 eta) of run r's block <-> a contiguous field.
+apfc_status copy_field(apfc_batch* b, int r, int part, bool to_state) {
+  const RunGeom& g = b->rg[r];
+  const size_t row = sizeof(double2) * (size_t)g.pts;
+  double2* blk = b->x64 + g.elem_off + part * g.pts;
+  if (to_state)
+    BK(cudaMemcpy2DAsync(blk, 2 * row, b->field, row, row, b->J, cudaMemcpyDeviceToDevice, b->stream));
+  else
+    BK(cudaMemcpy2DAsync(b->field, row, blk, 2 * row, row, b->J, cudaMemcpyDeviceToDevice, b->stream));
+  return APFC_OK;
+}
+
+// One step of size dt of every run on its own context.
+apfc_status alone_step(apfc_batch* b, double dt) {
+  if (b->alone.empty()) {
+    b->alone.assign(b->R, nullptr);
+    b->fresh.assign(b->R, 0);
+    long long most = 0;
+    for (const RunGeom& g : b->rg) most = std::max(most, g.pts);
+    BK(cudaMalloc(&b->field, sizeof(double2) * (size_t)b->J * (size_t)most));
+  }
+  b->have_prev = false;
+  for (int r = 0; r < b->R; ++r) {
+    apfc_ctx*& c = b->alone[r];
+    apfc_status st = APFC_OK;
+    auto run_fail = [&](const std::string& what) {
+      return bfail(b, st, "run " + std::to_string(r) + ": " + what);
+    };
+    if (c == nullptr) {
+      const apfc_grid g{{b->nx[r], b->ny[r], 1}, {b->gmax.h[0], b->gmax.h[1], 1.0}};
+      if ((st = apfc_init(&c, &b->lat, &b->par, &g, &b->opts, b->stream)) != APFC_OK)
+        return run_fail(apfc_last_error(nullptr));
+    }
+    if (!b->fresh[r]) {
+      if ((st = apfc_set_opts(c, &b->opts)) != APFC_OK) return run_fail(apfc_last_error(c));
+      if ((st = copy_field(b, r, 1, false)) != APFC_OK) return st;
+      if ((st = apfc_set_amplitudes(c, b->field, APFC_DEVICE, APFC_C128)) != APFC_OK) return run_fail(apfc_last_error(c));
+      b->fresh[r] = 1;
+    }
+    if ((st = apfc_step(c, dt, 1)) != APFC_OK) return run_fail(apfc_last_error(c));
+    apfc_stats_t one;
+    apfc_stats(c, &one);
+    apfc_stats_t& t = b->stats[r];
+    t.steps += 1;
+    t.iters_last = one.iters_last;
+    t.iters_total += one.iters_last;
+    t.refine_last = one.refine_last;
+    t.resid_last = one.resid_last;
+    if ((st = apfc_get_amplitudes(c, b->field, APFC_DEVICE, APFC_C128)) != APFC_OK) return run_fail(apfc_last_error(c));
+    if ((st = copy_field(b, r, 1, true)) != APFC_OK) return st;
+    if ((st = apfc_get_zeta(c, b->field, APFC_DEVICE)) != APFC_OK) return run_fail(apfc_last_error(c));
+    if ((st = copy_field(b, r, 0, true)) != APFC_OK) return st;
+  }
+  return APFC_OK;
+}
+
 // One step of every run: FP32 Chebyshev solves inside FP64 iterative refinement.
 apfc_status batch_step(apfc_batch* b) {
+  if (!b->schur_ok) return alone_step(b, b->coef_dt);
+  std::fill(b->fresh.begin(), b->fresh.end(), 0);
   cudaStream_t s = b->stream;
   double* part = reinterpret_cast<double*>(b->part_fix);
   bool resid_ready = false;
@@ -254,7 +317,7 @@ apfc_status batch_step(apfc_batch* b) {
   for (;; ++sweep) {
     if (sweep == 0) launch_schur_plan(prhs, b->ks64, s, &b->bl);
     if (!resid_ready) {
-      launch_resid_schur2d<float>(b->b64, b->x64, b->r[0], b->r64_prev, b->rpart, b->coef, false, s, &b->bl);
+      launch_resid_schur2d<float>(b->b64, b->x64, b->r[0], b->r64_prev, b->rpart, b->coef, false, schur_resid_f64(b->schur, b->opts.tol), s, &b->bl);
       launch_schur_plan(plan, b->ks64, s, &b->bl);
     }
     resid_ready = false;
@@ -338,6 +401,8 @@ void free_batch(apfc_batch* b) {
   for (auto& p : b->d) cudaFree(p);
   cudaFree(b->u);
   cudaFree(b->tab);
+  for (apfc_ctx* c : b->alone) apfc_destroy(c);
+  cudaFree(b->field);
   cudaFree(b->rpart);
   cudaFree(b->part_fix);
   cudaFree(b->ks64);
@@ -488,6 +553,7 @@ apfc_status apfc_batch_set_opts(apfc_batch* b, const apfc_opts* opts) {
   std::string e;
   if (!valid_batch_opts(*opts, e)) return bfail(b, APFC_EINVAL, e);
   b->opts = *opts;
+  std::fill(b->fresh.begin(), b->fresh.end(), 0);
   const double dt = b->coef_dt;
   b->coef_dt = -1.0;  // tau_mode or the degree may have changed
   if (!set_coef(b, dt > 0 ? dt : 1.0, e)) return bfail(b, APFC_EINVAL, e);
@@ -509,6 +575,7 @@ apfc_status apfc_batch_set_amplitudes(apfc_batch* b, int run, const void* eta, i
   BK(cudaStreamSynchronize(b->stream));
   b->has_state[run] = 1;
   b->have_prev = false;
+  if (!b->fresh.empty()) b->fresh[run] = 0;
   b->failed = false;  // as on a context: new amplitudes clear a sticky error
   b->err.clear();
   b->stats[run] = apfc_stats_t{};
@@ -568,12 +635,18 @@ apfc_status apfc_batch_autotune(apfc_batch* b, double dt, int* tile_out, int* ro
     if (!b->has_state[r]) return bfail(b, APFC_ESTATE, "no amplitudes set for run " + std::to_string(r));
   std::string e;
   if (!set_coef(b, dt, e)) return bfail(b, APFC_EINVAL, e);
+  if (!b->schur_ok) {  // the runs are stepped alone: nothing to choose
+    if (tile_out) *tile_out = b->opts.tile;
+    if (rows_out) *rows_out = rows_of(b);
+    if (ms_out) *ms_out = 0.0;
+    return APFC_OK;
+  }
   cudaStream_t s = b->stream;
   // the first refinement residual of a step from the current state is the right-hand side
   // every candidate iterates on; u is never added to the state (the passes stop before the
   // last of the ks64[].iters set here)
   launch_rhs(b->x64, b->b64, b->coef, b->nt, s, &b->bl);
-  launch_resid_schur2d<float>(b->b64, b->x64, b->r[0], nullptr, b->rpart, b->coef, false, s, &b->bl);
+  launch_resid_schur2d<float>(b->b64, b->x64, b->r[0], nullptr, b->rpart, b->coef, false, schur_resid_f64(b->schur, b->opts.tol), s, &b->bl);
   b->have_prev = false;
   std::memset(b->ks64_host, 0, sizeof(KScal) * b->R * b->J);
   for (int i = 0; i < b->R * b->J; ++i) b->ks64_host[i].iters = kTunePasses + 1;

@@ -1211,12 +1211,11 @@ void launch_extrapolate(double2* x, double2* xp, const OpCoef& c, cudaStream_t s
 }
 
 void launch_zeta(double2* x, const OpCoef& c, cudaStream_t s) {
-  if (c.dim == 3) {
-    launch3d_zeta(x, c, s);
-    return;
-  }
   ProfScope ps_(KID_ZETA, s);
-  k_zeta<2><<<grid_pts3(c), kThreads, 0, s>>>(x, c);
+  if (c.dim == 3)
+    k_zeta<3><<<grid_pts3(c), kThreads, 0, s>>>(x, c);
+  else
+    k_zeta<2><<<grid_pts3(c), kThreads, 0, s>>>(x, c);
 }
 void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const double2* r_prev, float2* r32,
                       double* partials, const OpCoef& c, const NonlinTable& nt, bool schur, cudaStream_t s,

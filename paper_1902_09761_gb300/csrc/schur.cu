@@ -150,8 +150,16 @@ bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s) {
     s.lmax[j] = c.a[j] + c.kt[j] * g * g;
     kappa = std::max(kappa, s.lmax[j] / s.lmin[j]);
   }
+  s.kappa = kappa;
   if (!finish(s)) return false;
-  if (!(kappa > 40.0) || c.dim != 2) return true;
+  if (c.dim == 3) {
+    // no preconditioned variant: on fine grids, where a solve would need about 100 terms, an
+    // iteration of BiCGStab with its preconditioner costs 7 (FP64) to 11 (FP32) of them
+    for (int j = 0; j < c.J; ++j)
+      if (s.lnrate[j] < 0.1) return false;
+    return true;
+  }
+  if (!(kappa > 40.0)) return true;
   schur_spectrum(c, grid, m, q.lmin, q.lmax);
   if (!finish(q)) return true;
   double slow_q = 1e300;
@@ -159,6 +167,7 @@ bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s) {
     slow = std::min(slow, s.lnrate[j]);
     slow_q = std::min(slow_q, q.lnrate[j]);
   }
+  q.kappa = kappa;
   if (slow_q > 2.0 * slow) s = q;
   return true;
 }
@@ -287,8 +296,8 @@ __global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, in
 // G_h eta at row t - 1 and r at row t - 2 of its column, the y-neighbours in registers (the row
 // below is the one just formed), the x-neighbours from two-row shared-memory rings.  Every
 // double is split once.  Writes zeta into the state (the solve never reads it, so it always
-// belongs to the latest eta), r as FP32 (RED: or FP64), optionally r in FP64, and per block the
-// sums ||r||^2 and, on request, ||b||^2.
+// belongs to the latest eta), r as RT, optionally r in FP64, and per block the sums ||r||^2 and,
+// on request, ||b||^2.  F64: in FP64 arithmetic (see SchurCoef::kappa), bound by the FP64 pipe.
 // ---------------------------------------------------------------------------
 constexpr int kRsNT = 256, kRsPF = 2, kRsV = kRsNT - 4;
 
@@ -318,9 +327,9 @@ __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src));
 }
 
-template <bool F64>
+template <bool F64, typename RT>
 __global__ void __launch_bounds__(kRsNT, 2)
-    k_resid_schur2d(const double2* __restrict__ b, double2* x, void* r_out, double2* __restrict__ r64,
+    k_resid_schur2d(const double2* __restrict__ b, double2* x, RT* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
                     int want_b, const RunGeom* rg) {
   using RV = RsVal<F64>;
@@ -350,14 +359,13 @@ __global__ void __launch_bounds__(kRsNT, 2)
   const int sy = blockIdx.x / nstrips, sx = blockIdx.x - sy * nstrips;
   if (c.prof != nullptr && blockIdx.x == 0 && t == 0)
     atomicAdd(c.prof + KID_RESID_REFINE,
-              (unsigned long long)pts * (3 * sizeof(double2) + (F64 ? sizeof(double2) : sizeof(float2)) +
+              (unsigned long long)pts * (3 * sizeof(double2) + sizeof(RT) +
                                          (r64 != nullptr ? sizeof(double2) : 0)));
   double2* zt = x + 2LL * j * pts;
   const double2* et = zt + pts;
   const double2* bt = b + (2LL * j + 1) * pts;
   fo += (long long)j * pts;
-  [[maybe_unused]] float2* r32 = reinterpret_cast<float2*>(r_out) + fo;
-  [[maybe_unused]] double2* rd = reinterpret_cast<double2*>(r_out) + fo;
+  r_out += fo;
   if (r64 != nullptr) r64 += fo;
 
   [[maybe_unused]] ResidCoef<2> q;
@@ -440,7 +448,11 @@ __global__ void __launch_bounds__(kRsNT, 2)
           const double Gx = lx - (ax * (zr.y - zl.y) + ay * (z0.y - z2.y));
           const double Gy = ly + (ax * (zr.x - zl.x) + ay * (z0.x - z2.x));
           const double2 rv = make_double2(bv.x - (kt * Gx + aa * e2.x), bv.y - (kt * Gy + aa * e2.y));
-          rd[p] = rv;
+          if constexpr (sizeof(RT) == 16)
+            r_out[p] = rv;
+          else
+            r_out[p] = make_float2((float)rv.x, (float)rv.y);
+          if (r64 != nullptr) r64[p] = rv;
           rrd += rv.x * rv.x + rv.y * rv.y;
           if (want_b) bbd += bv.x * bv.x + bv.y * bv.y;
         } else {
@@ -455,7 +467,7 @@ __global__ void __launch_bounds__(kRsNT, 2)
           a.fma(ma.h, ma.l, e2);
           float2 f, l;
           a.result(f, l);
-          r32[p] = f;
+          r_out[p] = f;
           if (r64 != nullptr) r64[p] = make_double2(df_to_d(DF{f.x, l.x}), df_to_d(DF{f.y, l.y}));
           rr = fmaf(f.x, f.x, fmaf(f.y, f.y, rr));
           if (want_b) bb = fmaf(bp.h.x, bp.h.x, fmaf(bp.h.y, bp.h.y, bb));
@@ -528,23 +540,29 @@ int schur_resid_parts(int nx, int ny, int J) {
 
 template <typename T>
 void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
-                          bool want_b, cudaStream_t s, const BatchLaunch* bl) {
+                          bool want_b, bool f64, cudaStream_t s, const BatchLaunch* bl) {
   ProfScope ps_(KID_RESID_REFINE, s);
-  constexpr bool F64 = sizeof(T) == 8;
+  const int Ly = schur_resid_rows(c.nx, c.ny, c.J);
+  const int ns = (c.nx + kRsV - 1) / kRsV, ng = (c.ny + Ly - 1) / Ly;
+  dim3 grid(ns * ng, c.J);
   if (bl != nullptr) {
     int most = 0;
     for (int i = 0; i < bl->R; ++i) most = std::max(most, bl->host[i].npart_r);
-    k_resid_schur2d<F64><<<dim3(most, c.J, bl->R), kRsNT, 0, s>>>(b, x, r, r64, part, c, 0, 0, 0, want_b, bl->dev);
-    return;
+    grid = dim3(most, c.J, bl->R);
   }
-  const int Ly = schur_resid_rows(c.nx, c.ny, c.J);
-  const int ns = (c.nx + kRsV - 1) / kRsV, ng = (c.ny + Ly - 1) / Ly;
-  k_resid_schur2d<F64><<<dim3(ns * ng, c.J), kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, nullptr);
+  const RunGeom* rg = bl != nullptr ? bl->dev : nullptr;
+  if constexpr (sizeof(T) == 4) {
+    if (!f64) {
+      k_resid_schur2d<false, float2><<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
+      return;
+    }
+  }
+  k_resid_schur2d<true, cplx<T>><<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
 }
 template void launch_resid_schur2d<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool,
-                                          cudaStream_t, const BatchLaunch*);
+                                          bool, cudaStream_t, const BatchLaunch*);
 template void launch_resid_schur2d<double>(const double2*, double2*, double2*, double2*, double*, const OpCoef&, bool,
-                                           cudaStream_t, const BatchLaunch*);
+                                           bool, cudaStream_t, const BatchLaunch*);
 
 template <typename T>
 void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s) {

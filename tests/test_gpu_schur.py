@@ -27,8 +27,9 @@ def lib():
 
 
 def _steps(shape, h, n, bound, dt=1.0, seed=81, **opts):
-    ctx, L = context("hex", shape, h, **opts)
-    eta = inputs.random_amplitudes(3, shape, seed=seed, scale=0.15)
+    kind = "hex" if len(shape) == 2 else "bcc"
+    ctx, L = context(kind, shape, h, **opts)
+    eta = inputs.random_amplitudes(L.J, shape, seed=seed, scale=0.15 if kind == "hex" else 0.1)
     ctx.set_amplitudes(eta)
     for _ in range(n):
         ctx.step(dt)
@@ -98,3 +99,40 @@ def test_batch_on_a_fine_grid_equals_the_runs_alone():
         ctx.step(1.0, 2)
         assert np.array_equal(ctx.get_amplitudes(), got[r]), s
         ctx.close()
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("shape", [(3, 3, 3), (4, 3, 5), (9, 16, 32), (5, 17, 33), (70, 31, 30), (21, 33, 67), (16, 40, 64)])
+def test_3d_grids_around_tile_and_halo_widths(prec, shape):
+    # tiles of 32 x 16 points: exact, one point more, one less; grids smaller than the halo of
+    # two; odd rows take single-value copies.  cond(S) < 50 at h = pi/2 in 3D
+    _steps(shape, (np.pi / 2,) * 3, 2, 1e-10, tol=1e-13, precision=prec)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("shape", [(12, 8, 64), (20, 12, 40), (70, 13, 67)])
+def test_3d_per_pass_bicgstab(prec, shape):
+    # fused = 0 keeps the per-pass kernels (TMA-staged planes where nx % 64 == 0 and ny % 8 == 0)
+    _steps(shape, (1.0, 1.3, 0.9), 2, 1e-10, dt=0.5, tol=1e-13, precision=prec, fused=0, cheb_degree=2)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+def test_3d_fine_grid_falls_back_to_bicgstab(prec):
+    # at h = 0.35 a solve would need more than 100 terms; cond(S) < 9100 there
+    _steps((10, 12, 16), (0.35,) * 3, 1, 2e-8, tol=1e-12, precision=prec)
+
+
+def test_batch_beyond_the_chebyshev_iteration_steps_its_runs_alone():
+    # tol below the noise of the Schur residual on this grid (kappa about 1100): BiCGStab
+    L = O.hex_lattice()
+    shapes, h = [(24, 28), (20, 33)], (0.5, 0.5)
+    o = A.apfc_default_opts(precision=A.APFC_FP32_REFINED, tol=5e-13)
+    states = [inputs.random_amplitudes(3, s, seed=95 + r, scale=0.15) for r, s in enumerate(shapes)]
+    with A.Batch(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), shapes, h, o) as b:
+        for r, e in enumerate(states):
+            b.set_amplitudes(r, e)
+        b.step(1.0, 2)
+        for r, s in enumerate(shapes):
+            ref = O.run(states[r], 1.0, 2, P, L, h)[-1]
+            assert max(rel_l2_per_amp(b.get_amplitudes(r), ref)) <= 2e-9
+            assert b.stats(r)["resid_last"] <= 5e-13 and b.stats(r)["steps"] == 2
