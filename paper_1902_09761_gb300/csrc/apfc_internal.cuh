@@ -437,12 +437,12 @@ int schur_auto_rows(const SchurCoef& sc, const int* nx, const int* ny, int n, in
 template <typename T>
 bool launch_cheb2d(int m, const OpCoef& c, const ChebStep* w, const ChebPass& cp, int Ly, const ChebBufs<T>& b,
                    int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
-template <typename T>
-bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Ly,
-                    const ChebBufs<T>& b, int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
-template <typename T>
-bool launch_gauge3d(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, const ChebBufs<T>& b, int pass,
-                    int sms, cudaStream_t s);
+bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
+                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
+bool launch_gauge3d(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
+                    int pass, int sms, cudaStream_t s);
+bool launch_gauge64(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeights& w, const ChebBufs<double>& b,
+                    int pass, cudaStream_t s);
 // tab[j][d][i] = e^{i phi_d i}, 0 <= i <= n_d (sizes of GaugeTab)
 template <typename T>
 void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s);
@@ -452,9 +452,12 @@ bool launch_schur_pass(const SchurCoef& sc, int m, int tile, const OpCoef& c, co
                        const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int pass, cudaStream_t s,
                        int sms, const BatchLaunch* bl = nullptr) {
   const int ni = schur_ni<T>(sc, c.dim, m);
-  if (c.dim == 3) return launch_gauge3d<T>(c, gt, gauge_weights(sc, c.J, pass, ni), b, pass, sms, s);
-  return sc.plain ? launch_gauge2d<T>(tile, c, gt, gauge_weights(sc, c.J, pass, ni), Ly, b, pass, s, bl)
-                  : launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, pass, ni), Ly, b, pass, s, bl);
+  if (!sc.plain) return launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, pass, ni), Ly, b, pass, s, bl);
+  const GaugeWeights gw = gauge_weights(sc, c.J, pass, ni);
+  if constexpr (sizeof(T) == 8)
+    return launch_gauge64(c, gt, gw, b, pass, s);
+  else
+    return c.dim == 3 ? launch_gauge3d(c, gt, gw, b, pass, sms, s) : launch_gauge2d(tile, c, gt, gw, Ly, b, pass, s, bl);
 }
 // r = b - (a + kt G^2) eta from the eta-parts of x, b; zeta = G eta written into x; r [J][pts] in
 // T, r64 (nullable) the same in FP64; part [J][2][schur_resid_parts] sums of ||r||^2, ||b||^2;

@@ -20,9 +20,8 @@ bool go(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int L
 
 // Strips of 128 columns (tiles 0, 1, 3) or 256 (2, 4, 5): as fast at 4096^2, the narrow ones ahead
 // on grids that give an SM few blocks (1024^2: 37 against 51 us a pass).
-template <>
-bool launch_gauge2d<float>(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
-                           const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl) {
+bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
+                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl) {
   return tile == 2 || tile == 4 || tile == 5 ? go<128>(c, gt, w, Ly, b, pass, s, bl)
                                              : go<64>(c, gt, w, Ly, b, pass, s, bl);
 }

@@ -16,11 +16,14 @@ namespace apfc {
 
 namespace {
 
-template <typename T, int V_, int TXV_, int TYV_, int PF_, bool START_>
+// A warp spans a row of the tile with its halo (32 lanes of V points), so that shared-memory
+// accesses have no bank conflicts (36-column tiles with rows across warps took two wavefronts for
+// each) and rows are uniform over a warp.
+template <typename T, int V_, int TYV_, int PF_, bool START_>
 struct Gauge3Shape {
-  static constexpr int V = V_, TXV = TXV_, TYV = TYV_, PF = PF_;
-  static constexpr int OX = TXV + 4, OY = TYV + 4;   // tile with its halo
-  static constexpr int PX = OX / V, NT = PX * (OY / 2);
+  static constexpr int V = V_, TYV = TYV_, PF = PF_;
+  static constexpr int OX = 32 * V, TXV = OX - 4, OY = TYV + 4;  // tile with its halo
+  static constexpr int PX = 32, NT = PX * (OY / 2);
   static constexpr int RW = PX + 2, PLANE = (OY + 2) * RW;  // one part of a ring plane, padded
   static constexpr int SLOTS = PF + 1;
   static constexpr size_t ring_elems = 2ull * 2 * V * PLANE;  // v, g' x two planes
@@ -46,13 +49,13 @@ struct Gauge3Param {
 
 // Grid (tiles, z-chunks, J).  START: v is the residual; forms b (negated) and v_1, writes both
 // and v_2.  vp: v_(n-1) in, v_(n+1) out (START: v_2); v1_out: START's v_1.
-template <typename T, int V, int TXV, int TYV, int PF, int MINB, bool START>
-__global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MINB)
+template <typename T, int V, int TYV, int PF, int MINB, bool START>
+__global__ void __launch_bounds__(Gauge3Shape<T, V, TYV, PF, START>::NT, MINB)
     k_gauge3d(const __grid_constant__ Gauge3Param<T> c, Gauge3Geom g, const cplx<T>* v_in, cplx<T>* vp, cplx<T>* b_io,
               cplx<T>* v1_out, double2* x64, const KScal* ks, int pass, int kid) {
-  using SH = Gauge3Shape<T, V, TXV, TYV, PF, START>;
+  using SH = Gauge3Shape<T, V, TYV, PF, START>;
   using C = cplx<T>;
-  constexpr int NT = SH::NT, PX = SH::PX, OX = SH::OX, OY = SH::OY, RW = SH::RW, PLANE = SH::PLANE;
+  constexpr int NT = SH::NT, TXV = SH::TXV, OX = SH::OX, OY = SH::OY, RW = SH::RW, PLANE = SH::PLANE;
   extern __shared__ __align__(16) unsigned char gauge3_smem[];
   C* ring = reinterpret_cast<C*>(gauge3_smem);  // [v, g'][2 planes][V][PLANE]
   C* stg = ring + SH::ring_elems;               // [SLOTS][NT][2][V]
@@ -81,40 +84,32 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
 
   // cells: columns V px .. of rows 2 ry and 2 ry + 1 of the tile; positions beyond the grid are
   // the periodic image times the wraps' phases
-  const int ry = t / PX, px = t - ry * PX;
+  const int ry = __shfl_sync(0xffffffffu, t >> 5, 0), px = t & 31;  // row pair: uniform over the warp
   const int tyi = blockIdx.x / g.ntx, txi = blockIdx.x - tyi * g.ntx;
   const int X0 = txi * TXV - 2 + V * px, Y0 = tyi * TYV - 2 + 2 * ry;
-  int gx[V], goff[2];
-  bool wrapped = false, own[2][V];
-  C fac[2][V], ph[2][V];  // wraps' phase in (x, y); e^{i phi.(x, y)}
-  {
-    const C ex = tabx[g.nx], ey = taby[g.ny];
-    C fx[V];
+  int gx[V], gyr[2], goff[2];
+  bool wrapped = false, xown[V], yown[2];
+  C colf[V], rowf[2];
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      int x = (X0 + v) % g.nx;
-      if (x < 0) x += g.nx;
-      gx[v] = x;
-      fx[v] = g_pow(ex, (X0 + v - x) / g.nx, one);
-      wrapped = wrapped || X0 + v != x;
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      int y = (Y0 + r) % g.ny;
-      if (y < 0) y += g.ny;
-      goff[r] = y * g.nx;
-      const C fy = g_pow(ey, (Y0 + r - y) / g.ny, one);
-      wrapped = wrapped || Y0 + r != y;
-      const bool yo = 2 * ry + r >= 2 && 2 * ry + r < OY - 2 && Y0 + r < g.ny;
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        fac[r][v] = g_cmul(fx[v], fy);
-        own[r][v] = yo && V * px + v >= 2 && V * px + v < OX - 2 && X0 + v < g.nx;
-        ph[r][v] = one;
-        if (START || last) ph[r][v] = g_cmul(g_cmul(tabx[gx[v]], taby[y]), fac[r][v]);
-      }
-    }
+  for (int v = 0; v < V; ++v) {
+    int x = (X0 + v) % g.nx;
+    if (x < 0) x += g.nx;
+    gx[v] = x;
+    colf[v] = g_pow(tabx[g.nx], (X0 + v - x) / g.nx, one);
+    wrapped = wrapped || X0 + v != x;
+    xown[v] = V * px + v >= 2 && V * px + v < OX - 2 && X0 + v < g.nx;
   }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    int y = (Y0 + r) % g.ny;
+    if (y < 0) y += g.ny;
+    gyr[r] = y;
+    goff[r] = y * g.nx;
+    rowf[r] = g_pow(taby[g.ny], (Y0 + r - y) / g.ny, one);
+    wrapped = wrapped || Y0 + r != y;
+    yown[r] = 2 * ry + r >= 2 && 2 * ry + r < OY - 2 && Y0 + r < g.ny;
+  }
+  const bool rows_own = yown[0] || yown[1];  // stage B's rows: the warps of the halo skip it
   const bool vec = V == 1 || (g.nx & 1) == 0;
   const long long plane = (long long)g.nx * g.ny;
   const int z0 = blockIdx.y * g.Lz, nzc = min(g.nz, z0 + g.Lz) - z0, steps = nzc + 4;
@@ -152,17 +147,17 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
     for (int r = 0; r < 2; ++r) {
       const C* p = src + zo + goff[r] + gx[0];
       if constexpr (V == 1) {
-        if (own[r][0]) d[r][0] = p[0];
+        if (yown[r] && xown[0]) d[r][0] = p[0];
       } else {
         if (vec) {
-          if (own[r][0]) {
+          if (yown[r] && xown[0]) {
             const float4 w = *reinterpret_cast<const float4*>(p);
             d[r][0] = make_float2(w.x, w.y);
             d[r][1] = make_float2(w.z, w.w);
           }
         } else {
-          if (own[r][0]) d[r][0] = p[0];
-          if (own[r][1]) d[r][1] = src[zo + goff[r] + gx[1]];
+          if (yown[r] && xown[0]) d[r][0] = p[0];
+          if (yown[r] && xown[V - 1]) d[r][1] = src[zo + goff[r] + gx[V - 1]];
         }
       }
     }
@@ -172,13 +167,13 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
     for (int r = 0; r < 2; ++r) {
       C* p = dst + zo + goff[r] + gx[0];
       if constexpr (V == 1) {
-        if (own[r][0]) p[0] = d[r][0];
+        if (yown[r] && xown[0]) p[0] = d[r][0];
       } else {
         if (vec) {
-          if (own[r][0]) *reinterpret_cast<float4*>(p) = make_float4(d[r][0].x, d[r][0].y, d[r][1].x, d[r][1].y);
+          if (yown[r] && xown[0]) *reinterpret_cast<float4*>(p) = make_float4(d[r][0].x, d[r][0].y, d[r][1].x, d[r][1].y);
         } else {
-          if (own[r][0]) p[0] = d[r][0];
-          if (own[r][1]) dst[zo + goff[r] + gx[1]] = d[r][1];
+          if (yown[r] && xown[0]) p[0] = d[r][0];
+          if (yown[r] && xown[V - 1]) dst[zo + goff[r] + gx[V - 1]] = d[r][1];
         }
       }
     }
@@ -230,7 +225,8 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
       for (int r = 0; r < 2; ++r)
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-          const C w = g_cmul(g_cmul(pz, ph[r][v]), F[r][v]);
+          const C pr = g_cmul(pz, g_cmul(taby[gyr[r]], rowf[r]));
+          const C w = g_cmul(g_cmul(pr, g_cmul(tabx[gx[v]], colf[v])), F[r][v]);
           bt[r][v] = mkc<T>(-w.x, -w.y);
           F[r][v] = q_mul(q.mith, bt[r][v]);
         }
@@ -242,7 +238,7 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
 #pragma unroll
       for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int v = 0; v < V; ++v) F[r][v] = g_cmul(g_cmul(zf, fac[r][v]), F[r][v]);
+        for (int v = 0; v < V; ++v) F[r][v] = g_cmul(g_cmul(g_cmul(zf, rowf[r]), colf[v]), F[r][v]);
     }
     auto put = [&](int w, const C (&f)[2][V]) {
       C* d = ring + ((size_t)w * 2 + par) * V * PLANE + cell;
@@ -271,7 +267,7 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
     C G[2][V];
     stencil(0, v1, v2, F, nullptr, G);  // plane tt - 1
     put(1, G);
-    {
+    if (rows_own) {
       // r^ = a v - b + N g' at plane tt - 2
       C av[2 * V], rh[2][V], out[2][V];
 #pragma unroll
@@ -295,8 +291,8 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
           for (int r = 0; r < 2; ++r)
 #pragma unroll
             for (int v = 0; v < V; ++v) {
-              if (!own[r][v]) continue;
-              const C un = g_cmul(g_conj(g_cmul(pz, ph[r][v])), out[r][v]);
+              if (!(yown[r] && xown[v])) continue;
+              const C un = g_cmul(g_conj(g_cmul(g_cmul(pz, taby[gyr[r]]), tabx[gx[v]])), out[r][v]);
               double2* xp = x64 + zo + goff[r] + gx[v];
               double2 xv = *xp;
               if constexpr (sizeof(T) == 4) {
@@ -338,10 +334,11 @@ __global__ void __launch_bounds__(Gauge3Shape<T, V, TXV, TYV, PF, START>::NT, MI
   asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
-template <typename T, int V, int TXV, int TYV, int PF, int MINB, bool START>
+template <typename T, int V, int TYV, int PF, int MINB, bool START>
 bool launch_gauge3_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Lz, const ChebBufs<T>& b,
                         int pass, cudaStream_t s) {
-  using SH = Gauge3Shape<T, V, TXV, TYV, PF, START>;
+  using SH = Gauge3Shape<T, V, TYV, PF, START>;
+  constexpr int TXV = SH::TXV;
   static_assert(SH::OX % V == 0 && SH::OY % 2 == 0 && SH::NT <= 1024, "tile");
   const int kid = kid_of<T>(KID_FUSED_APINV);
   ProfScope ps_(kid, s);
@@ -365,7 +362,7 @@ bool launch_gauge3_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeigh
     a.mc2 = (T)(-w.c2[0][j]);
     a.mith = (T)(-w.inv_theta[j]);
   }
-  auto kern = k_gauge3d<T, V, TXV, TYV, PF, MINB, START>;
+  auto kern = k_gauge3d<T, V, TYV, PF, MINB, START>;
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::smem);
   if (attr != cudaSuccess) return false;
   // START: v_1 into r[1], v_2 into d[0]; pass p >= 1 reads v from d[0] / r[1] and replaces the other

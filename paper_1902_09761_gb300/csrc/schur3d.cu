@@ -302,19 +302,15 @@ static int gauge3_planes(const OpCoef& c, int txv, int tyv, int res, int sms) {
   return bl;
 }
 
-template <>
-bool launch_gauge3d<float>(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
-                           int pass, int sms, cudaStream_t s) {
-  const int Lz = gauge3_planes(c, 32, 16, 2, sms);
-  return pass == 0 ? launch_gauge3_pass<float, 2, 32, 16, 2, 2, true>(c, gt, w, Lz, b, pass, s)
-                   : launch_gauge3_pass<float, 2, 32, 16, 2, 2, false>(c, gt, w, Lz, b, pass, s);
-}
-template <>
-bool launch_gauge3d<double>(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeights& w,
-                            const ChebBufs<double>& b, int pass, int sms, cudaStream_t s) {
-  const int Lz = gauge3_planes(c, 32, 16, 1, sms);
-  return pass == 0 ? launch_gauge3_pass<double, 1, 32, 16, 2, 1, true>(c, gt, w, Lz, b, pass, s)
-                   : launch_gauge3_pass<double, 1, 32, 16, 2, 1, false>(c, gt, w, Lz, b, pass, s);
+// 60 x 12 points a tile, two blocks of 256 threads per SM, one plane ahead.  Measured at 256^3 x 6
+// (us a term; its 32 bytes a point take 481 at the copy rate): 718; 60 x 16 in one block 1005, in
+// two (spilled) 892, 60 x 28 750; with 36-column tiles (rows across warps, bank conflicts) 32 x 16
+// 744, 64 x 16 863.
+bool launch_gauge3d(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
+                    int pass, int sms, cudaStream_t s) {
+  const int Lz = gauge3_planes(c, 60, 12, 2, sms);
+  return pass == 0 ? launch_gauge3_pass<float, 2, 12, 1, 2, true>(c, gt, w, Lz, b, pass, s)
+                   : launch_gauge3_pass<float, 2, 12, 1, 2, false>(c, gt, w, Lz, b, pass, s);
 }
 
 }  // namespace apfc
