@@ -113,7 +113,10 @@ typedef struct {
   double tol;                /* stop at ||b - A x||_2 <= tol ||b||_2 (block norm, per amplitude) */
   double tol_inner;          /* relative tolerance of each FP32 inner solve         */
   int tile;                  /* fused 2D kernel variant 0..5 (columns per block and
-                                rows of look-ahead), default 3                     */
+                                rows of look-ahead), default 3: with it the FP32
+                                Chebyshev solves of small grids (up to about 900^2
+                                with three amplitudes) run on tiles, whatever
+                                tile_rows                                          */
   int tile_rows;             /* rows per block of the fused 2D kernels of the
                                 iteration; 0 (default): automatic, by the grid size
                                 (BiCGStab: the tallest of 128, 64, 32 rows that

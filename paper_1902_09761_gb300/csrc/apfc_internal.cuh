@@ -438,7 +438,18 @@ template <typename T>
 bool launch_cheb2d(int m, const OpCoef& c, const ChebStep* w, const ChebPass& cp, int Ly, const ChebBufs<T>& b,
                    int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
 bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
-                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl = nullptr);
+                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl, int take);
+// Two units (of kGaugeNI32 terms) on tiles of 40 x 56 points, one to a multiprocessor at a time:
+// shorter than two streamed passes up to some 1500 tiles (three amplitudes, us per unit against a
+// streamed pass: 256^2, 105 tiles, 5.6 against 13; 768^2, 840, 23 against 30; 1024^2, 1482, 38 against
+// 39; 1531 x 997, 2106, 59 against 58).
+constexpr int kTileUnits = 2, kTileX = 40, kTileY = 56;
+inline bool gauge_tiled(int nx, int ny, int J) {
+  const long long tx = (nx + kTileX - 1) / kTileX, ty = (ny + kTileY - 1) / kTileY;
+  return tx * ty * J <= 1200;
+}
+bool launch_gauge_tile(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
+                       int pass, int sms, cudaStream_t s, const BatchLaunch* bl);
 bool launch_gauge3d(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
                     int pass, int sms, cudaStream_t s);
 bool launch_gauge64(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeights& w, const ChebBufs<double>& b,
@@ -446,18 +457,42 @@ bool launch_gauge64(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeig
 // tab[j][d][i] = e^{i phi_d i}, 0 <= i <= n_d (sizes of GaugeTab)
 template <typename T>
 void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s);
-// pass `pass` of a solve, by either iteration
+// The first np passes of a solve, by either iteration; variant 3 takes the tiles where the grid is
+// small enough.
 template <typename T>
-bool launch_schur_pass(const SchurCoef& sc, int m, int tile, const OpCoef& c, const ChebStep* w,
-                       const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int pass, cudaStream_t s,
-                       int sms, const BatchLaunch* bl = nullptr) {
+bool launch_schur_passes(const SchurCoef& sc, int m, int tile, const OpCoef& c, const ChebStep* w,
+                         const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int np, cudaStream_t s, int sms,
+                         const BatchLaunch* bl = nullptr) {
   const int ni = schur_ni<T>(sc, c.dim, m);
-  if (!sc.plain) return launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, pass, ni), Ly, b, pass, s, bl);
-  const GaugeWeights gw = gauge_weights(sc, c.J, pass, ni);
-  if constexpr (sizeof(T) == 8)
-    return launch_gauge64(c, gt, gw, b, pass, s);
-  else
-    return c.dim == 3 ? launch_gauge3d(c, gt, gw, b, pass, sms, s) : launch_gauge2d(tile, c, gt, gw, Ly, b, pass, s, bl);
+  int take = 0;
+  if constexpr (sizeof(T) == 4) {
+    if (sc.plain && c.dim == 2 && tile == 3) {
+      int tiled = 0;
+      if (bl != nullptr)
+        for (int i = 0; i < bl->R; ++i) tiled += gauge_tiled(bl->host[i].nx, bl->host[i].ny, c.J);
+      else
+        tiled = gauge_tiled(c.nx, c.ny, c.J);
+      for (int p = 0; tiled > 0 && p * kTileUnits < np; ++p)
+        if (!launch_gauge_tile(c, gt, gauge_weights(sc, c.J, p, ni * kTileUnits), b, p, sms, s, bl)) return false;
+      if (tiled == (bl != nullptr ? bl->R : 1)) return true;
+      if (tiled > 0) take = -1;
+    }
+  }
+  for (int p = 0; p < np; ++p) {
+    bool ok;
+    if (!sc.plain) {
+      ok = launch_cheb2d<T>(m, c, w, schur_pass(sc, c.J, p, ni), Ly, b, p, s, bl);
+    } else {
+      const GaugeWeights gw = gauge_weights(sc, c.J, p, ni);
+      if constexpr (sizeof(T) == 8)
+        ok = launch_gauge64(c, gt, gw, b, p, s);
+      else
+        ok = c.dim == 3 ? launch_gauge3d(c, gt, gw, b, p, sms, s)
+                        : launch_gauge2d(tile, c, gt, gw, Ly, b, p, s, bl, take);
+    }
+    if (!ok) return false;
+  }
+  return true;
 }
 // r = b - (a + kt G^2) eta from the eta-parts of x, b; zeta = G eta written into x; r [J][pts] in
 // T, r64 (nullable) the same in FP64; part [J][2][schur_resid_parts] sums of ||r||^2, ||b||^2;

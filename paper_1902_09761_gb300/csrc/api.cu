@@ -895,9 +895,9 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       worst = KS_NOCONV;
       break;
     }
-    for (int p = 0; p < np; ++p)
-      if (!launch_schur_pass<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, p, s, ctx->sms))
-        return fail(ctx, APFC_ECUDA, "the Chebyshev pass cannot be launched");
+    if (!launch_schur_passes<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, np, s,
+                                ctx->sms))
+      return fail(ctx, APFC_ECUDA, "the Chebyshev passes cannot be launched");
     if (np > 0) total += (nt0 + ni * np + 1) / 2;  // two applications, as in a BiCGStab iteration
   }
   CK(cudaGetLastError());
@@ -1571,6 +1571,8 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
     const int rows = (ny + s - 1) / s;
     if (rows >= 32 && rows <= ny && std::find(cand.begin(), cand.end(), rows) == cand.end()) cand.push_back(rows);
   }
+  if (schur && ctx->schur.plain && ctx->opts.tile == 3 && gauge_tiled(ctx->grid.n[0], ny, ctx->J))
+    cand.resize(1);  // the tiles have no height
   const size_t blk = sizeof(double2) * 2 * (size_t)ctx->J * (size_t)ctx->pts;
   double2* saved = nullptr;
   if (cudaMalloc(&saved, blk) != cudaSuccess) {

@@ -168,10 +168,7 @@ bool issue_passes(apfc_batch* b, int np, int tile, int rows) {
   const int m = b->opts.cheb_degree;
   const GaugeTab<float> gt{b->tab, b->gmax.n[0] + 1, b->gmax.n[1] + 1, 0};
   const ChebBufs<float> bufs{b->r[0], {b->r[0], b->r[1]}, {b->d[0], b->d[1]}, b->u, b->x64, b->ks64};
-  for (int p = 0; p < np; ++p)
-    if (!launch_schur_pass<float>(b->schur, m, tile, b->coef, b->cw.data(), gt, rows, bufs, p, b->stream, b->sms, &b->bl))
-      return false;
-  return true;
+  return launch_schur_passes<float>(b->schur, m, tile, b->coef, b->cw.data(), gt, rows, bufs, np, b->stream, b->sms, &b->bl);
 }
 
 apfc_status sync_ks(apfc_batch* b) {

@@ -540,13 +540,16 @@ inline ChebGeom cheb_geom(int nx, int ny, int S, int NC, int Ly) {
   return g;
 }
 
-// The launch table of runs r0 .. of a batch; returns their count, the most blocks of one in *maxblk.
-inline int cheb_table(const BatchLaunch& bl, int r0, int S, int NC, int Ly, int J, ChebTab& tab, int& maxblk) {
+// The launch table of runs r0 .. of a batch; returns their count, the most blocks of one in maxblk.
+// take: all runs (0), those on tiles (1) or the others (-1; gauge_tiled).
+inline int cheb_table(const BatchLaunch& bl, int r0, int S, int NC, int Ly, int J, ChebTab& tab, int& maxblk,
+                      int take = 0) {
   const int nr = std::min(kChebRuns, bl.R - r0);
   std::memset(&tab, 0, sizeof(tab));
   maxblk = 0;
   for (int i = 0; i < nr; ++i) {
     const RunGeom& q = bl.host[r0 + i];
+    if (take != 0 && (take > 0) != gauge_tiled(q.nx, q.ny, J)) continue;
     const ChebGeom g = cheb_geom(q.nx, q.ny, S, NC, Ly);
     ChebRun& e = tab.run[i];
     e.pts = q.pts;

@@ -419,14 +419,8 @@ __global__ void __launch_bounds__(NT, MINB)
   asm volatile("cp.async.wait_group 0;\n" ::);
 }
 
-// One pass over one grid or, with bl, over every run of a batch.
-template <typename T, int NI, int V, int NT, int PF, int MINB, bool START>
-bool launch_gauge_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Ly, const ChebBufs<T>& b,
-                       int pass, cudaStream_t s, const BatchLaunch* bl) {
-  using SH = GaugeShape<T, NI, V, NT, PF, START>;
-  static_assert(NI <= kGaugeMaxNI && SH::S % V == 0 && (SH::NC - 2 * SH::S) % V == 0, "strips start on a pair");
-  const int kid = kid_of<T>(KID_FUSED_APINV);
-  ProfScope ps_(kid, s);
+template <typename T>
+GaugeParam<T> gauge_param(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int terms) {
   GaugeParam<T> in;
   std::memset(&in, 0, sizeof(in));
   in.prof = c.prof;
@@ -441,12 +435,24 @@ bool launch_gauge_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeight
     a.nx = (T)(sk * gauge_w(c, j, 0));
     a.ny = (T)(sk * gauge_w(c, j, 1));
     a.a = (T)c.a[j];
-    for (int i = 0; i < NI; ++i) {
+    for (int i = 0; i < terms; ++i) {
       a.c1[i] = (T)w.c1[i][j];
       a.mc2[i] = (T)(-w.c2[i][j]);
     }
     a.mith = (T)(-w.inv_theta[j]);
   }
+  return in;
+}
+
+// One pass over one grid or, with bl, over every run of a batch.
+template <typename T, int NI, int V, int NT, int PF, int MINB, bool START>
+bool launch_gauge_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeights& w, int Ly, const ChebBufs<T>& b,
+                       int pass, cudaStream_t s, const BatchLaunch* bl, int take = 0) {
+  using SH = GaugeShape<T, NI, V, NT, PF, START>;
+  static_assert(NI <= kGaugeMaxNI && SH::S % V == 0 && (SH::NC - 2 * SH::S) % V == 0, "strips start on a pair");
+  const int kid = kid_of<T>(KID_FUSED_APINV);
+  ProfScope ps_(kid, s);
+  const GaugeParam<T> in = gauge_param<T>(c, gt, w, NI);
   // fields: v in r / d by pass parity (r0 the residual), b in u
   const int cur = pass & 1;
   const cplx<T>* vin = START ? b.r0 : b.r[cur];
@@ -470,7 +476,8 @@ bool launch_gauge_pass(const OpCoef& c, const GaugeTab<T>& gt, const GaugeWeight
     for (int r0 = 0; r0 < bl->R; r0 += kChebRuns) {
       ChebTab tab;
       int maxblk = 0;
-      const int nr = cheb_table(*bl, r0, SH::S, SH::NC, Ly, c.J, tab, maxblk);
+      const int nr = cheb_table(*bl, r0, SH::S, SH::NC, Ly, c.J, tab, maxblk, take);
+      if (maxblk == 0) continue;
       kern<<<dim3(maxblk, nr), NT, SH::smem, s>>>(in, ChebGeom{0, 0, 0, SH::NC - 2 * SH::S, 0, 0, 0}, vin, b.d[cur],
                                                   b.r[1 - cur], b.d[1 - cur], b.u, b.x64, b.ks, pass, kid, tab);
     }

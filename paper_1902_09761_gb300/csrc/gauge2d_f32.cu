@@ -10,20 +10,20 @@ namespace {
 // registers, two blocks of 128 threads per SM); one point per thread 172 at best.
 template <int NT>
 bool go(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly, const ChebBufs<float>& b, int pass,
-        cudaStream_t s, const BatchLaunch* bl) {
+        cudaStream_t s, const BatchLaunch* bl, int take) {
   constexpr int MB = 384 / NT;
-  return pass == 0 ? launch_gauge_pass<float, kGaugeNI32, 2, NT, 3, MB, true>(c, gt, w, Ly, b, pass, s, bl)
-                   : launch_gauge_pass<float, kGaugeNI32, 2, NT, 3, MB, false>(c, gt, w, Ly, b, pass, s, bl);
+  return pass == 0 ? launch_gauge_pass<float, kGaugeNI32, 2, NT, 3, MB, true>(c, gt, w, Ly, b, pass, s, bl, take)
+                   : launch_gauge_pass<float, kGaugeNI32, 2, NT, 3, MB, false>(c, gt, w, Ly, b, pass, s, bl, take);
 }
 
 }  // namespace
 
-// Strips of 128 columns (tiles 0, 1, 3) or 256 (2, 4, 5): as fast at 4096^2, the narrow ones ahead
+// Strips of 128 columns (variants 0, 1, 3) or 256 (2, 4, 5): as fast at 4096^2, the narrow ones ahead
 // on grids that give an SM few blocks (1024^2: 37 against 51 us a pass).
 bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
-                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl) {
-  return tile == 2 || tile == 4 || tile == 5 ? go<128>(c, gt, w, Ly, b, pass, s, bl)
-                                             : go<64>(c, gt, w, Ly, b, pass, s, bl);
+                    const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl, int take) {
+  return tile == 2 || tile == 4 || tile == 5 ? go<128>(c, gt, w, Ly, b, pass, s, bl, take)
+                                             : go<64>(c, gt, w, Ly, b, pass, s, bl, take);
 }
 
 }  // namespace apfc

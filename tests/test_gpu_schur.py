@@ -136,3 +136,35 @@ def test_batch_beyond_the_chebyshev_iteration_steps_its_runs_alone():
             ref = O.run(states[r], 1.0, 2, P, L, h)[-1]
             assert max(rel_l2_per_amp(b.get_amplitudes(r), ref)) <= 2e-9
             assert b.stats(r)["resid_last"] <= 5e-13 and b.stats(r)["steps"] == 2
+
+
+@pytest.mark.parametrize("shape", [(56, 40), (57, 41), (55, 39), (112, 121), (23, 200), (7, 43), (331, 402)])
+def test_tiles_around_their_widths(shape):
+    # tiles own 40 columns of 56 rows and reach 12 further on each side: exact, one more, one less,
+    # grids that the reach wraps around, several tiles a block; odd rows take single-value copies
+    _steps(shape, H2, 2, 1e-10, tol=1e-13, precision=A.APFC_FP32_REFINED)
+
+
+@pytest.mark.parametrize("shape", [(3, 4), (40, 117), (131, 6), (16, 116)])
+def test_narrow_strips_on_small_grids(shape):
+    # variant 3 takes the tiles on these, variant 0 keeps the strips of 128 columns
+    _steps(shape, H2, 2, 1e-10, tol=1e-13, precision=A.APFC_FP32_REFINED, tile=0)
+
+
+def test_batch_of_tiled_and_streamed_runs_equals_the_runs_alone():
+    # 896 x 880 has 22 x 16 x 3 = 1056 tiles (tiled), 960 x 961 has 25 x 18 x 3 = 1350 (streamed)
+    L = O.hex_lattice()
+    shapes = [(896, 880), (40, 48), (960, 961), (33, 131)]
+    o = A.apfc_default_opts(precision=A.APFC_FP32_REFINED, tol=1e-12, tile_rows=64)
+    states = [inputs.random_amplitudes(3, s, seed=95 + r, scale=0.15) for r, s in enumerate(shapes)]
+    with A.Batch(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), shapes, H2, o) as b:
+        for r, e in enumerate(states):
+            b.set_amplitudes(r, e)
+        b.step(1.0, 2)
+        got = [b.get_amplitudes(r) for r in range(len(shapes))]
+    for r, s in enumerate(shapes):
+        ctx, _ = context("hex", s, H2, precision=A.APFC_FP32_REFINED, tol=1e-12, tile_rows=64)
+        ctx.set_amplitudes(states[r])
+        ctx.step(1.0, 2)
+        assert np.array_equal(ctx.get_amplitudes(), got[r]), s
+        ctx.close()
