@@ -35,31 +35,37 @@ struct DF {
 // (an absolute error below 1e-22, far under the precision of the sums these
 // values enter); NaN, Inf and |v| >= 2^127 give (NaN, 0) so that non-finite
 // states still surface as NaN residual norms.
+//
+// h is the double's sign, its exponent less 896 (the low 8 bits of E + 128) and 23 mantissa bits, all
+// in one funnel shift.  l's 29 bits are the mantissas of two floats a, b with exponents 23 and 29
+// below h's; a - A and b - B (A, B: the same floats with mantissa zero) are exact.  12 instructions
+// and the range check; the field-by-field form took about 26.
 __device__ __forceinline__ DF split_d(double v) {
   const unsigned hw = (unsigned)__double2hiint(v);
   const unsigned lw = (unsigned)__double2loint(v);
-  const unsigned E = (hw >> 20) & 0x7ffu;
-  const unsigned sign = hw & 0x80000000u;
-  if (E < 949u) return DF{0.f, 0.f};
-  if (E >= 1151u) return DF{__uint_as_float(0x7fc00000u), 0.f};
-  const float h = __uint_as_float(sign | ((E - 896u) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29));
-  const unsigned q = lw & 0x1fffffffu;  // low 29 mantissa bits, in units of 2^(E-1075)
-  // q >> 6 and q & 63 are below 2^23: exact floats by the 2^23 magic-number trick
-  const float qa = __fsub_rn(__uint_as_float(0x4B000000u | (q >> 6)), 8388608.f);
-  const float qb = __fsub_rn(__uint_as_float(0x4B000000u | (q & 63u)), 8388608.f);
-  const float qf = __fmaf_rn(qa, 64.f, qb);                    // q rounded to 24 bits
-  const float sc = __uint_as_float(sign | ((E - 948u) << 23));  // +-2^(E-1075), a normal float
-  return DF{h, __fmul_rn(qf, sc)};
+  unsigned h = ((__funnelshift_l(lw, hw, 3) + 0x40000000u) & 0x7fffffffu) | (hw & 0x80000000u);
+  const unsigned A = (h & 0xff800000u) - (23u << 23), B = A - (6u << 23);
+  const float la = __fsub_rn(__uint_as_float(A | ((lw >> 6) & 0x7fffffu)), __uint_as_float(A));
+  const float lb = __fsub_rn(__uint_as_float(B | (lw & 63u)), __uint_as_float(B));
+  float l = __fadd_rn(la, lb);  // rounded to 24 bits
+  const unsigned m = (hw & 0x7fffffffu) - (949u << 20);  // |v|'s exponent field above the least kept
+  if (m >= (202u << 20)) {
+    h = (int)m < 0 ? 0u : 0x7fc00000u;
+    l = 0.f;
+  }
+  return DF{__uint_as_float(h), l};
 }
 
 // Exact double of a float (zero and subnormal floats give 0, Inf and NaN give NaN).
 __device__ __forceinline__ double f2d(float f) {
-  const unsigned u = __float_as_uint(f);
-  const unsigned e = (u >> 23) & 0xffu;
-  if (e == 0u) return 0.0;
-  if (e == 255u) return __hiloint2double(0x7ff80000, 0);
-  const unsigned hi = (u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7fffffu) >> 3);
-  return __hiloint2double((int)hi, (int)(u << 29));
+  const unsigned u = __float_as_uint(f), t = u & 0x7f800000u;
+  int hi = (((int)u >> 3) & (int)0x8fffffffu) + 0x38000000;  // sign, exponent + 896, 20 mantissa bits
+  unsigned lo = u << 29;
+  if (t - 0x00800000u >= 0x7f000000u) {
+    hi = t == 0u ? 0 : 0x7ff80000;
+    lo = 0u;
+  }
+  return __hiloint2double(hi, (int)lo);
 }
 
 // The double nearest h + l (one FP64 addition of two exact conversions).

@@ -43,8 +43,9 @@ __device__ __forceinline__ PDF pdf_add(PDF a, PDF b) {
 __device__ __forceinline__ PDF pdf_sub(PDF a, PDF b) {
   return pdf_add(a, PDF{make_float2(-b.h.x, -b.h.y), make_float2(-b.l.x, -b.l.y)});
 }
-__device__ __forceinline__ float4 pdf_pack(PDF v) { return make_float4(v.h.x, v.l.x, v.h.y, v.l.y); }
-__device__ __forceinline__ PDF pdf_unpack(float4 v) { return PDF{make_float2(v.x, v.z), make_float2(v.y, v.w)}; }
+// (re, im) pairs side by side: 16-byte accesses leave them in the registers the packed instructions read
+__device__ __forceinline__ float4 pdf_pack(PDF v) { return make_float4(v.h.x, v.h.y, v.l.x, v.l.y); }
+__device__ __forceinline__ PDF pdf_unpack(float4 v) { return PDF{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
 
 // Coefficients of amplitude j: G_h (centre, neighbour sums, swapped neighbour
 // differences with lane signs (-1, +1)) and -kt G_h; a is passed per point.
