@@ -347,6 +347,8 @@ void launch_adj_nonlin(const double2* eta0, const double2* xg, const double2* et
                        double* out, const OpCoef& c, const NonlinTable& nt, cudaStream_t s);
 // Picard iteration of Alg. 1: b_j = eta_prev_j/dt - kap_j (N_j - D_j eta_j) from the
 // previous iterate (eta-parts of x); jd (nullable) receives kap_j D_j, D_j = dN_j/d eta_j
+// keys[2 j], keys[2 j + 1]: order-preserving keys of jd's least and greatest value over amplitude j
+void launch_jac_range(const double* jd, long long* keys, const OpCoef& c, cudaStream_t s);
 void launch_rhs_picard(const double2* x, const double2* eta_prev, double2* b, double* jd, float2* jd32,
                        const OpCoef& c, const NonlinTable& nt, cudaStream_t s);
 // Rotation diagnostic and adaptivity map (Sec. II.D): per point the rotation
@@ -428,6 +430,7 @@ int schur_t0(const SchurCoef& s, int dim, int m) {
   return s.plain ? 1 : 2 - schur_ni<T>(s, dim, m);
 }
 bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s);
+bool schur_widen(const SchurCoef& s, const double* dmin, const double* dmax, int J, SchurCoef& out);
 ChebPass schur_pass(const SchurCoef& s, int J, int pass, int ni);
 GaugeWeights gauge_weights(const SchurCoef& s, int J, int pass, int ni);
 int schur_terms(double tin, double lnrate);  // terms that reduce the residual by tin
@@ -458,7 +461,7 @@ bool launch_gauge64(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeig
 template <typename T>
 void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, cudaStream_t s);
 // The first np passes of a solve, by either iteration; variant 3 takes the tiles where the grid is
-// small enough.
+// small enough, Picard with the Jacobian (2D) on any grid.
 template <typename T>
 bool launch_schur_passes(const SchurCoef& sc, int m, int tile, const OpCoef& c, const ChebStep* w,
                          const GaugeTab<T>& gt, int Ly, const ChebBufs<T>& b, int np, cudaStream_t s, int sms,
@@ -466,12 +469,12 @@ bool launch_schur_passes(const SchurCoef& sc, int m, int tile, const OpCoef& c, 
   const int ni = schur_ni<T>(sc, c.dim, m);
   int take = 0;
   if constexpr (sizeof(T) == 4) {
-    if (sc.plain && c.dim == 2 && tile == 3) {
+    if (sc.plain && c.dim == 2 && (tile == 3 || c.jd32 != nullptr)) {
       int tiled = 0;
       if (bl != nullptr)
         for (int i = 0; i < bl->R; ++i) tiled += gauge_tiled(bl->host[i].nx, bl->host[i].ny, c.J);
       else
-        tiled = gauge_tiled(c.nx, c.ny, c.J);
+        tiled = c.jd32 != nullptr || gauge_tiled(c.nx, c.ny, c.J);  // the streamed kernel has no diagonal
       for (int p = 0; tiled > 0 && p * kTileUnits < np; ++p)
         if (!launch_gauge_tile(c, gt, gauge_weights(sc, c.J, p, ni * kTileUnits), b, p, sms, s, bl)) return false;
       if (tiled == (bl != nullptr ? bl->R : 1)) return true;

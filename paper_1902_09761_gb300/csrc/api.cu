@@ -229,6 +229,10 @@ struct apfc_ctx {
   double2* eta_step = nullptr;
   double* jd = nullptr;
   float2* jd32 = nullptr;
+  long long* jkeys = nullptr;       // range of jd per amplitude (device, pinned host)
+  long long* jkeys_host = nullptr;
+  SchurCoef schur_jac{};            // schur widened by it, of the Picard iteration at hand
+  bool schur_jac_ok = false;
   // contiguous device copy of host amplitudes (one full-bandwidth host-to-device copy)
   double2* stage = nullptr;
 };
@@ -764,15 +768,19 @@ apfc_status status_of(apfc_ctx* ctx, int worst) {
   return APFC_OK;
 }
 
+const SchurCoef& schur_of(const apfc_ctx* ctx) { return ctx->coef.jd != nullptr ? ctx->schur_jac : ctx->schur; }
+
 // Whether the solve runs as the Chebyshev iteration on the Schur complement: constant
-// coefficients (no Jacobian), the fused pipeline, a tolerance above the residual's noise, and no
+// coefficients or a Jacobian that keeps it well conditioned, the fused pipeline, a tolerance above the residual's noise, and no
 // more operator applications than max_iter BiCGStab iterations (two each) may take.
 bool use_schur(const apfc_ctx* ctx) {
-  if (!ctx->schur_ok || ctx->opts.fused == 0 || ctx->coef.jd != nullptr) return false;
-  if (!schur_resid_ok(ctx->schur, ctx->opts.tol)) return false;
+  if (!ctx->schur_ok || ctx->opts.fused == 0) return false;
+  if (ctx->coef.jd != nullptr && !ctx->schur_jac_ok) return false;
+  const SchurCoef& sc = schur_of(ctx);
+  if (!schur_resid_ok(sc, ctx->opts.tol)) return false;
   const double tin = ctx->opts.precision == APFC_FP64 ? 0.9 * ctx->opts.tol : ctx->opts.tol_inner;
   for (int j = 0; j < ctx->J; ++j)
-    if (schur_terms(tin, ctx->schur.lnrate[j]) > 2LL * ctx->opts.max_iter) return false;
+    if (schur_terms(tin, sc.lnrate[j]) > 2LL * ctx->opts.max_iter) return false;
   return true;
 }
 
@@ -822,16 +830,17 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   constexpr bool fp64 = sizeof(T) == 8;
   cudaStream_t s = ctx->stream;
   const apfc_opts& o = ctx->opts;
-  const int m = o.cheb_degree, ni = schur_ni<T>(ctx->schur, ctx->dim, m), nt0 = schur_t0<T>(ctx->schur, ctx->dim, m), J = ctx->J;
+  const SchurCoef& sc = schur_of(ctx);
+  const int m = o.cheb_degree, ni = schur_ni<T>(sc, ctx->dim, m), nt0 = schur_t0<T>(sc, ctx->dim, m), J = ctx->J;
   const int most = fp64 ? 4 : o.max_refine;
   const auto cw = cheb_weights(ctx);
   const int rows = o.tile_rows > 0 ? o.tile_rows
-                                   : schur_auto_rows(ctx->schur, &ctx->grid.n[0], &ctx->grid.n[1], 1, J, m,
+                                   : schur_auto_rows(sc, &ctx->grid.n[0], &ctx->grid.n[1], 1, J, m,
                                                      (int)sizeof(cplx<T>), o.tile, ctx->sms);
   SchurPlan plan{};
   plan.tol = o.tol;
   plan.tol_inner = o.tol_inner;
-  for (int j = 0; j < J; ++j) plan.lnrate[j] = ctx->schur.lnrate[j];
+  for (int j = 0; j < J; ++j) plan.lnrate[j] = sc.lnrate[j];
   plan.t0 = nt0;
   plan.ni = ni;
   plan.max_pass = (int)std::min<long long>(1 << 30, std::max(1LL, (2LL * o.max_iter - nt0 + ni - 1) / ni));
@@ -852,7 +861,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   plan.amp_stride = 2LL * plan.npart;
   const auto [none, tx, ty, tz] = gauge_sizes(ctx);
   const GaugeTab<T> gt{w.tab, tx, ty, tz};
-  const bool f64 = fp64 || schur_resid_f64(ctx->schur, o.tol);
+  const bool f64 = fp64 || schur_resid_f64(sc, o.tol);
   const ChebBufs<T> bufs{w.r[0], {w.r[0], w.r[1]}, {w.d[0], w.d[1]}, w.u, x, ctx->ks64};
   int total = 0, worst = KS_CONVERGED, sweep = 0;
   const double tol2 = o.tol * o.tol;
@@ -895,7 +904,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       worst = KS_NOCONV;
       break;
     }
-    if (!launch_schur_passes<T>(ctx->schur, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, np, s,
+    if (!launch_schur_passes<T>(sc, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, np, s,
                                 ctx->sms))
       return fail(ctx, APFC_ECUDA, "the Chebyshev passes cannot be launched");
     if (np > 0) total += (nt0 + ni * np + 1) / 2;  // two applications, as in a BiCGStab iteration
@@ -1277,6 +1286,33 @@ apfc_status ensure_states(apfc_ctx* ctx, double2** buf, size_t* cap, size_t n) {
   return APFC_OK;
 }
 
+// Bounds of S + d(x) for the Chebyshev iteration, from the range of this iteration's Jacobian.
+apfc_status jac_bounds(apfc_ctx* ctx) {
+  ctx->schur_jac_ok = false;
+  if (ctx->dim != 2 || !ctx->schur_ok || !ctx->schur.plain) return APFC_OK;
+  const int J = ctx->J;
+  const size_t bytes = sizeof(long long) * 2 * kMaxJ;
+  if (!ctx->jkeys) CK(cudaMalloc(&ctx->jkeys, bytes));
+  if (!ctx->jkeys_host) CK(cudaMallocHost(&ctx->jkeys_host, bytes));
+  for (int j = 0; j < J; ++j) {  // above every key, below every key
+    CK(cudaMemsetAsync(ctx->jkeys + 2 * j, 0x7f, sizeof(long long), ctx->stream));
+    CK(cudaMemsetAsync(ctx->jkeys + 2 * j + 1, 0x80, sizeof(long long), ctx->stream));
+  }
+  launch_jac_range(ctx->jd, ctx->jkeys, ctx->coef, ctx->stream);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(ctx->jkeys_host, ctx->jkeys, bytes, cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaStreamSynchronize(ctx->stream));
+  double d[2][kMaxJ];
+  for (int j = 0; j < J; ++j)
+    for (int e = 0; e < 2; ++e) {
+      long long k = ctx->jkeys_host[2 * j + e];
+      k ^= (k >> 63) & 0x7fffffffffffffffLL;
+      std::memcpy(&d[e][j], &k, sizeof(double));
+    }
+  ctx->schur_jac_ok = schur_widen(ctx->schur, d[0], d[1], J, ctx->schur_jac);
+  return APFC_OK;
+}
+
 // One step of Alg. 1 with K = picard_iters iterations, the Jacobian optional.
 apfc_status step_picard(apfc_ctx* ctx) {
   const size_t fe = field_elems(ctx);
@@ -1295,6 +1331,11 @@ apfc_status step_picard(apfc_ctx* ctx) {
                       ctx->coef, ctx->nt, ctx->stream);
     ctx->coef.jd = jac ? ctx->jd : nullptr;
     ctx->coef.jd32 = jac ? ctx->jd32 : nullptr;
+    if (jac && (st = jac_bounds(ctx)) != APFC_OK) {
+      ctx->coef.jd = nullptr;
+      ctx->coef.jd32 = nullptr;
+      return st;
+    }
     int it = 0;
     st = solve_block(ctx, ctx->b64, ctx->x64, &it);
     ctx->coef.jd = nullptr;
@@ -1684,6 +1725,8 @@ void apfc_destroy(apfc_ctx* ctx) {
   cudaFree(ctx->eta_step);
   cudaFree(ctx->jd);
   cudaFree(ctx->jd32);
+  cudaFree(ctx->jkeys);
+  cudaFreeHost(ctx->jkeys_host);
   cudaFree(ctx->stage);
   delete ctx;
 }

@@ -22,6 +22,7 @@ struct G64Param {
   G64Amp amp[kMaxJ];
   unsigned long long* prof;
   const double2* tab;
+  const double* jd;  // Picard with the Jacobian: d(x), else null
   int J, nx, ny, nz, tx, ty, tz;
 };
 
@@ -129,7 +130,8 @@ __global__ void __launch_bounds__(256)
   const G64Amp& a = c.amp[q.j];
   double2 s = make_double2(0.0, 0.0);
   if (q.in) {
-    s = q_fma(a.mb, b[o + q.p], q_mul(a.m0, v[o + q.p]));
+    const double m0 = c.jd != nullptr ? fma(a.mb, c.jd[o + q.p], a.m0) : a.m0;  // a + d(x): Picard with the Jacobian
+    s = q_fma(a.mb, b[o + q.p], q_mul(m0, v[o + q.p]));
     if (pass > 0) s = q_fma(a.mp, vp[o + q.p], s);
   }
   s = g64_stencil<DIM>(g + o, q, c, tab, s, a.u0, a.u);
@@ -165,6 +167,7 @@ bool launch_gauge64(const OpCoef& c, const GaugeTab<double>& gt, const GaugeWeig
   G64Param in;
   std::memset(&in, 0, sizeof(in));
   in.prof = c.prof;
+  in.jd = c.jd;
   in.tab = gt.tab;
   in.tx = gt.tx;
   in.ty = gt.ty;

@@ -10,8 +10,11 @@ namespace apfc {
 // / 20.8 / 39 / 115.
 bool launch_gauge_tile(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
                        int pass, int sms, cudaStream_t s, const BatchLaunch* bl) {
-  using SH = TileShape<8, 10, kTileUnits, false>;
+  using SH = TileShape<8, 10, kTileUnits, false, false>;
   static_assert(SH::TX == kTileX && SH::TY == kTileY, "gauge_tiled counts these tiles");
+  if (c.jd32 != nullptr)
+    return pass == 0 ? launch_tile_pass<8, 10, kTileUnits, 1, true, true>(c, gt, w, b, pass, sms, s, bl)
+                     : launch_tile_pass<8, 10, kTileUnits, 1, false, true>(c, gt, w, b, pass, sms, s, bl);
   return pass == 0 ? launch_tile_pass<8, 10, kTileUnits, 1, true>(c, gt, w, b, pass, sms, s, bl)
                    : launch_tile_pass<8, 10, kTileUnits, 1, false>(c, gt, w, b, pass, sms, s, bl);
 }

@@ -16,6 +16,9 @@
 // Terms are counted in the streamed kernel's passes of three and evaluated by the same operations;
 // only values carried across the periodic boundary inside a launch round differently.  What a point
 // gets does not depend on the launch's other grids: a run of a batch equals the run alone.
+//
+// JAC: S = a + d(x) + kt G_h^2 with a Picard iteration's real diagonal d (SchurCoef's bounds widened
+// by its range); d commutes with the gauge.  Its values wait in shared memory, two tiles deep.
 #pragma once
 #include "gauge2d.cuh"
 
@@ -23,12 +26,13 @@ namespace apfc {
 
 namespace {
 
-template <int NW, int R, int UNITS, bool START>
+template <int NW, int R, int UNITS, bool START, bool JAC>
 struct TileShape {
   static constexpr int H = 2 * kGaugeNI32 * UNITS, OX = 64, OY = R * NW, TX = OX - 2 * H, TY = OY - 2 * H;
   static constexpr int NF = START ? 1 : 3;  // fields staged: v (START: the residual), v_(n-1), b
-  static constexpr size_t xrow = 2 * NW * 2 * 32, stage = (size_t)NF * R * NW * 32;  // in float4
-  static constexpr size_t smem = sizeof(float4) * (xrow + stage);
+  static constexpr size_t xrow = 2 * NW * 2 * 32, stage = (size_t)NF * R * NW * 32,  // in float4
+                          diag = JAC ? 2ull * R * NW * 32 : 0;
+  static constexpr size_t smem = sizeof(float4) * (xrow + stage + diag);
 };
 
 // Tiles of one grid.
@@ -39,17 +43,19 @@ struct TileGrid {
 };
 
 // unit: first unit (three terms) of this launch; ks[].iters units in all.
-template <int NW, int R, int UNITS, int MINB, bool START, class TAB>
+template <int NW, int R, int UNITS, int MINB, bool START, bool JAC, class TAB>
 __global__ void __launch_bounds__(32 * NW, MINB)
     k_gauge_tile(const __grid_constant__ GaugeParam<float> c, ChebGeom g1, int total, const float2* v_in,
-                 const float2* vp_in, float2* v_out, float2* vp_out, float2* b_io, double2* x64, const KScal* ks,
+                 const float2* vp_in, float2* v_out, float2* vp_out, float2* b_io, double2* x64, const float2* jd, const KScal* ks,
                  int unit, int kid, const __grid_constant__ TAB tab) {
-  using SH = TileShape<NW, R, UNITS, START>;
+  using SH = TileShape<NW, R, UNITS, START, JAC>;
   using C = float2;
   constexpr bool BATCH = std::is_same<TAB, ChebTab>::value;
   extern __shared__ __align__(16) unsigned char tile_smem[];
   float4* xr = reinterpret_cast<float4*>(tile_smem);       // [v, g'][warp][first, last row][32]
   float4* stg = xr + SH::xrow + threadIdx.x;               // [field][row][thread]
+  [[maybe_unused]] float4* dg = stg + SH::stage;           // JAC: [two tiles][row][thread]
+  [[maybe_unused]] int dbuf = 0;                           // of the tile fetched last
   __shared__ int its[(BATCH ? kChebRuns : 1) * kMaxJ];
   const int t = threadIdx.x, px = t & 31, w = __shfl_sync(0xffffffffu, t >> 5, 0);
   const C one = make_float2(1.f, 0.f), zero = make_float2(0.f, 0.f);
@@ -98,9 +104,9 @@ __global__ void __launch_bounds__(32 * NW, MINB)
       for (int r = 0; r < R; ++r) {
         const long long p = o + (long long)y * q.nx;
 #pragma unroll
-        for (int f = 0; f < SH::NF; ++f) {
-          const C* src = (f == 0 ? v_in : f == 1 ? vp_in : b_io) + p;
-          C* dst = reinterpret_cast<C*>(stg + (f * R + r) * (32 * NW));
+        for (int f = 0; f < SH::NF + JAC; ++f) {
+          const C* src = (f == SH::NF ? jd : f == 0 ? v_in : f == 1 ? vp_in : b_io) + p;
+          C* dst = reinterpret_cast<C*>(f == SH::NF ? dg + (dbuf * R + r) * (32 * NW) : stg + (f * R + r) * (32 * NW));
           if (vec) {
             cheb_cp_async16(dst, src + x0);
           } else {
@@ -210,7 +216,9 @@ __global__ void __launch_bounds__(32 * NW, MINB)
       }
     }
     __syncthreads();  // the slots have been read
+    [[maybe_unused]] const float4* dd = dg + dbuf * R * (32 * NW);
     if (next < total) {
+      dbuf ^= 1;
       locate(next);
       fetch();
     }
@@ -243,7 +251,11 @@ __global__ void __launch_bounds__(32 * NW, MINB)
       exchange(xr + NW * 64, h);
       const float c1 = q_.c1[i], mc2 = q_.mc2[i];
       stencil(
-          xr + NW * 64, h, [&](int r, int k) { return q_fma(n0, h[r][k], q_fma(aa, v[r][k], b[r][k])); },
+          xr + NW * 64, h, [&](int r, int k) {
+            float a = aa;
+            if constexpr (JAC) a += k == 0 ? dd[r * (32 * NW)].x : dd[r * (32 * NW)].z;
+            return q_fma(n0, h[r][k], q_fma(a, v[r][k], b[r][k]));
+          },
           [&](int r, int k, C rh) {
             const C nv = q_fma(mc2, rh, q_fma(c1, q_sub(v[r][k], vp[r][k]), v[r][k]));
             vp[r][k] = v[r][k];
@@ -277,10 +289,10 @@ __global__ void __launch_bounds__(32 * NW, MINB)
 }
 
 // Launch `pass` of a solve: units UNITS pass .. UNITS pass + UNITS - 1.
-template <int NW, int R, int UNITS, int MINB, bool START>
+template <int NW, int R, int UNITS, int MINB, bool START, bool JAC = false>
 bool launch_tile_pass(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
                       int pass, int sms, cudaStream_t s, const BatchLaunch* bl) {
-  using SH = TileShape<NW, R, UNITS, START>;
+  using SH = TileShape<NW, R, UNITS, START, JAC>;
   static_assert(kGaugeNI32 * UNITS <= kGaugeMaxNI && SH::H % 2 == 0 && SH::TX > 0 && SH::TY > 0, "tile");
   const int kid = kid_of<float>(KID_FUSED_APINV);
   ProfScope ps_(kid, s);
@@ -288,18 +300,19 @@ bool launch_tile_pass(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWei
   const int cur = pass & 1;
   const float2* vin = START ? b.r0 : b.r[cur];
   if (bl == nullptr) {
-    auto kern = k_gauge_tile<NW, R, UNITS, MINB, START, ChebNoTab>;
+    auto kern = k_gauge_tile<NW, R, UNITS, MINB, START, JAC, ChebNoTab>;
     static const cudaError_t attr =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::smem);
     if (attr != cudaSuccess) return false;
     const ChebGeom g = cheb_geom(c.nx, c.ny, SH::H, SH::OX, SH::TY);
     const int total = g.nstrips * g.nsegs * c.J;
     kern<<<std::min(total, MINB * sms), 32 * NW, SH::smem, s>>>(in, g, total, vin, b.d[cur], b.r[1 - cur],
-                                                                b.d[1 - cur], b.u, b.x64, b.ks, UNITS * pass, kid,
-                                                                ChebNoTab{});
+                                                                b.d[1 - cur], b.u, b.x64, c.jd32, b.ks, UNITS * pass,
+                                                                kid, ChebNoTab{});
     return true;
   }
-  auto kern = k_gauge_tile<NW, R, UNITS, MINB, START, ChebTab>;
+  if constexpr (JAC) return false;  // batched runs have no Jacobian
+  auto kern = k_gauge_tile<NW, R, UNITS, MINB, START, false, ChebTab>;
   static const cudaError_t attr =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::smem);
   if (attr != cudaSuccess) return false;
@@ -310,7 +323,8 @@ bool launch_tile_pass(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWei
     for (int i = 0; i < nr; ++i) total += tab.run[i].nblk;
     if (total == 0) continue;
     kern<<<std::min(total, MINB * sms), 32 * NW, SH::smem, s>>>(in, ChebGeom{}, total, vin, b.d[cur], b.r[1 - cur],
-                                                                b.d[1 - cur], b.u, b.x64, b.ks, UNITS * pass, kid, tab);
+                                                                b.d[1 - cur], b.u, b.x64, nullptr, b.ks, UNITS * pass,
+                                                                kid, tab);
   }
   return true;
 }

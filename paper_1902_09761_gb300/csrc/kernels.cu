@@ -910,6 +910,30 @@ __global__ void k_rhs_picard(const double2* __restrict__ x, const double2* __res
   }
 }
 
+// A double as a signed integer of the same order (NaN beyond the infinities).
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+// Range of jd per amplitude (blockIdx.y); keys hold 0x7f.. and 0x80.. bytes before.
+__global__ void __launch_bounds__(256) k_jac_range(const double* __restrict__ jd, long long* keys, long long pts) {
+  jd += blockIdx.y * pts;
+  long long lo = 0x7fffffffffffffffLL, hi = ~lo;
+  for (long long p = (long long)blockIdx.x * 256 + threadIdx.x; p < pts; p += (long long)gridDim.x * 256) {
+    const long long k = order_key(jd[p]);
+    lo = min(lo, k);
+    hi = max(hi, k);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(keys + 2 * blockIdx.y, lo);
+    atomicMax(keys + 2 * blockIdx.y + 1, hi);
+  }
+}
+
 __global__ void k_adj_nonlin(const double2* __restrict__ eta0, const double2* __restrict__ xg,
                              const double2* __restrict__ eta1, double2* __restrict__ lam,
                              double* __restrict__ partials, OpCoef c, NonlinTable nt) {
@@ -1254,6 +1278,9 @@ void launch_rotation(const double2* x, double* omega, double* amp, double* hmap,
   ProfScope ps_(KID_ROTATION, s);
   const dim3 g((unsigned)((c.nx + 31) / 32), (unsigned)((c.ny + 7) / 8), (unsigned)(c.dim == 3 ? c.nz : 1));
   k_rotation<<<g, 256, 0, s>>>(x, omega, amp, hmap, rp, c);
+}
+void launch_jac_range(const double* jd, long long* keys, const OpCoef& c, cudaStream_t s) {
+  k_jac_range<<<dim3((unsigned)std::min<long long>((c.pts + 1023) / 1024, 304), c.J), 256, 0, s>>>(jd, keys, c.pts);
 }
 void launch_rhs_picard(const double2* x, const double2* eta_prev, double2* b, double* jd, float2* jd32,
                        const OpCoef& c, const NonlinTable& nt, cudaStream_t s) {

@@ -172,6 +172,25 @@ bool schur_build(const OpCoef& c, const apfc_grid& grid, int m, SchurCoef& s) {
   return true;
 }
 
+// S + d(x), d real within [dmin, dmax]: both ends of the spectrum move by no more than d's.  False
+// (NaN included) where it may not be positive, or where a solve would need about 100 terms; an
+// iteration of BiCGStab with its preconditioner costs about 12 of them (512^2: 100 of its
+// iterations 10 ms, three terms 12 us).
+bool schur_widen(const SchurCoef& s, const double* dmin, const double* dmax, int J, SchurCoef& out) {
+  if (!s.plain) return false;
+  out = s;
+  out.kappa = 0.0;
+  for (int j = 0; j < J; ++j) {
+    out.lmin[j] += dmin[j];
+    out.lmax[j] += dmax[j];
+    if (!(out.lmin[j] > 0.0) || !(out.lmax[j] > out.lmin[j]) || !std::isfinite(out.lmax[j])) return false;
+    out.lnrate[j] = std::acosh((out.lmax[j] + out.lmin[j]) / (out.lmax[j] - out.lmin[j]));
+    if (!(out.lnrate[j] >= 0.1)) return false;
+    out.kappa = std::max(out.kappa, out.lmax[j] / out.lmin[j]);
+  }
+  return true;
+}
+
 // Saad, Alg. 12.1: rho_0 = 1/sigma, d_0 = z/theta; rho_k = 1/(2 sigma - rho_(k-1)),
 // d_k = rho_k rho_(k-1) d_(k-1) + (2 rho_k / delta) z_k: weights of d_first .. d_(first+count-1).
 namespace {
@@ -297,7 +316,7 @@ __global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, in
 // below is the one just formed), the x-neighbours from two-row shared-memory rings.  Every
 // double is split once.  Writes zeta into the state (the solve never reads it, so it always
 // belongs to the latest eta), r as RT, optionally r in FP64, and per block the sums ||r||^2 and,
-// on request, ||b||^2.  F64: in FP64 arithmetic (see SchurCoef::kappa), bound by the FP64 pipe.
+// on request, ||b||^2.  JAC: a + d(x) in place of a (Picard with the Jacobian).  F64: in FP64 arithmetic (see SchurCoef::kappa), bound by the FP64 pipe.
 // ---------------------------------------------------------------------------
 constexpr int kRsNT = 256, kRsPF = 2, kRsV = kRsNT - 4;
 
@@ -327,7 +346,7 @@ __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src));
 }
 
-template <bool F64, typename RT>
+template <bool F64, bool JAC, typename RT>
 __global__ void __launch_bounds__(kRsNT, 2)
     k_resid_schur2d(const double2* __restrict__ b, double2* x, RT* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
@@ -410,6 +429,11 @@ __global__ void __launch_bounds__(kRsNT, 2)
   for (int tt = 0; tt < steps; ++tt) {
     issue(tt + kRsPF, islot);
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kRsPF));
+    const int lr = tt - 2;
+    [[maybe_unused]] double jd = 0.0;  // JAC: on its way while zeta is formed
+    if constexpr (JAC) {
+      if (col_own && lr >= 2) jd = c.jd[(long long)j * pts + (long long)(y0 + lr - 2) * nx + xo];
+    }
     const V e0 = RV::in(stg[slot][0][t]);
     ring[0][par][t + 1] = RV::pack(e0);
     // zeta at row tt - 1
@@ -436,7 +460,6 @@ __global__ void __launch_bounds__(kRsNT, 2)
     const int lz = tt - 1;
     if (col_own && lz >= 2 && lz < rows + 2) zt[(long long)(y0 + lz - 2) * nx + xo] = zd;
     // r at row tt - 2
-    const int lr = tt - 2;
     if (lr >= 2) {
       const V zl = RV::unpack(ring[1][par ^ 1][t]), zr = RV::unpack(ring[1][par ^ 1][t + 2]);
       if (col_own) {
@@ -447,7 +470,8 @@ __global__ void __launch_bounds__(kRsNT, 2)
           const double ly = fma(gy, z2.y + z0.y, fma(gx, zl.y + zr.y, g0 * z1.y));
           const double Gx = lx - (ax * (zr.y - zl.y) + ay * (z0.y - z2.y));
           const double Gy = ly + (ax * (zr.x - zl.x) + ay * (z0.x - z2.x));
-          const double2 rv = make_double2(bv.x - (kt * Gx + aa * e2.x), bv.y - (kt * Gy + aa * e2.y));
+          const double ap = JAC ? aa + jd : aa;
+          const double2 rv = make_double2(bv.x - (kt * Gx + ap * e2.x), bv.y - (kt * Gy + ap * e2.y));
           if constexpr (sizeof(RT) == 16)
             r_out[p] = rv;
           else
@@ -464,6 +488,7 @@ __global__ void __launch_bounds__(kRsNT, 2)
           a.fma(q.kl[1].h, q.kl[1].l, pdf_add(z0, z2));
           a.fma(q.ka[0].h, q.ka[0].l, pdf_swap(pdf_sub(zr, zl)));
           a.fma(q.ka[1].h, q.ka[1].l, pdf_swap(pdf_sub(z0, z2)));
+          if constexpr (JAC) ma = lane_c(c.a[j] + jd, -1.f, -1.f);
           a.fma(ma.h, ma.l, e2);
           float2 f, l;
           a.result(f, l);
@@ -553,11 +578,13 @@ void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64
   const RunGeom* rg = bl != nullptr ? bl->dev : nullptr;
   if constexpr (sizeof(T) == 4) {
     if (!f64) {
-      k_resid_schur2d<false, float2><<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
+      const auto k = c.jd != nullptr ? k_resid_schur2d<false, true, float2> : k_resid_schur2d<false, false, float2>;
+      k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
       return;
     }
   }
-  k_resid_schur2d<true, cplx<T>><<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
+  const auto k = c.jd != nullptr ? k_resid_schur2d<true, true, cplx<T>> : k_resid_schur2d<true, false, cplx<T>>;
+  k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
 }
 template void launch_resid_schur2d<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool,
                                           bool, cudaStream_t, const BatchLaunch*);

@@ -11,6 +11,7 @@ import numpy as np
 import pytest
 
 import oracle as O
+from oracle import picard as PC
 from paper_1902_09761_gb300 import apfc as A
 from paper_1902_09761_gb300 import inputs
 
@@ -168,3 +169,18 @@ def test_batch_of_tiled_and_streamed_runs_equals_the_runs_alone():
         ctx.step(1.0, 2)
         assert np.array_equal(ctx.get_amplitudes(), got[r]), s
         ctx.close()
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("shape,h", [((61, 93), H2), ((130, 41), H2), ((37, 45), (0.5, 0.5))])
+def test_picard_with_the_jacobian_across_tiles(prec, shape, h):
+    # d(x) >= 0 for hexagonal amplitudes and below 0.5 here: cond(S + d) is no larger than cond(S) as
+    # in the bounds above.  h = 0.5 is beyond the plain iteration and keeps BiCGStab
+    kind = "hex"
+    ctx, L = context(kind, shape, h, precision=prec, tol=1e-12, picard_iters=2, jacobian=1)
+    eta = inputs.random_amplitudes(3, shape, seed=97, scale=0.1)
+    ctx.set_amplitudes(eta)
+    ctx.step(1.0)
+    ref, _ = PC.step_picard(eta, 1.0, P, L, h, 2, jacobian=True)
+    assert max(rel_l2_per_amp(ctx.get_amplitudes(), ref)) <= 2e-9
+    ctx.close()
