@@ -56,6 +56,13 @@ __device__ __forceinline__ DF split_d(double v) {
   return DF{__uint_as_float(h), l};
 }
 
+// A double rounded to a float (through 48 bits: half an ulp and 2^-24 more; tiny values give 0, those
+// from 2^127 NaN).
+__device__ __forceinline__ float d2f(double v) {
+  const DF d = split_d(v);
+  return __fadd_rn(d.h, d.l);
+}
+
 // Exact double of a float (zero and subnormal floats give 0, Inf and NaN give NaN).
 __device__ __forceinline__ double f2d(float f) {
   const unsigned u = __float_as_uint(f), t = u & 0x7f800000u;

@@ -732,7 +732,84 @@ __global__ void __launch_bounds__(256) k_rhs_resid_tab(const double2* __restrict
   }
 }
 
-// Energy density summed per block.
+// The triangular lattice's three amplitudes in closed form: FP64 kernels bound by the FP64 pipe (two
+// operations a clock and multiprocessor), so the operations of a point are counted: amplitudes in
+// registers, factors folded, the stencil as one chain of FMAs (18).  Each block takes tiles of
+// 32 x 8 points.
+struct HexTile {
+  long long p, xm, xp, ym, yp;
+  bool in;
+};
+__device__ __forceinline__ long long hex_tiles(const OpCoef& c) {
+  return (long long)((c.nx + 31) / 32) * ((c.ny + 7) / 8);
+}
+__device__ __forceinline__ HexTile hex_tile(long long tile, const OpCoef& c) {
+  const unsigned ntx = (c.nx + 31) / 32, ty = (unsigned)(tile / ntx), tx = (unsigned)(tile - (long long)ty * ntx);
+  const int x = tx * 32 + (threadIdx.x & 31), y = ty * 8 + (threadIdx.x >> 5);
+  HexTile t;
+  t.in = x < c.nx && y < c.ny;
+  t.p = (long long)y * c.nx + x;
+  t.xm = x == 0 ? t.p + c.nx - 1 : t.p - 1;
+  t.xp = x + 1 == c.nx ? t.p - x : t.p + 1;
+  t.ym = y == 0 ? t.p + (long long)(c.ny - 1) * c.nx : t.p - c.nx;
+  t.yp = y + 1 == c.ny ? t.p - (long long)y * c.nx : t.p + c.nx;
+  return t;
+}
+// f G_h's coefficients
+struct HexG {
+  double c0, hx, hy, kx[3], ky[3];
+};
+HexG hex_coef(const OpCoef& c, double f) {
+  HexG g{f * c.c0, f * c.ih2[0], f * c.ih2[1], {}, {}};
+  for (int j = 0; j < 3; ++j) g.kx[j] = f * c.kh[j][0], g.ky[j] = f * c.kh[j][1];
+  return g;
+}
+// init + f G_h u
+__device__ __forceinline__ double2 hex_G(const double2* __restrict__ u, double2 uc, const HexTile& t, const HexG& q,
+                                         int j, double2 init) {
+  const double2 r = u[t.xp], l = u[t.xm], n = u[t.yp], s = u[t.ym];
+  double2 g;
+  g.x = fma(-q.ky[j], n.y - s.y,
+            fma(-q.kx[j], r.y - l.y, fma(q.hy, n.x + s.x, fma(q.hx, r.x + l.x, fma(q.c0, uc.x, init.x)))));
+  g.y = fma(q.ky[j], n.x - s.x,
+            fma(q.kx[j], r.x - l.x, fma(q.hy, n.y + s.y, fma(q.hx, r.y + l.y, fma(q.c0, uc.y, init.y)))));
+  return g;
+}
+
+// Energy density: 88 operations a point (the general kernel with the closed form took 102, its
+// amplitudes in local memory): 1024^2 217 -> 185 us.
+__global__ void __launch_bounds__(kThreads) k_energy_hex(const double2* __restrict__ x, double* __restrict__ partials,
+                                                         const __grid_constant__ OpCoef c,
+                                                         const __grid_constant__ HexG q, EnergyTable et, double Bx) {
+  prof_add(c, KID_ENERGY, (unsigned long long)c.J * c.pts * sizeof(double2));
+  double acc[1] = {0.0};
+  const long long nt = hex_tiles(c);
+  for (long long i = blockIdx.x; i < nt; i += gridDim.x) {
+    const HexTile t = hex_tile(i, c);
+    if (!t.in) continue;
+    double2 e[3];
+    double S2 = 0.0, S4 = 0.0, grad = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const double2* u = x + (2LL * j + 1) * c.pts;
+      e[j] = u[t.p];
+      const double m2 = fma(e[j].x, e[j].x, e[j].y * e[j].y);
+      S2 += m2;
+      S4 = fma(m2, m2, S4);
+      const double2 g = hex_G(u, e[j], t, q, j, make_double2(0.0, 0.0));
+      grad = fma(g.x, g.x, fma(g.y, g.y, grad));
+    }
+    const double2 p01 = make_double2(fma(e[0].x, e[1].x, -(e[0].y * e[1].y)), fma(e[0].x, e[1].y, e[0].y * e[1].x));
+    const double cub = fma(p01.x, e[2].x, -(p01.y * e[2].y));
+    // dB/2 A^2 + 3v/4 A^4 - 3v/2 sum |eta|^4 - 4t Re(eta_0 eta_1 eta_2), A^2 = 2 S2
+    const double f = fma(S2, fma(3.0 * et.v, S2, et.dB), fma(-1.5 * et.v, S4, -4.0 * et.t * cub));
+    acc[0] += fma(Bx, grad, f);
+  }
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
+}
+
+// Energy density summed per block (any lattice but the triangular one).
 __global__ void k_energy(const double2* __restrict__ x, double* __restrict__ partials, OpCoef c, EnergyTable et,
                          double Bx) {
   prof_add(c, KID_ENERGY, (unsigned long long)c.J * c.pts * sizeof(double2));
@@ -741,30 +818,23 @@ __global__ void k_energy(const double2* __restrict__ x, double* __restrict__ par
        p += (long long)gridDim.x * blockDim.x) {
     const Nb n = neighbours(p, c);
     double2 eta[kMaxJ];
-    double S2 = 0.0, S4 = 0.0, grad = 0.0;
+    double S2 = 0.0, grad = 0.0;
     for (int j = 0; j < c.J; ++j) {
       const double2* e = x + (2LL * j + 1) * c.pts;
       eta[j] = e[p];
-      const double m2 = eta[j].x * eta[j].x + eta[j].y * eta[j].y;
-      S2 += m2;
-      S4 += m2 * m2;
+      S2 += eta[j].x * eta[j].x + eta[j].y * eta[j].y;
       const double2 g = opG<double>(e, n, c, j);
       grad += g.x * g.x + g.y * g.y;
     }
     const double A2 = 2.0 * S2;
     double f = 0.5 * et.dB * A2;
-    if (et.hex) {
-      const double2 cub = cm(cm(eta[0], eta[1]), eta[2]);
-      f += 0.75 * et.v * A2 * A2 - 1.5 * et.v * S4 - 4.0 * et.t * cub.x;
-    } else {
-      for (int q = 0; q < et.ne; ++q) {
-        double2 prod = make_double2(et.coef[q], 0.0);
-        for (int ff = 0; ff < et.nf[q]; ++ff) {
-          const int code = et.f[q][ff];
-          prod = cm(prod, (code & 1) ? cconj(eta[code >> 1]) : eta[code >> 1]);
-        }
-        f += prod.x;
+    for (int q = 0; q < et.ne; ++q) {
+      double2 prod = make_double2(et.coef[q], 0.0);
+      for (int ff = 0; ff < et.nf[q]; ++ff) {
+        const int code = et.f[q][ff];
+        prod = cm(prod, (code & 1) ? cconj(eta[code >> 1]) : eta[code >> 1]);
       }
+      f += prod.x;
     }
     acc[0] += f + Bx * grad;
   }
@@ -790,8 +860,9 @@ inline dim3 grid_pts3(const OpCoef& c) {
 // ---------------------------------------------------------------------------
 
 // N_j(eta) at one point (closed form on the triangular lattice, else the table).
+template <bool HEX>
 __device__ __forceinline__ double2 nonlin_at(const double2* eta, int j, const OpCoef& c, const NonlinTable& nt) {
-  if (nt.hex) {
+  if constexpr (HEX) {
     double A2 = 0.0;
     for (int m = 0; m < 3; ++m) A2 += eta[m].x * eta[m].x + eta[m].y * eta[m].y;
     A2 *= 2.0;
@@ -817,32 +888,9 @@ __device__ __forceinline__ double2 nonlin_at(const double2* eta, int j, const Op
 __device__ __forceinline__ double2 cadd2(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ double2 csub2(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 
-// out_k -= sum_j [w_j conj(dN_j/deta_k) + conj(w_j) dN_j/dconj(eta_k)] at one point.
+// out_k -= sum_j [w_j conj(dN_j/deta_k) + conj(w_j) dN_j/dconj(eta_k)] at one point (table lattices).
 __device__ __forceinline__ void nonlin_vjp_sub(const double2* eta, const double2* w, double2* out, const OpCoef& c,
                                                const NonlinTable& nt) {
-  if (nt.hex) {
-    double A2 = 0.0;
-    for (int m = 0; m < 3; ++m) A2 += eta[m].x * eta[m].x + eta[m].y * eta[m].y;
-    A2 *= 2.0;
-    for (int j = 0; j < 3; ++j) {
-      // dN_j/deta_j = 3v A^2 (real), dN_j/dconj(eta_j) = 3v eta_j^2
-      const double a = 3.0 * nt.v * A2;
-      const double2 e2 = cm(eta[j], eta[j]);
-      const double2 b = make_double2(3.0 * nt.v * e2.x, 3.0 * nt.v * e2.y);
-      out[j] = csub2(out[j], cadd2(make_double2(a * w[j].x, a * w[j].y), cm(cconj(w[j]), b)));
-      for (int m = 0; m < 3; ++m) {
-        if (m == j) continue;
-        const int o = 3 - j - m;
-        // dN_j/deta_m = 6v eta_j conj(eta_m); dN_j/dconj(eta_m) = 6v eta_j eta_m - 2t conj(eta_o)
-        const double2 am = cm(eta[j], cconj(eta[m]));
-        const double2 em = cm(eta[j], eta[m]);
-        const double2 a6 = make_double2(6.0 * nt.v * am.x, 6.0 * nt.v * am.y);
-        const double2 b6 = make_double2(6.0 * nt.v * em.x - 2.0 * nt.t * eta[o].x, 6.0 * nt.v * em.y + 2.0 * nt.t * eta[o].y);
-        out[m] = csub2(out[m], cadd2(cm(w[j], cconj(a6)), cm(cconj(w[j]), b6)));
-      }
-    }
-    return;
-  }
   for (int j = 0; j < c.J; ++j) {
     for (int q = nt.start[j]; q < nt.start[j + 1]; ++q) {
       for (int f = 0; f < nt.nf[q]; ++f) {
@@ -864,8 +912,9 @@ __device__ __forceinline__ void nonlin_vjp_sub(const double2* eta, const double2
 // triangular lattice, else the derivative of every table monomial by its unconjugated
 // eta_j factors.  The exact value is real (a mixed second derivative of the real bulk
 // density); the real part is returned.
+template <bool HEX>
 __device__ __forceinline__ double jac_diag_at(const double2* eta, int j, const OpCoef& c, const NonlinTable& nt) {
-  if (nt.hex) {
+  if constexpr (HEX) {
     double A2 = 0.0;
     for (int m = 0; m < 3; ++m) A2 += eta[m].x * eta[m].x + eta[m].y * eta[m].y;
     return 3.0 * nt.v * 2.0 * A2;
@@ -889,17 +938,24 @@ __device__ __forceinline__ double jac_diag_at(const double2* eta, int j, const O
 // Right-hand side of Picard iteration k (Alg. 1): from the previous iterate eta (the
 // eta-parts of x), b_j = eta_prev_j/dt - kap_j (N_j - D_j eta_j) and jd_j = kap_j D_j
 // (jd == nullptr: plain Picard, D = 0).
+template <bool HEX>
 __global__ void k_rhs_picard(const double2* __restrict__ x, const double2* __restrict__ eta_prev,
                              double2* __restrict__ b, double* __restrict__ jd, float2* __restrict__ jd32, OpCoef c,
                              NonlinTable nt) {
   prof_add(c, KID_RHS, (unsigned long long)c.J * c.pts * (3 * sizeof(double2) + (jd ? sizeof(double) : 0)));
   for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < c.pts;
        p += (long long)gridDim.x * blockDim.x) {
-    double2 eta[kMaxJ];
-    for (int j = 0; j < c.J; ++j) eta[j] = x[(2LL * j + 1) * c.pts + p];
-    for (int j = 0; j < c.J; ++j) {
-      const double2 N = nonlin_at(eta, j, c, nt);
-      const double D = jd != nullptr ? jac_diag_at(eta, j, c, nt) : 0.0;
+    constexpr int MJ = HEX ? 3 : kMaxJ;  // the triangular lattice's amplitudes stay in registers
+    const int J = HEX ? 3 : c.J;
+    double2 eta[MJ];
+#pragma unroll
+    for (int j = 0; j < MJ; ++j)
+      if (j < J) eta[j] = x[(2LL * j + 1) * c.pts + p];
+#pragma unroll
+    for (int j = 0; j < MJ; ++j) {
+      if (j >= J) break;
+      const double2 N = nonlin_at<HEX>(eta, j, c, nt);
+      const double D = jd != nullptr ? jac_diag_at<HEX>(eta, j, c, nt) : 0.0;
       const double kap = c.kap[j];
       const double2 ep = eta_prev[j * c.pts + p];
       b[(2LL * j + 1) * c.pts + p] = make_double2(ep.x * c.inv_dt - kap * (N.x - D * eta[j].x),
@@ -934,6 +990,48 @@ __global__ void __launch_bounds__(256) k_jac_range(const double* __restrict__ jd
   }
 }
 
+// The triangular lattice's adjoint of the explicit part: N is the gradient of a real density, so its
+// VJP is its directional derivative,
+//   dN_j(w) = 3v [(2S - |eta_j|^2) w_j + (4D - 2 d_j) eta_j] - 2t conj(eta_k w_l + w_k eta_l),
+// S = sum |eta|^2, d_j = Re(conj(eta_j) w_j), D = sum d_j: 98 operations a point instead of about 250.
+// 256^2: 39 -> 24 us.
+__global__ void __launch_bounds__(kThreads)
+    k_adj_nonlin_hex(const double2* __restrict__ eta0, const double2* __restrict__ xg, const double2* __restrict__ eta1,
+                     double2* __restrict__ lam, double* __restrict__ partials, const __grid_constant__ OpCoef c,
+                     double t, double v) {
+  prof_add(c, KID_ADJ_NONLIN, 4ull * c.J * (unsigned long long)c.pts * sizeof(double2));
+  double acc[1] = {0.0};
+  const double v3 = 3.0 * v, t2 = 2.0 * t;
+  for (long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x; p < c.pts;
+       p += (long long)gridDim.x * blockDim.x) {
+    double2 e[3], w[3], g[3];
+    double m2[3], d[3], S = 0.0, D = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      e[j] = eta0[j * c.pts + p];
+      g[j] = xg[(2LL * j + 1) * c.pts + p];
+      const double2 e1 = eta1[j * c.pts + p];
+      acc[0] = fma(c.kap[j], fma(g[j].x, e1.x, g[j].y * e1.y), acc[0]);
+      w[j] = make_double2(c.kap[j] * g[j].x, c.kap[j] * g[j].y);
+      m2[j] = fma(e[j].x, e[j].x, e[j].y * e[j].y);
+      d[j] = fma(e[j].x, w[j].x, e[j].y * w[j].y);
+      S += m2[j];
+      D += d[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int k = (j + 1) % 3, l = (j + 2) % 3;
+      const double a = v3 * fma(2.0, S, -m2[j]), b = v3 * fma(4.0, D, -2.0 * d[j]);
+      const double qx = fma(e[k].x, w[l].x, fma(w[k].x, e[l].x, -fma(e[k].y, w[l].y, w[k].y * e[l].y)));
+      const double qy = fma(e[k].x, w[l].y, fma(e[k].y, w[l].x, fma(w[k].x, e[l].y, w[k].y * e[l].x)));
+      lam[j * c.pts + p] = make_double2(fma(g[j].x, c.inv_dt, fma(t2, qx, -fma(a, w[j].x, b * e[j].x))),
+                                        fma(g[j].y, c.inv_dt, fma(-t2, qy, -fma(a, w[j].y, b * e[j].y))));
+    }
+  }
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
+}
+
 __global__ void k_adj_nonlin(const double2* __restrict__ eta0, const double2* __restrict__ xg,
                              const double2* __restrict__ eta1, double2* __restrict__ lam,
                              double* __restrict__ partials, OpCoef c, NonlinTable nt) {
@@ -957,6 +1055,42 @@ __global__ void k_adj_nonlin(const double2* __restrict__ eta0, const double2* __
   if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
 }
 
+// The triangular lattice's scale (dB eta_j + Bx G_h zeta_j + N_j) and the block sums of |eta|^2: 92
+// operations a point; 1024^2 365 -> 199 us.
+__global__ void __launch_bounds__(kThreads)
+    k_energy_grad_hex(const double2* __restrict__ x, double2* __restrict__ grad, double scale, double dB,
+                      double* __restrict__ partials, const __grid_constant__ OpCoef c, const __grid_constant__ HexG q,
+                      double t, double v) {
+  prof_add(c, KID_ENERGY_GRAD, 3ull * c.J * (unsigned long long)c.pts * sizeof(double2));
+  double acc[1] = {0.0};
+  const double v3 = 3.0 * v * scale, t2 = 2.0 * t * scale, sdB = scale * dB;
+  const long long nt = hex_tiles(c);
+  for (long long i = blockIdx.x; i < nt; i += gridDim.x) {
+    const HexTile n = hex_tile(i, c);
+    if (!n.in) continue;
+    double2 e[3];
+    double m2[3], S = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      e[j] = x[(2LL * j + 1) * c.pts + n.p];
+      m2[j] = fma(e[j].x, e[j].x, e[j].y * e[j].y);
+      S += m2[j];
+    }
+    acc[0] += S;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int k = (j + 1) % 3, l = (j + 2) % 3;
+      const double s = fma(v3, fma(2.0, S, -m2[j]), sdB);
+      const double px = fma(e[k].x, e[l].x, -(e[k].y * e[l].y)), py = fma(e[k].x, e[l].y, e[k].y * e[l].x);
+      const double2 init = make_double2(fma(s, e[j].x, -t2 * px), fma(s, e[j].y, t2 * py));
+      const double2* z = x + 2LL * j * c.pts;
+      grad[j * c.pts + n.p] = hex_G(z, z[n.p], n, q, j, init);
+    }
+  }
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
+}
+
 __global__ void k_energy_grad(const double2* __restrict__ x, double2* __restrict__ grad, double scale, double dB,
                               double Bx, double* __restrict__ partials, OpCoef c, NonlinTable nt) {
   prof_add(c, KID_ENERGY_GRAD, 3ull * c.J * (unsigned long long)c.pts * sizeof(double2));
@@ -971,7 +1105,7 @@ __global__ void k_energy_grad(const double2* __restrict__ x, double2* __restrict
     }
     for (int j = 0; j < c.J; ++j) {
       const double2 gz = opG<double>(x + 2LL * j * c.pts, n, c, j);
-      const double2 N = nonlin_at(e, j, c, nt);
+      const double2 N = nonlin_at<false>(e, j, c, nt);
       grad[j * c.pts + p] = make_double2(scale * (dB * e[j].x + Bx * gz.x + N.x), scale * (dB * e[j].y + Bx * gz.y + N.y));
     }
   }
@@ -986,7 +1120,8 @@ __global__ void k_energy_grad(const double2* __restrict__ x, double2* __restrict
 // One thread per point on a (32 x 8)-point tile grid with z in blockIdx.z.  A = sqrt(2
 // sum |eta_j|^2) is formed once per point of the tile and its one-point (x, y) halo in
 // shared memory (FP64: A and |grad A| decide the branches of Eq. hhh); z-neighbours
-// in 3D are formed directly.  The phases go through FP32: eta converted on load, the
+// in 3D are formed directly.  The phases go through FP32: eta converted on load (by integer
+// and FP32 operations: 24 conversions a point on the FP64 pipe made 1024^2 take 158 us, now 109), the
 // product a conj(b) and atan2f in FP32 (about 1e-7 rad per difference), the weighted
 // sums and omega in FP32.  The branches compare squares: |grad A|^2 >= eps^2 and
 // A^2 > A_min^2.
@@ -1014,7 +1149,9 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
     for (int i = threadIdx.x; i < 10 * 34; i += 256) {
       const int ly = i / 34, lx = i - ly * 34;
       // periodic wrap (the halo of a partial tile can lie several points past a small grid)
-      const int gx = ((x0 + lx - 1) % c.nx + c.nx) % c.nx, gy = ((y0 + ly - 1) % c.ny + c.ny) % c.ny;
+      int gx = x0 + lx - 1, gy = y0 + ly - 1;
+      gx = gx < 0 ? gx + c.nx : gx < c.nx ? gx : gx % c.nx;
+      gy = gy < 0 ? gy + c.ny : gy < c.ny ? gy : gy % c.ny;
       sA[ly][lx] = amp_at(x, zoff + (long long)gy * c.nx + gx, c);
     }
     __syncthreads();
@@ -1040,7 +1177,7 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
     for (int d = 0; d < 3; ++d) {
       if (d >= dim) break;
       const double2 ad = e[nbp[d]], bd = e[nbm[d]];
-      const float ax = (float)ad.x, ay = (float)ad.y, bx = (float)bd.x, by = (float)bd.y;
+      const float ax = d2f(ad.x), ay = d2f(ad.y), bx = d2f(bd.x), by = d2f(bd.y);
       // arg(a conj(b)): central difference of the unwrapped phase
       const float g = atan2f(ay * bx - ax * by, ax * bx + ay * by) * rp.inv2h[d];
 #pragma unroll
@@ -1062,7 +1199,7 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
   float wmax = 0.0f;
   for (int q = 0; q < nc; ++q) {
     if (!ok) om[q] = 0.0f;
-    omega[q * c.pts + p] = (double)om[q];
+    omega[q * c.pts + p] = f2d(om[q]);
     wmax = fmaxf(wmax, fabsf(om[q]));
   }
   if (!want_h && amp == nullptr) return;
@@ -1083,7 +1220,7 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
       // theta = asin(w); sin(theta/2) = w / sqrt(2 (1 + cos(theta)))
       const float w = fminf(wmax, 1.0f);
       const float s = w / sqrtf(2.0f * (1.0f + sqrtf(1.0f - w * w)));
-      const double h_amp = s > 0.0f ? rp.pi_over_nk / (double)s : INFINITY;
+      const double h_amp = s > 0.0f ? rp.pi_over_nk / f2d(s) : INFINITY;
       hv = fmin(fmax(h_amp, rp.h_int), rp.h_max);
     } else {
       hv = rp.h_max;
@@ -1256,20 +1393,30 @@ void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const
 void launch_energy(const double2* x, double* partials, double* out, const OpCoef& c, const EnergyTable& et, double Bx,
                    cudaStream_t s) {
   ProfScope ps_(KID_ENERGY, s);
-  k_energy<<<kDotBlocks, kThreads, 0, s>>>(x, partials, c, et, Bx);
+  if (et.hex)
+    k_energy_hex<<<kDotBlocks, kThreads, 0, s>>>(x, partials, c, hex_coef(c, 1.0), et, Bx);
+  else
+    k_energy<<<kDotBlocks, kThreads, 0, s>>>(x, partials, c, et, Bx);
   k_sum_partials<<<1, kThreads, 0, s>>>(partials, kDotBlocks, out);
 }
 
 void launch_adj_nonlin(const double2* eta0, const double2* xg, const double2* eta1, double2* lam, double* partials,
                        double* out, const OpCoef& c, const NonlinTable& nt, cudaStream_t s) {
   ProfScope ps_(KID_ADJ_NONLIN, s);
-  k_adj_nonlin<<<kDotBlocks, kThreads, 0, s>>>(eta0, xg, eta1, lam, partials, c, nt);
+  if (nt.hex)
+    k_adj_nonlin_hex<<<kDotBlocks, kThreads, 0, s>>>(eta0, xg, eta1, lam, partials, c, nt.t, nt.v);
+  else
+    k_adj_nonlin<<<kDotBlocks, kThreads, 0, s>>>(eta0, xg, eta1, lam, partials, c, nt);
   k_sum_partials<<<1, kThreads, 0, s>>>(partials, kDotBlocks, out);
 }
 void launch_energy_grad(const double2* x, double2* grad, double scale, double dB, double Bx, double* partials,
                         double* out, const OpCoef& c, const NonlinTable& nt, cudaStream_t s) {
   ProfScope ps_(KID_ENERGY_GRAD, s);
-  k_energy_grad<<<kDotBlocks, kThreads, 0, s>>>(x, grad, scale, dB, Bx, partials, c, nt);
+  if (nt.hex)
+    k_energy_grad_hex<<<kDotBlocks, kThreads, 0, s>>>(x, grad, scale, dB, partials, c, hex_coef(c, scale * Bx), nt.t,
+                                                      nt.v);
+  else
+    k_energy_grad<<<kDotBlocks, kThreads, 0, s>>>(x, grad, scale, dB, Bx, partials, c, nt);
   k_sum_partials<<<1, kThreads, 0, s>>>(partials, kDotBlocks, out);
 }
 
@@ -1285,7 +1432,8 @@ void launch_jac_range(const double* jd, long long* keys, const OpCoef& c, cudaSt
 void launch_rhs_picard(const double2* x, const double2* eta_prev, double2* b, double* jd, float2* jd32,
                        const OpCoef& c, const NonlinTable& nt, cudaStream_t s) {
   ProfScope ps_(KID_RHS, s);
-  k_rhs_picard<<<(unsigned)std::min<long long>((c.pts + kThreads - 1) / kThreads, 8 * kDotBlocks), kThreads, 0, s>>>(
+  const auto k = nt.hex ? k_rhs_picard<true> : k_rhs_picard<false>;
+  k<<<(unsigned)std::min<long long>((c.pts + kThreads - 1) / kThreads, 8 * kDotBlocks), kThreads, 0, s>>>(
       x, eta_prev, b, jd, jd32, c, nt);
 }
 #define APFC_INST(T)                                                                                                 \
