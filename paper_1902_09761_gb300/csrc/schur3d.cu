@@ -302,15 +302,24 @@ static int gauge3_planes(const OpCoef& c, int txv, int tyv, int res, int sms) {
   return bl;
 }
 
-// 60 x 12 points a tile, two blocks of 256 threads per SM, one plane ahead.  Measured at 256^3 x 6
-// (us a term; its 32 bytes a point take 481 at the copy rate): 718; 60 x 16 in one block 1005, in
-// two (spilled) 892, 60 x 28 750; with 36-column tiles (rows across warps, bank conflicts) 32 x 16
-// 744, 64 x 16 863.
+// Tiles of 60 columns: of 28 rows (eight warps of four, one block per SM) or of 12 (eight warps of
+// two, two blocks), one plane ahead.  Measured at 256^3 x 6 (us a term; its 32 bytes a point take
+// 481 at the copy rate): 28 rows 670, 12 rows 745 (718 with every x-neighbour from shared memory);
+// 26 rows in ten warps of three 727, 28 in sixteen of two 720; v_(n-1) and b through shared memory
+// 702 to 816.  A covered row costs the tall tile 0.85 of the short one's; with fewer than two
+// rounds of blocks the short one's finer grain wins (70 x 90 x 101: 54 against 58).
 bool launch_gauge3d(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
                     int pass, int sms, cudaStream_t s) {
+  const long long rows28 = (c.ny + 27) / 28, rows12 = (c.ny + 11) / 12;
+  const long long blocks = (c.nx + 59) / 60 * rows28 * ((c.nz + 31) / 32) * c.J;
+  if (0.85 * 28 * rows28 < 12.0 * rows12 && blocks >= 2 * sms) {
+    const int Lz = gauge3_planes(c, 60, 28, 1, sms);
+    return pass == 0 ? launch_gauge3_pass<4, 8, 1, 1, true>(c, gt, w, Lz, b, pass, s)
+                     : launch_gauge3_pass<4, 8, 1, 1, false>(c, gt, w, Lz, b, pass, s);
+  }
   const int Lz = gauge3_planes(c, 60, 12, 2, sms);
-  return pass == 0 ? launch_gauge3_pass<float, 2, 12, 1, 2, true>(c, gt, w, Lz, b, pass, s)
-                   : launch_gauge3_pass<float, 2, 12, 1, 2, false>(c, gt, w, Lz, b, pass, s);
+  return pass == 0 ? launch_gauge3_pass<2, 8, 1, 2, true>(c, gt, w, Lz, b, pass, s)
+                   : launch_gauge3_pass<2, 8, 1, 2, false>(c, gt, w, Lz, b, pass, s);
 }
 
 }  // namespace apfc
