@@ -15,7 +15,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libapfc.so")
-SOURCES = ["fused2d_v.cu", "fused2d_t.cu", "fused2d.cu", "kernels.cu", "stream3d.cu", "reduce.cu", "api.cu", "batch.cu", "noalloc.cu", "probe.cu", "resid2d.cu", "cheb2d_f32.cu", "cheb2d_f64.cu", "gauge2d_f32.cu", "gauge_tile.cu", "gauge_f64.cu", "schur.cu", "schur3d.cu"]
+SOURCES = ["fused2d_v.cu", "fused2d_t.cu", "fused2d.cu", "kernels.cu", "stream3d.cu", "reduce.cu", "api.cu", "batch.cu", "noalloc.cu", "probe.cu", "resid2d.cu", "cheb2d_f32.cu", "cheb2d_f64.cu", "gauge2d_f32.cu", "gauge_tile.cu", "gauge_f64.cu", "resid_f64.cu", "schur.cu", "schur3d.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -508,6 +508,10 @@ template <typename T>
 bool launch_resid_schur3d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
                           bool want_b, bool f64, cudaStream_t s);
 int schur_resid3_parts(int nx, int ny, int nz, int J);
+// either, in FP64 arithmetic (resid_f64.cu)
+template <typename T>
+void launch_resid64(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c, bool want_b,
+                    int npart, cudaStream_t s, const BatchLaunch* bl);
 int schur_resid_rows(int nx, int ny, int J);
 int schur_resid_parts(int nx, int ny, int J);
 // ks[j].rnorm2 / bnorm2 from partial sums and ks[j].iters, the passes of the next solve

@@ -316,45 +316,22 @@ __global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, in
 // below is the one just formed), the x-neighbours from two-row shared-memory rings.  Every
 // double is split once.  Writes zeta into the state (the solve never reads it, so it always
 // belongs to the latest eta), r as RT, optionally r in FP64, and per block the sums ||r||^2 and,
-// on request, ||b||^2.  JAC: a + d(x) in place of a (Picard with the Jacobian).  F64: in FP64 arithmetic (see SchurCoef::kappa), bound by the FP64 pipe.
+// on request, ||b||^2.  JAC: a + d(x) in place of a (Picard with the Jacobian).Where
+// SchurCoef::kappa asks for FP64 arithmetic resid_f64.cu's kernels run instead.
 // ---------------------------------------------------------------------------
 constexpr int kRsNT = 256, kRsPF = 2, kRsV = kRsNT - 4;
-
-template <bool F64>
-struct RsVal;
-template <>
-struct RsVal<false> {
-  using V = PDF;
-  using S = float4;
-  static __device__ __forceinline__ V in(double2 v) { return pdf_split(v); }
-  static __device__ __forceinline__ S pack(V v) { return pdf_pack(v); }
-  static __device__ __forceinline__ V unpack(S v) { return pdf_unpack(v); }
-  static __device__ __forceinline__ V zero() { return PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-};
-template <>
-struct RsVal<true> {
-  using V = double2;
-  using S = double2;
-  static __device__ __forceinline__ V in(double2 v) { return v; }
-  static __device__ __forceinline__ S pack(V v) { return v; }
-  static __device__ __forceinline__ V unpack(S v) { return v; }
-  static __device__ __forceinline__ V zero() { return make_double2(0.0, 0.0); }
-};
 
 __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src));
 }
 
-template <bool F64, bool JAC, typename RT>
+template <bool JAC>
 __global__ void __launch_bounds__(kRsNT, 2)
-    k_resid_schur2d(const double2* __restrict__ b, double2* x, RT* __restrict__ r_out, double2* __restrict__ r64,
+    k_resid_schur2d(const double2* __restrict__ b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
                     int want_b, const RunGeom* rg) {
-  using RV = RsVal<F64>;
-  using V = typename RV::V;
-  using SV = typename RV::S;
-  __shared__ SV ring[2][2][kRsNT + 2];             // eta, zeta
+  __shared__ float4 ring[2][2][kRsNT + 2];             // eta, zeta
   __shared__ double2 stg[kRsPF + 1][2][kRsNT];     // eta, b rows in flight
   __shared__ double shn[2][kRsNT / 32];
   const int j = blockIdx.y, t = threadIdx.x;
@@ -378,7 +355,7 @@ __global__ void __launch_bounds__(kRsNT, 2)
   const int sy = blockIdx.x / nstrips, sx = blockIdx.x - sy * nstrips;
   if (c.prof != nullptr && blockIdx.x == 0 && t == 0)
     atomicAdd(c.prof + KID_RESID_REFINE,
-              (unsigned long long)pts * (3 * sizeof(double2) + sizeof(RT) +
+              (unsigned long long)pts * (3 * sizeof(double2) + sizeof(float2) +
                                          (r64 != nullptr ? sizeof(double2) : 0)));
   double2* zt = x + 2LL * j * pts;
   const double2* et = zt + pts;
@@ -387,15 +364,9 @@ __global__ void __launch_bounds__(kRsNT, 2)
   r_out += fo;
   if (r64 != nullptr) r64 += fo;
 
-  [[maybe_unused]] ResidCoef<2> q;
-  [[maybe_unused]] LaneC ma;
-  [[maybe_unused]] double g0, gx, gy, ax, ay, kt, aa;
-  if constexpr (F64) {
-    g0 = c.c0, gx = c.ih2[0], gy = c.ih2[1], ax = c.kh[j][0], ay = c.kh[j][1], kt = c.kt[j], aa = c.a[j];
-  } else {
-    q = resid_coef<2>(c, j);
-    ma = lane_c(c.a[j], -1.f, -1.f);
-  }
+  const ResidCoef<2> q = resid_coef<2>(c, j);
+  LaneC ma = lane_c(c.a[j], -1.f, -1.f);
+  const PDF zero{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 
   const int x_first = sx * kRsV - 2;
   int gxx = (x_first + t) % nx;
@@ -416,15 +387,14 @@ __global__ void __launch_bounds__(kRsNT, 2)
   };
   if (t == 0) {
     for (int k = 0; k < 2; ++k)
-      for (int p = 0; p < 2; ++p) ring[k][p][0] = ring[k][p][kRsNT + 1] = RV::pack(RV::zero());
+      for (int p = 0; p < 2; ++p) ring[k][p][0] = ring[k][p][kRsNT + 1] = pdf_pack(zero);
   }
   for (int k = 0; k < 2; ++k)
-    for (int p = 0; p < 2; ++p) ring[k][p][t + 1] = RV::pack(RV::zero());
+    for (int p = 0; p < 2; ++p) ring[k][p][t + 1] = pdf_pack(zero);
   for (int tf = 0; tf < kRsPF; ++tf) issue(tf, tf);
   __syncthreads();
-  V e1 = RV::zero(), e2 = RV::zero(), z1 = RV::zero(), z2 = RV::zero();  // rows formed 1 and 2 steps ago
+  PDF e1 = zero, e2 = zero, z1 = zero, z2 = zero;  // rows formed 1 and 2 steps ago
   float rr = 0.f, bb = 0.f;
-  double rrd = 0.0, bbd = 0.0;
   int slot = 0, islot = kRsPF, par = 0;
   for (int tt = 0; tt < steps; ++tt) {
     issue(tt + kRsPF, islot);
@@ -434,20 +404,15 @@ __global__ void __launch_bounds__(kRsNT, 2)
     if constexpr (JAC) {
       if (col_own && lr >= 2) jd = c.jd[(long long)j * pts + (long long)(y0 + lr - 2) * nx + xo];
     }
-    const V e0 = RV::in(stg[slot][0][t]);
-    ring[0][par][t + 1] = RV::pack(e0);
+    const PDF e0 = pdf_split(stg[slot][0][t]);
+    ring[0][par][t + 1] = pdf_pack(e0);
     // zeta at row tt - 1
-    const V el = RV::unpack(ring[0][par ^ 1][t]), er = RV::unpack(ring[0][par ^ 1][t + 2]);
-    V z0;
+    const PDF el = pdf_unpack(ring[0][par ^ 1][t]), er = pdf_unpack(ring[0][par ^ 1][t + 2]);
+    PDF z0;
     double2 zd;
-    if constexpr (F64) {
-      const double lx = fma(gy, e2.x + e0.x, fma(gx, el.x + er.x, g0 * e1.x));
-      const double ly = fma(gy, e2.y + e0.y, fma(gx, el.y + er.y, g0 * e1.y));
-      z0 = make_double2(lx - (ax * (er.y - el.y) + ay * (e0.y - e2.y)), ly + (ax * (er.x - el.x) + ay * (e0.x - e2.x)));
-      zd = z0;
-    } else {
+    {
       PAcc a;
-      a.init(RV::zero());
+      a.init(zero);
       a.fma(q.g0.h, q.g0.l, e1);
       a.fma(q.gl[0].h, q.gl[0].l, pdf_add(er, el));
       a.fma(q.gl[1].h, q.gl[1].l, pdf_add(e0, e2));
@@ -456,30 +421,16 @@ __global__ void __launch_bounds__(kRsNT, 2)
       a.result(z0.h, z0.l);
       zd = make_double2(df_to_d(DF{z0.h.x, z0.l.x}), df_to_d(DF{z0.h.y, z0.l.y}));
     }
-    ring[1][par][t + 1] = RV::pack(z0);
+    ring[1][par][t + 1] = pdf_pack(z0);
     const int lz = tt - 1;
     if (col_own && lz >= 2 && lz < rows + 2) zt[(long long)(y0 + lz - 2) * nx + xo] = zd;
     // r at row tt - 2
     if (lr >= 2) {
-      const V zl = RV::unpack(ring[1][par ^ 1][t]), zr = RV::unpack(ring[1][par ^ 1][t + 2]);
+      const PDF zl = pdf_unpack(ring[1][par ^ 1][t]), zr = pdf_unpack(ring[1][par ^ 1][t + 2]);
       if (col_own) {
         const double2 bv = stg[slot][1][t];
         const long long p = (long long)(y0 + lr - 2) * nx + xo;
-        if constexpr (F64) {
-          const double lx = fma(gy, z2.x + z0.x, fma(gx, zl.x + zr.x, g0 * z1.x));
-          const double ly = fma(gy, z2.y + z0.y, fma(gx, zl.y + zr.y, g0 * z1.y));
-          const double Gx = lx - (ax * (zr.y - zl.y) + ay * (z0.y - z2.y));
-          const double Gy = ly + (ax * (zr.x - zl.x) + ay * (z0.x - z2.x));
-          const double ap = JAC ? aa + jd : aa;
-          const double2 rv = make_double2(bv.x - (kt * Gx + ap * e2.x), bv.y - (kt * Gy + ap * e2.y));
-          if constexpr (sizeof(RT) == 16)
-            r_out[p] = rv;
-          else
-            r_out[p] = make_float2((float)rv.x, (float)rv.y);
-          if (r64 != nullptr) r64[p] = rv;
-          rrd += rv.x * rv.x + rv.y * rv.y;
-          if (want_b) bbd += bv.x * bv.x + bv.y * bv.y;
-        } else {
+        {
           const PDF bp = pdf_split(bv);
           PAcc a;
           a.init(bp);
@@ -509,7 +460,7 @@ __global__ void __launch_bounds__(kRsNT, 2)
     __syncthreads();
   }
   asm volatile("cp.async.wait_group 0;\n" ::);
-  if constexpr (!F64) rrd = (double)rr, bbd = (double)bb;
+  double rrd = (double)rr, bbd = (double)bb;
   for (int o = 16; o > 0; o >>= 1) {
     rrd += __shfl_xor_sync(0xffffffffu, rrd, o);
     bbd += __shfl_xor_sync(0xffffffffu, bbd, o);
@@ -566,7 +517,6 @@ int schur_resid_parts(int nx, int ny, int J) {
 template <typename T>
 void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
                           bool want_b, bool f64, cudaStream_t s, const BatchLaunch* bl) {
-  ProfScope ps_(KID_RESID_REFINE, s);
   const int Ly = schur_resid_rows(c.nx, c.ny, c.J);
   const int ns = (c.nx + kRsV - 1) / kRsV, ng = (c.ny + Ly - 1) / Ly;
   dim3 grid(ns * ng, c.J);
@@ -575,16 +525,15 @@ void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64
     for (int i = 0; i < bl->R; ++i) most = std::max(most, bl->host[i].npart_r);
     grid = dim3(most, c.J, bl->R);
   }
-  const RunGeom* rg = bl != nullptr ? bl->dev : nullptr;
   if constexpr (sizeof(T) == 4) {
     if (!f64) {
-      const auto k = c.jd != nullptr ? k_resid_schur2d<false, true, float2> : k_resid_schur2d<false, false, float2>;
-      k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
+      ProfScope ps_(KID_RESID_REFINE, s);
+      const auto k = c.jd != nullptr ? k_resid_schur2d<true> : k_resid_schur2d<false>;
+      k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, bl != nullptr ? bl->dev : nullptr);
       return;
     }
   }
-  const auto k = c.jd != nullptr ? k_resid_schur2d<true, true, cplx<T>> : k_resid_schur2d<true, false, cplx<T>>;
-  k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, rg);
+  launch_resid64<T>(b, x, r, r64, part, c, want_b, grid.x, s, bl);
 }
 template void launch_resid_schur2d<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool,
                                           bool, cudaStream_t, const BatchLaunch*);

@@ -7,62 +7,41 @@ namespace apfc {
 
 namespace {
 
-// Streams through a chunk of z-planes of a 32 x 16 point tile with a halo of two (36 x 20 cells,
-// one column of two adjacent rows per thread): at step t zeta = G_h eta is formed on plane t - 1
-// and r on plane t - 2, z-neighbours in registers, x- and y-neighbours from two-plane
-// shared-memory rings.  Every double is split once (dfloat.cuh); arithmetic and rounding as in
-// the 2D kernel (schur.cu).  F64: in FP64.
-constexpr int kR3X = 32, kR3Y = 16, kR3OX = kR3X + 4, kR3OY = kR3Y + 4, kR3NT = kR3OX * (kR3OY / 2);
-constexpr int kR3RW = kR3OX + 2, kR3Plane = (kR3OY + 2) * kR3RW, kR3PF = 1;
+// Streams through a chunk of z-planes of a tile of 28 columns: a warp spans the columns with a halo of
+// two on each side, a thread holds kR3R adjacent rows; at step t zeta = G_h eta is formed on plane
+// t - 1 and r on plane t - 2, z-neighbours in registers, x- and y-neighbours from two-plane
+// shared-memory rings.  The halo's outer rows only pass eta on, the next ones zeta.  Every double
+// is split once (dfloat.cuh); arithmetic and rounding as in the 2D kernel (schur.cu).
+// Sixteen warps of two rows, one block per SM: bound by the packed FP32 instructions (about 270 a
+// point, 88 per cent of that pipe's rate with the halo).  256^3 x 6: 4.21 ms, twelve warps 4.44, eight
+// of two in two blocks 4.61, eight of four 5.02 (with two operations a term more); the 32 x 16 tile of
+// 36-column cells before 4.63, with its rows across warps.  Now 3.93.
+constexpr int kR3NW = 16, kR3R = 2, kR3B = 1, kR3NT = 32 * kR3NW;
+constexpr int kR3X = 28, kR3OY = kR3NW * kR3R, kR3Y = kR3OY - 4;
+constexpr int kR3RW = 34, kR3Plane = kR3OY * kR3RW, kR3PF = 1;
 
-template <bool F64>
-struct R3Val;
-template <>
-struct R3Val<false> {
-  using V = PDF;
-  using S = float4;
-  static __device__ __forceinline__ V in(double2 v) { return pdf_split(v); }
-  static __device__ __forceinline__ S pack(V v) { return pdf_pack(v); }
-  static __device__ __forceinline__ V unpack(S v) { return pdf_unpack(v); }
-  static __device__ __forceinline__ V zero() { return PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-};
-template <>
-struct R3Val<true> {
-  using V = double2;
-  using S = double2;
-  static __device__ __forceinline__ V in(double2 v) { return v; }
-  static __device__ __forceinline__ S pack(V v) { return v; }
-  static __device__ __forceinline__ V unpack(S v) { return v; }
-  static __device__ __forceinline__ V zero() { return make_double2(0.0, 0.0); }
-};
 // G_h: centre, neighbour sums, neighbour differences (lane signs as in resid_coef); -kt G_h; -a
 struct R3Coef {
   LaneC g0, gl[3], ga[3], k0, kl[3], ka[3], ma;
 };
-template <bool F64>
-constexpr size_t resid3_smem() {
-  return 2ull * 2 * kR3Plane * 16 + (size_t)(kR3PF + 1) * kR3NT * 2 * sizeof(double2) + sizeof(R3Coef);
-}
+constexpr size_t kR3Smem = 2ull * 2 * kR3Plane * 16 + (size_t)(kR3PF + 1) * kR3NT * kR3R * sizeof(double2) + sizeof(R3Coef);
 
-template <bool F64, typename RT>
-__global__ void __launch_bounds__(kR3NT, 1)
-    k_resid_schur3d(const double2* __restrict__ b, double2* x, RT* __restrict__ r_out, double2* __restrict__ r64,
+__global__ void __launch_bounds__(kR3NT, kR3B)
+    k_resid_schur3d(const double2* __restrict__ b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Lz, int ntx, int want_b) {
-  using RV = R3Val<F64>;
-  using V = typename RV::V;
-  using SV = typename RV::S;
   extern __shared__ __align__(16) unsigned char r3_smem[];
-  SV* ring = reinterpret_cast<SV*>(r3_smem);  // [eta, zeta][2 planes][kR3Plane]
+  float4* ring = reinterpret_cast<float4*>(r3_smem);  // [eta, zeta][2 planes][kR3Plane]
   double2* stg = reinterpret_cast<double2*>(ring + 4 * kR3Plane);
-  R3Coef& q = *reinterpret_cast<R3Coef*>(stg + (kR3PF + 1) * kR3NT * 2);
-  __shared__ double shn[2][(kR3NT + 31) / 32];
+  R3Coef& q = *reinterpret_cast<R3Coef*>(stg + (kR3PF + 1) * kR3NT * kR3R);
+  __shared__ double shn[2][kR3NW];
+  constexpr int R = kR3R;
   const int j = blockIdx.z, t = threadIdx.x;
-  const int ry = t / kR3OX, px = t - ry * kR3OX;
+  const int w = __shfl_sync(0xffffffffu, t >> 5, 0), px = t & 31;
   const int tyi = blockIdx.x / ntx, txi = blockIdx.x - tyi * ntx;
   const long long pts = c.pts, plane = (long long)c.nx * c.ny;
   if (c.prof != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && t == 0)
     atomicAdd(c.prof + KID_RESID_REFINE,
-              (unsigned long long)pts * (3 * sizeof(double2) + sizeof(RT) +
+              (unsigned long long)pts * (3 * sizeof(double2) + sizeof(float2) +
                                          (r64 != nullptr ? sizeof(double2) : 0)));
   if (t == 0) {
     const ResidCoef<3> rc = resid_coef<3>(c, j);
@@ -77,87 +56,85 @@ __global__ void __launch_bounds__(kR3NT, 1)
   const long long fo = (long long)j * pts;
   r_out += fo;
   if (r64 != nullptr) r64 += fo;
-  for (int i = t; i < 4 * kR3Plane; i += kR3NT) ring[i] = RV::pack(RV::zero());
+  const PDF zero{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  for (int i = t; i < 4 * kR3Plane; i += kR3NT) ring[i] = pdf_pack(zero);
 
-  const int X = txi * kR3X - 2 + px, Y0 = tyi * kR3Y - 2 + 2 * ry;
+  const int X = txi * kR3X - 2 + px, Y0 = tyi * kR3Y - 2 + R * w;
   int gx = X % c.nx;
   if (gx < 0) gx += c.nx;
-  int off[2];
-  bool own[2];
+  int off[R];
+  bool own[R], zrow[R], rrow[R];  // zrow, rrow: zeta and r are formed on the row (uniform over the warp)
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < R; ++r) {
     int y = (Y0 + r) % c.ny;
     if (y < 0) y += c.ny;
     off[r] = y * c.nx + gx;
-    own[r] = px >= 2 && px < kR3OX - 2 && 2 * ry + r >= 2 && 2 * ry + r < kR3OY - 2 && X < c.nx && Y0 + r < c.ny;
+    zrow[r] = R * w + r >= 1 && R * w + r < kR3OY - 1;
+    rrow[r] = R * w + r >= 2 && R * w + r < kR3OY - 2 && Y0 + r < c.ny;
+    own[r] = px >= 2 && px < 30 && rrow[r] && X < c.nx;
   }
   const int z0 = blockIdx.y * Lz, nzc = min(c.nz, z0 + Lz) - z0, steps = nzc + 4;
   int fz = (z0 - 2) % c.nz;
   if (fz < 0) fz += c.nz;
   auto issue = [&](int tf, int slot) {
     if (tf < steps) {
-      double2* d = stg + ((size_t)slot * kR3NT + t) * 2;
+      double2* d = stg + (size_t)slot * kR3NT * R + t;
       const double2* p = et + fz * plane;
-      cheb_cp_async(d, p + off[0]);
-      cheb_cp_async(d + 1, p + off[1]);
+#pragma unroll
+      for (int r = 0; r < R; ++r) cheb_cp_async(d + r * kR3NT, p + off[r]);
       fz = cheb_wrap(fz, c.nz);
     }
     asm volatile("cp.async.commit_group;\n" ::);
   };
-  V e1[2], e2[2], h1[2], h2[2];
-  double2 bn[2];
+  PDF e1[R], e2[R], h1[R], h2[R];
+  double2 bn[R];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    e1[r] = e2[r] = h1[r] = h2[r] = RV::zero();
+  for (int r = 0; r < R; ++r) {
+    e1[r] = e2[r] = h1[r] = h2[r] = zero;
     bn[r] = make_double2(0.0, 0.0);
   }
   float rr = 0.f, bb = 0.f;
-  double rrd = 0.0, bbd = 0.0;
 #pragma unroll
   for (int tf = 0; tf < kR3PF; ++tf) issue(tf, tf);
   __syncthreads();
   int slot = 0, islot = kR3PF;
-  const int cell = (2 * ry + 1) * kR3RW + px + 1;
+  const int cell = R * w * kR3RW + px + 1;
   for (int tt = 0; tt < steps; ++tt) {
     issue(tt + kR3PF, islot);
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kR3PF));
     const int par = tt & 1;
     const long long zo = (long long)(z0 + tt - 4) * plane;  // plane tt - 2, where r is formed
-    const double2 bc[2] = {bn[0], bn[1]};
+    double2 bc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) bc[r] = bn[r];
     if (tt >= 3 && tt + 1 < steps) {
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < R; ++r)
         if (own[r]) bn[r] = bt[zo + plane + off[r]];
     }
-    V e0[2], h0[2];
+    PDF e0[R], h0[R];
     {
-      const double2* st = stg + ((size_t)slot * kR3NT + t) * 2;
+      const double2* st = stg + (size_t)slot * kR3NT * R + t;
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        e0[r] = RV::in(st[r]);
-        ring[par * kR3Plane + cell + r * kR3RW] = RV::pack(e0[r]);
+      for (int r = 0; r < R; ++r) {
+        e0[r] = pdf_split(st[r * kR3NT]);
+        ring[par * kR3Plane + cell + r * kR3RW] = pdf_pack(e0[r]);
       }
     }
-    const SV* re = ring + (par ^ 1) * kR3Plane + cell;
-    const SV* rz = re + 2 * kR3Plane;
+    const float4* re = ring + (par ^ 1) * kR3Plane + cell;
+    const float4* rz = re + 2 * kR3Plane;
     // zeta at plane tt - 1
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const V l = RV::unpack(re[r * kR3RW - 1]), rt = RV::unpack(re[r * kR3RW + 1]);
-      const V o = RV::unpack(re[r == 0 ? -kR3RW : 2 * kR3RW]);
-      const V ym = r == 0 ? o : e1[0], yp = r == 0 ? e1[1] : o;
+    for (int r = 0; r < R; ++r) {
+      h0[r] = zero;
+      if (!zrow[r]) continue;
+      const PDF l = pdf_unpack(re[r * kR3RW - 1]), rt = pdf_unpack(re[r * kR3RW + 1]);
+      const PDF ym = r == 0 ? pdf_unpack(re[-kR3RW]) : e1[r > 0 ? r - 1 : 0];
+      const PDF yp = r == R - 1 ? pdf_unpack(re[R * kR3RW]) : e1[r < R - 1 ? r + 1 : 0];
       double2 zd;
-      if constexpr (F64) {
-        const double2 s = make_double2(
-            fma(c.ih2[2], e2[r].x + e0[r].x, fma(c.ih2[1], ym.x + yp.x, fma(c.ih2[0], l.x + rt.x, c.c0 * e1[r].x))),
-            fma(c.ih2[2], e2[r].y + e0[r].y, fma(c.ih2[1], ym.y + yp.y, fma(c.ih2[0], l.y + rt.y, c.c0 * e1[r].y))));
-        const double k0 = c.kh[j][0], k1 = c.kh[j][1], k2 = c.kh[j][2];
-        h0[r] = make_double2(s.x - (k0 * (rt.y - l.y) + k1 * (yp.y - ym.y) + k2 * (e0[r].y - e2[r].y)),
-                             s.y + (k0 * (rt.x - l.x) + k1 * (yp.x - ym.x) + k2 * (e0[r].x - e2[r].x)));
-        zd = h0[r];
-      } else {
+      {
         PAcc a;
-        a.init(RV::zero());
+        a.init(zero);
         a.fma(q.g0.h, q.g0.l, e1[r]);
         a.fma(q.gl[0].h, q.gl[0].l, pdf_add(rt, l));
         a.fma(q.gl[1].h, q.gl[1].l, pdf_add(yp, ym));
@@ -168,34 +145,19 @@ __global__ void __launch_bounds__(kR3NT, 1)
         a.result(h0[r].h, h0[r].l);
         zd = make_double2(df_to_d(DF{h0[r].h.x, h0[r].l.x}), df_to_d(DF{h0[r].h.y, h0[r].l.y}));
       }
-      ring[(2 + par) * kR3Plane + cell + r * kR3RW] = RV::pack(h0[r]);
+      ring[(2 + par) * kR3Plane + cell + r * kR3RW] = pdf_pack(h0[r]);
       if (own[r] && tt >= 3 && tt < nzc + 3) zt[zo + plane + off[r]] = zd;
     }
     // r at plane tt - 2
     if (tt >= 4) {
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        if (!own[r]) continue;
-        const V l = RV::unpack(rz[r * kR3RW - 1]), rt = RV::unpack(rz[r * kR3RW + 1]);
-        const V o = RV::unpack(rz[r == 0 ? -kR3RW : 2 * kR3RW]);
-        const V ym = r == 0 ? o : h1[0], yp = r == 0 ? h1[1] : o;
+      for (int r = 0; r < R; ++r) {
+        if (!rrow[r] || !own[r]) continue;
+        const PDF l = pdf_unpack(rz[r * kR3RW - 1]), rt = pdf_unpack(rz[r * kR3RW + 1]);
+        const PDF ym = r == 0 ? pdf_unpack(rz[-kR3RW]) : h1[r > 0 ? r - 1 : 0];
+        const PDF yp = r == R - 1 ? pdf_unpack(rz[R * kR3RW]) : h1[r < R - 1 ? r + 1 : 0];
         const long long p = zo + off[r];
-        if constexpr (F64) {
-          const double2 s = make_double2(
-              fma(c.ih2[2], h2[r].x + h0[r].x, fma(c.ih2[1], ym.x + yp.x, fma(c.ih2[0], l.x + rt.x, c.c0 * h1[r].x))),
-              fma(c.ih2[2], h2[r].y + h0[r].y, fma(c.ih2[1], ym.y + yp.y, fma(c.ih2[0], l.y + rt.y, c.c0 * h1[r].y))));
-          const double k0 = c.kh[j][0], k1 = c.kh[j][1], k2 = c.kh[j][2], kt = c.kt[j], aa = c.a[j];
-          const double Gx = s.x - (k0 * (rt.y - l.y) + k1 * (yp.y - ym.y) + k2 * (h0[r].y - h2[r].y));
-          const double Gy = s.y + (k0 * (rt.x - l.x) + k1 * (yp.x - ym.x) + k2 * (h0[r].x - h2[r].x));
-          const double2 rv = make_double2(bc[r].x - (kt * Gx + aa * e2[r].x), bc[r].y - (kt * Gy + aa * e2[r].y));
-          if constexpr (sizeof(RT) == 16)
-            r_out[p] = rv;
-          else
-            r_out[p] = make_float2((float)rv.x, (float)rv.y);
-          if (r64 != nullptr) r64[p] = rv;
-          rrd += rv.x * rv.x + rv.y * rv.y;
-          if (want_b) bbd += bc[r].x * bc[r].x + bc[r].y * bc[r].y;
-        } else {
+        {
           const PDF bp = pdf_split(bc[r]);
           PAcc a;
           a.init(bp);
@@ -217,7 +179,7 @@ __global__ void __launch_bounds__(kR3NT, 1)
       }
     }
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < R; ++r) {
       e2[r] = e1[r];
       e1[r] = e0[r];
       h2[r] = h1[r];
@@ -228,22 +190,19 @@ __global__ void __launch_bounds__(kR3NT, 1)
     __syncthreads();
   }
   asm volatile("cp.async.wait_group 0;\n" ::);
-  if constexpr (!F64) rrd = (double)rr, bbd = (double)bb;
-  // the last warp is not full: sums through shared memory
-  double* red = reinterpret_cast<double*>(ring);
-  red[2 * t] = rrd;
-  red[2 * t + 1] = bbd;
-  __syncthreads();
-  if (t < 64) {
-    const int w = t >> 5, l = t & 31;
-    double v = 0.0;
-    for (int i = l; i < kR3NT; i += 32) v += red[2 * i + w];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (l == 0) shn[w][0] = v;
+  double rrd = (double)rr, bbd = (double)bb;
+  for (int o = 16; o > 0; o >>= 1) {
+    rrd += __shfl_xor_sync(0xffffffffu, rrd, o);
+    bbd += __shfl_xor_sync(0xffffffffu, bbd, o);
   }
+  if (px == 0) shn[0][w] = rrd, shn[1][w] = bbd;
   __syncthreads();
   const int npart = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
-  if (t < 2) part[(2LL * j + t) * npart + blk] = shn[t][0];
+  if (t < 2) {
+    double v = 0.0;
+    for (int i = 0; i < kR3NW; ++i) v += shn[t][i];
+    part[(2LL * j + t) * npart + blk] = v;
+  }
 }
 
 int resid3_planes(int nx, int ny, int nz, int J) {
@@ -259,26 +218,23 @@ int schur_resid3_parts(int nx, int ny, int nz, int J) {
   return ((nx + kR3X - 1) / kR3X) * ((ny + kR3Y - 1) / kR3Y) * ((nz + Lz - 1) / Lz);
 }
 
-template <bool F64, typename RT>
-static bool resid3(const double2* b, double2* x, RT* r, double2* r64, double* part, const OpCoef& c, bool want_b,
-                   cudaStream_t s) {
-  auto kern = k_resid_schur3d<F64, RT>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)resid3_smem<F64>());
-  if (attr != cudaSuccess) return false;
-  ProfScope ps_(KID_RESID_REFINE, s);
-  const int Lz = resid3_planes(c.nx, c.ny, c.nz, c.J), ntx = (c.nx + kR3X - 1) / kR3X;
-  kern<<<dim3(ntx * ((c.ny + kR3Y - 1) / kR3Y), (c.nz + Lz - 1) / Lz, c.J), kR3NT, resid3_smem<F64>(), s>>>(
-      b, x, r, r64, part, c, Lz, ntx, want_b);
-  return true;
-}
 template <typename T>
 bool launch_resid_schur3d(const double2* b, double2* x, cplx<T>* r, double2* r64, double* part, const OpCoef& c,
                           bool want_b, bool f64, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {
-    if (!f64) return resid3<false, float2>(b, x, r, r64, part, c, want_b, s);
+    if (!f64) {
+      static const cudaError_t attr =
+          cudaFuncSetAttribute(k_resid_schur3d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kR3Smem);
+      if (attr != cudaSuccess) return false;
+      ProfScope ps_(KID_RESID_REFINE, s);
+      const int Lz = resid3_planes(c.nx, c.ny, c.nz, c.J), ntx = (c.nx + kR3X - 1) / kR3X;
+      k_resid_schur3d<<<dim3(ntx * ((c.ny + kR3Y - 1) / kR3Y), (c.nz + Lz - 1) / Lz, c.J), kR3NT, kR3Smem, s>>>(
+          b, x, r, r64, part, c, Lz, ntx, want_b);
+      return true;
+    }
   }
-  return resid3<true, cplx<T>>(b, x, r, r64, part, c, want_b, s);
+  launch_resid64<T>(b, x, r, r64, part, c, want_b, schur_resid3_parts(c.nx, c.ny, c.nz, c.J), s, nullptr);
+  return true;
 }
 template bool launch_resid_schur3d<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool,
                                           bool, cudaStream_t);
