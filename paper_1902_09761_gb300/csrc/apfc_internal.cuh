@@ -525,6 +525,7 @@ struct SchurPlan {
   double lnrate[kMaxJ];
   int t0, ni, max_pass, fp64, J;      // L passes make t0 + ni L terms
 };
+int schur_most_passes(const SchurPlan& p);
 void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl = nullptr);
 
 // ---------------------------------------------------------------------------

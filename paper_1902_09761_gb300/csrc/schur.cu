@@ -243,7 +243,7 @@ int schur_terms(double tin, double lnrate) {
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr double kSchurLast64 = 0.4, kSchurLast32 = 1.0 / 16.0;
+constexpr float kSchurLast64 = 0.4f, kSchurLast32 = 1.f / 16.f, kSchurLeast = 0.05f;
 
 // Sums the partials of ||r||^2 and ||b||^2 (have bits 1, 2) of amplitude blockIdx.x of the run
 // and sets the number of passes of its next solve.
@@ -284,18 +284,20 @@ __global__ void __launch_bounds__(256) k_schur_plan(const __grid_constant__ Schu
   // The residual that a Chebyshev solve leaves sits in the low end of the spectrum, where it
   // weighs most in the error: the solve that is to meet the outer tolerance goes further below
   // it than a Krylov solve has to for the same error.
-  const double want = b2 > 0.0 ? p.tol * sqrt(b2 / r2) : p.tol_inner;
-  double tin;
+  // (FP32 is plenty for a number of terms; the FP64 pipe's square roots and logarithms took 3 us.)
+  const float tol = (float)p.tol, tol_inner = (float)p.tol_inner;
+  const float want = b2 > 0.0 ? tol * sqrtf((float)(b2 / r2)) : tol_inner;
+  float tin;
   if (p.fp64) {
-    tin = kSchurLast64 * (b2 > 0.0 ? want : p.tol);
+    tin = kSchurLast64 * (b2 > 0.0 ? want : tol);
   } else {
-    tin = fmin(0.5, fmax(p.tol_inner, 0.25 * want));
-    if (tin <= want) tin = fmin(tin, fmax(0.05 * p.tol_inner, kSchurLast32 * want));
+    tin = fminf(0.5f, fmaxf(tol_inner, 0.25f * want));
+    if (tin <= want) tin = fminf(tin, fmaxf(kSchurLeast * tol_inner, kSchurLast32 * want));
   }
-  const double x = 1.0 / tin;
-  const double need = x > 1.0 ? log(x + sqrt(x * x - 1.0)) / p.lnrate[j] : 0.0;
-  const double n = fmin(fmax(2.0, ceil(need)), 1e9);
-  k.iters = min(max(1, (int)ceil((n - p.t0) / p.ni)), p.max_pass);
+  const float x = 1.f / tin;
+  const float need = x > 1.f ? logf(x + sqrtf(x * x - 1.f)) / (float)p.lnrate[j] : 0.f;
+  const float n = fminf(fmaxf(2.f, ceilf(need)), 1e9f);
+  k.iters = min(max(1, (int)ceilf((n - p.t0) / p.ni)), p.max_pass);
 }
 
 // e^{i phi_d i}: blockIdx.y = amplitude
@@ -311,15 +313,21 @@ __global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, in
 
 // ---------------------------------------------------------------------------
 // Outer residual r = b - a eta - kt G_h (G_h eta) on 2D grids, streamed down the rows: a block
-// owns 256 columns (252 of them valid) and a segment of rows; at step t a thread forms zeta =
+// owns 64 columns (60 of them valid) and a segment of rows; at step t a thread forms zeta =
 // G_h eta at row t - 1 and r at row t - 2 of its column, the y-neighbours in registers (the row
 // below is the one just formed), the x-neighbours from two-row shared-memory rings.  Every
 // double is split once.  Writes zeta into the state (the solve never reads it, so it always
 // belongs to the latest eta), r as RT, optionally r in FP64, and per block the sums ||r||^2 and,
-// on request, ||b||^2.  JAC: a + d(x) in place of a (Picard with the Jacobian).Where
+// on request, ||b||^2.  JAC: a + d(x) in place of a (Picard with the Jacobian).  Where
 // SchurCoef::kappa asks for FP64 arithmetic resid_f64.cu's kernels run instead.
 // ---------------------------------------------------------------------------
-constexpr int kRsNT = 256, kRsPF = 2, kRsV = kRsNT - 4;
+// Two warps a block, twelve blocks per SM (80 registers): bound by the packed FP32 instructions (about
+// 190 a point) and the conversions' integer ones, at half of either's rate.  us, three amplitudes, at
+// 128^2 / 256^2 / 512^2 / 1024^2 / 1531 x 997 / 4096^2: 8.7 / 15 / 30 / 88 / 115 / 1023; four warps in
+// six blocks 10.6 / 15 / 33 / 88 / 116 / 1017, in four (126 registers) 12.5 / 15 / 33 / 91 / 120 / 1052;
+// eight in two 15 / 23 / 42 / 109 / 142 / 1147; one in 24 8.7 / 15 / 29 / 87 / 119 / 1078; tiles of
+// 28 x 28 held by a block 8.8 / 13 / 31 / 95 / 125 / 1220.
+constexpr int kRsNT = 64, kRsPF = 2, kRsV = kRsNT - 4;
 
 __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -327,7 +335,7 @@ __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
 }
 
 template <bool JAC>
-__global__ void __launch_bounds__(kRsNT, 2)
+__global__ void __launch_bounds__(kRsNT, 12)
     k_resid_schur2d(const double2* __restrict__ b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
                     int want_b, const RunGeom* rg) {
@@ -504,10 +512,13 @@ int schur_auto_rows(const SchurCoef& sc, const int* nx, const int* ny, int n, in
   return best_rows;
 }
 
+// Rows per segment: two rounds of the resident blocks, at least eight rows (and four of halo), or four
+// where eight leave every other multiprocessor idle (128^2: 12.3 against 8.7 us).
 int schur_resid_rows(int nx, int ny, int J) {
   const long long strips = (nx + kRsV - 1) / kRsV;
-  const long long rows = (long long)ny * strips * J / 912;  // about six blocks per SM
-  return (int)std::min<long long>(128, std::max<long long>(8, rows));
+  const long long rows = (long long)ny * strips * J / 3648;
+  const long long least = (ny + 7) / 8 * strips * J < 304 ? 4 : 8;
+  return (int)std::min<long long>(128, std::max(least, rows));
 }
 int schur_resid_parts(int nx, int ny, int J) {
   const int Ly = schur_resid_rows(nx, ny, J);
@@ -546,6 +557,16 @@ void launch_gauge_table(cplx<T>* tab, const OpCoef& c, int tx, int ty, int tz, c
 }
 template void launch_gauge_table<float>(float2*, const OpCoef&, int, int, int, cudaStream_t);
 template void launch_gauge_table<double>(double2*, const OpCoef&, int, int, int, cudaStream_t);
+
+// Passes that no FP32 solve of plan p exceeds (one to spare for the rounding of the device's logarithm).
+int schur_most_passes(const SchurPlan& p) {
+  long long n = 1;
+  for (int j = 0; j < p.J; ++j) {
+    const long long terms = schur_terms(kSchurLeast * p.tol_inner, p.lnrate[j]);
+    n = std::max(n, (terms - p.t0 + p.ni - 1) / p.ni + 1);
+  }
+  return (int)std::min<long long>(n, p.max_pass);
+}
 
 void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl) {
   ProfScope ps_(kid_of<double>(KID_FINALIZE), s);
