@@ -195,7 +195,8 @@ struct apfc_ctx {
   Work<double> w64;
   Work<float> w32;
   KScal* ks64 = nullptr;       // refinement norms (device)
-  KScal* ks64_host = nullptr;  // pinned
+  KScal* ks64_host = nullptr;  // pinned, of up to three checks
+  int last_sweeps = 0;         // FP32 solves of the last refinement by the Chebyshev iteration
   void* part64 = nullptr;      // refinement partials
   SchurWork<double> s64;
   SchurWork<float> s32;
@@ -862,16 +863,17 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   const auto [none, tx, ty, tz] = gauge_sizes(ctx);
   const GaugeTab<T> gt{w.tab, tx, ty, tz};
   const bool f64 = fp64 || schur_resid_f64(sc, o.tol);
+  bool want_b = !bnorm_ready;
   const ChebBufs<T> bufs{w.r[0], {w.r[0], w.r[1]}, {w.d[0], w.d[1]}, w.u, x, ctx->ks64};
   int total = 0, worst = KS_CONVERGED, sweep = 0;
   const double tol2 = o.tol * o.tol;
-  for (;; ++sweep) {
+  // residual, norms and passes of solve `sweep`, its scalars on their way to the host
+  auto check = [&](KScal* host) -> apfc_status {
     if (resid_ready) {
       prhs.have = 3;
       launch_schur_plan(prhs, ctx->ks64, s);
     } else {
-      const bool want_b = sweep == 0 && !bnorm_ready;
-      if (sweep == 0 && bnorm_ready) {
+      if (bnorm_ready) {
         prhs.have = 2;
         launch_schur_plan(prhs, ctx->ks64, s);
       }
@@ -882,15 +884,44 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       plan.have = want_b ? 3 : 1;
       launch_schur_plan(plan, ctx->ks64, s);
     }
-    *stencil_last = !resid_ready;
-    resid_ready = false;
+    resid_ready = bnorm_ready = want_b = false;  // of the first check alone
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(ctx->ks64_host, ctx->ks64, sizeof(KScal) * J, cudaMemcpyDeviceToHost, s));
-    CK(cudaStreamSynchronize(s));
+    CK(cudaMemcpyAsync(host, ctx->ks64, sizeof(KScal) * J, cudaMemcpyDeviceToHost, s));
+    return APFC_OK;
+  };
+  auto passes = [&](int n) -> apfc_status {
+    if (!launch_schur_passes<T>(sc, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, n, s, ctx->sms))
+      return fail(ctx, APFC_ECUDA, "the Chebyshev passes cannot be launched");
+    return APFC_OK;
+  };
+  // On small grids the host's waits (about 12 us each) weigh as much as the solves.  Where the last
+  // solve took two or more, the first two go out at their greatest number of passes without a look
+  // at the norms between them: passes beyond an amplitude's own return at once, and so do all of
+  // them once the residual is small enough.
+  const bool ahead = !fp64 && most >= 2 && ctx->last_sweeps >= 2 && ctx->dim == 2 && sc.plain && o.tile == 3 &&
+                     gauge_tiled(ctx->grid.n[0], ctx->grid.n[1], J);
+  KScal* rec = ctx->ks64_host;  // of the check at hand
+  int queued = 0;
+  for (;; ++sweep) {
+    if (queued > 0) {
+      --queued;
+      rec += J;
+      *stencil_last = true;
+    } else {
+      rec = ctx->ks64_host;
+      *stencil_last = !resid_ready;
+      if ((st = check(rec)) != APFC_OK) return st;
+      if (sweep == 0 && ahead)
+        for (queued = 0; queued < 2; ++queued) {
+          if ((st = passes(schur_most_passes(plan))) != APFC_OK) return st;
+          if ((st = check(rec + (queued + 1) * J)) != APFC_OK) return st;
+        }
+      CK(cudaStreamSynchronize(s));
+    }
     bool done = true, bad = false;
     int np = 0;
     for (int j = 0; j < J; ++j) {
-      const KScal& k = ctx->ks64_host[j];
+      const KScal& k = rec[j];
       if (!std::isfinite(k.rnorm2) || !std::isfinite(k.bnorm2)) bad = true;
       if (k.rnorm2 > tol2 * k.bnorm2) done = false;
       np = std::max(np, k.iters);
@@ -904,16 +935,15 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       worst = KS_NOCONV;
       break;
     }
-    if (!launch_schur_passes<T>(sc, m, o.tile, ctx->coef, cw.data(), gt, rows, bufs, np, s,
-                                ctx->sms))
-      return fail(ctx, APFC_ECUDA, "the Chebyshev passes cannot be launched");
+    if (queued == 0 && (st = passes(np)) != APFC_OK) return st;
     if (np > 0) total += (nt0 + ni * np + 1) / 2;  // two applications, as in a BiCGStab iteration
   }
   CK(cudaGetLastError());
   *total_it = total;
   *sweeps = sweep;
   *worst_out = worst;
-  ctx->resid = max_rel_resid(ctx->ks64_host, J);
+  if (!fp64) ctx->last_sweeps = sweep;
+  ctx->resid = max_rel_resid(rec, J);
   return APFC_OK;
 }
 
@@ -1513,7 +1543,7 @@ apfc_status apfc_init(apfc_ctx** out, const apfc_lattice* lat, const apfc_params
   if ((st = check(cudaMallocHost(&ctx->eout_host, sizeof(double)), "cudaMallocHost (energy)")) != APFC_OK) return st;
   if ((st = check(cudaMalloc(&ctx->ks64, sizeof(KScal) * ctx->J), "cudaMalloc (Krylov scalars)")) != APFC_OK)
     return st;
-  if ((st = check(cudaMallocHost(&ctx->ks64_host, sizeof(KScal) * ctx->J), "cudaMallocHost (Krylov scalars)")) !=
+  if ((st = check(cudaMallocHost(&ctx->ks64_host, 3 * sizeof(KScal) * ctx->J), "cudaMallocHost (Krylov scalars)")) !=
       APFC_OK)
     return st;
   if ((st = check(cudaMalloc(&ctx->part64, 16ull * kDotSlots * kDotBlocks * ctx->J), "cudaMalloc (partials)")) !=
