@@ -122,6 +122,33 @@ __host__ __device__ constexpr int kid_of(int k) {
 // Host side (api.cu): called by every launch wrapper around its launch.
 void prof_launch_begin(int kid, cudaStream_t s);
 void prof_launch_end(int kid, cudaStream_t s);
+// Programmatic dependent launch for the kernels of a solve, each of which is short and needs the last
+// one's results: a kernel launched by launch_dependent may be set up while its predecessor still runs,
+// and waits (dependent_wait, before its first access to memory) until that has completed and its
+// writes are visible; only then may its own successor be set up.  Its inputs are not declared
+// __restrict__: read-only loads could be moved above the wait.
+// Measured: 128^2, 4 steps 0.819 -> 0.724 ms; FP64 512^2 5.26 -> 4.90; rollout at 256^2 9.76 -> 9.33.
+// The streamed 2D passes are launched plainly: their blocks, placed as the last launch's drain, spread
+// unevenly (1024^2: 2.41 -> 2.55 ms).
+__device__ __forceinline__ void dependent_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+template <typename... P, typename... A>
+void launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 struct ProfScope {
   int kid;
   cudaStream_t s;

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
   float4* ring = reinterpret_cast<float4*>(gauge3_smem);  // [v, g'][2 planes][NW][first, last row][32]
   float4* stg = ring + SH::ring + threadIdx.x;            // [SLOTS][R][NT]
   const int j = blockIdx.z, t = threadIdx.x;
+  dependent_wait();
   const int npass = ks[j].iters;
   if (pass >= npass) return;
   const bool last = pass + 1 == npass;
@@ -340,7 +341,7 @@ bool launch_gauge3_pass(const OpCoef& c, const GaugeTab<float>& gt, const GaugeW
   float2* two[2] = {b.r[1], b.d[0]};
   const Gauge3Geom g{c.nx, c.ny, c.nz, Lz, (c.nx + TXV - 1) / TXV, c.pts};
   const dim3 grid((unsigned)(g.ntx * ((c.ny + TYV - 1) / TYV)), (unsigned)((c.nz + Lz - 1) / Lz), (unsigned)c.J);
-  kern<<<grid, SH::NT, SH::smem, s>>>(in, g, START ? b.r0 : two[pass & 1], START ? two[1] : two[1 - (pass & 1)], b.u,
+  launch_dependent(kern, grid, SH::NT, SH::smem, s, in, g, START ? b.r0 : two[pass & 1], START ? two[1] : two[1 - (pass & 1)], b.u,
                                       START ? two[0] : nullptr, b.x64, b.ks, pass, kid);
   return true;
 }

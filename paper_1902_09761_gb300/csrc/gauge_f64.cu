@@ -55,8 +55,8 @@ __noinline__ __device__ double2 g64_edge(const double2* wrap, double2 v, double 
 
 // add + n0 c + sum_d w_d (minus + plus)
 template <int DIM>
-__device__ __forceinline__ double2 g64_stencil(const double2* __restrict__ f, const G64Point<DIM>& q, const G64Param& c,
-                                               const double2* __restrict__ tab, double2 add, double n0,
+__device__ __forceinline__ double2 g64_stencil(const double2* f, const G64Point<DIM>& q, const G64Param& c,
+                                               const double2* tab, double2 add, double n0,
                                                const double* w) {
   const long long plane = (long long)c.nx * c.ny;
   double2 m[DIM], p[DIM];
@@ -90,9 +90,10 @@ __device__ __forceinline__ double2 g64_phase(const G64Param& c, const double2* t
 
 // b = -e^{i phi.x} r, v_1 = b / theta
 template <int DIM>
-__global__ void __launch_bounds__(256) k_g64_start(const __grid_constant__ G64Param c, const double2* __restrict__ r,
-                                                   double2* __restrict__ b, double2* __restrict__ v1, const KScal* ks) {
+__global__ void __launch_bounds__(256) k_g64_start(const __grid_constant__ G64Param c, const double2* r,
+                                                   double2* b, double2* v1, const KScal* ks) {
   const G64Point<DIM> q = g64_point<DIM>(c);
+  dependent_wait();
   if (ks[q.j].iters == 0 || !q.in) return;
   const long long pts = (long long)c.nx * c.ny * c.nz, i = q.j * pts + q.p;
   const double2* tab = c.tab + (long long)q.j * (c.tx + c.ty + c.tz);
@@ -103,9 +104,10 @@ __global__ void __launch_bounds__(256) k_g64_start(const __grid_constant__ G64Pa
 }
 
 template <int DIM>
-__global__ void __launch_bounds__(256) k_g64_n(const __grid_constant__ G64Param c, const double2* __restrict__ v,
-                                               double2* __restrict__ g, const KScal* ks, int pass) {
+__global__ void __launch_bounds__(256) k_g64_n(const __grid_constant__ G64Param c, const double2* v,
+                                               double2* g, const KScal* ks, int pass) {
   const G64Point<DIM> q = g64_point<DIM>(c);
+  dependent_wait();
   if (pass >= ks[q.j].iters) return;
   const long long o = (long long)q.j * c.nx * c.ny * c.nz;
   const double2* tab = c.tab + (long long)q.j * (c.tx + c.ty + c.tz);
@@ -117,10 +119,11 @@ __global__ void __launch_bounds__(256) k_g64_n(const __grid_constant__ G64Param 
 // vp: v_(n-1) in (first: zero), v_(n+1) out; an amplitude's last pass adds it to the state instead
 template <int DIM>
 __global__ void __launch_bounds__(256)
-    k_g64_update(const __grid_constant__ G64Param c, const double2* __restrict__ g, const double2* __restrict__ v,
-                 const double2* __restrict__ b, double2* __restrict__ vp, double2* __restrict__ x64, const KScal* ks,
+    k_g64_update(const __grid_constant__ G64Param c, const double2* g, const double2* v,
+                 const double2* b, double2* vp, double2* x64, const KScal* ks,
                  int pass, int kid) {
   const G64Point<DIM> q = g64_point<DIM>(c);
+  dependent_wait();
   const int npass = ks[q.j].iters;
   if (pass >= npass) return;
   const long long pts = (long long)c.nx * c.ny * c.nz, o = q.j * pts;
@@ -154,9 +157,9 @@ void pass64(const G64Param& in, const ChebBufs<double>& b, int pass, cudaStream_
   ProfScope ps_(kid, s);
   const dim3 grid((in.nx + kGX - 1) / kGX, (in.ny + kGY - 1) / kGY, in.nz * in.J);
   double2* two[2] = {b.r[1], b.d[0]};  // v of even and odd passes; g' in d[1], b in u
-  if (pass == 0) k_g64_start<DIM><<<grid, kGX * kGY, 0, s>>>(in, b.r0, b.u, two[0], b.ks);
-  k_g64_n<DIM><<<grid, kGX * kGY, 0, s>>>(in, two[pass & 1], b.d[1], b.ks, pass);
-  k_g64_update<DIM><<<grid, kGX * kGY, 0, s>>>(in, b.d[1], two[pass & 1], b.u, two[1 - (pass & 1)], b.x64, b.ks, pass,
+  if (pass == 0) launch_dependent(k_g64_start<DIM>, grid, kGX * kGY, 0, s, in, b.r0, b.u, two[0], b.ks);
+  launch_dependent(k_g64_n<DIM>, grid, kGX * kGY, 0, s, in, two[pass & 1], b.d[1], b.ks, pass);
+  launch_dependent(k_g64_update<DIM>, grid, kGX * kGY, 0, s, in, b.d[1], two[pass & 1], b.u, two[1 - (pass & 1)], b.x64, b.ks, pass,
                                              kid);
 }
 

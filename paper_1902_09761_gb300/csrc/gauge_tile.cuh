@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(32 * NW, MINB)
   __shared__ int its[(BATCH ? kChebRuns : 1) * kMaxJ];
   const int t = threadIdx.x, px = t & 31, w = __shfl_sync(0xffffffffu, t >> 5, 0);
   const C one = make_float2(1.f, 0.f), zero = make_float2(0.f, 0.f);
+  dependent_wait();
   if constexpr (BATCH) {
     for (int i = t; i < kChebRuns * c.J; i += 32 * NW) its[i] = ks[(long long)tab.run[i / c.J].run * c.J + i % c.J].iters;
   } else {
@@ -306,7 +307,7 @@ bool launch_tile_pass(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWei
     if (attr != cudaSuccess) return false;
     const ChebGeom g = cheb_geom(c.nx, c.ny, SH::H, SH::OX, SH::TY);
     const int total = g.nstrips * g.nsegs * c.J;
-    kern<<<std::min(total, MINB * sms), 32 * NW, SH::smem, s>>>(in, g, total, vin, b.d[cur], b.r[1 - cur],
+    launch_dependent(kern, std::min(total, MINB * sms), 32 * NW, SH::smem, s, in, g, total, vin, b.d[cur], b.r[1 - cur],
                                                                 b.d[1 - cur], b.u, b.x64, c.jd32, b.ks, UNITS * pass,
                                                                 kid, ChebNoTab{});
     return true;

@@ -71,6 +71,7 @@ __device__ __forceinline__ R64Geom r64_geom(const OpCoef& c, const RunGeom* rg) 
 
 template <int DIM>
 __global__ void __launch_bounds__(256) k_zeta64(double2* x, const __grid_constant__ OpCoef c, const RunGeom* rg) {
+  dependent_wait();
   const R64Geom g = r64_geom(c, rg);
   if ((int)blockIdx.x >= g.npart) return;
   const int j = blockIdx.y;
@@ -85,9 +86,10 @@ __global__ void __launch_bounds__(256) k_zeta64(double2* x, const __grid_constan
 
 template <int DIM, typename RT>
 __global__ void __launch_bounds__(256)
-    k_resid64(const double2* __restrict__ b, const double2* __restrict__ x, RT* __restrict__ r_out,
+    k_resid64(const double2* b, const double2* x, RT* __restrict__ r_out,
               double2* __restrict__ r64, double* __restrict__ part, const __grid_constant__ OpCoef c, int want_b,
               const RunGeom* rg) {
+  dependent_wait();
   const R64Geom g = r64_geom(c, rg);
   if ((int)blockIdx.x >= g.npart) return;
   const int j = blockIdx.y;
@@ -139,11 +141,11 @@ void launch_resid64(const double2* b, double2* x, cplx<T>* r, double2* r64, doub
   const dim3 grid(npart, c.J, bl != nullptr ? bl->R : 1);
   const RunGeom* rg = bl != nullptr ? bl->dev : nullptr;
   if (c.dim == 3) {
-    k_zeta64<3><<<grid, 256, 0, s>>>(x, c, rg);
-    k_resid64<3, cplx<T>><<<grid, 256, 0, s>>>(b, x, r, r64, part, c, want_b, rg);
+    launch_dependent(k_zeta64<3>, grid, 256, 0, s, x, c, rg);
+    launch_dependent(k_resid64<3, cplx<T>>, grid, 256, 0, s, b, x, r, r64, part, c, want_b, rg);
   } else {
-    k_zeta64<2><<<grid, 256, 0, s>>>(x, c, rg);
-    k_resid64<2, cplx<T>><<<grid, 256, 0, s>>>(b, x, r, r64, part, c, want_b, rg);
+    launch_dependent(k_zeta64<2>, grid, 256, 0, s, x, c, rg);
+    launch_dependent(k_resid64<2, cplx<T>>, grid, 256, 0, s, b, x, r, r64, part, c, want_b, rg);
   }
 }
 template void launch_resid64<float>(const double2*, double2*, float2*, double2*, double*, const OpCoef&, bool, int,

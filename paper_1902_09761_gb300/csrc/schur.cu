@@ -249,6 +249,7 @@ constexpr float kSchurLast64 = 0.4f, kSchurLast32 = 1.f / 16.f, kSchurLeast = 0.
 // and sets the number of passes of its next solve.
 __global__ void __launch_bounds__(256) k_schur_plan(const __grid_constant__ SchurPlan p, KScal* ks, const RunGeom* rg) {
   const int run = rg != nullptr ? blockIdx.x / p.J : 0, j = blockIdx.x - run * p.J;
+  dependent_wait();
   const double* part = p.part;
   int npart = p.npart;
   long long ss = p.slot_stride, sj = p.amp_stride;
@@ -336,13 +337,14 @@ __device__ __forceinline__ void rs_copy16(void* dst, const void* src) {
 
 template <bool JAC>
 __global__ void __launch_bounds__(kRsNT, 12)
-    k_resid_schur2d(const double2* __restrict__ b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
+    k_resid_schur2d(const double2* b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Ly, int nstrips, int nsegs,
                     int want_b, const RunGeom* rg) {
   __shared__ float4 ring[2][2][kRsNT + 2];             // eta, zeta
   __shared__ double2 stg[kRsPF + 1][2][kRsNT];     // eta, b rows in flight
   __shared__ double shn[2][kRsNT / 32];
   const int j = blockIdx.y, t = threadIdx.x;
+  dependent_wait();
   int nx = c.nx, ny = c.ny;
   long long pts = c.pts, fo = 0;
   if (rg != nullptr) {
@@ -540,7 +542,7 @@ void launch_resid_schur2d(const double2* b, double2* x, cplx<T>* r, double2* r64
     if (!f64) {
       ProfScope ps_(KID_RESID_REFINE, s);
       const auto k = c.jd != nullptr ? k_resid_schur2d<true> : k_resid_schur2d<false>;
-      k<<<grid, kRsNT, 0, s>>>(b, x, r, r64, part, c, Ly, ns, ng, want_b, bl != nullptr ? bl->dev : nullptr);
+      launch_dependent(k, grid, kRsNT, 0, s, b, x, r, r64, part, c, Ly, ns, ng, want_b, bl != nullptr ? bl->dev : nullptr);
       return;
     }
   }
@@ -570,7 +572,7 @@ int schur_most_passes(const SchurPlan& p) {
 
 void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl) {
   ProfScope ps_(kid_of<double>(KID_FINALIZE), s);
-  k_schur_plan<<<(bl ? bl->R : 1) * p.J, 256, 0, s>>>(p, ks, bl ? bl->dev : nullptr);
+  launch_dependent(k_schur_plan, (bl ? bl->R : 1) * p.J, 256, 0, s, p, ks, bl ? bl->dev : nullptr);
 }
 
 }  // namespace apfc

@@ -27,7 +27,7 @@ struct R3Coef {
 constexpr size_t kR3Smem = 2ull * 2 * kR3Plane * 16 + (size_t)(kR3PF + 1) * kR3NT * kR3R * sizeof(double2) + sizeof(R3Coef);
 
 __global__ void __launch_bounds__(kR3NT, kR3B)
-    k_resid_schur3d(const double2* __restrict__ b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
+    k_resid_schur3d(const double2* b, double2* x, float2* __restrict__ r_out, double2* __restrict__ r64,
                     double* __restrict__ part, const __grid_constant__ OpCoef c, int Lz, int ntx, int want_b) {
   extern __shared__ __align__(16) unsigned char r3_smem[];
   float4* ring = reinterpret_cast<float4*>(r3_smem);  // [eta, zeta][2 planes][kR3Plane]
@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kR3NT, kR3B)
   const int j = blockIdx.z, t = threadIdx.x;
   const int w = __shfl_sync(0xffffffffu, t >> 5, 0), px = t & 31;
   const int tyi = blockIdx.x / ntx, txi = blockIdx.x - tyi * ntx;
+  dependent_wait();
   const long long pts = c.pts, plane = (long long)c.nx * c.ny;
   if (c.prof != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && t == 0)
     atomicAdd(c.prof + KID_RESID_REFINE,
@@ -228,7 +229,8 @@ bool launch_resid_schur3d(const double2* b, double2* x, cplx<T>* r, double2* r64
       if (attr != cudaSuccess) return false;
       ProfScope ps_(KID_RESID_REFINE, s);
       const int Lz = resid3_planes(c.nx, c.ny, c.nz, c.J), ntx = (c.nx + kR3X - 1) / kR3X;
-      k_resid_schur3d<<<dim3(ntx * ((c.ny + kR3Y - 1) / kR3Y), (c.nz + Lz - 1) / Lz, c.J), kR3NT, kR3Smem, s>>>(
+      launch_dependent(
+          k_resid_schur3d, dim3(ntx * ((c.ny + kR3Y - 1) / kR3Y), (c.nz + Lz - 1) / Lz, c.J), kR3NT, kR3Smem, s,
           b, x, r, r64, part, c, Lz, ntx, want_b);
       return true;
     }
