@@ -94,7 +94,7 @@ def workload_config(n, steps_note=None):
         "dt": 1.0,
         "params": {"dB": PARAMS[0], "Bx": PARAMS[1], "t": PARAMS[2], "v": PARAMS[3]},
         "tol": TOL,
-        "krylov": "right-preconditioned BiCGStab, Schur-complement preconditioner",
+        "krylov": "Chebyshev iteration on the Schur complement in the real gauge, inside FP64 refinement",
         "cheb_degree": CHEB,
         "tol_inner": TOL_INNER,
         "picard_iters": PICARD[0],
@@ -120,7 +120,7 @@ def measured_peaks():
 # hexagonal FP32-refined step, counted from their source: (FP64 arithmetic, FP64 <-> FP32
 # conversions).  Both kernels do their arithmetic in FP32 on doubles split by integer
 # operations; only the FP64 outputs cost FP64 additions.
-#   residual_refine_f64 (k_resid2d_tma): r64 = f2d(hi) + f2d(lo), 4 per DOF.
+#   residual_refine_f64 (k_resid_schur2d): zeta and r64 = f2d(hi) + f2d(lo), 4 per DOF.
 #   rhs_f64 (k_rhs_resid_hex): the new right-hand side as a double, 2 per DOF.
 FP64_PIPE_OPS = {"residual_refine_f64": (4.0, 0.0), "rhs_f64": (2.0, 0.0)}
 

@@ -11,9 +11,8 @@
 // products instead of 1 + 4 DIM; the pair sum's error, about 2^-47 of the
 // neighbours' magnitude, stays below what the compensated sum keeps anyway.
 //
-// The single-grid kernel (resid2d.cu, TMA tiles) and the batched kernel
-// (kernels.cu, plain loads) both evaluate points here, so that a run alone and
-// in a batch round alike.
+// Evaluated by the residual of the block system (resid2d.cu, TMA tiles); the Schur
+// complement's residuals (schur.cu, schur3d.cu) take its pair sums and coefficients.
 #pragma once
 
 #include "apfc_internal.cuh"
