@@ -486,30 +486,36 @@ __global__ void __launch_bounds__(kRsNT, 12)
 
 }  // namespace
 
-// Rows per segment of the passes: each step of a block costs about the same, so the heights
-// are compared by (what the busiest multiprocessor has to run) x (rows + 2S).
+// Rows per segment of the passes: each step of a block costs about the same, so the heights ceil(ny / s)
+// are compared by (what the busiest multiprocessor has to run) x (rows + 2S).  One or two of its blocks
+// together cost 1, a full round of them 1.56 (wide strips 1.5), and blocks drift apart (0.2).  Two
+// steps, ms by height: 4096^2 512 23.5, 342 25.7, 296 24.4, 256 23.3, 205 24.4, 171 23.1, 164 22.8, 147
+// 24.0, 128 23.3, 64 23.8; 3000^2 334 14.2, 160 13.7, 100 13.4, 64 13.7; 2048^2 187 7.2, 128 6.6, 100
+// 7.6, 64 6.8; 1024^2 64 2.65, 47 2.37, 32 2.23.
 int schur_auto_rows(const SchurCoef& sc, const int* nx, const int* ny, int n, int J, int m, int elem_bytes, int tile,
                     int sms) {
   const bool f32 = elem_bytes == 8, wide = f32 && sc.plain && (tile == 2 || tile == 4 || tile == 5);
   const int S = sc.plain ? 2 * (f32 ? kGaugeNI32 : kGaugeNI64) : (f32 && m == 1 ? 8 : 2 + 2 * m);
   const int NC = wide ? 256 : 128;
   const int res = wide ? 3 : 6;       // resident blocks per SM
-  const double thr = wide ? 0.5 : 0.26;  // a step of one among several, a lone block's being 1
+  const double thr = wide ? 0.5 : 0.26;  // a step of one block of a full round, a lone block's being 1
   int most = 1;
   for (int i = 0; i < n; ++i) most = std::max(most, ny[i]);
   double best = 1e300;
   int best_rows = std::min(most, 128);
-  for (int rows = 4; rows <= 512; rows += rows < 64 ? 4 : 8) {
+  for (int seg = (most + 511) / 512; seg <= most; ++seg) {
+    const int rows = (most + seg - 1) / seg;
+    if (rows < 4 && seg > 1) break;
     long long blocks = 0;
     for (int i = 0; i < n; ++i)
       blocks += (long long)((nx[i] + NC - 2 * S - 1) / (NC - 2 * S)) * ((ny[i] + rows - 1) / rows) * J;
     const long long per = (blocks + sms - 1) / sms;  // blocks of the busiest SM
     const long long full = per / res, rest = per - full * res;
-    double t = full * std::max(1.0, res * thr);
-    if (rest > 0) t += std::max(1.0, rest * thr);
+    const double round = res * thr;
+    double t = full * round + 0.2;
+    if (rest > 0) t += std::max(1.0, 1.0 + (rest - 2) * (round - 1.0) / (res - 2));
     t *= std::min(rows, most) + 2 * S + 4;
     if (t < best) best = t, best_rows = rows;
-    if (rows >= most) break;
   }
   return best_rows;
 }
