@@ -114,7 +114,7 @@ typedef struct {
   double tol_inner;          /* relative tolerance of each FP32 inner solve         */
   int tile;                  /* fused 2D kernel variant 0..5 (columns per block and
                                 rows of look-ahead), default 3: with it the FP32
-                                Chebyshev solves of small grids (up to about 900^2
+                                Chebyshev solves of small grids (up to about 700^2
                                 with three amplitudes) run on tiles, whatever
                                 tile_rows                                          */
   int tile_rows;             /* rows per block of the fused 2D kernels of the

@@ -470,13 +470,13 @@ bool launch_cheb2d(int m, const OpCoef& c, const ChebStep* w, const ChebPass& cp
 bool launch_gauge2d(int tile, const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, int Ly,
                     const ChebBufs<float>& b, int pass, cudaStream_t s, const BatchLaunch* bl, int take);
 // Two units (of kGaugeNI32 terms) on tiles of 40 x 56 points, one to a multiprocessor at a time:
-// shorter than two streamed passes up to some 1500 tiles (three amplitudes, us per unit against a
-// streamed pass: 256^2, 105 tiles, 5.6 against 13; 768^2, 840, 23 against 30; 1024^2, 1482, 38 against
-// 39; 1531 x 997, 2106, 59 against 58).
+// shorter than two streamed passes up to some 700 tiles (three amplitudes, two steps, ms, tiles against
+// streamed: 256^2, 105 tiles, 0.53 / 0.69; 512^2, 390, 0.89 / 1.03; 700^2, 702, 1.37 / 1.43; 768^2, 840,
+// 1.58 / 1.51; 900^2, 1173, 2.00 / 1.84).
 constexpr int kTileUnits = 2, kTileX = 40, kTileY = 56;
 inline bool gauge_tiled(int nx, int ny, int J) {
   const long long tx = (nx + kTileX - 1) / kTileX, ty = (ny + kTileY - 1) / kTileY;
-  return tx * ty * J <= 1200;
+  return tx * ty * J <= 720;
 }
 bool launch_gauge_tile(const OpCoef& c, const GaugeTab<float>& gt, const GaugeWeights& w, const ChebBufs<float>& b,
                        int pass, int sms, cudaStream_t s, const BatchLaunch* bl);

@@ -323,7 +323,7 @@ __global__ void k_gauge_table(cplx<T>* tab, const __grid_constant__ OpCoef c, in
 // SchurCoef::kappa asks for FP64 arithmetic resid_f64.cu's kernels run instead.
 // ---------------------------------------------------------------------------
 // Two warps a block, twelve blocks per SM (80 registers): bound by the packed FP32 instructions (about
-// 190 a point) and the conversions' integer ones, at half of either's rate.  us, three amplitudes, at
+// 190 a point, that pipe busy 59 per cent of the time) and the conversions' integer ones (44).  us, three amplitudes, at
 // 128^2 / 256^2 / 512^2 / 1024^2 / 1531 x 997 / 4096^2: 8.7 / 15 / 30 / 88 / 115 / 1023; four warps in
 // six blocks 10.6 / 15 / 33 / 88 / 116 / 1017, in four (126 registers) 12.5 / 15 / 33 / 91 / 120 / 1052;
 // eight in two 15 / 23 / 42 / 109 / 142 / 1147; one in 24 8.7 / 15 / 29 / 87 / 119 / 1078; tiles of

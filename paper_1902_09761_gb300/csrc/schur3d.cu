@@ -13,7 +13,8 @@ namespace {
 // shared-memory rings.  The halo's outer rows only pass eta on, the next ones zeta.  Every double
 // is split once (dfloat.cuh); arithmetic and rounding as in the 2D kernel (schur.cu).
 // Sixteen warps of two rows, one block per SM: bound by the packed FP32 instructions (about 270 a
-// point, 88 per cent of that pipe's rate with the halo).  256^3 x 6: 4.21 ms, twelve warps 4.44, eight
+// point; with the halo they keep that pipe busy 52 per cent of the time) and the barriers between
+// planes.  256^3 x 6: 4.21 ms, twelve warps 4.44, eight
 // of two in two blocks 4.61, eight of four 5.02 (with two operations a term more); the 32 x 16 tile of
 // 36-column cells before 4.63, with its rows across warps.  Now 3.93.
 constexpr int kR3NW = 16, kR3R = 2, kR3B = 1, kR3NT = 32 * kR3NW;
