@@ -201,7 +201,8 @@ apfc_status apfc_step(apfc_ctx* ctx, double dt, int n);
  * 64 rows and every height ceil(ny / s) between 96 and 256 rows (t-kernel variant as set),
  * then, where the solve is BiCGStab, every t-kernel variant at the best height.  Keeps the
  * fastest in the context's options (opts.tile_rows stays 0 where the automatic height is;
- * *tile_rows is then BiCGStab's automatic height).  The state and the
+ * *tile_rows is then BiCGStab's automatic height; grids whose solves run on tiles have no other
+ * candidate).  The state and the
  * statistics are restored (the next step takes a stencil initial residual).  Only
  * the FP32-refined fused path on 2D grids has a choice to make: other
  * configurations return APFC_OK with their options unchanged and ms_per_step 0.

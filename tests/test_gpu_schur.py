@@ -184,3 +184,17 @@ def test_picard_with_the_jacobian_across_tiles(prec, shape, h):
     ref, _ = PC.step_picard(eta, 1.0, P, L, h, 2, jacobian=True)
     assert max(rel_l2_per_amp(ctx.get_amplitudes(), ref)) <= 2e-9
     ctx.close()
+
+
+@pytest.mark.parametrize("kind,shape", [("hex", (7, 33)), ("hex", (8, 32)), ("hex", (9, 31)), ("hex", (353, 997)),
+                                        ("hex", (352, 992)), ("bcc", (3, 5, 33)), ("bcc", (60, 33, 31))])
+def test_zeta_of_new_amplitudes_around_block_edges(kind, shape):
+    # blocks of 32 x 8 points, of 32 x 32 from 304 blocks on.  Seven products of FP32 pairs, each
+    # good to about 2^-44 of the largest term: below 1e-12 relative
+    h = H2 if kind == "hex" else (np.pi / 2,) * 3
+    ctx, L = context(kind, shape, h, precision=A.APFC_FP32_REFINED)
+    eta = inputs.random_amplitudes(L.J, shape, seed=98, scale=0.1)
+    ctx.set_amplitudes(eta)
+    ref = np.stack([O.apply_G(eta[j], L.k[j], h) for j in range(L.J)])
+    assert max(rel_l2_per_amp(ctx.get_zeta(), ref)) <= 1e-12
+    ctx.close()
