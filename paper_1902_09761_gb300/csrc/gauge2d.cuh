@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(NT, MINB)
 
   const C zero = mkc<T>((T)0, (T)0), one = mkc<T>((T)1, (T)0);
   for (int i = t; i < (int)(SH::ring_elems + SH::b_elems); i += NT) ring[i] = zero;
+  __syncthreads();  // the first fetches land in b's ring, over zeros that other threads have stored
 
   // columns of this thread: V t .. V t + V - 1 of the strip; a column beyond the grid is the
   // periodic image times e^{i phi_x nx m}

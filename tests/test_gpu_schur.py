@@ -198,3 +198,20 @@ def test_zeta_of_new_amplitudes_around_block_edges(kind, shape):
     ref = np.stack([O.apply_G(eta[j], L.k[j], h) for j in range(L.J)])
     assert max(rel_l2_per_amp(ctx.get_zeta(), ref)) <= 1e-12
     ctx.close()
+
+
+@pytest.mark.parametrize("opts", [dict(tile=0), dict(tile=5), dict(tile=0, tile_rows=9), dict(tile=0, tile_rows=1)])
+@pytest.mark.parametrize("shape", [(61, 233), (40, 464)])
+def test_streamed_passes_repeat_bit_for_bit(shape, opts):
+    # the streamed passes (strips of 128 and 256 columns) fetch their first rows into shared memory
+    # that the block has just cleared: many blocks, the same bits from every one of them each time
+    ctx, L = context("hex", shape, H2, precision=A.APFC_FP32_REFINED, tol=1e-12, **opts)
+    eta = inputs.random_amplitudes(3, shape, seed=99, scale=0.15)
+    first = None
+    for _ in range(20):
+        ctx.set_amplitudes(eta)
+        ctx.step(1.0, 2)
+        got = ctx.get_amplitudes()
+        first = got if first is None else first
+        assert np.array_equal(got, first)
+    ctx.close()
