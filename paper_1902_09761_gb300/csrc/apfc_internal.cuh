@@ -551,6 +551,7 @@ struct SchurPlan {
   double tol, tol_inner;
   double lnrate[kMaxJ];
   int t0, ni, max_pass, fp64, J;      // L passes make t0 + ni L terms
+  int follow;                        // not the first check of a queue: nothing where that one found nothing to do
 };
 int schur_most_passes(const SchurPlan& p);
 void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const BatchLaunch* bl = nullptr);

@@ -196,7 +196,7 @@ struct apfc_ctx {
   Work<float> w32;
   KScal* ks64 = nullptr;       // refinement norms (device)
   KScal* ks64_host = nullptr;  // pinned, of up to three checks
-  int last_sweeps = 0;         // FP32 solves of the last refinement by the Chebyshev iteration
+  int last_sweeps = 0;         // FP32 solves expected of the next refinement: the last one's
   void* part64 = nullptr;      // refinement partials
   SchurWork<double> s64;
   SchurWork<float> s32;
@@ -769,6 +769,10 @@ apfc_status status_of(apfc_ctx* ctx, int worst) {
   return APFC_OK;
 }
 
+// What the first refinement from new amplitudes or with new options may need, whatever went before:
+// an FP32 solve gains at most tol_inner.
+void expect_sweeps(apfc_ctx* ctx) { ctx->last_sweeps = ctx->opts.tol < ctx->opts.tol_inner ? 2 : 0; }
+
 const SchurCoef& schur_of(const apfc_ctx* ctx) { return ctx->coef.jd != nullptr ? ctx->schur_jac : ctx->schur; }
 
 // Whether the solve runs as the Chebyshev iteration on the Schur complement: constant
@@ -868,7 +872,8 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   int total = 0, worst = KS_CONVERGED, sweep = 0;
   const double tol2 = o.tol * o.tol;
   // residual, norms and passes of solve `sweep`, its scalars on their way to the host
-  auto check = [&](KScal* host) -> apfc_status {
+  auto check = [&](KScal* host, bool follow = false) -> apfc_status {
+    plan.follow = follow;
     if (resid_ready) {
       prhs.have = 3;
       launch_schur_plan(prhs, ctx->ks64, s);
@@ -897,7 +902,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   // On small grids the host's waits (about 12 us each) weigh as much as the solves.  Where the last
   // solve took two or more, the first two go out at their greatest number of passes without a look
   // at the norms between them: passes beyond an amplitude's own return at once, and so do all of
-  // them once the residual is small enough.
+  // them once the residual is small enough.  The state's bits do not depend on it.
   const bool ahead = !fp64 && most >= 2 && ctx->last_sweeps >= 2 && ctx->dim == 2 && sc.plain && o.tile == 3 &&
                      gauge_tiled(ctx->grid.n[0], ctx->grid.n[1], J);
   KScal* rec = ctx->ks64_host;  // of the check at hand
@@ -914,7 +919,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
       if (sweep == 0 && ahead)
         for (queued = 0; queued < 2; ++queued) {
           if ((st = passes(schur_most_passes(plan))) != APFC_OK) return st;
-          if ((st = check(rec + (queued + 1) * J)) != APFC_OK) return st;
+          if ((st = check(rec + (queued + 1) * J, true)) != APFC_OK) return st;
         }
       CK(cudaStreamSynchronize(s));
     }
@@ -1565,6 +1570,7 @@ apfc_status apfc_set_opts(apfc_ctx* ctx, const apfc_opts* opts) {
   ctx->coef_dt = -1.0;  // tau_mode may have changed
   ctx->have_prev = false;
   ctx->have_xprev = false;
+  expect_sweeps(ctx);
   return APFC_OK;
 }
 
@@ -1575,6 +1581,7 @@ apfc_status apfc_set_amplitudes(apfc_ctx* ctx, const void* eta, int where, int d
   ctx->err.clear();
   ctx->have_prev = false;
   ctx->have_xprev = false;
+  expect_sweeps(ctx);
   apfc_status st = copy_part(ctx, const_cast<void*>(eta), where, 1, true, dtype);
   if (st != APFC_OK) return st;
   std::string e;

@@ -281,7 +281,17 @@ __global__ void __launch_bounds__(256) k_schur_plan(const __grid_constant__ Schu
   if (p.have & 2) k.bnorm2 = s[1];
   const double r2 = k.rnorm2, b2 = k.bnorm2;
   k.iters = 0;
-  if (!isfinite(r2) || !isfinite(b2) || r2 <= p.tol * p.tol * b2) return;
+  const bool more = isfinite(r2) && isfinite(b2) && r2 > p.tol * p.tol * b2;
+  if (p.follow) {
+    // A stencil residual may exceed the tolerance where the first check's, formed pointwise, met it:
+    // the refinement ended there, and what was queued behind it must leave the state alone.
+    bool any = false;
+    for (int i = 0; i < p.J; ++i) any = any || ks[i].active != 0;
+    if (!any) return;
+  } else {
+    k.active = more;
+  }
+  if (!more) return;
   // The residual that a Chebyshev solve leaves sits in the low end of the spectrum, where it
   // weighs most in the error: the solve that is to meet the outer tolerance goes further below
   // it than a Krylov solve has to for the same error.
