@@ -957,11 +957,18 @@ apfc_status solve_fp64(apfc_ctx* ctx, const double2* b, double2* x, int* iters, 
   if (use_schur(ctx)) {
     int sweeps = 0;
     bool stencil = false;
-    return schur_solve<double>(ctx, ctx->s64, b, x, nullptr, false, false, iters, &sweeps, worst, &stencil);
+    const apfc_status st =
+        schur_solve<double>(ctx, ctx->s64, b, x, nullptr, false, false, iters, &sweeps, worst, &stencil);
+    if (st != APFC_OK || *worst != KS_NOCONV) return st;
+    // its solves did not suffice: BiCGStab goes on from where they ended
+  } else {
+    *iters = 0;
   }
   apfc_status st = alloc_work<double>(ctx, ctx->w64);
   if (st != APFC_OK) return st;
-  st = krylov<double>(ctx, ctx->w64, b, x, ctx->opts.tol, ctx->opts.max_iter, iters, worst);
+  int it = 0;
+  st = krylov<double>(ctx, ctx->w64, b, x, ctx->opts.tol, ctx->opts.max_iter, &it, worst);
+  *iters += it;
   if (st == APFC_OK) ctx->resid = max_rel_resid(ctx->w64.ks_host, ctx->J);
   return st;
 }

@@ -50,78 +50,75 @@ struct Symbol {
     const double p = (1.0 - cheb(m + 1, (theta[j] - d) / delta[j]) / tsig[j]) / d;
     return (c.a[j] + c.kt[j] * g * g) * p * p;
   }
-  double at(int j, const double* q) const {
-    double K = 0.0, A = 0.0;
+  // Of all wave numbers with the same K = 2 sum_d (1 - cos q_d) / h_d^2 (d takes no other part in
+  // S p(D)^2), those where A = 2 sum_d (k_d / h_d) sin q_d is largest: sin is concave in 1 - cos, so
+  // there is one such point for every K, tan q_d = k_d h_d / lambda, and lambda from infinity to
+  // minus infinity makes the curve of them.  At lambda = 0 a dimension with k_d = 0 runs from 0 to
+  // pi.  s in [0, 3]: lambda > 0, that stretch, lambda < 0.
+  void curve(int j, double s, double* K, double* A) const {
+    const double th = 1.57079632679489661923 * (s < 1.0 ? s : s < 2.0 ? 1.0 : s - 1.0);
+    const double sn = std::sin(th), cs = s < 1.0 || s > 2.0 ? std::cos(th) : 0.0;
+    *K = *A = 0.0;
     for (int d = 0; d < c.dim; ++d) {
-      const double s = std::sin(0.5 * q[d]);
-      K += 4.0 * s * s / (h[d] * h[d]);
-      A += 2.0 * c.kh[j][d] * std::sin(q[d]);
+      const double ih2 = 1.0 / (h[d] * h[d]), kh = std::fabs(c.kh[j][d]) / ih2 * sn;  // |k_d| h_d sin(theta)
+      double sq = 0.0, cq = s < 1.0 ? 1.0 : s < 2.0 ? std::cos(3.14159265358979323846 * (s - 1.0)) : -1.0;
+      if (kh > 1e-12) {
+        const double ir = 1.0 / std::sqrt(kh * kh + cs * cs);
+        sq = kh * ir;
+        cq = cs * ir;
+      }
+      *K += 2.0 * ih2 * (1.0 - cq);
+      *A += 2.0 * std::fabs(c.kh[j][d]) * sq;
     }
-    return of(j, K, -K - A);
   }
 };
 
 }  // namespace
 
-// Bounds of the spectrum of S_j p(D)^2 over all wave numbers: sampled on a mesh, then the best
-// few samples improved by a pattern search, with 1% to spare on both sides.
+// Bounds of the spectrum of S_j p(D)^2 over all wave numbers.  G_h's symbol is -K - A, and -A occurs
+// with every A: for each K the symbol lies between its values at |G| = max(0, K - A) and K + A with A
+// at its largest, so the extremes over the curve of these points bound it.  The curve is sampled, and
+// every extremum of the samples narrowed down (golden section); 1% to spare on both sides.  Against
+// dense samples of the symbol (1024^2 wave numbers, h 0.2 to 1.5, dt 0.1 to 100, degrees 1 to 4) both
+// ends are within 0.4%.  A 32 x 32 sample improved by a pattern search left the least eigenvalue up to
+// 1.5 times too high: the symbol has a narrow valley along G = 0.
 void schur_spectrum(const OpCoef& c, const apfc_grid& grid, int m, double* lmin, double* lmax) {
   const Symbol sym(c, grid.h, m);
-  const int n = c.dim == 2 ? 32 : 20;
-  constexpr double kTwoPi = 6.283185307179586476925286766559;
-  std::vector<double> K1(3 * n, 0.0), S1(3 * n, 0.0);
-  for (int d = 0; d < c.dim; ++d)
-    for (int i = 0; i < n; ++i) {
-      const double q = kTwoPi * i / n, s = std::sin(0.5 * q);
-      K1[d * n + i] = 4.0 * s * s / (grid.h[d] * grid.h[d]);
-      S1[d * n + i] = 2.0 * std::sin(q);
-    }
-  constexpr int kBest = 4;
-  struct Cand {
-    double v;
-    int i[3];
-  };
+  constexpr int n = 128;  // samples of each stretch
+  constexpr double kGolden = 0.61803398874989484820;
+  std::vector<double> at, v[2];
   for (int j = 0; j < c.J; ++j) {
-    Cand best[2][kBest];
-    for (auto& b : best)
-      for (auto& e : b) e = Cand{1e300, {0, 0, 0}};
-    const int nz = c.dim == 3 ? n : 1;
-    for (int iz = 0; iz < nz; ++iz)
-      for (int iy = 0; iy < n; ++iy)
-        for (int ix = 0; ix < n; ++ix) {
-          double K = K1[ix] + K1[n + iy], A = c.kh[j][0] * S1[ix] + c.kh[j][1] * S1[n + iy];
-          if (c.dim == 3) K += K1[2 * n + iz], A += c.kh[j][2] * S1[2 * n + iz];
-          const double v = sym.of(j, K, -K - A);
-          for (int w = 0; w < 2; ++w) {
-            const double key = w == 0 ? v : -v;
-            if (key >= best[w][kBest - 1].v) continue;
-            int p = kBest - 1;
-            while (p > 0 && best[w][p - 1].v > key) best[w][p] = best[w][p - 1], --p;
-            best[w][p] = Cand{key, {ix, iy, iz}};
-          }
-        }
+    bool free = false;
+    for (int d = 0; d < c.dim; ++d) free = free || std::fabs(c.kh[j][d]) * grid.h[d] * grid.h[d] <= 1e-12;
+    at.clear();  // where every k_d is nonzero, lambda = 0 is the one point s = 1, and s = 2 + follows on it
+    for (int i = 0; i <= 3 * n; ++i)
+      if (free || i <= n || i > 2 * n) at.push_back((double)i / n);
+    auto value = [&](int w, double s) {
+      double K, A;
+      sym.curve(j, s, &K, &A);
+      const double g = w == 0 ? std::max(0.0, K - A) : K + A;
+      return w == 0 ? sym.of(j, K, g) : -sym.of(j, K, g);
+    };
+    const int ns = (int)at.size();
     double ext[2] = {1e300, 1e300};
-    for (int w = 0; w < 2; ++w)
-      for (const Cand& e : best[w]) {
-        if (e.v >= 1e300) continue;
-        double q[3], v = e.v;
-        for (int d = 0; d < 3; ++d) q[d] = kTwoPi * e.i[d] / n;
-        for (double step = kTwoPi / (2 * n); step > 1e-3;) {
-          bool moved = false;
-          for (int d = 0; d < c.dim; ++d)
-            for (double sg : {-1.0, 1.0}) {
-              const double old = q[d];
-              q[d] += sg * step;
-              const double f = w == 0 ? sym.at(j, q) : -sym.at(j, q);
-              if (f < v)
-                v = f, moved = true;
-              else
-                q[d] = old;
-            }
-          if (!moved) step *= 0.5;
+    for (int w = 0; w < 2; ++w) {
+      v[w].resize(ns);
+      for (int i = 0; i < ns; ++i) v[w][i] = value(w, at[i]);
+      for (int i = 0; i < ns; ++i) {
+        if ((i > 0 && v[w][i - 1] < v[w][i]) || (i + 1 < ns && v[w][i + 1] < v[w][i])) continue;
+        ext[w] = std::min(ext[w], v[w][i]);
+        const int i0 = std::max(i - 1, 0), i1 = std::min(i + 1, ns - 1);
+        double lo = at[i0], hi = at[i1];
+        const bool jump = !free && lo <= 1.0 && hi > 2.0;
+        if (jump) hi -= 1.0;
+        for (int it = 0; it < 30; ++it) {
+          const double x = hi - kGolden * (hi - lo), y = lo + kGolden * (hi - lo);
+          const double fx = value(w, jump && x > 1.0 ? x + 1.0 : x), fy = value(w, jump && y > 1.0 ? y + 1.0 : y);
+          ext[w] = std::min(ext[w], std::min(fx, fy));
+          (fx < fy ? hi : lo) = fx < fy ? y : x;
         }
-        ext[w] = std::min(ext[w], v);
       }
+    }
     lmin[j] = 0.99 * ext[0];
     lmax[j] = -1.01 * ext[1];
   }

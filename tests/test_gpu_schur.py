@@ -272,3 +272,42 @@ def test_solves_queued_ahead_do_not_change_a_converged_state():
                 assert plain.stats()["resid_last"] == ahead.stats()["resid_last"] == p
             met += 1
     assert met > 0, tried
+
+
+def _preconditioned_bounds(k, h, dt, m, n=1024):
+    # least and greatest value of the symbol of S p(D)^2 over n^2 wave numbers
+    kap = float(k @ k)
+    a, kt, q = 1.0 / dt + kap * P.dB, kap * P.Bx, 2.0 * np.pi * np.arange(n) / n
+    sD, mu, kmax = np.sqrt(a), np.sqrt(kt), sum(4.0 / x**2 for x in h)
+    K = sum(np.expand_dims(4.0 * np.sin(q / 2) ** 2 / h[d] ** 2, 1 - d) for d in range(2))
+    G = -K - sum(np.expand_dims(2.0 * k[d] / h[d] * np.sin(q), 1 - d) for d in range(2))
+    theta, delta = sD + 0.5 * mu * kmax, 0.5 * mu * kmax
+    cheb = np.polynomial.Chebyshev.basis(m + 1)
+    p = (1.0 - cheb((theta - sD - mu * K) / delta) / cheb(theta / delta)) / (sD + mu * K)
+    s = (a + kt * G**2) * p**2
+    return s.min(), s.max()
+
+
+@pytest.mark.parametrize("h,dt,m", [(0.49, 20.0, 3), (0.475, 10.0, 3), (0.363, 10.0, 4), (0.5, 20.0, 2), (0.45, 10.0, 1)])
+def test_fine_grids_with_long_steps_take_the_one_solve_planned(h, dt, m):
+    # An FP64 solve is planned to end below 0.4 of the tolerance: with the spectrum's true bounds
+    # (allowing 3% on their ratio) about acosh(1 / reduction) / rate terms, two to an iteration, do.
+    # A bound inside the spectrum leaves modes that shrink too slowly, and further solves.
+    shape, tol = (96, 100), 1e-10
+    ctx, L = context("hex", shape, (h, h), precision=A.APFC_FP64, tol=tol, cheb_degree=m)
+    eta = inputs.random_amplitudes(3, shape, seed=102, scale=0.15)
+    b = O.rhs(eta, dt, P, L)
+    most = 0.0
+    for j in range(3):
+        lo, hi = _preconditioned_bounds(L.k[j], (h, h), dt, m)
+        r = b[j] - np.fft.ifft2(O.schur_symbol(L.k[j], dt, P, shape, (h, h)) * np.fft.fft2(eta[j]))
+        reduction = 0.4 * tol * np.linalg.norm(b[j]) / np.linalg.norm(r)
+        rate = np.arccosh((1.03 * hi + lo) / (1.03 * hi - lo))
+        most = max(most, np.arccosh(1.0 / reduction) / rate)
+    ctx.set_amplitudes(eta)
+    ctx.step(dt)
+    assert ctx.stats()["iters_last"] <= most / 2 + 2
+    # a right-hand side with a residual spread over every mode
+    lam = inputs.random_amplitudes(3, shape, seed=103, scale=0.1)
+    ctx.adjoint_step(dt, eta, eta, lam)
+    ctx.close()
