@@ -453,30 +453,28 @@ __global__ void k_rhs(const double2* __restrict__ x, double2* __restrict__ b, co
   }
 }
 
-// zeta-part of the state = G_h (eta-part)
-// zeta = G_h eta from the state's eta-parts, FP64-accurate without the FP64 pipe: the point
+// zeta = G_h eta from the state's eta-parts on 2D grids, FP64-accurate without the FP64 pipe: the point
 // and its neighbours split into FP32 pairs and G_h as one compensated sum of products with
-// the residual's grouping (resid_point.cuh), rounded to the nearest double at the end.
-// A block forms 32 x ROWS points of a plane: a double is split once for all its readers, and a thread's
-// coefficients (as many splits) serve ROWS / 8 points.  us at 1024^2 x 3 / 4096^2 x 3 / 256^3 x 6: a thread
-// per point reading its neighbours 58 / 811 / 2281, 8 rows 58 / 803 / 2139, 32 rows 46 / 636 / 1674; 8
-// where 32 give fewer than two blocks per SM (128^2 x 3: 8.4 against 11.7).
-template <int DIM, int ROWS>
+// the residual's grouping (resid_point.cuh), rounded to the nearest double at the end.  (3D grids:
+// FP64 arithmetic, stream3d.cu.)
+// A block forms 32 x ROWS points: a double is split once for all its readers, and a thread's
+// coefficients (as many splits) serve ROWS / 8 points.  us at 1024^2 x 3 / 4096^2 x 3: a thread
+// per point reading its neighbours 58 / 811, 8 rows 58 / 803, 32 rows 46 / 636; 8 where 32 give
+// fewer than two blocks per SM (128^2 x 3: 8.4 against 11.7).
+template <int ROWS>
 __global__ void __launch_bounds__(256) k_zeta(double2* __restrict__ x, const __grid_constant__ OpCoef c) {
   prof_add3(c, KID_ZETA, 2ull * (unsigned long long)c.pts * sizeof(double2));
   __shared__ float4 tile[ROWS + 2][34];  // the points' pairs and their (x, y) neighbours'
-  const int j = amp_of(c), z = (int)(blockIdx.z - (unsigned)j * (unsigned)c.nz);
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * ROWS;
-  const long long plane = (long long)c.nx * c.ny;
+  const int j = blockIdx.z, x0 = blockIdx.x * 32, y0 = blockIdx.y * ROWS;
   const double2* e = x + (2LL * j + 1) * c.pts;
   for (int i = threadIdx.x; i < (ROWS + 2) * 34; i += 256) {
     const int ly = i / 34, lx = i - ly * 34;
     int gx = x0 + lx - 1, gy = y0 + ly - 1;
     gx = gx < 0 ? gx + c.nx : gx < c.nx ? gx : gx % c.nx;
     gy = gy < 0 ? gy + c.ny : gy < c.ny ? gy : gy % c.ny;
-    tile[ly][lx] = pdf_pack(pdf_split(e[z * plane + (long long)gy * c.nx + gx]));
+    tile[ly][lx] = pdf_pack(pdf_split(e[(long long)gy * c.nx + gx]));
   }
-  const ResidCoef<DIM> q = resid_coef<DIM>(c, j);
+  const ResidCoef<2> q = resid_coef<2>(c, j);
   const int tx = threadIdx.x & 31;
   __syncthreads();
   if (x0 + tx >= c.nx) return;
@@ -484,26 +482,19 @@ __global__ void __launch_bounds__(256) k_zeta(double2* __restrict__ x, const __g
   for (int r = 0; r < ROWS / 8; ++r) {
     const int ty = r * 8 + (threadIdx.x >> 5);
     if (y0 + ty >= c.ny) return;
-    const long long p = z * plane + (long long)(y0 + ty) * c.nx + x0 + tx;
-    PDF en[DIM][2];
-    en[0][0] = pdf_unpack(tile[ty + 1][tx]);
-    en[0][1] = pdf_unpack(tile[ty + 1][tx + 2]);
-    en[1][0] = pdf_unpack(tile[ty][tx + 1]);
-    en[1][1] = pdf_unpack(tile[ty + 2][tx + 1]);
-    if constexpr (DIM == 3) {
-      en[2][0] = pdf_split(e[z == 0 ? p + (c.nz - 1) * plane : p - plane]);
-      en[2][1] = pdf_split(e[z + 1 == c.nz ? p - z * plane : p + plane]);
-    }
+    const PDF xm = pdf_unpack(tile[ty + 1][tx]), xp = pdf_unpack(tile[ty + 1][tx + 2]);
+    const PDF ym = pdf_unpack(tile[ty][tx + 1]), yp = pdf_unpack(tile[ty + 2][tx + 1]);
     PAcc a;
     a.init(PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)});
     a.fma(q.g0.h, q.g0.l, pdf_unpack(tile[ty + 1][tx + 1]));
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) a.fma(q.gl[d].h, q.gl[d].l, pdf_add(en[d][1], en[d][0]));
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) a.fma(q.ga[d].h, q.ga[d].l, pdf_swap(pdf_sub(en[d][1], en[d][0])));
+    a.fma(q.gl[0].h, q.gl[0].l, pdf_add(xp, xm));
+    a.fma(q.gl[1].h, q.gl[1].l, pdf_add(yp, ym));
+    a.fma(q.ga[0].h, q.ga[0].l, pdf_swap(pdf_sub(xp, xm)));
+    a.fma(q.ga[1].h, q.ga[1].l, pdf_swap(pdf_sub(yp, ym)));
     float2 hi, lo;
     a.result(hi, lo);
-    x[2LL * j * c.pts + p] = make_double2(df_to_d(DF{hi.x, lo.x}), df_to_d(DF{hi.y, lo.y}));
+    x[2LL * j * c.pts + (long long)(y0 + ty) * c.nx + x0 + tx] =
+        make_double2(df_to_d(DF{hi.x, lo.x}), df_to_d(DF{hi.y, lo.y}));
   }
 }
 
@@ -1394,14 +1385,16 @@ void launch_extrapolate(double2* x, double2* xp, const OpCoef& c, cudaStream_t s
 }
 
 void launch_zeta(double2* x, const OpCoef& c, cudaStream_t s) {
+  if (c.dim == 3) {
+    launch3d_zeta(x, c, s);
+    return;
+  }
   ProfScope ps_(KID_ZETA, s);
-  const unsigned nx = (c.nx + 31) / 32, nz = (unsigned)(c.nz * c.J);
-  const dim3 tall(nx, (c.ny + 31) / 32, nz), flat(nx, (c.ny + 7) / 8, nz);
-  const bool wide = (long long)tall.x * tall.y * tall.z >= 304;
-  if (c.dim == 3)
-    wide ? k_zeta<3, 32><<<tall, 256, 0, s>>>(x, c) : k_zeta<3, 8><<<flat, 256, 0, s>>>(x, c);
+  const dim3 tall((c.nx + 31) / 32, (c.ny + 31) / 32, c.J), flat((c.nx + 31) / 32, (c.ny + 7) / 8, c.J);
+  if ((long long)tall.x * tall.y * tall.z >= 304)
+    k_zeta<32><<<tall, 256, 0, s>>>(x, c);
   else
-    wide ? k_zeta<2, 32><<<tall, 256, 0, s>>>(x, c) : k_zeta<2, 8><<<flat, 256, 0, s>>>(x, c);
+    k_zeta<8><<<flat, 256, 0, s>>>(x, c);
 }
 void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const double2* r_prev, float2* r32,
                       double* partials, const OpCoef& c, const NonlinTable& nt, bool schur, cudaStream_t s,

@@ -1,7 +1,7 @@
 // z-streaming stencil passes of the APFC step on 3D grids (arXiv:1902.09761, Sec. II):
 // the block operator A_j of Eq. linear_system2 (M = I), the steps of the preconditioner of
 // Eq. preconditioner (f = beta2 - kt G beta1, the Chebyshev applications of the diffusion
-// solves, step 4) and the residual r = b - A x, each one kernel that
+// solves, step 4), the residual r = b - A x and zeta = G_h eta of new amplitudes, each one kernel that
 // streams (x, y) tiles through chunks of z-planes.  The Krylov inner products of A P^{-1}
 // come out of the A passes.
 #include <algorithm>
@@ -405,6 +405,24 @@ struct OpChebSweep3 {
       R.at(j)[p] = rn;
       Dn.at(j)[p] = dn;
     }
+  }
+};
+
+// zeta-part of the state = G_h (eta-part), FP64 arithmetic (256^3 x 6: 5.5 ms, bound by the FP64 pipe;
+// FP32 pairs as in 2D take 1.7, but flush what lies below 2^-74 and keep 48 bits)
+struct OpZeta3 {
+  static constexpr int NS = 1, ND = 0, NQ = 0, MINB = 3;
+  double2* x;
+  long long pts;
+  int kid;
+  unsigned long long bytes;
+  template <typename Q>
+  __device__ void coef(Q&, int) const {}
+  __host__ __device__ const double2* src(int, int j) const { return x + (2LL * j + 1) * pts; }
+  __host__ __device__ const double2* qsrc(int, int) const { return nullptr; }
+  __device__ void apply(int j, long long p, const N7<double> (&n)[1], const OpCoef& c, const Coef7<double>& q,
+                        Acc<double>*, const double2*) const {
+    x[2LL * j * pts + p] = G7(n[0], q);
   }
 };
 
@@ -908,6 +926,11 @@ void launch3d_cheb_sweep(CFieldRef<T> Dd, FieldRef<T> X, FieldRef<T> R, FieldRef
                      kid_of<T>(KID_CHEB_SWEEP),
                      (last ? (fold ? 7ull : 4ull) : 6ull) * (unsigned long long)c.pts * sizeof(cplx<T>)};
   stream3d<T, OpChebSweep3<T>>(c, op, act, s);
+}
+void launch3d_zeta(double2* x, const OpCoef& c, cudaStream_t s) {
+  ProfScope ps3_(KID_ZETA, s);
+  OpZeta3 op{x, c.pts, KID_ZETA, 2ull * (unsigned long long)c.pts * sizeof(double2)};
+  k_stream3d<double, OpZeta3><<<grid_stream3d<double>(c), 256, 0, s>>>(c, op, nullptr);
 }
 #define APFC_INST3(T)                                                                                                \
   template void launch3d_apply_A<T>(const cplx<T>*, cplx<T>*, const OpCoef&, const KScal*, cudaStream_t);           \

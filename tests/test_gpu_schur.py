@@ -311,3 +311,19 @@ def test_fine_grids_with_long_steps_take_the_one_solve_planned(h, dt, m):
     lam = inputs.random_amplitudes(3, shape, seed=103, scale=0.1)
     ctx.adjoint_step(dt, eta, eta, lam)
     ctx.close()
+
+
+@pytest.mark.parametrize("scale", [0.1, 1e-25])
+@pytest.mark.parametrize("prec", PRECISIONS)
+def test_3d_zeta_of_new_amplitudes_in_fp64(prec, scale):
+    # 26 roundings of 2^-53 each (white amplitudes: the sum is as large as its terms), twice in the
+    # gradient; amplitudes of any size (FP32 pairs take those below 2^-74 for zero)
+    shape, h = (9, 16, 37), (np.pi / 2, 1.3, 1.1)
+    ctx, L = context("bcc", shape, h, precision=prec)
+    eta = inputs.random_amplitudes(6, shape, seed=104, scale=scale)
+    ctx.set_amplitudes(eta)
+    ref = np.stack([O.apply_G(eta[j], L.k[j], h) for j in range(6)])
+    assert max(rel_l2_per_amp(ctx.get_zeta(), ref)) <= 3e-15
+    ref = 2.0 * np.prod(h) * O.energy_gradient(eta, P, L, h)
+    assert max(rel_l2_per_amp(ctx.energy_gradient(eta)[0], ref)) <= 6e-15
+    ctx.close()
