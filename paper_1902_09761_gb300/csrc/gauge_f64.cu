@@ -33,13 +33,22 @@ struct G64Point {
   long long p;  // within the amplitude's field
   bool in;
 };
+// blockIdx.y = amplitude; blockIdx.x counts the tiles of all planes (a grid's other dimensions end at
+// 65535, which long boxes have more of)
 template <int DIM>
 __device__ __forceinline__ G64Point<DIM> g64_point(const G64Param& c) {
+  const unsigned ntx = (c.nx + kGX - 1) / kGX, row = blockIdx.x / ntx;
   G64Point<DIM> q;
-  q.j = DIM == 3 ? blockIdx.z / c.nz : blockIdx.z;
-  q.z = DIM == 3 ? blockIdx.z - q.j * c.nz : 0;
-  q.x = blockIdx.x * kGX + (threadIdx.x & 31);
-  q.y = blockIdx.y * kGY + (threadIdx.x >> 5);
+  q.j = blockIdx.y;
+  unsigned ty = row;
+  q.z = 0;
+  if constexpr (DIM == 3) {
+    const unsigned nty = (c.ny + kGY - 1) / kGY;
+    q.z = row / nty;
+    ty = row - q.z * nty;
+  }
+  q.x = (blockIdx.x - row * ntx) * kGX + (threadIdx.x & 31);
+  q.y = ty * kGY + (threadIdx.x >> 5);
   q.in = q.x < c.nx && q.y < c.ny;
   q.p = ((long long)q.z * c.ny + q.y) * c.nx + q.x;
   return q;
@@ -156,7 +165,7 @@ template <int DIM>
 void pass64(const G64Param& in, const ChebBufs<double>& b, int pass, cudaStream_t s) {
   const int kid = kid_of<double>(KID_FUSED_APINV);
   ProfScope ps_(kid, s);
-  const dim3 grid((in.nx + kGX - 1) / kGX, (in.ny + kGY - 1) / kGY, in.nz * in.J);
+  const dim3 grid((unsigned)((in.nx + kGX - 1) / kGX) * ((in.ny + kGY - 1) / kGY) * in.nz, in.J);
   double2* two[2] = {b.r[1], b.d[0]};  // v of even and odd passes; g' in d[1], b in u
   if (pass == 0) launch_dependent(k_g64_start<DIM>, grid, kGX * kGY, 0, s, in, b.r0, b.u, two[0], b.ks);
   launch_dependent(k_g64_n<DIM>, grid, kGX * kGY, 0, s, in, two[pass & 1], b.d[1], b.ks, pass);

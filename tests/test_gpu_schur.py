@@ -327,3 +327,11 @@ def test_3d_zeta_of_new_amplitudes_in_fp64(prec, scale):
     ref = 2.0 * np.prod(h) * O.energy_gradient(eta, P, L, h)
     assert max(rel_l2_per_amp(ctx.energy_gradient(eta)[0], ref)) <= 6e-15
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("kind,shape", [("bcc", (11000, 3, 4)), ("hex", (530000, 3))])
+def test_boxes_longer_than_a_grid_dimension(kind, shape, prec):
+    # 6 x 11000 planes and 530000 / 8 rows of tiles: more than 65535
+    h = (np.pi / 2,) * len(shape)
+    _steps(shape, h, 1, 1e-10, tol=1e-13, precision=prec)
