@@ -335,3 +335,19 @@ def test_boxes_longer_than_a_grid_dimension(kind, shape, prec):
     # 6 x 11000 planes and 530000 / 8 rows of tiles: more than 65535
     h = (np.pi / 2,) * len(shape)
     _steps(shape, h, 1, 1e-10, tol=1e-13, precision=prec)
+
+
+@pytest.mark.parametrize("kind,shape", [("hex", (128, 128)), ("hex", (190, 251)), ("bcc", (24, 30, 33))])
+def test_refined_steps_end_well_below_the_tolerance(kind, shape):
+    # The solve that can meet the tolerance aims at 1/16 of it, or at 0.03 tol_inner of its own
+    # residual where that is more: at most 0.15 of the tolerance.  One that cannot is aimed to leave
+    # at least five times the tolerance, so that none ends just beneath it.
+    h, tol = (np.pi / 2,) * len(shape), 1e-10
+    ctx, L = context(kind, shape, h, precision=A.APFC_FP32_REFINED, tol=tol)
+    phi = O.uniform_solid_hex(P) if kind == "hex" else O.uniform_solid_bcc(P)
+    for seed in range(4):
+        ctx.set_amplitudes(inputs.single_grain(L.k, phi, shape, h, 0.3 * min(shape) * h[0], 5.0 + seed, seed=105 + seed, noise=1e-3))
+        for _ in range(5):
+            ctx.step(1.0)
+            assert ctx.stats()["resid_last"] <= 0.2 * tol
+    ctx.close()
