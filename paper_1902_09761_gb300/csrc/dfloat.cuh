@@ -56,11 +56,25 @@ __device__ __forceinline__ DF split_d(double v) {
   return DF{__uint_as_float(h), l};
 }
 
-// A double rounded to a float (through 48 bits: half an ulp and 2^-24 more; tiny values give 0, those
-// from 2^127 NaN).
+// (float)v and (double)f to the bit, by integer operations where the float is normal or zero: on the
+// FP64 pipe a conversion costs as much as 64 FP32 instructions.  The rest are calls, so that no
+// predicated-off conversion takes the pipe's time either.
+static __noinline__ __device__ float d2f_convert(double v) { return (float)v; }
+static __noinline__ __device__ double f2d_convert(float f) { return (double)f; }
 __device__ __forceinline__ float d2f(double v) {
-  const DF d = split_d(v);
-  return __fadd_rn(d.h, d.l);
+  const unsigned hw = (unsigned)__double2hiint(v), lw = (unsigned)__double2loint(v), e = hw & 0x7ff00000u;
+  if (e - (897u << 20) >= (254u << 20)) {            // not in [2^-126, 2^128)
+    if (e >= (873u << 20)) return d2f_convert(v);    // from 2^-150 on: subnormal, infinity, NaN
+    return __uint_as_float(hw & 0x80000000u);
+  }
+  unsigned h = ((__funnelshift_l(lw, hw, 3) + 0x40000000u) & 0x7fffffffu) | (hw & 0x80000000u);
+  h += (lw & 0x1fffffffu) + (h & 1u) > 0x10000000u;  // to nearest, ties to even
+  return __uint_as_float(h);
+}
+__device__ __forceinline__ double f2d_exact(float f) {
+  const unsigned u = __float_as_uint(f), t = u & 0x7f800000u;
+  if (t - 0x00800000u >= 0x7f000000u) return (u << 1) == 0u ? __hiloint2double((int)u, 0) : f2d_convert(f);
+  return __hiloint2double((((int)u >> 3) & (int)0x8fffffffu) + 0x38000000, (int)(u << 29));
 }
 
 // Exact double of a float (zero and subnormal floats give 0, Inf and NaN give NaN).

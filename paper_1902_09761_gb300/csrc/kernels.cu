@@ -1133,8 +1133,8 @@ __global__ void k_energy_grad(const double2* __restrict__ x, double2* __restrict
 // One thread per point on a (32 x 8)-point tile grid with z in blockIdx.z.  A = sqrt(2
 // sum |eta_j|^2) is formed once per point of the tile and its one-point (x, y) halo in
 // shared memory (FP64: A and |grad A| decide the branches of Eq. hhh); z-neighbours
-// in 3D are formed directly.  The phases go through FP32: eta converted on load (by integer
-// and FP32 operations: 24 conversions a point on the FP64 pipe made 1024^2 take 158 us, now 109), the
+// in 3D are formed directly.  The phases go through FP32: eta converted on load (to the bit, by integer
+// operations: 24 conversions a point on the FP64 pipe made 1024^2 take 158 us, now 109), the
 // product a conj(b) and atan2f in FP32 (about 1e-7 rad per difference), the weighted
 // sums and omega in FP32.  The branches compare squares: |grad A|^2 >= eps^2 and
 // A^2 > A_min^2.
@@ -1212,7 +1212,7 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
   float wmax = 0.0f;
   for (int q = 0; q < nc; ++q) {
     if (!ok) om[q] = 0.0f;
-    omega[q * c.pts + p] = f2d(om[q]);
+    omega[q * c.pts + p] = f2d_exact(om[q]);
     wmax = fmaxf(wmax, fabsf(om[q]));
   }
   if (!want_h && amp == nullptr) return;
@@ -1233,7 +1233,7 @@ __global__ void __launch_bounds__(256) k_rotation(const double2* __restrict__ x,
       // theta = asin(w); sin(theta/2) = w / sqrt(2 (1 + cos(theta)))
       const float w = fminf(wmax, 1.0f);
       const float s = w / sqrtf(2.0f * (1.0f + sqrtf(1.0f - w * w)));
-      const double h_amp = s > 0.0f ? rp.pi_over_nk / f2d(s) : INFINITY;
+      const double h_amp = s > 0.0f ? rp.pi_over_nk / f2d_exact(s) : INFINITY;
       hv = fmin(fmax(h_amp, rp.h_int), rp.h_max);
     } else {
       hv = rp.h_max;
