@@ -70,6 +70,7 @@ struct OpCoef {
   double mu[kMaxJ];         //                       mu = sqrt(kt)
   double inv_mu[kMaxJ];
   double inv_theta[kMaxJ];  // Chebyshev: 1/theta, theta = centre of D's interval
+  float zero;               // 0, known at run time alone (PAcc, dfloat.cuh)
   unsigned long long* prof; // device byte counters per kernel id (nullptr: not measuring)
   const double* jd;         // Picard with Jacobian: kap_j D_j per point, [J][pts] (nullptr: none)
   const float2* jd32;       // the same as {value, 0} for the FP32 fused kernels' staged fetch

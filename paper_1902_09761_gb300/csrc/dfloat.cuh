@@ -186,20 +186,16 @@ struct PDF {
 __device__ __forceinline__ PDF pdf_of(CDF a) { return PDF{make_float2(a.x.h, a.y.h), make_float2(a.x.l, a.y.l)}; }
 __device__ __forceinline__ PDF pdf_split(double2 v) { return pdf_of(cdf_split(v)); }
 
-// Zero that the compiler cannot see (the kernels that sum have blockDim.y = 1): a packed
-// multiplication whose only use is an addition would be contracted with it, .rn or not, and the sum's
-// error would no longer be what follows computes (measured: 1e-8 instead of 6e-15).
-__device__ __forceinline__ float2 run_time_zero() {
-  const float z = __int_as_float((int)blockDim.y - 1);
-  return make_float2(z, z);
-}
-
-// Sum of products: s holds the running leading sum, e every error term.
+// Sum of products: s holds the running leading sum, e every error term.  nil: zero, from a kernel
+// argument, where the compiler cannot see it: a packed multiplication whose only use is an addition
+// would be contracted with it, .rn or not, and the sum's error would no longer be what fma() computes
+// (measured: 1e-8 instead of 6e-15).
 struct PAcc {
-  float2 s, e;
-  __device__ __forceinline__ void init(PDF v) {
+  float2 s, e, nil;
+  __device__ __forceinline__ void init(PDF v, float zero) {
     s = v.h;
     e = v.l;
+    nil = make_float2(zero, zero);
   }
   // s + e += v (coefficient +-1: sg = +1 or -1 in both lanes)
   __device__ __forceinline__ void add(PDF v, float sg) {
@@ -214,7 +210,7 @@ struct PAcc {
   // operations; with TwoSum and TwoProd apart and three additions to e it was twelve, and 1.2 to 1.4
   // times the error (sums of 5 to 8 terms)
   __device__ __forceinline__ void fma(float2 ch, float2 cl, PDF v) {
-    const float2 p = p_fma(ch, v.h, run_time_zero());
+    const float2 p = p_fma(ch, v.h, nil);
     const float2 t = p_add(s, p);
     const float2 nb = p_sub(s, t);                 // -(t - s)
     const float2 w = p_sub(s, p_add(t, nb));       // s's part of the sum's error

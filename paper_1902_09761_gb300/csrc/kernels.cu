@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(256) k_zeta(double2* __restrict__ x, const __g
     const PDF xm = pdf_unpack(tile[ty + 1][tx]), xp = pdf_unpack(tile[ty + 1][tx + 2]);
     const PDF ym = pdf_unpack(tile[ty][tx + 1]), yp = pdf_unpack(tile[ty + 2][tx + 1]);
     PAcc a;
-    a.init(PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)});
+    a.init(PDF{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, c.zero);
     a.fma(q.g0.h, q.g0.l, pdf_unpack(tile[ty + 1][tx + 1]));
     a.fma(q.gl[0].h, q.gl[0].l, pdf_add(xp, xm));
     a.fma(q.gl[1].h, q.gl[1].l, pdf_add(yp, ym));

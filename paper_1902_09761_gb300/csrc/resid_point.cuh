@@ -52,11 +52,13 @@ template <int DIM>
 struct ResidCoef {
   LaneC g0, gl[DIM], ga[DIM];
   LaneC k0, kl[DIM], ka[DIM];
+  float zero;
 };
 template <int DIM>
 __device__ __forceinline__ ResidCoef<DIM> resid_coef(const OpCoef& c, int j) {
   ResidCoef<DIM> q;
   const double kt = c.kt[j];
+  q.zero = c.zero;
   q.g0 = lane_c(c.c0, 1.f, 1.f);
   q.k0 = lane_c(kt * c.c0, -1.f, -1.f);
 #pragma unroll
@@ -77,7 +79,7 @@ __device__ __forceinline__ void resid_point(const ResidCoef<DIM>& q, LaneC ma, P
                                             float2& l1, float2& f2, float2& l2) {
   // r1 = b1 - zeta + G_h eta: centre, neighbour sums, neighbour differences
   PAcc a1;
-  a1.init(b1);
+  a1.init(b1, q.zero);
   a1.add(zc, -1.f);
   a1.fma(q.g0.h, q.g0.l, ec);
 #pragma unroll
@@ -86,7 +88,7 @@ __device__ __forceinline__ void resid_point(const ResidCoef<DIM>& q, LaneC ma, P
   for (int d = 0; d < DIM; ++d) a1.fma(q.ga[d].h, q.ga[d].l, pdf_swap(pdf_sub(en[d][1], en[d][0])));
   // r2 = b2 - kt G_h zeta - a eta
   PAcc a2;
-  a2.init(b2);
+  a2.init(b2, q.zero);
   a2.fma(q.k0.h, q.k0.l, zc);
 #pragma unroll
   for (int d = 0; d < DIM; ++d) a2.fma(q.kl[d].h, q.kl[d].l, pdf_add(zn[d][1], zn[d][0]));

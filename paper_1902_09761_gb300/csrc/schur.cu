@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kRsNT, 12)
     double2 zd;
     {
       PAcc a;
-      a.init(zero);
+      a.init(zero, c.zero);
       a.fma(q.g0.h, q.g0.l, e1);
       a.fma(q.gl[0].h, q.gl[0].l, pdf_add(er, el));
       a.fma(q.gl[1].h, q.gl[1].l, pdf_add(e0, e2));
@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(kRsNT, 12)
         {
           const PDF bp = pdf_split(bv);
           PAcc a;
-          a.init(bp);
+          a.init(bp, c.zero);
           a.fma(q.k0.h, q.k0.l, z1);
           a.fma(q.kl[0].h, q.kl[0].l, pdf_add(zr, zl));
           a.fma(q.kl[1].h, q.kl[1].l, pdf_add(z0, z2));

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kR3NT, kR3B)
       double2 zd;
       {
         PAcc a;
-        a.init(zero);
+        a.init(zero, c.zero);
         a.fma(q.g0.h, q.g0.l, e1[r]);
         a.fma(q.gl[0].h, q.gl[0].l, pdf_add(rt, l));
         a.fma(q.gl[1].h, q.gl[1].l, pdf_add(yp, ym));
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kR3NT, kR3B)
         {
           const PDF bp = pdf_split(bc[r]);
           PAcc a;
-          a.init(bp);
+          a.init(bp, c.zero);
           a.fma(q.k0.h, q.k0.l, h1[r]);
           a.fma(q.kl[0].h, q.kl[0].l, pdf_add(rt, l));
           a.fma(q.kl[1].h, q.kl[1].l, pdf_add(yp, ym));
