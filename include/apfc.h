@@ -200,9 +200,9 @@ apfc_status apfc_step(apfc_ctx* ctx, double dt, int n);
  * after one untimed step; first the automatic height, BiCGStab's automatic height, 32, 48 and
  * 64 rows and every height ceil(ny / s) between 96 and 256 rows (t-kernel variant as set),
  * then, where the solve is BiCGStab, every t-kernel variant at the best height.  Keeps the
- * fastest in the context's options (opts.tile_rows stays 0 where the automatic height is;
- * *tile_rows is then BiCGStab's automatic height; grids whose solves run on tiles have no other
- * candidate).  The state and the
+ * fastest in the context's options (opts.tile_rows stays 0 where the automatic height is, and
+ * *tile_rows is that height; grids whose solves run on tiles have no height to choose, and
+ * *tile_rows is BiCGStab's automatic one).  The state and the
  * statistics are restored (the next step takes a stencil initial residual).  Only
  * the FP32-refined fused path on 2D grids has a choice to make: other
  * configurations return APFC_OK with their options unchanged and ms_per_step 0.

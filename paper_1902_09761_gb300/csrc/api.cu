@@ -789,6 +789,14 @@ bool use_schur(const apfc_ctx* ctx) {
   return true;
 }
 
+// rows per segment of the 2D Chebyshev passes
+int schur_rows(const apfc_ctx* ctx, int elem_bytes) {
+  const apfc_opts& o = ctx->opts;
+  if (o.tile_rows > 0) return o.tile_rows;
+  return schur_auto_rows(schur_of(ctx), &ctx->grid.n[0], &ctx->grid.n[1], 1, ctx->J, o.cheb_degree, elem_bytes, o.tile,
+                         ctx->sms);
+}
+
 int resid_parts(const apfc_ctx* ctx) {
   const int* n = ctx->grid.n;
   return ctx->dim == 3 ? schur_resid3_parts(n[0], n[1], n[2], ctx->J) : schur_resid_parts(n[0], n[1], ctx->J);
@@ -839,9 +847,7 @@ apfc_status schur_solve(apfc_ctx* ctx, SchurWork<T>& w, const double2* b, double
   const int m = o.cheb_degree, ni = schur_ni<T>(sc, ctx->dim, m), nt0 = schur_t0<T>(sc, ctx->dim, m), J = ctx->J;
   const int most = fp64 ? 4 : o.max_refine;
   const auto cw = cheb_weights(ctx);
-  const int rows = o.tile_rows > 0 ? o.tile_rows
-                                   : schur_auto_rows(sc, &ctx->grid.n[0], &ctx->grid.n[1], 1, J, m,
-                                                     (int)sizeof(cplx<T>), o.tile, ctx->sms);
+  const int rows = schur_rows(ctx, (int)sizeof(cplx<T>));
   SchurPlan plan{};
   plan.tol = o.tol;
   plan.tol_inner = o.tol_inner;
@@ -1656,8 +1662,8 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
     const int rows = (ny + s - 1) / s;
     if (rows >= 32 && rows <= ny && std::find(cand.begin(), cand.end(), rows) == cand.end()) cand.push_back(rows);
   }
-  if (schur && ctx->schur.plain && ctx->opts.tile == 3 && gauge_tiled(ctx->grid.n[0], ny, ctx->J))
-    cand.resize(1);  // the tiles have no height
+  const bool tiled = schur && ctx->schur.plain && ctx->opts.tile == 3 && gauge_tiled(ctx->grid.n[0], ny, ctx->J);
+  if (tiled) cand.resize(1);  // the tiles have no height
   const size_t blk = sizeof(double2) * 2 * (size_t)ctx->J * (size_t)ctx->pts;
   double2* saved = nullptr;
   if (cudaMalloc(&saved, blk) != cudaSuccess) {
@@ -1711,7 +1717,7 @@ apfc_status apfc_autotune(apfc_ctx* ctx, double dt, int* tile_rows, int* tile_t,
   ctx->opts.tile_rows = st == APFC_OK ? best_rows : saved_rows;
   ctx->opts.tile_t = st == APFC_OK ? best_tt : saved_tt;
   if (st != APFC_OK) return st;
-  if (tile_rows) *tile_rows = fused_rows(ctx);
+  if (tile_rows) *tile_rows = schur && !tiled ? schur_rows(ctx, (int)sizeof(float2)) : fused_rows(ctx);
   if (tile_t) *tile_t = best_tt;
   if (ms_per_step) *ms_per_step = best;
   return APFC_OK;
