@@ -351,3 +351,10 @@ def test_refined_steps_end_well_below_the_tolerance(kind, shape):
             ctx.step(1.0)
             assert ctx.stats()["resid_last"] <= 0.2 * tol
     ctx.close()
+
+
+@pytest.mark.parametrize("shape", [(9, 11, 59), (8, 12, 60), (9, 13, 61), (10, 27, 61), (9, 28, 60), (8, 29, 59), (97, 56, 361)])
+def test_3d_boxes_around_the_tiles_of_the_passes(shape):
+    # the FP32 passes own 60 columns of 12 rows, or of 28 where that gives two rounds of blocks (the
+    # last box: 7 x 2 tiles x 4 chunks x 6 amplitudes, one column over, odd rows); the residual 28 x 28
+    _steps(shape, (np.pi / 2,) * 3, 2, 1e-10, tol=1e-13, precision=A.APFC_FP32_REFINED)
