@@ -162,19 +162,33 @@ __device__ __forceinline__ void prof_add(const OpCoef& c, int kid, unsigned long
 }
 
 // Batched runs: every run's block vectors sit one after another in shared
-// arrays; elem_off is the run's first element (of [J][2][pts]).
+// arrays; elem_off is the run's first element (of [J][2][pts]).  BiCGStab's kernels write
+// partial sums from a run's 16-byte slot part_off (v-kernel) or part_off_t (t-kernel) on.
 struct RunGeom {
   int nx, ny;
   long long pts, elem_off;
   long long field_off;             // the run's first element in a [run][J][pts] field (even)
   long long part_off_r;            // residual kernel: first partial sum, partials, rows per segment
   int npart_r, rows_r;
+  long long part_off, part_off_t;
+  int npart, npart_t;              // partial-sum slots per amplitude in each layout
 };
 struct BatchLaunch {
   const RunGeom* dev;   // device copy of the run table (per-point kernels, reductions)
   const RunGeom* host;  // host copy (the fused kernels carry it in their parameters)
   int R;
+  int tlay;  // 1: partial sums in the t-kernel layout (its own tile variant)
 };
+
+// Point a kernel's grid sizes at run `run`; returns the run's first element.
+__device__ __forceinline__ long long select_run(const RunGeom* rg, int run, OpCoef& c) {
+  const RunGeom& q = rg[run];
+  c.nx = q.nx;
+  c.ny = q.ny;
+  c.nz = 1;
+  c.pts = q.pts;
+  return q.elem_off;
+}
 
 // Chebyshev recurrence weights for one application (per amplitude):
 // d_{k+1} = c1 d_k + c2 r_{k+1}.
@@ -348,6 +362,10 @@ void launch_extrapolate(double2* x, double2* xp, const OpCoef& c, cudaStream_t s
 // complex64 [J][pts] <-> part (0 zeta, 1 eta) of the FP64 state block, rounding to nearest
 void launch_c64_to_part(const float2* src, double2* x, long long pts, int J, int part, cudaStream_t s);
 void launch_part_to_c64(const double2* x, float2* dst, long long pts, int J, int part, cudaStream_t s);
+// 2D grids of a batch (no Jacobian): the residual of the block system with FP32 (and optional FP64)
+// output and the partial ||r||^2 per run and amplitude
+void launch_residual_refine2d(const double2* b, const double2* x, float2* r32, double2* r64, double* partials,
+                              const OpCoef& c, cudaStream_t s, const BatchLaunch& bl);
 // One 2D or 3D grid: the residual with its tiles staged by TMA and the partial ||r||^2
 // per amplitude (resid2d.cu); false, with *err set, if the tensor maps cannot be built
 // (nothing is launched then)
@@ -360,7 +378,7 @@ unsigned long long stream3d_timeouts();
 // Start of an FP32 solve from x0 = 0: r = b, rhat = b rounded to bf16 with its packed copy
 // rh16 [J][pts] (bf16pair.cuh), partials of (r, r), (b, b), (rhat, r) in slots 0-2 (k_dots' layout)
 void launch_init32(const float2* b, float2* r, float2* rhat, uint2* rh16, void* partials, const OpCoef& c,
-                   cudaStream_t s);
+                   cudaStream_t s, const BatchLaunch* bl = nullptr);
 // new RHS and initial residual r0 = b - b_prev + r_prev (pointwise); b_prev = r_prev = null:
 // the RHS and the ||b||^2 partials only (the ||r0||^2 slot holds 0, r32 is not written).
 // schur: r_prev and r32 are [J][pts] fields (the Schur complement's residual), else block vectors
@@ -408,7 +426,7 @@ int fused2d_tiles();  // number of tile variants
 // x64 += P^{-1} u
 template <typename T>
 bool launch_fused_pinv_add(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* u, double2* x64,
-                           cudaStream_t s);
+                           cudaStream_t s, const BatchLaunch* bl = nullptr);
 // blocks of one fused launch over an nx x ny grid (J amplitudes); *npart = blocks per amplitude
 int fused2d_blocks(int nx, int ny, int J, int m, int Ly, int elem_bytes, int tile, bool with_a, int* npart);
 // x = P^{-1} b
@@ -422,15 +440,16 @@ template <typename T>
 bool launch_fused_merged_v(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
                            const cplx<T>* t, const cplx<T>* p, cplx<T>* u, cplx<T>* r_new, cplx<T>* p_new,
                            cplx<T>* v_new, const cplx<T>* rhat, const uint2* rh16, const KScal* act, void* partials,
-                           cudaStream_t s);
+                           cudaStream_t s, const BatchLaunch* bl = nullptr);
 // t = A P^{-1} s, s = r - alpha v; partials (t, s), (t, t), (s, s), (rhat, s), (rhat, t)
 template <typename T>
 bool launch_fused_merged_t(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
-                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s);
+                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s,
+                           const BatchLaunch* bl = nullptr);
 // the pending u += alpha p + omega (r - alpha v) of amplitudes that stopped in this iteration
 template <typename T>
 void launch_final_update(const cplx<T>* r, const cplx<T>* v, const cplx<T>* p, cplx<T>* u, const KScal* ks,
-                         const OpCoef& c, cudaStream_t s);
+                         const OpCoef& c, cudaStream_t s, const BatchLaunch* bl = nullptr);
 // ---------------------------------------------------------------------------
 // cheb2d_f32.cu, cheb2d_f64.cu: passes of the Chebyshev iteration on the Schur complement (2D
 // grids, degree m in 1..4 of p).  schur.cu: its spectrum, weights, outer residual and plan.
@@ -561,13 +580,19 @@ void launch_schur_plan(const SchurPlan& p, KScal* ks, cudaStream_t s, const Batc
 // ---------------------------------------------------------------------------
 // reduce.cu
 // ---------------------------------------------------------------------------
+// bl != nullptr: one launch over every run of a batch (partials of run r from slot r J kDotSlots kDotBlocks)
 template <typename T>
 void launch_dots(int npair, const DotPairs<T>& pr, void* partials, const OpCoef& c, const KScal* act,
-                 cudaStream_t s);
+                 cudaStream_t s, const BatchLaunch* bl = nullptr);
 // npart: partial-sum slots per (amplitude, pair); layout [J][kDotSlots][npart].
 template <typename T>
 void launch_finalize(int npair, const void* partials, KScal* k, int op, int J, cudaStream_t s,
                      int npart = kDotBlocks);
+// batched runs: Krylov scalars k[run J + j]; npart_fixed > 0 for the k_dots layout
+// (kDotBlocks), 0 for the fused-pipeline layout (RunGeom part_off, npart)
+template <typename T>
+void launch_finalize_batch(int npair, const void* partials, int npart_fixed, const BatchLaunch& bl, int J, KScal* k,
+                           int op, cudaStream_t s);
 // partials in FP64 double2 layout regardless of T (for the fused FP64 residual)
 void launch_finalize64(int npair, const void* partials, KScal* k, int op, int J, cudaStream_t s);
 }  // namespace apfc

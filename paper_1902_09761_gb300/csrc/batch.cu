@@ -8,6 +8,12 @@
 // each (run, amplitude) takes its own number of passes.  A run that has
 // converged idles (its blocks return at once) while the others go on.  The
 // passes of a solve can be replayed from captured CUDA graphs.
+//
+// Where the Chebyshev iteration does not serve (tolerances beneath its residual's noise, more
+// terms than max_iter allows) the solves are BiCGStab on the block system (FP32 in FP64
+// refinement, fused2d.cuh), batched the same way: each (run, amplitude) keeps its own Krylov
+// scalars.  Run by run on contexts of their own, 24 runs of 96^2 to 256^2 took 3 to 10 times as
+// long (h = 0.7, dt = 10, tol 1e-12: 71 against 517 ms a step).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -23,7 +29,9 @@ using namespace apfc;
 namespace {
 
 constexpr int kMaxRuns = 65536;
-constexpr int kTunePasses = 6;     // Chebyshev passes timed per autotuner candidate
+constexpr int kTunePasses = 6;     // Chebyshev passes or BiCGStab iterations timed per autotuner candidate
+constexpr int kBlocks = 10;        // BiCGStab: r, rhat, p, v, u, t, r32, p', v', r'
+constexpr int kBicgRows = 128;     // its rows per block segment when opts.tile_rows is 0
 constexpr int kTuneRows[] = {32, 48, 64, 96, 128, 192, 256};
 
 }  // namespace
@@ -61,17 +69,24 @@ struct apfc_batch {
   void* part_fix = nullptr;  // right-hand-side kernel partials: R J kDotSlots kDotBlocks slots
   SchurCoef schur{};
   bool schur_ok = false;
-  // runs stepped alone where the Chebyshev iteration does not serve (very fine grids, tolerances
-  // beneath its residual's noise), each by a context of its own; fresh[r]: it holds run r's state
-  std::vector<apfc_ctx*> alone;
-  std::vector<char> fresh;
-  double2* field = nullptr;  // [J][pts] of the largest run
+  // BiCGStab on the block system (alloc_bicg)
+  float2* blk[kBlocks] = {};
+  uint2* rh16 = nullptr;         // rhat as packed bf16 pairs, [run][J][pts] (bf16pair.cuh)
+  double2* r64_blk = nullptr;    // the last step's residual
+  void* part_pipe = nullptr;     // fused-pipeline partials (run table layout)
+  long long part_pipe_cap = 0;
+  KScal* ks = nullptr;
+  KScal* ks_host = nullptr;
+  BatchLaunch bl_t{};            // t-kernel partial layout (its own tile variant)
+  int layout[4] = {-1, 0, 0, 0}; // tile, rows, tile_t, degree that the run table's partial layouts belong to
+  cudaGraphExec_t gblock[2] = {nullptr, nullptr};  // captured iterations, by starting side of the ping-pong buffers
   KScal* ks64 = nullptr;
   KScal* ks64_host = nullptr;
   double* epart = nullptr;
   double* eout = nullptr;
   double* eout_host = nullptr;
   bool have_prev = false;
+  bool prev_schur = false;  // r64_prev holds the previous residual, else r64_blk
   double prev_dt = 0.0;
   std::vector<char> has_state;
   std::vector<apfc_stats_t> stats;
@@ -133,6 +148,8 @@ bool make_table(apfc_batch* b) {
 void drop_graphs(apfc_batch* b) {
   for (auto& g : b->gexec) cudaGraphExecDestroy(g.second);
   b->gexec.clear();
+  for (auto& g : b->gblock)
+    if (g) cudaGraphExecDestroy(g), g = nullptr;
 }
 
 // The automatic segment height of the current options and coefficients.
@@ -171,9 +188,9 @@ bool issue_passes(apfc_batch* b, int np, int tile, int rows) {
   return launch_schur_passes<float>(b->schur, m, tile, b->coef, b->cw.data(), gt, rows, bufs, np, b->stream, b->sms, &b->bl);
 }
 
-apfc_status sync_ks(apfc_batch* b) {
+apfc_status sync_ks(apfc_batch* b, KScal* dev, KScal* host) {
   BK(cudaGetLastError());
-  BK(cudaMemcpyAsync(b->ks64_host, b->ks64, sizeof(KScal) * b->R * b->J, cudaMemcpyDeviceToHost, b->stream));
+  BK(cudaMemcpyAsync(host, dev, sizeof(KScal) * b->R * b->J, cudaMemcpyDeviceToHost, b->stream));
   BK(cudaStreamSynchronize(b->stream));
   return APFC_OK;
 }
@@ -222,70 +239,276 @@ apfc_status solve(apfc_batch* b, int np) {
   return APFC_OK;
 }
 
-// One part (0 zeta, 1 eta) of run r's block <-> a contiguous field.
-apfc_status copy_field(apfc_batch* b, int r, int part, bool to_state) {
-  const RunGeom& g = b->rg[r];
-  const size_t row = sizeof(double2) * (size_t)g.pts;
-  double2* blk = b->x64 + g.elem_off + part * g.pts;
-  if (to_state)
-    BK(cudaMemcpy2DAsync(blk, 2 * row, b->field, row, row, b->J, cudaMemcpyDeviceToDevice, b->stream));
-  else
-    BK(cudaMemcpy2DAsync(b->field, row, blk, 2 * row, row, b->J, cudaMemcpyDeviceToDevice, b->stream));
+// ---- BiCGStab on the block system ------------------------------------------
+int bicg_rows(const apfc_opts& o) { return o.tile_rows > 0 ? o.tile_rows : kBicgRows; }
+int tile_t_of(const apfc_opts& o) { return o.tile_t >= 0 ? o.tile_t : o.tile; }
+
+apfc_status alloc_bicg(apfc_batch* b) {
+  if (b->ks_host) return APFC_OK;
+  const size_t n = (size_t)b->elems, nks = sizeof(KScal) * (size_t)b->R * b->J;
+  for (auto& q : b->blk)
+    if (!q) BK(cudaMalloc(&q, sizeof(float2) * n));
+  if (!b->rh16) BK(cudaMalloc(&b->rh16, sizeof(uint2) * (n / 2)));
+  if (!b->r64_blk) BK(cudaMalloc(&b->r64_blk, sizeof(double2) * n));
+  if (!b->ks) BK(cudaMalloc(&b->ks, nks));
+  BK(cudaMallocHost(&b->ks_host, nks));
   return APFC_OK;
 }
 
-// One step of size dt of every run on its own context.
-apfc_status alone_step(apfc_batch* b, double dt) {
-  if (b->alone.empty()) {
-    b->alone.assign(b->R, nullptr);
-    b->fresh.assign(b->R, 0);
-    long long most = 0;
-    for (const RunGeom& g : b->rg) most = std::max(most, g.pts);
-    BK(cudaMalloc(&b->field, sizeof(double2) * (size_t)b->J * (size_t)most));
+// The partial-sum offsets of (tile, rows) of the v-kernel and tile_t of the t-kernel into the run table.
+apfc_status set_layout(apfc_batch* b, int tile, int rows, int tile_t) {
+  apfc_status st = alloc_bicg(b);
+  if (st != APFC_OK) return st;
+  const int m = b->opts.cheb_degree, eb = (int)sizeof(float2), want[4] = {tile, rows, tile_t, m};
+  if (std::equal(want, want + 4, b->layout)) return APFC_OK;
+  long long poff = 0, poff_t = 0;
+  for (RunGeom& g : b->rg) {
+    g.part_off = poff;
+    g.part_off_t = poff_t;
+    fused2d_blocks(g.nx, g.ny, b->J, m, rows, eb, tile, true, &g.npart);
+    fused2d_blocks(g.nx, g.ny, b->J, m, rows, eb, tile_t, true, &g.npart_t);
+    poff += (long long)b->J * kDotSlots * g.npart;
+    poff_t += (long long)b->J * kDotSlots * g.npart_t;
+  }
+  b->layout[0] = -1;  // until the table is on the device
+  const long long need = std::max(poff, poff_t);  // the two kernels use the buffer in turn
+  BK(cudaMemcpyAsync(b->rg_dev, b->rg.data(), sizeof(RunGeom) * b->R, cudaMemcpyHostToDevice, b->stream));
+  BK(cudaStreamSynchronize(b->stream));
+  if (need > b->part_pipe_cap) {
+    cudaFree(b->part_pipe);
+    b->part_pipe = nullptr;
+    b->part_pipe_cap = 0;
+    BK(cudaMalloc(&b->part_pipe, 16ull * (size_t)need));
+    b->part_pipe_cap = need;
+  }
+  b->bl_t = b->bl;
+  b->bl_t.tlay = 1;
+  drop_graphs(b);
+  std::copy(want, want + 4, b->layout);
+  return APFC_OK;
+}
+
+// ping-pong views of the Krylov vectors
+struct Vecs {
+  float2 *r[2], *p[2], *v[2], *rhat, *u, *t, *r32;
+};
+Vecs vecs(apfc_batch* b) {
+  Vecs v;
+  v.r[0] = b->blk[0];
+  v.r[1] = b->blk[9];
+  v.rhat = b->blk[1];
+  v.p[0] = b->blk[2];
+  v.p[1] = b->blk[7];
+  v.v[0] = b->blk[3];
+  v.v[1] = b->blk[8];
+  v.u = b->blk[4];
+  v.t = b->blk[5];
+  v.r32 = b->blk[6];
+  return v;
+}
+
+// `every` merged BiCGStab iterations over all runs, starting on side `cur`.
+bool issue_block(apfc_batch* b, int cur, int every, int tile, int rows, int tile_t) {
+  const Vecs x = vecs(b);
+  const int m = b->opts.cheb_degree;
+  cudaStream_t s = b->stream;
+  for (int q = 0; q < every; ++q) {
+    if (!launch_fused_merged_v<float>(m, rows, tile, b->coef, b->cw.data(), x.r[cur], x.v[cur], x.t, x.p[cur], x.u,
+                                      x.r[1 - cur], x.p[1 - cur], x.v[1 - cur], x.rhat, b->rh16, b->ks, b->part_pipe, s,
+                                      &b->bl))
+      return false;
+    launch_finalize_batch<float>(1, b->part_pipe, 0, b->bl, b->J, b->ks, OP_ALPHA, s);
+    if (!launch_fused_merged_t<float>(m, rows, tile_t, b->coef, b->cw.data(), x.r[1 - cur], x.v[1 - cur], x.t,
+                                      x.rhat, b->ks, b->part_pipe, s, &b->bl_t))
+      return false;
+    launch_finalize_batch<float>(5, b->part_pipe, 0, b->bl_t, b->J, b->ks, OP_OMEGA5, s);
+    launch_final_update<float>(x.r[1 - cur], x.v[1 - cur], x.p[1 - cur], x.u, b->ks, b->coef, s, &b->bl);
+    cur = 1 - cur;
+  }
+  return true;
+}
+
+// Start a BiCGStab solve of A P^{-1} u = r32 for every (run, amplitude); runs with
+// skip[r] start converged.  fixed_tol >= 0: that relative tolerance for all; else the
+// refinement's per-amplitude choice (inner_tol) from the outer residual norms.
+// Leaves the scalars on the host; *any: some are active.
+apfc_status krylov_init(apfc_batch* b, const std::vector<char>& skip, int max_iter, bool* any,
+                        double fixed_tol = -1.0) {
+  const Vecs x = vecs(b);
+  cudaStream_t s = b->stream;
+  const size_t bytes = sizeof(float2) * (size_t)b->elems;
+  for (int r = 0; r < b->R; ++r)
+    for (int j = 0; j < b->J; ++j) {
+      KScal& k = b->ks_host[r * b->J + j];
+      // r0 = b: a relative tolerance >= 1 stops at once; otherwise the run alone's choice
+      const KScal& o = b->ks64_host[r * b->J + j];
+      const double tj = skip[r]           ? 2.0
+                        : fixed_tol >= 0.0 ? fixed_tol
+                                           : inner_tol(b->opts.tol, b->opts.tol_inner, o.rnorm2, o.bnorm2);
+      std::memset(&k, 0, sizeof(k));
+      k.tolrel2 = tj * tj;
+      k.max_iter = max_iter;
+    }
+  BK(cudaMemcpyAsync(b->ks, b->ks_host, sizeof(KScal) * b->R * b->J, cudaMemcpyHostToDevice, s));
+  BK(cudaMemsetAsync(x.p[0], 0, bytes, s));
+  BK(cudaMemsetAsync(x.v[0], 0, bytes, s));
+  BK(cudaMemsetAsync(x.u, 0, bytes, s));
+  BK(cudaMemsetAsync(x.t, 0, bytes, s));
+  // r = r32 and the shadow residual rounded to bf16, as in a context alone: rho0 = (rhat, r0)
+  launch_init32(x.r32, x.r[0], x.rhat, b->rh16, b->part_fix, b->coef, s, &b->bl);
+  launch_finalize_batch<float>(3, b->part_fix, kDotBlocks, b->bl, b->J, b->ks, OP_INIT3, s);
+  apfc_status st = sync_ks(b, b->ks, b->ks_host);
+  if (st != APFC_OK) return st;
+  *any = false;
+  for (int i = 0; i < b->R * b->J; ++i) {
+    if (b->ks_host[i].status == KS_NAN) return bfail(b, APFC_ENAN, "run " + std::to_string(i / b->J) + ": NaN/Inf");
+    *any = *any || b->ks_host[i].active;
+  }
+  return APFC_OK;
+}
+
+// Iterate until every (run, amplitude) has stopped.
+apfc_status krylov_iterate(apfc_batch* b, int max_iter, int tile, int rows, int tile_t) {
+  const int every = std::max(1, b->opts.check_every);
+  const bool graph = (b->flags & APFC_BATCH_GRAPH) && !profiler_on();
+  int cur = 0;
+  long long launched = 0, blocks = 0;
+  while (true) {
+    if (launched > (long long)max_iter + every) return bfail(b, APFC_ENOCONV, "Krylov iteration cap exceeded");
+    launched += every;
+    if (graph && blocks > 0) {
+      // the first block ran eagerly (kernel attributes are set on first use)
+      if (!b->gblock[cur]) {
+        cudaGraph_t g = nullptr;
+        BK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+        const bool ok = issue_block(b, cur, every, tile, rows, tile_t);
+        const cudaError_t ec = cudaStreamEndCapture(b->stream, &g);
+        if (!ok) {
+          if (g) cudaGraphDestroy(g);
+          return bfail(b, APFC_EINVAL, "fused pipeline cannot run these options");
+        }
+        BK(ec);
+        const cudaError_t ei = cudaGraphInstantiate(&b->gblock[cur], g, 0);
+        cudaGraphDestroy(g);
+        BK(ei);
+      }
+      BK(cudaGraphLaunch(b->gblock[cur], b->stream));
+      b->graph_replays += 1;
+    } else if (!issue_block(b, cur, every, tile, rows, tile_t)) {
+      return bfail(b, APFC_EINVAL, "fused pipeline cannot run these options");
+    }
+    ++blocks;
+    if (every & 1) cur = 1 - cur;
+    apfc_status st = sync_ks(b, b->ks, b->ks_host);
+    if (st != APFC_OK) return st;
+    bool run = false;
+    for (int i = 0; i < b->R * b->J; ++i) run = run || b->ks_host[i].active;
+    if (!run) return APFC_OK;
+  }
+}
+
+// One step of every run by BiCGStab: FP32 solves inside FP64 iterative refinement.
+apfc_status bicg_step(apfc_batch* b) {
+  cudaStream_t s = b->stream;
+  const int tile = b->opts.tile, rows = bicg_rows(b->opts), tile_t = tile_t_of(b->opts);
+  const apfc_status sl = set_layout(b, tile, rows, tile_t);
+  if (sl != APFC_OK) return sl;
+  const Vecs x = vecs(b);
+  double* part = reinterpret_cast<double*>(b->part_fix);
+  bool resid_ready = false;
+  if (b->have_prev && b->prev_dt == b->coef_dt && !b->prev_schur) {
+    // r0 = b - b_prev + r_prev; the new RHS goes to the other buffer
+    launch_rhs_resid(b->x64, b->b64_prev, b->b64, b->r64_blk, x.r32, part, b->coef, b->nt, false, s, &b->bl);
+    std::swap(b->b64, b->b64_prev);
+    resid_ready = true;
+  } else {
+    // the new RHS and ||b||^2 (the same kernel as a context alone), r0 by stencil below
+    launch_rhs_resid(b->x64, b->b64, nullptr, nullptr, x.r32, part, b->coef, b->nt, false, s, &b->bl);
   }
   b->have_prev = false;
+  const double tol2 = b->opts.tol * b->opts.tol;
+  std::vector<char> done(b->R, 0);
+  std::vector<int> solves(b->R, 0), iters(b->R, 0);
+  int sweep = 0;
+  for (;; ++sweep) {
+    // the right-hand side's partial sums: ||b||^2 and, with a previous residual, ||r0||^2
+    if (sweep == 0) launch_finalize_batch<double>(2, part, kDotBlocks, b->bl, b->J, b->ks64, OP_NORMS, s);
+    if (!resid_ready) {
+      launch_residual_refine2d(b->b64, b->x64, x.r32, b->r64_blk, part, b->coef, s, b->bl);
+      launch_finalize_batch<double>(1, part, kDotBlocks, b->bl, b->J, b->ks64, OP_RNORM, s);
+    }
+    resid_ready = false;
+    apfc_status st = sync_ks(b, b->ks64, b->ks64_host);
+    if (st != APFC_OK) return st;
+    bool all = true;
+    for (int r = 0; r < b->R; ++r) {
+      bool ok = true;
+      for (int j = 0; j < b->J; ++j) {
+        const KScal& k = b->ks64_host[r * b->J + j];
+        if (!std::isfinite(k.rnorm2) || !std::isfinite(k.bnorm2))
+          return bfail(b, APFC_ENAN, "run " + std::to_string(r) + ": residual norm is not finite");
+        if (k.rnorm2 > tol2 * k.bnorm2) ok = false;
+      }
+      if (ok && !done[r]) done[r] = 1;
+      all = all && done[r];
+    }
+    if (all) {
+      // the last check of every run was a stencil residual of its final state
+      b->have_prev = sweep > 0;
+      b->prev_schur = false;
+      b->prev_dt = b->coef_dt;
+      break;
+    }
+    if (sweep >= b->opts.max_refine) {
+      for (int r = 0; r < b->R; ++r)
+        if (!done[r]) return bfail(b, APFC_ENOCONV, "run " + std::to_string(r) + ": refinement did not converge");
+    }
+    bool any = false;
+    st = krylov_init(b, done, b->opts.max_iter, &any);
+    if (st != APFC_OK) return st;
+    if (any) {
+      st = krylov_iterate(b, b->opts.max_iter, tile, rows, tile_t);
+      if (st != APFC_OK) return st;
+      // x += P^{-1} u (u = 0 for runs that did not iterate)
+      if (!launch_fused_pinv_add<float>(b->opts.cheb_degree, rows, tile, b->coef, b->cw.data(), x.u, b->x64, s,
+                                        &b->bl))
+        return bfail(b, APFC_EINVAL, "fused pipeline cannot run these options");
+    }
+    for (int r = 0; r < b->R; ++r) {
+      if (done[r]) continue;
+      solves[r] += 1;
+      int mx = 0;
+      for (int j = 0; j < b->J; ++j) {
+        const KScal& k = b->ks_host[r * b->J + j];
+        if (k.status == KS_NAN) return bfail(b, APFC_ENAN, "run " + std::to_string(r) + ": NaN in the Krylov solve");
+        mx = std::max(mx, k.iters);
+      }
+      iters[r] += mx;
+    }
+  }
   for (int r = 0; r < b->R; ++r) {
-    apfc_ctx*& c = b->alone[r];
-    apfc_status st = APFC_OK;
-    auto run_fail = [&](const std::string& what) {
-      return bfail(b, st, "run " + std::to_string(r) + ": " + what);
-    };
-    if (c == nullptr) {
-      const apfc_grid g{{b->nx[r], b->ny[r], 1}, {b->gmax.h[0], b->gmax.h[1], 1.0}};
-      if ((st = apfc_init(&c, &b->lat, &b->par, &g, &b->opts, b->stream)) != APFC_OK)
-        return run_fail(apfc_last_error(nullptr));
-    }
-    if (!b->fresh[r]) {
-      if ((st = apfc_set_opts(c, &b->opts)) != APFC_OK) return run_fail(apfc_last_error(c));
-      if ((st = copy_field(b, r, 1, false)) != APFC_OK) return st;
-      if ((st = apfc_set_amplitudes(c, b->field, APFC_DEVICE, APFC_C128)) != APFC_OK) return run_fail(apfc_last_error(c));
-      b->fresh[r] = 1;
-    }
-    if ((st = apfc_step(c, dt, 1)) != APFC_OK) return run_fail(apfc_last_error(c));
-    apfc_stats_t one;
-    apfc_stats(c, &one);
     apfc_stats_t& t = b->stats[r];
     t.steps += 1;
-    t.iters_last = one.iters_last;
-    t.iters_total += one.iters_last;
-    t.refine_last = one.refine_last;
-    t.resid_last = one.resid_last;
-    if ((st = apfc_get_amplitudes(c, b->field, APFC_DEVICE, APFC_C128)) != APFC_OK) return run_fail(apfc_last_error(c));
-    if ((st = copy_field(b, r, 1, true)) != APFC_OK) return st;
-    if ((st = apfc_get_zeta(c, b->field, APFC_DEVICE)) != APFC_OK) return run_fail(apfc_last_error(c));
-    if ((st = copy_field(b, r, 0, true)) != APFC_OK) return st;
+    t.iters_last = iters[r];
+    t.iters_total += iters[r];
+    t.refine_last = solves[r];
+    double rr = 0.0;
+    for (int j = 0; j < b->J; ++j) {
+      const KScal& k = b->ks64_host[r * b->J + j];
+      rr = std::max(rr, std::sqrt(k.rnorm2 / (k.bnorm2 > 0 ? k.bnorm2 : 1.0)));
+    }
+    t.resid_last = rr;
   }
   return APFC_OK;
 }
 
 // One step of every run: FP32 Chebyshev solves inside FP64 iterative refinement.
 apfc_status batch_step(apfc_batch* b) {
-  if (!b->schur_ok) return alone_step(b, b->coef_dt);
-  std::fill(b->fresh.begin(), b->fresh.end(), 0);
+  if (!b->schur_ok) return bicg_step(b);
   cudaStream_t s = b->stream;
   double* part = reinterpret_cast<double*>(b->part_fix);
   bool resid_ready = false;
-  if (b->have_prev && b->prev_dt == b->coef_dt) {
+  if (b->have_prev && b->prev_dt == b->coef_dt && b->prev_schur) {
     // r0 = b - b_prev + r_prev; the new RHS goes to the other buffer
     launch_rhs_resid(b->x64, b->b64_prev, b->b64, b->r64_prev, b->r[0], part, b->coef, b->nt, true, s, &b->bl);
     std::swap(b->b64, b->b64_prev);
@@ -318,7 +541,7 @@ apfc_status batch_step(apfc_batch* b) {
       launch_schur_plan(plan, b->ks64, s, &b->bl);
     }
     resid_ready = false;
-    apfc_status st = sync_ks(b);
+    apfc_status st = sync_ks(b, b->ks64, b->ks64_host);
     if (st != APFC_OK) return st;
     bool all = true, patch = false;
     int np = 0;
@@ -349,6 +572,7 @@ apfc_status batch_step(apfc_batch* b) {
     if (all) {
       // the last check of every run was a stencil residual of its final state
       b->have_prev = sweep > 0;
+      b->prev_schur = true;
       b->prev_dt = b->coef_dt;
       break;
     }
@@ -375,6 +599,63 @@ apfc_status batch_step(apfc_batch* b) {
   return APFC_OK;
 }
 
+// The autotuner for BiCGStab: merged iterations on the first refinement residual of a step, for every
+// tile variant and height of both kernels, then for every variant of the t-kernel alone.
+apfc_status bicg_tune(apfc_batch* b, int* tile_out, int* rows_out, double* ms_out) {
+  apfc_status st = alloc_bicg(b);
+  if (st != APFC_OK) return st;
+  cudaStream_t s = b->stream;
+  const Vecs x = vecs(b);
+  double* part = reinterpret_cast<double*>(b->part_fix);
+  launch_rhs(b->x64, b->b64, b->coef, b->nt, s, &b->bl);
+  launch_residual_refine2d(b->b64, b->x64, x.r32, nullptr, part, b->coef, s, b->bl);
+  b->have_prev = false;
+  cudaEvent_t e0, e1;
+  BK(cudaEventCreate(&e0));
+  BK(cudaEventCreate(&e1));
+  int best_tile = b->opts.tile, best_rows = bicg_rows(b->opts), best_t = tile_t_of(b->opts);
+  double best = 1e300;
+  const std::vector<char> none(b->R, 0);
+  auto time_candidate = [&](int tile, int rows, int tile_t, double* ms) -> apfc_status {
+    apfc_status s2 = set_layout(b, tile, rows, tile_t);
+    if (s2 != APFC_OK) return s2;
+    for (int rep = 0; rep < 2; ++rep) {  // the first pass warms up
+      bool any = false;
+      // a tolerance that no solve reaches within kTunePasses iterations
+      if ((s2 = krylov_init(b, none, 1 << 20, &any, 1e-30)) != APFC_OK) return s2;
+      BK(cudaEventRecord(e0, s));
+      if (!issue_block(b, 0, kTunePasses, tile, rows, tile_t))
+        return bfail(b, APFC_EINVAL, "fused pipeline cannot run these options");
+      BK(cudaEventRecord(e1, s));
+      BK(cudaEventSynchronize(e1));
+      float f = 0.f;
+      BK(cudaEventElapsedTime(&f, e0, e1));
+      *ms = f;
+    }
+    return APFC_OK;
+  };
+  double ms = 1e300;
+  for (int tile = 0; tile < fused2d_tiles() && st == APFC_OK; ++tile)
+    for (int rows : kTuneRows) {
+      if ((st = time_candidate(tile, rows, tile, &ms)) != APFC_OK) break;
+      if (ms < best) best = ms, best_tile = tile, best_rows = rows, best_t = tile;
+    }
+  for (int tile_t = 0; tile_t < fused2d_tiles() && st == APFC_OK; ++tile_t) {
+    if (tile_t == best_t) continue;
+    if ((st = time_candidate(best_tile, best_rows, tile_t, &ms)) == APFC_OK && ms < best) best = ms, best_t = tile_t;
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (st != APFC_OK) return st;
+  b->opts.tile = best_tile;
+  b->opts.tile_rows = best_rows;
+  b->opts.tile_t = best_t;
+  if (tile_out) *tile_out = best_tile;
+  if (rows_out) *rows_out = best_rows;
+  if (ms_out) *ms_out = best / kTunePasses;
+  return APFC_OK;
+}
+
 bool valid_batch_opts(const apfc_opts& o, std::string& e) {
   if (!valid_opts(o, e)) return false;
   if (o.precision != APFC_FP32_REFINED) e = "batched runs use precision APFC_FP32_REFINED";
@@ -398,8 +679,12 @@ void free_batch(apfc_batch* b) {
   for (auto& p : b->d) cudaFree(p);
   cudaFree(b->u);
   cudaFree(b->tab);
-  for (apfc_ctx* c : b->alone) apfc_destroy(c);
-  cudaFree(b->field);
+  for (auto& p : b->blk) cudaFree(p);
+  cudaFree(b->rh16);
+  cudaFree(b->r64_blk);
+  cudaFree(b->part_pipe);
+  cudaFree(b->ks);
+  if (b->ks_host) cudaFreeHost(b->ks_host);
   cudaFree(b->rpart);
   cudaFree(b->part_fix);
   cudaFree(b->ks64);
@@ -550,7 +835,6 @@ apfc_status apfc_batch_set_opts(apfc_batch* b, const apfc_opts* opts) {
   std::string e;
   if (!valid_batch_opts(*opts, e)) return bfail(b, APFC_EINVAL, e);
   b->opts = *opts;
-  std::fill(b->fresh.begin(), b->fresh.end(), 0);
   const double dt = b->coef_dt;
   b->coef_dt = -1.0;  // tau_mode or the degree may have changed
   if (!set_coef(b, dt > 0 ? dt : 1.0, e)) return bfail(b, APFC_EINVAL, e);
@@ -572,7 +856,6 @@ apfc_status apfc_batch_set_amplitudes(apfc_batch* b, int run, const void* eta, i
   BK(cudaStreamSynchronize(b->stream));
   b->has_state[run] = 1;
   b->have_prev = false;
-  if (!b->fresh.empty()) b->fresh[run] = 0;
   b->failed = false;  // as on a context: new amplitudes clear a sticky error
   b->err.clear();
   b->stats[run] = apfc_stats_t{};
@@ -632,12 +915,7 @@ apfc_status apfc_batch_autotune(apfc_batch* b, double dt, int* tile_out, int* ro
     if (!b->has_state[r]) return bfail(b, APFC_ESTATE, "no amplitudes set for run " + std::to_string(r));
   std::string e;
   if (!set_coef(b, dt, e)) return bfail(b, APFC_EINVAL, e);
-  if (!b->schur_ok) {  // the runs are stepped alone: nothing to choose
-    if (tile_out) *tile_out = b->opts.tile;
-    if (rows_out) *rows_out = rows_of(b);
-    if (ms_out) *ms_out = 0.0;
-    return APFC_OK;
-  }
+  if (!b->schur_ok) return bicg_tune(b, tile_out, rows_out, ms_out);
   cudaStream_t s = b->stream;
   // the first refinement residual of a step from the current state is the right-hand side
   // every candidate iterates on; u is never added to the state (the passes stop before the

@@ -24,12 +24,12 @@ int fused2d_blocks(int nx, int ny, int J, int m, int Ly, int elem_bytes, int til
 
 template <typename T>
 bool launch_fused_pinv_add(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* u, double2* x64,
-                           cudaStream_t s) {
+                           cudaStream_t s, const BatchLaunch* bl) {
   LoadPlain<T> ld{u, c.pts};
   EpAddX<T> ep{x64, c.pts};
   // reads u (2 fields); reads and writes the FP64 block x (2 FP64 fields each way)
   const int f = 2 + 4 * (int)(sizeof(double2) / sizeof(cplx<T>));
-  return dispatch<T, false>(m, tile, c, w, Ly, ld, ep, nullptr, nullptr, s, kid_of<T>(KID_FUSED_PINV), f);
+  return dispatch<T, false>(m, tile, c, w, Ly, ld, ep, nullptr, nullptr, s, kid_of<T>(KID_FUSED_PINV), f, bl);
 }
 
 template <typename T>
@@ -41,20 +41,25 @@ bool launch_fused_pinv_store(int m, int Ly, int tile, const OpCoef& c, const Che
 }
 
 // u += alpha p + omega (r - alpha v) for amplitudes whose solve stopped in this iteration.
-// FP32 vectors stream as 16-byte pairs of
+// Batched runs: blockIdx.z selects the run.  FP32 vectors stream as 16-byte pairs of
 // complex values (each amplitude's block starts at an even element of a 256-byte
 // aligned allocation, and holds an even number 2 pts of values).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_final_update(const cplx<T>* __restrict__ r,
                                                            const cplx<T>* __restrict__ v,
                                                            const cplx<T>* __restrict__ p, cplx<T>* __restrict__ u,
-                                                           const KScal* ks, OpCoef c) {
+                                                           const KScal* ks, OpCoef c, const RunGeom* rg) {
   const int j = blockIdx.y;
+  long long o = 0;
+  if (rg != nullptr) {
+    o = select_run(rg, blockIdx.z, c);
+    ks += (long long)blockIdx.z * c.J;
+  }
   if (ks[j].just_done == 0) return;
   prof_add(c, kid_of<T>(KID_BICG_UPDATE), 10ull * (unsigned long long)c.pts * sizeof(cplx<T>));
   const cplx<T> al = to_c<T>(ks[j].alpha), om = to_c<T>(ks[j].omega);
   const long long n = 2 * c.pts;
-  const long long o = 2LL * j * c.pts;
+  o += 2LL * j * c.pts;
   const long long stride = (long long)gridDim.x * blockDim.x;
   if constexpr (sizeof(T) == 4) {
     const float4* r4 = reinterpret_cast<const float4*>(r + o);
@@ -85,18 +90,22 @@ __global__ void __launch_bounds__(kThreads) k_final_update(const cplx<T>* __rest
 
 template <typename T>
 void launch_final_update(const cplx<T>* r, const cplx<T>* v, const cplx<T>* p, cplx<T>* u, const KScal* ks,
-                         const OpCoef& c, cudaStream_t s) {
+                         const OpCoef& c, cudaStream_t s, const BatchLaunch* bl) {
   ProfScope ps_(kid_of<T>(KID_BICG_UPDATE), s);
+  if (bl != nullptr) {
+    k_final_update<T><<<dim3(kDotBlocks, c.J, bl->R), kThreads, 0, s>>>(r, v, p, u, ks, c, bl->dev);
+    return;
+  }
   // usually one amplitude is done at a time: enough blocks for that one to fill the GPU
-  k_final_update<T><<<dim3(4 * kDotBlocks, c.J), kThreads, 0, s>>>(r, v, p, u, ks, c);
+  k_final_update<T><<<dim3(4 * kDotBlocks, c.J), kThreads, 0, s>>>(r, v, p, u, ks, c, nullptr);
 }
 
-#define APFC_FUSED_INST(T)                                                                                           \
-  template void launch_final_update<T>(const cplx<T>*, const cplx<T>*, const cplx<T>*, cplx<T>*, const KScal*,       \
-                                       const OpCoef&, cudaStream_t);                                                \
-  template bool launch_fused_pinv_add<T>(int, int, int, const OpCoef&, const ChebStep*, const cplx<T>*, double2*,    \
-                                         cudaStream_t);                                                             \
-  template bool launch_fused_pinv_store<T>(int, int, int, const OpCoef&, const ChebStep*, const cplx<T>*, cplx<T>*,  \
+#define APFC_FUSED_INST(T)                                                                                         \
+  template void launch_final_update<T>(const cplx<T>*, const cplx<T>*, const cplx<T>*, cplx<T>*, const KScal*,     \
+                                       const OpCoef&, cudaStream_t, const BatchLaunch*);                          \
+  template bool launch_fused_pinv_add<T>(int, int, int, const OpCoef&, const ChebStep*, const cplx<T>*, double2*,   \
+                                         cudaStream_t, const BatchLaunch*);                                        \
+  template bool launch_fused_pinv_store<T>(int, int, int, const OpCoef&, const ChebStep*, const cplx<T>*, cplx<T>*, \
                                            cudaStream_t);
 
 APFC_FUSED_INST(double)

@@ -173,6 +173,11 @@ struct LoadPlain {
   const cplx<T>* b;
   long long pts;
   long long off;
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    b += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal*) { off = 2LL * j * pts; }
   __device__ const cplx<T>* in(int i) const { return b + off + i * pts; }
   __device__ const cplx<T>* re(int) const { return b + off; }
@@ -193,6 +198,12 @@ struct LoadS {
   long long pts;
   cplx<T> alpha;
   long long off;
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    r += e;
+    v += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal* k) {
     alpha = to_c<T>(k[j].alpha);
     off = 2LL * j * pts;
@@ -224,6 +235,17 @@ struct LoadPR {
   long long pts;
   cplx<T> al, om, be;
   long long off;
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    r += e;
+    v += e;
+    t += e;
+    p += e;
+    u += e;
+    rn += e;
+    pn += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal* k) {
     al = to_c<T>(k[j].alpha);
     om = to_c<T>(k[j].omega);
@@ -280,6 +302,14 @@ struct EpT5 {
   long long off;
   cplx<T> alpha;
   Acc<T> acc[5];
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    t += e;
+    r += e;
+    v += e;
+    rhat += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal* k) {
     off = 2LL * j * pts;
     alpha = to_c<T>(k[j].alpha);
@@ -315,6 +345,11 @@ struct EpStore {  // out = y
   long long pts;
   long long off;
   Acc<T> acc[1];
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    out += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal*) { off = 2LL * j * pts; }
   __device__ const cplx<T>* ep(int) const { return nullptr; }
   __device__ void put(const cplx<T>*, int, long long p, cplx<T> y1, cplx<T> y2, cplx<T>, cplx<T>) {
@@ -330,6 +365,11 @@ struct EpAddX {  // x64 += y (the Krylov correction P^{-1} u)
   long long pts;
   long long off;
   Acc<T> acc[1];
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    x += e;
+    pts = n;
+  }
   __device__ void setup(int j, const KScal*) { off = 2LL * j * pts; }
   __device__ const cplx<T>* ep(int) const { return nullptr; }
   __device__ void put(const cplx<T>*, int, long long p, cplx<T> y1, cplx<T> y2, cplx<T>, cplx<T>) {
@@ -362,6 +402,16 @@ struct EpV {  // v = y; (rhat, v)
   long long pts;
   long long off;
   Acc<T> acc[1];
+  // batched runs: move every array to this run's block vectors
+  __device__ void rebase(long long e, long long n) {
+    v += e;
+    if constexpr (H16) {
+      rh16 += e / 2;
+    } else {
+      rhat += e;
+    }
+    pts = n;
+  }
   __device__ void setup(int j, const KScal*) { off = 2LL * j * pts; }
   __device__ const cplx<T>* ep(int i) const {
     if constexpr (H16) return reinterpret_cast<const cplx<T>*>(rh16 + off / 2);
@@ -500,14 +550,30 @@ __device__ __forceinline__ Nbh<T> fetch_d(const cplx<T>* ring, int mask, int row
 }
 
 
+// Batched runs: the geometry of up to kTabRuns runs of one launch travels in
+// the kernel parameters (a constant-bank table indexed by blockIdx.y), so that
+// the work-item indices and grid sizes stay block-uniform values.
+constexpr int kTabRuns = 64;
+struct RunRec {
+  long long pts, elem_off, part_off;
+  int nx, ny, Ly, nstrips, nsegs, nblk, run, pad;
+};
+struct RunTab {
+  RunRec run[kTabRuns];
+};
+struct NoTab {};
+
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int wrap_inc(int y, int n) { return y + 1 == n ? 0 : y + 1; }
 
-// Grid: (nstrips, nsegs, J).
+// Grid: (nstrips, nsegs, J) for one grid (TAB = NoTab); for batched runs
+// (TAB = RunTab) (blocks of the largest run, runs of the table), each block
+// taking item blockIdx.x = sx + nstrips (sy + nsegs j) of run blockIdx.y.
 // JAC: the (2,2) block of A carries the Jacobian diagonal c.jd of a Picard iteration.
-template <typename T, int M, bool WITH_A, int PF, int NT_, class LD, class EP, bool JAC>
+template <typename T, int M, bool WITH_A, int PF, int NT_, class LD, class EP, class TAB, bool JAC>
 __global__ void __launch_bounds__(NT_) k_pipe2d(OpCoef c, ChebAll cw, PipeGeom g, LD ld, EP ep, const KScal* act,
-                                                void* partials, int kid, int fields) {
+                                                void* partials, int kid, int fields,
+                                                const __grid_constant__ TAB tab) {
   using SH = PipeShape<T, M, WITH_A, PF, NT_, LD, EP>;
   constexpr int NT = SH::NT;
   constexpr int S = SH::S;
@@ -518,8 +584,31 @@ __global__ void __launch_bounds__(NT_) k_pipe2d(OpCoef c, ChebAll cw, PipeGeom g
   cplx<T>* keep = sm + SH::ring_elems;  // [KD][2][NT]: loader outputs of the own column
   cplx<T>* stage_buf = keep + SH::keep_elems;
 
-  // work item: strip sx, row segment sy, amplitude j
-  const int sx = blockIdx.x, sy = blockIdx.y, j = blockIdx.z;
+  // work item: strip sx, row segment sy, amplitude j (of run blockIdx.y when batched)
+  int sx, sy, j;
+  if constexpr (std::is_same<TAB, RunTab>::value) {
+    const RunRec& rq = tab.run[blockIdx.y];
+    const int b = blockIdx.x;
+    if (b >= rq.nblk) return;
+    g.nx = rq.nx;
+    g.ny = rq.ny;
+    g.Ly = rq.Ly;
+    g.nstrips = rq.nstrips;
+    g.nsegs = rq.nsegs;
+    g.npart = rq.nstrips * rq.nsegs;
+    g.pts = rq.pts;
+    sx = b % rq.nstrips;
+    sy = (b / rq.nstrips) % rq.nsegs;
+    j = b / g.npart;
+    ld.rebase(rq.elem_off, rq.pts);
+    ep.rebase(rq.elem_off, rq.pts);
+    if (act != nullptr) act += (long long)rq.run * c.J;
+    if (partials != nullptr) partials = reinterpret_cast<char*>(partials) + 16ll * rq.part_off;
+  } else {
+    sx = blockIdx.x;
+    sy = blockIdx.y;
+    j = blockIdx.z;
+  }
   if (act != nullptr && act[j].active == 0) return;
   const int t = threadIdx.x;
   const JCoef<T> q = jcoef<T>(c, j);
@@ -892,12 +981,12 @@ inline PipeGeom geom(const OpCoef& c, int S, int Ly, int NT) {
   return g;
 }
 
-template <typename T, int M, bool WITH_A, int PF, int NT, class LD, class EP, bool JAC>
+template <typename T, int M, bool WITH_A, int PF, int NT, class LD, class EP, class TAB, bool JAC>
 void set_smem_attr() {
   using SH = PipeShape<T, M, WITH_A, PF, NT, LD, EP>;
   static bool done = false;
   if (!done) {
-    cudaFuncSetAttribute(k_pipe2d<T, M, WITH_A, PF, NT, LD, EP, JAC>,
+    cudaFuncSetAttribute(k_pipe2d<T, M, WITH_A, PF, NT, LD, EP, TAB, JAC>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::smem);
     done = true;
   }
@@ -905,7 +994,7 @@ void set_smem_attr() {
 
 template <typename T, int M, bool WITH_A, int PF, int NT, class LD, class EP, bool JAC = false>
 bool launch_pipe(const OpCoef& c, const ChebStep* w, int Ly, LD ld, EP ep, const KScal* act, void* partials,
-                 cudaStream_t s, int kid, int fields) {
+                 cudaStream_t s, int kid, int fields, const BatchLaunch* bl) {
   using SH = PipeShape<T, M, WITH_A, PF, NT, LD, EP>;
   const PipeGeom g = geom(c, SH::S, Ly, NT);
   constexpr size_t sm = SH::smem;
@@ -916,10 +1005,47 @@ bool launch_pipe(const OpCoef& c, const ChebStep* w, int Ly, LD ld, EP ep, const
       ca.c1[k][i] = k < M ? w[k].c1[i] : 0.0;
       ca.c2[k][i] = k < M ? w[k].c2[i] : 0.0;
     }
-  set_smem_attr<T, M, WITH_A, PF, NT, LD, EP, JAC>();
-  k_pipe2d<T, M, WITH_A, PF, NT, LD, EP, JAC>
-      <<<dim3(g.nstrips, g.nsegs, c.J), NT, sm, s>>>(c, ca, g, ld, ep, act, partials, kid, fields);
-  return true;
+  if (bl == nullptr) {
+    set_smem_attr<T, M, WITH_A, PF, NT, LD, EP, NoTab, JAC>();
+    k_pipe2d<T, M, WITH_A, PF, NT, LD, EP, NoTab, JAC>
+        <<<dim3(g.nstrips, g.nsegs, c.J), NT, sm, s>>>(c, ca, g, ld, ep, act, partials, kid, fields, NoTab{});
+    return true;
+  }
+  if constexpr (sizeof(T) == 8 || JAC) {
+    return false;  // batched runs are FP32 and take the explicit step
+  } else {
+    set_smem_attr<T, M, WITH_A, PF, NT, LD, EP, RunTab, false>();
+    // one launch per kTabRuns runs; the table holds this launch's geometry of each run
+    for (int r0 = 0; r0 < bl->R; r0 += kTabRuns) {
+      const int nr = std::min(kTabRuns, bl->R - r0);
+      RunTab tab;
+      std::memset(&tab, 0, sizeof(tab));
+      int maxblk = 0;
+      for (int i = 0; i < nr; ++i) {
+        const RunGeom& q = bl->host[r0 + i];
+        OpCoef cr = c;
+        cr.nx = q.nx;
+        cr.ny = q.ny;
+        const PipeGeom gr = geom(cr, SH::S, Ly, NT);
+        RunRec& e = tab.run[i];
+        e.pts = q.pts;
+        e.elem_off = q.elem_off;
+        e.part_off = bl->tlay ? q.part_off_t : q.part_off;
+        e.nx = q.nx;
+        e.ny = q.ny;
+        e.Ly = gr.Ly;
+        e.nstrips = gr.nstrips;
+        e.nsegs = gr.nsegs;
+        e.nblk = gr.npart * c.J;
+        e.run = r0 + i;
+        if (WITH_A && gr.npart != (bl->tlay ? q.npart_t : q.npart)) return false;  // layout must match the table
+        maxblk = std::max(maxblk, e.nblk);
+      }
+      k_pipe2d<T, M, WITH_A, PF, NT, LD, EP, RunTab, false>
+          <<<dim3(maxblk, nr), NT, sm, s>>>(c, ca, g, ld, ep, act, partials, kid, fields, tab);
+    }
+    return true;
+  }
 }
 
 // Tile variants of the FP32 pipeline with one Chebyshev application (the default
@@ -940,12 +1066,12 @@ inline int tile_nt(int elem_bytes, int m, int tile) {
 // complex field of precision T) reported to the measurement counters.
 template <typename T, bool WITH_A, class LD, class EP>
 bool dispatch(int m, int tile, const OpCoef& c, const ChebStep* w, int Ly, LD ld, EP ep, const KScal* act,
-              void* partials, cudaStream_t s, int kid, int fields) {
+              void* partials, cudaStream_t s, int kid, int fields, const BatchLaunch* bl = nullptr) {
   if constexpr (WITH_A) {
     if (c.jd != nullptr) {  // Picard iteration with the Jacobian: one Chebyshev application only
-      if (m != 1) return false;
+      if (m != 1 || bl != nullptr) return false;
       if constexpr (sizeof(T) == 8) {
-        return launch_pipe<T, 1, true, 0, 256, LD, EP, true>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
+        return launch_pipe<T, 1, true, 0, 256, LD, EP, true>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
       } else {
         if (c.jd32 == nullptr) return false;
         EpJ<EP, T> ej{};
@@ -953,39 +1079,39 @@ bool dispatch(int m, int tile, const OpCoef& c, const ChebStep* w, int Ly, LD ld
         ej.jd32 = c.jd32;
         using EJ = EpJ<EP, T>;
         switch (tile) {
-          case 1: return launch_pipe<T, 1, true, 1, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
-          case 2: return launch_pipe<T, 1, true, 1, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
-          case 3: return launch_pipe<T, 1, true, 2, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
-          case 4: return launch_pipe<T, 1, true, 3, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
-          case 5: return launch_pipe<T, 1, true, 3, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
-          default: return launch_pipe<T, 1, true, 2, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields);
+          case 1: return launch_pipe<T, 1, true, 1, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
+          case 2: return launch_pipe<T, 1, true, 1, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
+          case 3: return launch_pipe<T, 1, true, 2, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
+          case 4: return launch_pipe<T, 1, true, 3, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
+          case 5: return launch_pipe<T, 1, true, 3, 256, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
+          default: return launch_pipe<T, 1, true, 2, 128, LD, EJ, true>(c, w, Ly, ld, ej, act, partials, s, kid, fields, bl);
         }
       }
     }
   }
   if constexpr (sizeof(T) == 8) {
     switch (m) {
-      case 1: return launch_pipe<T, 1, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-      case 2: return launch_pipe<T, 2, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-      case 3: return launch_pipe<T, 3, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-      case 4: return launch_pipe<T, 4, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
+      case 1: return launch_pipe<T, 1, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+      case 2: return launch_pipe<T, 2, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+      case 3: return launch_pipe<T, 3, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+      case 4: return launch_pipe<T, 4, WITH_A, 0, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
       default: return false;
     }
   } else {
     if (m == 1) {
       switch (tile) {
-        case 1: return launch_pipe<T, 1, WITH_A, 1, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-        case 2: return launch_pipe<T, 1, WITH_A, 1, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-        case 3: return launch_pipe<T, 1, WITH_A, 2, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-        case 4: return launch_pipe<T, 1, WITH_A, 3, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-        case 5: return launch_pipe<T, 1, WITH_A, 3, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-        default: return launch_pipe<T, 1, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
+        case 1: return launch_pipe<T, 1, WITH_A, 1, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+        case 2: return launch_pipe<T, 1, WITH_A, 1, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+        case 3: return launch_pipe<T, 1, WITH_A, 2, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+        case 4: return launch_pipe<T, 1, WITH_A, 3, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+        case 5: return launch_pipe<T, 1, WITH_A, 3, 256>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+        default: return launch_pipe<T, 1, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
       }
     }
     switch (m) {
-      case 2: return launch_pipe<T, 2, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-      case 3: return launch_pipe<T, 3, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
-      case 4: return launch_pipe<T, 4, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields);
+      case 2: return launch_pipe<T, 2, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+      case 3: return launch_pipe<T, 3, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
+      case 4: return launch_pipe<T, 4, WITH_A, 2, 128>(c, w, Ly, ld, ep, act, partials, s, kid, fields, bl);
       default: return false;
     }
   }

@@ -7,16 +7,18 @@ namespace apfc {
 
 template <typename T>
 bool launch_fused_merged_t(int m, int Ly, int tile, const OpCoef& c, const ChebStep* w, const cplx<T>* r, const cplx<T>* v,
-                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s) {
+                           cplx<T>* t_out, const cplx<T>* rhat, const KScal* act, void* partials, cudaStream_t s,
+                           const BatchLaunch* bl) {
   LoadS<T> ld{r, v, c.pts};
   EpT5<T> ep{t_out, r, v, rhat, c.pts};
   // reads r, v, rhat; writes t
-  return dispatch<T, true>(m, tile, c, w, Ly, ld, ep, act, partials, s, kid_of<T>(KID_FUSED_APINV_T), 8);
+  return dispatch<T, true>(m, tile, c, w, Ly, ld, ep, act, partials, s, kid_of<T>(KID_FUSED_APINV_T), 8, bl);
 }
 
-#define APFC_FUSED_T_INST(T)                                                                                            \
+#define APFC_FUSED_T_INST(T)                                                                                       \
   template bool launch_fused_merged_t<T>(int, int, int, const OpCoef&, const ChebStep*, const cplx<T>*, const cplx<T>*, \
-                                         cplx<T>*, const cplx<T>*, const KScal*, void*, cudaStream_t);
+                                         cplx<T>*, const cplx<T>*, const KScal*, void*, cudaStream_t,             \
+                                         const BatchLaunch*);
 
 APFC_FUSED_T_INST(double)
 APFC_FUSED_T_INST(float)

@@ -521,6 +521,81 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
   }
 }
 
+// FP64-accurate outer residual of a batch's 2D grids (blockIdx.z), r = b - A x with x, b FP64 in memory,
+// evaluated without the FP64 pipe: every input double is split into an FP32 pair
+// (h, l) by integer operations and each component of r1 = b1 - zeta + G_h eta and
+// r2 = b2 - kt G_h zeta - a eta is one compensated sum of products (dfloat.cuh);
+// residuals to about 1e-14 of the terms' size, beneath the 1e-10 and 1e-13
+// tolerances of the refinement.  Writes r as FP32 (the inner solve's right-hand
+// side) and, if r64 != nullptr, as FP64 (kept as the previous residual of the
+// next step).  32 x 8 point tiles whose (zeta, eta) values and one-point halo are
+// split once into shared memory.  The partial ||r||^2 per amplitude is
+// accumulated from the FP32-rounded residual (it only decides convergence,
+// where a relative error of 1e-5 in the norm is immaterial); ||b||^2 is not
+// recomputed: b is fixed within a step.
+constexpr int kRTX = 32, kRTY = 8;
+__global__ void __launch_bounds__(256, 3) k_residual_refine2d(const double2* __restrict__ b,
+                                                           const double2* __restrict__ x, float2* __restrict__ r32,
+                                                           double2* __restrict__ r64, double2* __restrict__ partials,
+                                                           const __grid_constant__ OpCoef c, const RunGeom* rg) {
+  const int j = blockIdx.y;
+  const RunGeom& g = rg[blockIdx.z];
+  const int nx = g.nx, ny = g.ny;
+  const long long pts = g.pts;
+  b += g.elem_off;
+  x += g.elem_off;
+  r32 += g.elem_off;
+  if (r64 != nullptr) r64 += g.elem_off;
+  partials += (long long)blockIdx.z * c.J * kDotSlots * kDotBlocks;
+  if (c.prof != nullptr && blockIdx.x == 0 && threadIdx.x == 0)
+    atomicAdd(c.prof + KID_RESID_REFINE, (unsigned long long)pts * (4 * sizeof(double2) + 2 * sizeof(float2) +
+                                                                   (r64 ? 2 * sizeof(double2) : 0)));
+  __shared__ float4 sz[kRTY + 2][kRTX + 2], se[kRTY + 2][kRTX + 2];
+  const long long o = 2LL * j * pts;
+  const double2* z = x + o;
+  const double2* e = z + pts;
+  const ResidCoef<2> q = resid_coef<2>(c, j);
+  const LaneC ma = lane_c(c.a[j], -1.f, -1.f);
+  const int tx_count = (nx + kRTX - 1) / kRTX, ntiles = tx_count * ((ny + kRTY - 1) / kRTY);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  float rr = 0.f;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int tyi = tile / tx_count;
+    const int x0 = (tile - tyi * tx_count) * kRTX, y0 = tyi * kRTY;
+    __syncthreads();  // the previous tile's shared values are no longer read
+    for (int i = threadIdx.x; i < (kRTX + 2) * (kRTY + 2); i += 256) {
+      const int ry = i / (kRTX + 2), rx = i - ry * (kRTX + 2);
+      int gxx = x0 - 1 + rx, gyy = y0 - 1 + ry;
+      gxx = gxx < 0 ? gxx + nx : (gxx >= nx ? gxx % nx : gxx);
+      gyy = gyy < 0 ? gyy + ny : (gyy >= ny ? gyy % ny : gyy);
+      const long long q = (long long)gyy * nx + gxx;
+      sz[ry][rx] = pdf_pack(pdf_split(z[q]));
+      se[ry][rx] = pdf_pack(pdf_split(e[q]));
+    }
+    __syncthreads();
+    const int xx = x0 + tx, yy = y0 + ty;
+    if (xx >= nx || yy >= ny) continue;
+    const long long pc = (long long)yy * nx + xx;
+    const PDF zn[2][2] = {{pdf_unpack(sz[ty + 1][tx]), pdf_unpack(sz[ty + 1][tx + 2])},
+                          {pdf_unpack(sz[ty][tx + 1]), pdf_unpack(sz[ty + 2][tx + 1])}};
+    const PDF en[2][2] = {{pdf_unpack(se[ty + 1][tx]), pdf_unpack(se[ty + 1][tx + 2])},
+                          {pdf_unpack(se[ty][tx + 1]), pdf_unpack(se[ty + 2][tx + 1])}};
+    float2 f1, l1, f2, l2;
+    resid_point<2>(q, ma, pdf_split(b[o + pc]), pdf_split(b[o + pts + pc]), pdf_unpack(sz[ty + 1][tx + 1]),
+                   pdf_unpack(se[ty + 1][tx + 1]), zn, en, f1, l1, f2, l2);
+    r32[o + pc] = f1;
+    r32[o + pts + pc] = f2;
+    if (r64 != nullptr) {
+      r64[o + pc] = make_double2(df_to_d(DF{f1.x, l1.x}), df_to_d(DF{f1.y, l1.y}));
+      r64[o + pts + pc] = make_double2(df_to_d(DF{f2.x, l2.x}), df_to_d(DF{f2.y, l2.y}));
+    }
+    rr = fmaf(f1.x, f1.x, fmaf(f1.y, f1.y, fmaf(f2.x, f2.x, fmaf(f2.y, f2.y, rr))));
+  }
+  double acc[1] = {(double)rr};
+  block_sum<1>(acc);
+  if (threadIdx.x == 0) partials[(j * kDotSlots + 0) * kDotBlocks + blockIdx.x] = make_double2(acc[0], 0.0);
+}
+
 // New right-hand side plus the initial outer residual of the step without a
 // stencil: with the previous step's final residual r_prev = b_prev - A x0,
 // r0 = b - A x0 = b - b_prev + r_prev (exact algebra, pointwise).  Writes b
@@ -1395,6 +1470,12 @@ void launch_zeta(double2* x, const OpCoef& c, cudaStream_t s) {
     k_zeta<32><<<tall, 256, 0, s>>>(x, c);
   else
     k_zeta<8><<<flat, 256, 0, s>>>(x, c);
+}
+void launch_residual_refine2d(const double2* b, const double2* x, float2* r32, double2* r64, double* partials,
+                              const OpCoef& c, cudaStream_t s, const BatchLaunch& bl) {
+  ProfScope ps_(KID_RESID_REFINE, s);
+  k_residual_refine2d<<<dim3(kDotBlocks, c.J, bl.R), 256, 0, s>>>(b, x, r32, r64, reinterpret_cast<double2*>(partials), c,
+                                                                  bl.dev);
 }
 void launch_rhs_resid(const double2* x, double2* b, const double2* b_prev, const double2* r_prev, float2* r32,
                       double* partials, const OpCoef& c, const NonlinTable& nt, bool schur, cudaStream_t s,

@@ -11,7 +11,8 @@
 // products instead of 1 + 4 DIM; the pair sum's error, about 2^-47 of the
 // neighbours' magnitude, stays below what the compensated sum keeps anyway.
 //
-// Evaluated by the residual of the block system (resid2d.cu, TMA tiles); the Schur
+// Evaluated by the residuals of the block system, of one grid (resid2d.cu, TMA tiles) and of a
+// batch's (kernels.cu, plain loads), so that a run alone and in a batch round alike; the Schur
 // complement's residuals (schur.cu, schur3d.cu) take its pair sums and coefficients.
 #pragma once
 

@@ -211,3 +211,71 @@ def test_full_size_batch_64_runs_autotuned():
     print(f"batch 64 runs: smallest run ({picks[0][0]}^2) rel L2 per amplitude vs oracle {errs}, "
           f"resid {b_resid}")
     assert max(errs) <= 1e-10
+
+
+# --- BiCGStab, where the Chebyshev iteration does not serve (test_gpu_bicgstab.py) ---------------
+
+FINE = (0.5, 0.5)
+
+
+def _fine(shapes, opts, dts, graph=True):
+    """Amplitudes and statistics of every run after each step: of a batch, and of the runs alone."""
+    L = O.hex_lattice()
+    states = [inputs.random_amplitudes(3, s, seed=120 + r, scale=0.1) for r, s in enumerate(shapes)]
+    got, ref = [], []
+    with A.Batch(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), shapes, FINE, opts, graph=graph) as b:
+        for r, e in enumerate(states):
+            b.set_amplitudes(r, e)
+        for dt in dts:
+            b.step(dt)
+            got.append([(b.get_amplitudes(r), b.stats(r)) for r in range(len(shapes))])
+        replays = b.graph_replays()
+        b.profile_start("fused_apinv_t_f32")
+        b.step(dts[-1])
+        launches = b.profile_read("fused_apinv_t_f32")["launches"]
+        b.profile_stop()
+    for s, e in zip(shapes, states):
+        with A.Context(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), s, FINE, opts) as c:
+            c.set_amplitudes(e)
+            ref.append([])
+            for dt in dts:
+                c.step(dt)
+                ref[-1].append((c.get_amplitudes(), c.stats()))
+    for r in range(len(shapes)):
+        for n in range(len(dts)):
+            assert np.array_equal(got[n][r][0], ref[r][n][0]), (shapes[r], n)
+            for key in ("iters_last", "refine_last"):
+                assert got[n][r][1][key] == ref[r][n][1][key]
+    return replays, launches
+
+
+@pytest.mark.parametrize("graph", [True, False])
+@pytest.mark.parametrize("m,tile,rows,tile_t", [(1, 3, 0, 1), (1, 0, 64, -1), (1, 5, 128, 0), (3, 0, 128, -1)])
+def test_bicgstab_of_a_batch_equals_the_runs_alone(m, tile, rows, tile_t, graph):
+    # tol 5e-13 < 9e-16 cond(S): one launch of each kernel over all runs, not the runs one by one
+    shapes = [(40, 48), (33, 131), (64, 64), (130, 250)]
+    opts = _opts(tol=5e-13, cheb_degree=m, tile=tile, tile_rows=rows or 128, tile_t=tile_t, check_every=3)
+    replays, launches = _fine(shapes, opts, [1.0, 1.0], graph)
+    assert (replays > 0) == graph and launches > 0
+
+
+def test_batch_that_changes_between_the_two_solvers():
+    # cond(S) is 640 at dt = 0.5 and 2400 at dt = 2: 1e-12 is above its noise at the first alone
+    shapes = [(40, 48), (33, 131)]
+    _, launches = _fine(shapes, _opts(tol=1e-12), [0.5, 2.0, 2.0, 0.5, 0.5, 2.0])
+    assert launches > 0
+
+
+def test_autotune_of_a_batch_on_bicgstab():
+    shapes = [(40, 48), (33, 131)]
+    L = O.hex_lattice()
+    with A.Batch(L.k, A.APFC_LATTICE_HEX2D, (P.dB, P.Bx, P.t, P.v), shapes, FINE, _opts(tol=5e-13)) as b:
+        for r, s in enumerate(shapes):
+            b.set_amplitudes(r, inputs.random_amplitudes(3, s, seed=130 + r, scale=0.1))
+        before = [b.get_amplitudes(r) for r in range(2)]
+        assert b.autotune(1.0)["ms_per_iter"] > 0
+        assert all(np.array_equal(b.get_amplitudes(r), before[r]) for r in range(2))
+        b.step(1.0)
+        for r, s in enumerate(shapes):
+            ref, _ = O.step(before[r], 1.0, P, L, FINE)
+            assert rel_l2(b.get_amplitudes(r), ref) <= 2e-9
