@@ -72,13 +72,16 @@ enum { APFC_C128 = 0, APFC_C64 = 1 };
  * n = sum_j (eta_j e^{i k_j.r} + c.c.) (Eq. density). */
 enum { APFC_LATTICE_CUSTOM = 0, APFC_LATTICE_HEX2D = 1, APFC_LATTICE_BCC3D = 2 };
 
-enum { APFC_FP64 = 0,         /* fields, Krylov iterates and reductions in FP64 */
-       APFC_FP32_REFINED = 1  /* FP32 Krylov inside FP64 iterative refinement   */ };
-/* The only value.  Systems with constant coefficients on 2D grids (no Jacobian, fused 1,
- * cheb_degree 1..4) are solved to the same tolerance by a Chebyshev iteration on the Schur
- * complement of the block system, a_j + kap_j Bx G_h^2 (preconditioned by Eq. preconditioner's
- * second factor squared where that pays, on fine grids); the others by BiCGStab, as is a system
- * whose Chebyshev iteration could need more operator applications than max_iter allows. */
+enum { APFC_FP64 = 0,         /* fields, solver iterates and reductions in FP64 */
+       APFC_FP32_REFINED = 1  /* FP32 solves inside FP64 iterative refinement   */ };
+/* The only value.  With fused 1 and cheb_degree 1..4, systems on 2D and 3D grids are solved to the
+ * same tolerance by a Chebyshev iteration on the Schur complement of the block system,
+ * a_j + kap_j Bx G_h^2 (2D grids: preconditioned by Eq. preconditioner's second factor squared
+ * where that pays, on fine grids, and with the Jacobian's diagonal added where that keeps it well
+ * conditioned).  BiCGStab on the block system solves the others: 3D grids too fine for it, 3D
+ * grids with the Jacobian, tolerances below about 9e-16 times the complement's condition
+ * number (the noise of its residual), and systems whose Chebyshev iteration could need more
+ * operator applications than max_iter allows. */
 enum { APFC_BICGSTAB = 0 };
 enum { APFC_TAU_FOLD = 0,     /* preconditioner uses 1/tau = 1/dt + kap dB      */
        APFC_TAU_PLAIN = 1     /* preconditioner uses tau = dt                    */ };
@@ -391,19 +394,21 @@ apfc_status apfc_rotation_field(apfc_ctx* ctx, void* omega, void* amp, void* hma
  * together by the step of apfc_step (Alg. 1 with one nonlinear iterate; Chebyshev
  * solves of the Schur complement) in precision APFC_FP32_REFINED with the fused
  * pipeline.  Every stage of the step is one launch over the work of
- * all runs; each (run, amplitude) takes its own number of iterations, and a run whose refinement has converged waits unchanged for the
- * others.  Run r follows the same arithmetic as run r alone on an apfc_ctx
+ * all runs; each (run, amplitude) takes its own number of iterations, and a run whose
+ * refinement has converged waits unchanged for the others.  Run r follows the same arithmetic as run r alone on an apfc_ctx
  * with the same options (its solves do not depend on the split into tiles, and its
  * norms are reduced in the same order).
  *
  * Storage: the batch owns the concatenated block vectors of all runs (FP64
  * state, right-hand sides and residuals; FP32 solver fields), about
- * J sum_r(nx ny) x (7 x 16 + 5 x 8) bytes.  Amplitude buffers of run r are
+ * J sum_r(nx ny) x (7 x 16 + 5 x 8) bytes; the first step that BiCGStab takes (see
+ * APFC_BICGSTAB) adds about 2 J sum_r(nx ny) x (16 + 10 x 8 + 4).  Amplitude buffers of run r are
  * [J][ny[r]][nx[r]] complex128, owned by the caller, copied in or out.
  *
- * flags: APFC_BATCH_GRAPH replays the passes of a solve from captured CUDA
- * graphs (one per number of passes); the first solve runs uncaptured.  With that flag a NULL stream makes the batch create and own
- * a non-blocking stream (graphs cannot be captured on the legacy stream).
+ * flags: APFC_BATCH_GRAPH replays the passes of a solve (BiCGStab: check_every
+ * iterations) from captured CUDA graphs; the first solve (block of iterations) runs
+ * uncaptured.  With that flag a NULL stream makes the batch create and own a
+ * non-blocking stream (graphs cannot be captured on the legacy stream).
  * Errors are sticky as on a context; ENAN / ENOCONV name the failing run in
  * apfc_batch_last_error(). */
 typedef struct apfc_batch apfc_batch;
@@ -438,7 +443,8 @@ apfc_status apfc_batch_stats(const apfc_batch* b, int run, apfc_stats_t* out);
  * passes over all runs for the narrow and the wide strips (tile 3 and 5) and every
  * segment height (32, 48, 64, 96, 128, 192, 256 rows); keep the fastest in the
  * batch's options (tile, tile_rows; see apfc_batch_get_opts) and return tile, rows
- * and ms per pass (null pointers skipped). */
+ * and ms per pass (null pointers skipped).  Where BiCGStab solves: its iterations, for
+ * every tile variant and height, then every variant of the t-kernel (tile_t). */
 apfc_status apfc_batch_autotune(apfc_batch* b, double dt, int* tile, int* tile_rows, double* ms_per_iter);
 
 /* Number of captured-graph replays since creation (-1 for a null batch). */

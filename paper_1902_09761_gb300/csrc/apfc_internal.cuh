@@ -260,7 +260,6 @@ struct GaugeTab {
 inline double gauge_w(const OpCoef& c, int j, int d) {
   return std::sqrt(c.ih2[d] * c.ih2[d] + c.kh[j][d] * c.kh[j][d]);
 }
-inline double gauge_phi(const OpCoef& c, int j, int d) { return std::atan2(c.kh[j][d], c.ih2[d]); }
 
 // Fields [J][pts] of such a solve: r0 the initial residual, r and d ping-pong pairs (r0 may be
 // r[0]), u the sum of the d; x64 the state block that receives u; ks[j].iters the passes of

@@ -7,7 +7,7 @@
 // approximant of D^{-1} (f = beta2 - kt G_h beta1 obeys f(A P^{-1} beta) = S p(D)^2 f(beta)).
 // All operators are constant-coefficient periodic stencils: they commute, S p(D)^2 is Hermitian
 // positive definite, and its spectrum is known from the stencils' symbols (schur_spectrum in
-// api.cu).  So the solve needs no inner products: the Chebyshev semi-iteration (Saad, Alg. 12.1)
+// schur.cu).  So the solve needs no inner products: the Chebyshev semi-iteration (Saad, Alg. 12.1)
 //   d_0 = p^2 r_0 / theta,  u = d_0;   r -= S d,  d = c1 d + c2 p^2 r,  u += d
 // reaches a given reduction in a number of applications known beforehand.
 //

@@ -11,8 +11,9 @@
 //
 // Without the preconditioner p(D)^2 an application of S costs two stencil stages instead of 2 + 2M.
 // At the spacings amplitudes need (about h <= pi/2: few points per atom) S is hardly worse
-// conditioned than S p(D)^2 (20.5 against 15.6 at h = pi/2, dt = 1), so the plain iteration needs
-// fewer stages; solve_plan (api.cu) compares the two and takes cheb2d.cuh's on finer grids.
+// conditioned than S p(D)^2 (16.5 against 15.4 at h = pi/2, dt = 1, degree 1), so the plain
+// iteration needs fewer stages; schur_build (schur.cu) compares the two and takes cheb2d.cuh's on
+// finer grids.
 //
 // k_gauge2d makes NI terms of the iteration (Saad, Alg. 12.1, in the two-vector form
 // v_(n+1) = v_n + c1 (v_n - v_(n-1)) + c2 (b - S v_n)) in one pass: stages

@@ -460,7 +460,7 @@ __global__ void k_rhs(const double2* __restrict__ x, double2* __restrict__ b, co
 // A block forms 32 x ROWS points: a double is split once for all its readers, and a thread's
 // coefficients (as many splits) serve ROWS / 8 points.  us at 1024^2 x 3 / 4096^2 x 3: a thread
 // per point reading its neighbours 58 / 811, 8 rows 58 / 803, 32 rows 46 / 636; 8 where 32 give
-// fewer than two blocks per SM (128^2 x 3: 8.4 against 11.7).
+// fewer than two blocks on each of 152 SMs (128^2 x 3: 8.4 against 11.7).
 template <int ROWS>
 __global__ void __launch_bounds__(256) k_zeta(double2* __restrict__ x, const __grid_constant__ OpCoef c) {
   prof_add3(c, KID_ZETA, 2ull * (unsigned long long)c.pts * sizeof(double2));

@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kR3NT, kR3B)
 
 int resid3_planes(int nx, int ny, int nz, int J) {
   const long long tiles = (long long)((nx + kR3X - 1) / kR3X) * ((ny + kR3Y - 1) / kR3Y) * J;
-  const long long rows = nz * tiles / 608;  // about two rounds of two blocks per SM
+  const long long rows = nz * tiles / 608;  // about four rounds of one block on each of 152 SMs
   return (int)std::min<long long>(nz, std::min<long long>(64, std::max<long long>(8, rows)));
 }
 
